@@ -26,6 +26,14 @@ wost_status cuda_fail(cudaError_t e, const char *what);
         if (_e != cudaSuccess) return wost::cuda_fail(_e, what); \
     } while (0)
 
+// A solve of at most this many walks runs them one per warp from the start,
+// and a larger one hands its last walks over when so many are left: that is
+// where the two forms run equally many steps per second (Koch workload: 4,864
+// walks one per warp 2.4e8 steps/s; 12,288 of them left over in 4,864 warps of
+// one-lane walks ~2e8, each step of such a warp taking 60 us).
+constexpr uint64_t kWarpWalks = 12288;
+constexpr unsigned kTailWalks = 12288;
+
 // device allocation owned by a scene or solve
 struct DevBuf {
     void *p = nullptr;
@@ -112,6 +120,7 @@ struct wost_solve_handle {
     int32_t walks = 0;
     int block = 128;
     int lanes = 1;                        // lanes per walk (persistent / resumable kernels)
+    bool warp_ok = false;                 // the scene's own traversal limits: walks may run one per warp
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     cudaStream_t poll_stream = nullptr;

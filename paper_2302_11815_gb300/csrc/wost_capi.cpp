@@ -338,6 +338,7 @@ wost_status wost::prepare_solve(wost_scene *scene, const wost_solve_desc *d, cud
     sp.vis_tmax = 1.f - 1e-4f;
     sp.stack_depth = d->stack_depth ? d->stack_depth : (lanes == 1 ? scene->stack_depth : scene->stack_depth_team);
     sp.visit_limit = (uint32_t)d->visit_limit;
+    h->warp_ok = !d->stack_depth && !d->visit_limit;
     sp.sigma = d->sigma;
     sp.sqrt_sigma = std::sqrt(d->sigma);
     sp.screen_after = d->screen_after;
@@ -390,7 +391,10 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
             CK(resume_grid(h->dim, h->block, h->sp.stack_depth, &h->resume_blocks, h->lanes), "occupancy");
             CK(h->slots.alloc((size_t)resume_slots(h->block, h->resume_blocks, h->lanes) * 3 * sizeof(float4)),
                "cudaMalloc slots");
-            CK(h->rstate.alloc(16), "cudaMalloc counters");
+            // counters (steps_run u64; live u32; the tail's work counter u32),
+            // then the list of the saved walks' slots
+            const size_t n_slots = (size_t)resume_slots(h->block, h->resume_blocks, h->lanes);
+            CK(h->rstate.alloc(16 + n_slots * sizeof(uint32_t)), "cudaMalloc counters");
             CK(cudaMemsetAsync(h->slots.p, 0, h->slots.bytes, stream), "memset");
             CK(cudaMemsetAsync(h->rstate.p, 0, 16, stream), "memset");
             if ((st = wait_for_copies(stream)) != WOST_OK) return st;
@@ -403,7 +407,13 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
         h->t_launch = std::chrono::steady_clock::now();
         CK(cudaEventRecord(h->ev_start, stream), "cudaEventRecord");
         cudaError_t le;
-        if (d->kernel == WOST_KERNEL_PLAIN) {
+        // one lane per walk under the scene's own traversal limits: the walks
+        // (few of them) or the last walks (of many) run one per warp
+        const uint64_t total = (uint64_t)d->n_points * (uint64_t)d->walks_per_point;
+        const bool warp_ok = h->lanes == 1 && h->warp_ok;
+        if (warp_ok && total <= kWarpWalks && d->kernel != WOST_KERNEL_COUNTING) {
+            le = launch_walk_warp(scene->view, sp, acc, TailWalks{}, total, stream);
+        } else if (d->kernel == WOST_KERNEL_PLAIN) {
             le = launch_walk_plain(scene->view, sp, acc, h->block, stream);
         } else if (d->kernel == WOST_KERNEL_COUNTING) {
             le = h->counts.alloc(10 * 8);
@@ -413,7 +423,17 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
         } else {
             int blocks = 0;
             le = persistent_grid(h->dim, h->block, sp.stack_depth, &blocks, h->lanes);
-            if (le == cudaSuccess) le = launch_walk_persistent(scene->view, sp, acc, h->block, blocks, stream, h->lanes);
+            HandOver ho{};
+            TailWalks tw{};
+            if (le == cudaSuccess && warp_ok) {
+                le = h->slots.alloc((size_t)kTailWalks * 3 * sizeof(float4));
+                unsigned int *ctr = (unsigned int *)((unsigned long long *)h->globals.p + 3);
+                ho = HandOver{(float4 *)h->slots.p, ctr, kTailWalks, 0};
+                tw = TailWalks{(float4 *)h->slots.p, nullptr, ctr, ctr + 1, nullptr};
+            }
+            if (le == cudaSuccess)
+                le = launch_walk_persistent(scene->view, sp, acc, h->block, blocks, stream, h->lanes, ho);
+            if (le == cudaSuccess && warp_ok) le = launch_walk_warp(scene->view, sp, acc, tw, kTailWalks, stream);
         }
         if (le != cudaSuccess) return cuda_fail(le, "kernel launch");
         CK(cudaEventRecord(h->ev_done, stream), "cudaEventRecord");
@@ -542,14 +562,19 @@ wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_so
 // Resumable solve whose latest launch has completed: finished when that
 // launch saved no walk and no walk is left to draw (or the solve was
 // cancelled, which stops the drawing).
-static wost_status resumable_finished(wost_solve_handle *h, bool *finished) {
+// *drained: no walk is left to draw; *live: walks saved by the launch.
+static wost_status resumable_finished(wost_solve_handle *h, bool *finished, bool *drained = nullptr,
+                                      unsigned int *live = nullptr) {
     unsigned long long g[4] = {0, 0, 0, 0};
     unsigned int st[4] = {0, 0, 0, 0};
     CK(cudaMemcpyAsync(g, h->globals.p, sizeof g, cudaMemcpyDeviceToHost, h->poll_stream), "poll copy");
     CK(cudaMemcpyAsync(st, h->rstate.p, sizeof st, cudaMemcpyDeviceToHost, h->poll_stream), "poll copy");
     CK(cudaStreamSynchronize(h->poll_stream), "poll sync");
     const uint64_t total = (uint64_t)h->n_points * (uint64_t)h->walks;
-    *finished = st[2] == 0 && (g[1] >= total || *(volatile int *)h->cancel_host != 0);
+    const bool none_left = g[1] >= total || *(volatile int *)h->cancel_host != 0;
+    *finished = st[2] == 0 && none_left;
+    if (drained) *drained = none_left;
+    if (live) *live = st[2];
     return WOST_OK;
 }
 
@@ -652,12 +677,36 @@ static wost_status advance_locked(wost_solve_handle *h, int iters, cudaStream_t 
     }
     unsigned int *live = (unsigned int *)((char *)h->rstate.p + 8);
     CK(cudaMemsetAsync(live, 0, sizeof(unsigned int), s), "memset");
-    ResumeState rs{(float4 *)h->slots.p, (unsigned long long *)h->rstate.p, live};
+    ResumeState rs{(float4 *)h->slots.p, (unsigned long long *)h->rstate.p, live,
+                   h->lanes == 1 ? (uint32_t *)((char *)h->rstate.p + 16) : nullptr};
     CK(launch_walk_resume(h->scene->view, h->sp, h->acc, rs, iters, h->block, h->resume_blocks, s, h->lanes),
        "kernel launch");
     CK(cudaEventRecord(h->ev_done, s), "cudaEventRecord");
     h->launches++;
     return WOST_OK;
+}
+
+// The next launch of a resumable solve while its caller waits: bounded as
+// wost_solve_advance's, or, once the last walks are few, one walk per warp to
+// their ends (caller holds h->mu; the previous launch has completed).
+static wost_status advance_waiting(wost_solve_handle *h) {
+    const bool warp_ok = h->lanes == 1 && h->warp_ok;
+    if (warp_ok && h->launches > 0) {
+        bool fin = false, drained = false;
+        unsigned int live = 0;
+        wost_status st = resumable_finished(h, &fin, &drained, &live);
+        if (st != WOST_OK) return st;
+        if (drained && live > 0 && live <= kTailWalks) {
+            unsigned int *ctr = (unsigned int *)((char *)h->rstate.p + 8);
+            TailWalks tw{(float4 *)h->slots.p, ctr + 2, ctr, ctr + 1, (unsigned long long *)h->rstate.p};
+            CK(launch_walk_warp(h->scene->view, h->sp, h->acc, tw, live, h->stream), "kernel launch");
+            CK(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned int), h->stream), "memset");
+            CK(cudaEventRecord(h->ev_done, h->stream), "cudaEventRecord");
+            h->launches++;
+            return WOST_OK;
+        }
+    }
+    return advance_locked(h, 2048, h->stream);
 }
 
 wost_status wost_solve_advance(wost_solve_handle *h, int32_t iterations, void *stream) {
@@ -687,7 +736,7 @@ wost_status wost_wait(wost_solve_handle *h, double timeout_s) {
             // a resumable solve advances while its caller waits: the next
             // launch as soon as the previous one has completed
             if (h->resumable() && (h->launches == 0 || cudaEventQuery(h->ev_done) == cudaSuccess))
-                if ((st = advance_locked(h, 2048, h->stream)) != WOST_OK) return st;
+                if ((st = advance_waiting(h)) != WOST_OK) return st;
         }
         double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         if (timeout_s >= 0 && el >= timeout_s) return fail(WOST_ERR_TIMEOUT, "solve not finished");

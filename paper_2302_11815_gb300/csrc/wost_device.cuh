@@ -952,8 +952,8 @@ struct NSample {
     float s0, s1;  // interpolation weights of z on the primitive
 };
 
-template <int D, bool CN = false>
-__device__ NSample q_sample(const TreeView &T, P3 x, float r, Stream &rng, Cnt<CN> &cnt) {
+template <int D, bool CN = false, class RNG>
+__device__ NSample q_sample(const TreeView &T, P3 x, float r, RNG &rng, Cnt<CN> &cnt) {
     NSample out;
     out.rec = -1;
     out.pdf = 0.f;
@@ -1160,6 +1160,7 @@ __device__ __forceinline__ float maxabs3(P3 a) { return fmaxf(fabsf(a.x), fmaxf(
 // queries with its own shared-memory stack.
 template <int D, bool CN>
 struct LaneQ {
+    static constexpr bool kWarp = false;
     Stack st;
     Cnt<CN> &cnt;
     __device__ Closest closest(const TreeView &T, P3 x, float bound2) { return q_closest<D, CN>(T, x, st, cnt, bound2); }
@@ -1220,8 +1221,8 @@ __device__ __forceinline__ bool in_bounds(const SceneView &sc, P3 x) {
 // One iteration of Alg. 1 for the walk w of this lane (act = the lane holds
 // a walk).  Returns true when an active walk has terminated (its estimate is
 // then w.acc).  Q answers the geometric queries (LaneQ: one lane per walk;
-// GroupQ: 8 cooperating lanes per walk, every lane of the group running this
-// same code on the same walk).
+// GroupQ, WarpQ: 8 or all 32 lanes per walk, every lane of the group running
+// this same code on the same walk).
 //
 // Warp-synchronous: all 32 lanes of the warp call it together, and the warp
 // meets at a __syncwarp() after every query.  Without those meeting points
@@ -1240,6 +1241,7 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
     // R13: a walk outside the grown bounding box of the boundary has left the
     // domain through a rounding gap; it ends like a capped walk (R5)
     const bool lost = act && !in_bounds<D>(sc, w.x);
+    if constexpr (Q::kWarp) q.begin_step(sp, w, lost);  // the whole warp holds this walk
     // distance to the Dirichlet boundary (Q.1).  The closest point of the
     // previous step is at most dbound away (triangle inequality), which
     // prunes the search; the result is the exact closest point either way,
@@ -1301,7 +1303,11 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
     // direction: uniform, flipped into the hemisphere about -n_x on the boundary
     const uint32_t k = (uint32_t)(w.steps - 1);
     uint4 rb = make_uint4(0u, 0u, 0u, 0u);
-    if (act) rb = philox10(make_uint4(w.index, w.point, k, 0u), sp.key0, sp.key1);
+    if constexpr (Q::kWarp) {
+        rb = q.slot0();
+    } else {
+        if (act) rb = philox10(make_uint4(w.index, w.point, k, 0u), sp.key0, sp.key1);
+    }
     P3 v;
     if constexpr (D == 2) {
         float s, c;
@@ -1325,9 +1331,13 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
     zs.s0 = zs.s1 = 0.f;
     if (__any_sync(FULL, want4)) {
         if (want4) {
-            Stream rng;
-            rng.init(sp.key0, sp.key1, w.index, w.point, k);
-            zs = q.sample(sc.N, w.x, r, rng);
+            if constexpr (Q::kWarp) {
+                zs = q.sample(sc.N, w.x, r);
+            } else {
+                Stream rng;
+                rng.init(sp.key0, sp.key1, w.index, w.point, k);
+                zs = q.sample(sc.N, w.x, r, rng);
+            }
         }
         __syncwarp();
     }

@@ -131,6 +131,7 @@ __device__ __forceinline__ bool gpop(const GStack &gs, int &sp, uint32_t &ref, f
 
 template <int D, bool CN>
 struct GroupQ {
+    static constexpr bool kWarp = false;
     Group g;
     GStack gs;
     Cnt<CN> &cnt;

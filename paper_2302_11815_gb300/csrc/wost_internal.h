@@ -121,6 +121,28 @@ struct ResumeState {
     float4 *slots;
     unsigned long long *steps_run;  // [1] walk steps executed by all launches
     unsigned int *live;             // [1] walks saved by the latest launch (cleared before it)
+    uint32_t *list;                 // slots of those walks (one entry per slot; null with 8-lane teams)
+};
+
+// Where a one-lane kernel hands its last walks over (slots as in
+// ResumeState, filled from the front; null: it keeps them): once the solve's
+// counter is exhausted and at most `most` walks are left, every warp saves
+// the walks it holds and ends.
+struct HandOver {
+    float4 *slots;
+    unsigned int *count;  // [1] walks saved
+    unsigned int most;    // capacity of `slots`
+    unsigned int lanes;   // walks the launch can hold at once
+};
+
+// The saved walks a one-walk-per-warp kernel runs to their ends (slots null:
+// none saved, it draws the solve's own walks).
+struct TailWalks {
+    float4 *slots;
+    const uint32_t *list;           // their slots (null: slots 0, 1, ...)
+    const unsigned int *count;      // [1] how many
+    unsigned int *next;             // [1] work counter
+    unsigned long long *steps_run;  // [1] receives the steps run (may be null)
 };
 
 // Accumulators of one solve, for the per-solve summary kernel.

@@ -154,10 +154,12 @@ cudaError_t persistent_grid(int dim, int block, int depth, int *blocks_out, int 
 }
 
 cudaError_t launch_walk_persistent(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, int block,
-                                   int blocks, cudaStream_t s, int lanes) {
-    if (sp.sigma > 0.f) return launch_walk_persistent_scr(sc, sp, acc, block, blocks, s);
+                                   int blocks, cudaStream_t s, int lanes, const HandOver &ho) {
     if (lanes == WOST_WIDE) return launch_walk_persistent_team(sc, sp, acc, block, blocks, s);
-    return walk_persistent_launch<false, 1>(sc, sp, acc, block, blocks, s);
+    HandOver h = ho;
+    h.lanes = (unsigned)blocks * (unsigned)block;
+    if (sp.sigma > 0.f) return launch_walk_persistent_scr(sc, sp, acc, h, block, blocks, s);
+    return walk_persistent_launch<false, 1>(sc, sp, acc, h, block, blocks, s);
 }
 
 // the resumable kernels share the persistent ones' occupancy (same body)

@@ -22,7 +22,10 @@ cudaError_t launch_walk_batch(int dim, const BatchHeader *hdr, const BatchJob *j
 // lanes: lanes per walk, 1 (binary trees) or 8 (8-lane teams over the 8-wide
 // trees; Poisson solves)
 cudaError_t launch_walk_persistent(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, int block,
-                                   int blocks, cudaStream_t s, int lanes = 1);
+                                   int blocks, cudaStream_t s, int lanes = 1, const HandOver &ho = HandOver{});
+// one walk per warp: `walks` walks (an upper bound), saved ones or the solve's own
+cudaError_t launch_walk_warp(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, const TailWalks &tw,
+                             uint64_t walks, cudaStream_t s);
 // resumable solves: grid of the fixed launch, its walk slots, one launch
 cudaError_t resume_grid(int dim, int block, int depth, int *blocks_out, int lanes = 1);
 int64_t resume_slots(int block, int blocks, int lanes = 1);

@@ -102,6 +102,31 @@ __device__ __forceinline__ void accumulate(const Accumulators &acc, const Walk &
     if (w.capped) atomicAdd(acc.capped, 1ull);
 }
 
+// saved walks (layout: ResumeState)
+__device__ __forceinline__ bool load_walk(const float4 *slot, Walk &w) {
+    const float4 c = slot[2];
+    const uint32_t flags = __float_as_uint(c.w);
+    if (!(flags & 1u)) return false;
+    const float4 a = slot[0], b = slot[1];
+    w.x = mk(a.x, a.y, a.z);
+    w.acc = a.w;
+    w.n = mk(b.x, b.y, b.z);
+    w.dbound = b.w;
+    w.steps = (int)__float_as_uint(c.x);
+    w.point = __float_as_uint(c.y);
+    w.index = __float_as_uint(c.z);
+    w.onN = (flags & 2u) != 0;
+    w.capped = (flags & 4u) != 0;
+    return true;
+}
+__device__ __forceinline__ void save_walk(float4 *slot, const Walk &w) {
+    const uint32_t flags = 1u | (w.onN ? 2u : 0u) | (w.capped ? 4u : 0u);
+    slot[0] = make_float4(w.x.x, w.x.y, w.x.z, w.acc);
+    slot[1] = make_float4(w.n.x, w.n.y, w.n.z, w.dbound);
+    slot[2] = make_float4(__uint_as_float((uint32_t)w.steps), __uint_as_float(w.point), __uint_as_float(w.index),
+                          __uint_as_float(flags));
+}
+
 template <int D, bool SCR>
 __global__ void WOST_WALK_BOUNDS k_walk_plain(const SceneView sc, const SolveParams sp, const Accumulators acc,
                                                     int warp_uniform_points) {
@@ -153,7 +178,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_plain(const SceneView sc, const SolvePar
 
 template <int D, bool SCR, int T>
 __global__ void WOST_WALK_BOUNDS k_walk_persistent(const SceneView sc, const SolveParams sp,
-                                                         const Accumulators acc) {
+                                                         const Accumulators acc, const HandOver ho) {
     Cnt<false> cnt;
     auto q = make_q<D, false, T>(sp.stack_depth, acc.guard, cnt, sp.visit_limit);
     const Group g = make_team<T>();
@@ -192,7 +217,26 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const SceneView sc, const Sol
                 }
             }
         }
-        if (!__any_sync(FULL, have)) break;
+        const unsigned held = __ballot_sync(FULL, have);
+        if (!held) break;
+        if constexpr (T == 1) {
+            // Once this warp has found the counter exhausted: every lane of
+            // the launch has failed once to draw (adding 1 to the counter)
+            // or holds a walk, so the counter tells how many are left.
+            if (ho.slots && held != FULL) {
+                unsigned first = 0xffffffffu;
+                if (lane == 0) {
+                    const unsigned long long drawn = *(volatile unsigned long long *)acc.next_walk;
+                    if (drawn >= total && ho.lanes - (unsigned)(drawn - total) <= ho.most)
+                        first = atomicAdd(ho.count, (unsigned)__popc(held));
+                }
+                first = __shfl_sync(FULL, first, 0);
+                if (first != 0xffffffffu) {
+                    if (have) save_walk(ho.slots + 3 * (size_t)(first + __popc(held & ((1u << lane) - 1u))), w);
+                    break;
+                }
+            }
+        }
         if (walk_step<D, SCR>(sc, sp, w, q, have)) {
             if (g.leader()) accumulate(acc, w);
             have = false;
@@ -219,23 +263,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_resume(const SceneView sc, const SolvePa
     float4 *slot = rs.slots + 3 * (((size_t)blockIdx.x * blockDim.x + threadIdx.x) / T);
     Walk w{};
     bool have = false, drained = false;  // uniform within a team
-    {
-        float4 c = slot[2];
-        uint32_t flags = __float_as_uint(c.w);
-        if (flags & 1u) {
-            float4 a = slot[0], b = slot[1];
-            w.x = mk(a.x, a.y, a.z);
-            w.acc = a.w;
-            w.n = mk(b.x, b.y, b.z);
-            w.dbound = b.w;
-            w.steps = (int)__float_as_uint(c.x);
-            w.point = __float_as_uint(c.y);
-            w.index = __float_as_uint(c.z);
-            w.onN = (flags & 2u) != 0;
-            w.capped = (flags & 4u) != 0;
-            have = true;
-        }
-    }
+    have = load_walk(slot, w);
     unsigned long long ran = 0;
     for (int it = 0; it < iters; ++it) {
         unsigned need = __ballot_sync(FULL, g.leader() && !have && !drained);
@@ -268,24 +296,22 @@ __global__ void WOST_WALK_BOUNDS k_walk_resume(const SceneView sc, const SolvePa
         __syncwarp();
     }
     if (g.leader()) {
-        if (have) {
-            uint32_t flags = 1u | (w.onN ? 2u : 0u) | (w.capped ? 4u : 0u);
-            slot[0] = make_float4(w.x.x, w.x.y, w.x.z, w.acc);
-            slot[1] = make_float4(w.n.x, w.n.y, w.n.z, w.dbound);
-            slot[2] = make_float4(__uint_as_float((uint32_t)w.steps), __uint_as_float(w.point),
-                                  __uint_as_float(w.index), __uint_as_float(flags));
-        } else {
-            slot[2] = make_float4(0.f, 0.f, 0.f, 0.f);  // flags 0: empty
-        }
+        if (have) save_walk(slot, w);
+        else slot[2] = make_float4(0.f, 0.f, 0.f, 0.f);  // flags 0: empty
     }
     // launch totals: steps run (one count per team) and walks saved
     unsigned long long r = g.leader() ? ran : 0ull;
-    unsigned saved = __popc(__ballot_sync(FULL, g.leader() && have));
+    const unsigned saved = __ballot_sync(FULL, g.leader() && have);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(FULL, r, o);
-    if (lane == 0) {
-        if (r) atomicAdd(rs.steps_run, r);
-        if (saved) atomicAdd(rs.live, saved);
+    if (lane == 0 && r) atomicAdd(rs.steps_run, r);
+    if (saved) {
+        unsigned first = 0;
+        if (lane == 0) first = atomicAdd(rs.live, (unsigned)__popc(saved));
+        if constexpr (T == 1) {
+            first = __shfl_sync(FULL, first, 0);
+            if (have) rs.list[first + __popc(saved & ((1u << lane) - 1u))] = blockIdx.x * blockDim.x + threadIdx.x;
+        }
     }
 }
 
@@ -365,30 +391,32 @@ static cudaError_t walk_count_launch(const SceneView &sc, const SolveParams &sp,
 
 // resident blocks of kernel k per SM times the SM count, its shared-memory
 // limit set
-static cudaError_t resident_grid(const void *k, int block, int depth, int *blocks_out, int lanes = 1) {
+static cudaError_t resident_blocks(const void *k, int block, size_t sm, int *blocks_out) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    size_t sm = smem_bytes(depth, block, lanes);
     if (e == cudaSuccess) e = smem_limit(k, sm);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, sm);
     if (e != cudaSuccess) return e;
     *blocks_out = sms * (per_sm > 0 ? per_sm : 1);
     return cudaSuccess;
 }
+static cudaError_t resident_grid(const void *k, int block, int depth, int *blocks_out, int lanes = 1) {
+    return resident_blocks(k, block, smem_bytes(depth, block, lanes), blocks_out);
+}
 
 template <bool SCR, int T>
 static cudaError_t walk_persistent_launch(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
-                                          int block, int blocks, cudaStream_t s) {
+                                          const HandOver &ho, int block, int blocks, cudaStream_t s) {
     size_t sm = smem_bytes(sp.stack_depth, block, T);
     const void *k =
         sc.dim == 2 ? (const void *)k_walk_persistent<2, SCR, T> : (const void *)k_walk_persistent<3, SCR, T>;
     cudaError_t e = smem_limit(k, sm);
     if (e != cudaSuccess) return e;
     if (sc.dim == 2)
-        k_walk_persistent<2, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc);
+        k_walk_persistent<2, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc, ho);
     else
-        k_walk_persistent<3, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc);
+        k_walk_persistent<3, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc, ho);
     return cudaGetLastError();
 }
 
@@ -412,7 +440,9 @@ cudaError_t launch_walk_plain_scr(const SceneView &sc, const SolveParams &sp, co
 cudaError_t launch_walk_count_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                   unsigned long long *stats, int block, cudaStream_t s);
 cudaError_t launch_walk_persistent_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
-                                       int block, int blocks, cudaStream_t s);
+                                       const HandOver &ho, int block, int blocks, cudaStream_t s);
+cudaError_t launch_walk_warp_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
+                                 const TailWalks &tw, uint64_t walks, cudaStream_t s);
 cudaError_t launch_walk_resume_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                    const ResumeState &rs, int iters, int block, int blocks, cudaStream_t s);
 // 8-lane team instantiations (Poisson), defined in wost_kernels_team.cu

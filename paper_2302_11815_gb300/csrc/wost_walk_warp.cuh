@@ -1,0 +1,110 @@
+// Walk kernels with one walk per warp (WarpQ, wost_warp.cuh): all of a small
+// solve's walks, or the last walks of a large one, which the one-lane kernels
+// hand over in saved-walk slots once too few of them are left to fill lanes.
+#pragma once
+
+#include "wost_walk.cuh"
+#include "wost_warp.cuh"
+
+// Register cap of the one-walk-per-warp kernels.
+#ifndef WOST_WARP_REGS
+#define WOST_WARP_REGS 96
+#endif
+
+namespace wost {
+
+constexpr int kWarpFrontier = 192;  // frontier entries per warp (an overflow falls back to the binary trees)
+
+// largest coordinate of the boundary
+__device__ __forceinline__ float scene_scale(const SceneView &sc) {
+    float m = 0.f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        m = fmaxf(m, fmaxf(fabsf(sc.D.root_lo[a]), fabsf(sc.D.root_hi[a])));
+        m = fmaxf(m, fmaxf(fabsf(sc.N.root_lo[a]), fabsf(sc.N.root_hi[a])));
+    }
+    return m;
+}
+
+template <int D>
+__device__ __forceinline__ WarpQ<D> make_warp_q(int depth, unsigned int *guard) {
+    extern __shared__ int2 smem_stack[];
+    WarpQ<D> q;
+    int2 *mine = smem_stack + (threadIdx.x >> 5) * (kWarpFrontier + depth);
+    q.fr = mine;
+    q.fcap = kWarpFrontier;
+    q.st = Stack{mine + kWarpFrontier, 1, depth, guard, 0u};
+    q.lane = threadIdx.x & 31;
+    q.new_walk();
+    return q;
+}
+
+// Walks drawn from the solve's counter, or saved ones (tw.slots).  Bound by
+// the latency of its dependent rounds: a step takes 10 us alone (Koch; one
+// lane 20 us, a full warp of one-lane walks 35 us).  Whole solves, before ->
+// after: 976 Koch walks 1,348 -> 426 ms, 6,144 keyhole walks 164 -> 36 ms, 768
+// walks by a crack 5.5 -> 1.7 ms, 544,096 torus walks (tail only) 391 -> 234 ms.
+template <int D, bool SCR>
+__global__ void __maxnreg__(WOST_WARP_REGS) k_walk_warp(const __grid_constant__ SceneView sc,
+                                                        const __grid_constant__ SolveParams sp,
+                                                        const Accumulators acc, const TailWalks tw) {
+    WarpQ<D> q = make_warp_q<D>(sp.stack_depth, acc.guard);
+    q.scale = scene_scale(sc);
+    q.eps = sp.epsilon;
+    const uint64_t total = (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
+    const unsigned n_saved = tw.slots ? *tw.count : 0u;
+    for (;;) {
+        unsigned long long my = 0;
+        if (q.lane == 0) {
+            if (tw.slots) my = atomicAdd(tw.next, 1u);
+            else my = (acc.cancel && *(volatile int *)acc.cancel) ? total : atomicAdd(acc.next_walk, 1ull);
+        }
+        my = __shfl_sync(0xffffffffu, my, 0);
+        Walk w{};
+        if (tw.slots) {
+            if (my >= n_saved) break;
+            float4 *slot = tw.slots + 3 * (size_t)(tw.list ? tw.list[my] : (uint32_t)my);
+            load_walk(slot, w);
+            __syncwarp();
+            if (q.lane == 0) slot[2] = make_float4(0.f, 0.f, 0.f, 0.f);  // taken
+        } else {
+            if (my >= total) break;
+            walk_init<D>(sp, w, (int64_t)(my / (uint64_t)sp.walks_per_point),
+                         (uint32_t)(my % (uint64_t)sp.walks_per_point) + sp.first_walk);
+        }
+        q.new_walk();
+        const int began = w.steps;
+        while (!walk_step<D, SCR>(sc, sp, w, q, true)) {
+        }
+        if (q.lane == 0) {
+            accumulate(acc, w);
+            if (tw.steps_run) atomicAdd(tw.steps_run, (unsigned long long)(w.steps - began));
+        }
+        __syncwarp();
+    }
+}
+
+template <int D, bool SCR>
+static cudaError_t walk_warp_launch_d(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
+                                      const TailWalks &tw, uint64_t walks, cudaStream_t s) {
+    const int block = 64;
+    const size_t sm = (size_t)(block / 32) * (kWarpFrontier + sp.stack_depth) * sizeof(int2);
+    const void *k = (const void *)k_walk_warp<D, SCR>;
+    cudaError_t e = smem_limit(k, sm);
+    int blocks = 0;
+    if (e == cudaSuccess) e = resident_blocks(k, block, sm, &blocks);
+    if (e != cudaSuccess) return e;
+    const uint64_t want = (walks + block / 32 - 1) / (block / 32);
+    if (want < (uint64_t)blocks) blocks = (int)want;
+    k_walk_warp<D, SCR><<<blocks, block, sm, s>>>(sc, sp, acc, tw);
+    return cudaGetLastError();
+}
+
+template <bool SCR>
+static cudaError_t walk_warp_launch(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
+                                    const TailWalks &tw, uint64_t walks, cudaStream_t s) {
+    return sc.dim == 2 ? walk_warp_launch_d<2, SCR>(sc, sp, acc, tw, walks, s)
+                       : walk_warp_launch_d<3, SCR>(sc, sp, acc, tw, walks, s);
+}
+
+}  // namespace wost

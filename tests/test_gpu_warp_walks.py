@@ -1,0 +1,111 @@
+"""Walks carried by whole warps (small solves, and the last walks of large
+ones) are those of the one-lane kernels, bit for bit: same step counts, means
+that differ by the order of the FP64 additions only (1e-9, as between the
+one-lane kernels).  A solve that gives its traversal limits itself (here: the
+scene's own) stays on the one-lane kernels, which are tested against the
+oracle."""
+import numpy as np
+import pytest
+
+from paper_2302_11815_gb300 import scenes
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def wost():
+    from paper_2302_11815_gb300 import build as libbuild
+    from paper_2302_11815_gb300 import wost as w
+
+    assert torch.cuda.is_available()
+    libbuild.build()
+    w.load()
+    return w
+
+
+def _disk(frac):
+    n = 300
+    return scenes.disk_scene(n, "exp_plane", (1.0, 1.2, -0.7, 0.0), neumann=np.arange(n) < frac * n)
+
+
+def _moved(sc, shift):
+    """The scene away from the origin: the rounding of positions grows with them."""
+    sc = dict(sc)
+    sc["vertices"] = (sc["vertices"] + np.float32(shift)).astype(np.float32)
+    return sc
+
+
+CASES = {
+    "flower": (lambda: scenes.config1(), 0, 0.0),
+    "flower_leaf16": (lambda: scenes.config1(data="per_vertex"), 16, 0.0),
+    "flower_far": (lambda: _moved(scenes.config1(), 30.0), 0, 0.0),
+    "koch3": (lambda: scenes.config2(grid=8, level=3), 0, 0.0),
+    "koch4_leaf1": (lambda: scenes.config2(grid=8, level=4), 1, 0.0),
+    "keyhole": (lambda: scenes.keyhole_scene(), 0, 0.0),
+    "square": (lambda: scenes.square_scene(200, neumann_sides=("left", "bottom")), 0, 0.0),
+    "crack": (lambda: scenes.crack_square_scene(), 0, 0.0),
+    "slit": (lambda: scenes.slit_square_scene(), 2, 0.0),
+    "sheet": (lambda: scenes.sheet_square_scene(m=60, n_sheet=90, data="per_corner_minus"), 0, 0.0),
+    "disk_screened": (lambda: _disk(0.5), 0, 1.9),
+    "disk_pure_neumann": (lambda: _disk(1.0), 0, 1.9),
+    "box_sphere": (lambda: scenes.box_sphere_scene(), 0, 0.0),
+    "cube_faces_leaf16": (lambda: scenes.cube_scene(8, neumann_faces=(0, 3)), 16, 0.0),
+    "cube_screened": (lambda: scenes.cube_scene(5, fn="exp_plane", params=(1.0, 0.8, -0.5, 0.6), neumann_faces=(0, 3)),
+                      0, 1.25),
+    "plate": (lambda: scenes.plate_cube_scene(), 0, 0.0),
+    "cube_torus": (lambda: scenes.config3(grid=8, nu=120, nv=48, cube_m=8), 0, 0.0),
+}
+
+
+def _points(sc, n, rng):
+    V = sc["vertices"].astype(np.float64)
+    lo, hi = V.min(0), V.max(0)
+    if sc["dim"] == 3:
+        p = lo + (hi - lo) * rng.uniform(0.03, 0.97, (8 * n, 3))
+        rho = np.hypot(np.hypot(p[:, 0], p[:, 1]) - 0.5, p[:, 2])
+        return p[(rho > 0.24) & (np.linalg.norm(p, axis=1) > 0.45)][:n].astype(np.float32)
+    c = 0.5 * (lo + hi)
+    if len(V) > 2000 or "koch" in sc.get("name", ""):  # the Koch scenes' domain: between hole and inner disk
+        r, t = rng.uniform(0.36, 0.5, n), rng.uniform(0, 2 * np.pi, n)
+        return np.c_[r * np.cos(t), r * np.sin(t)].astype(np.float32)
+    if "keyhole" in sc.get("name", ""):
+        return np.c_[rng.uniform(-1.9, -0.1, n), rng.uniform(-0.9, 0.9, n)].astype(np.float32)
+    return (c + 0.25 * (hi - lo) * rng.uniform(-1, 1, (n, 2))).astype(np.float32)
+
+
+def _both(wost, sc, leaf, sigma, pts, walks, kernel, cap=2048, **kw):
+    S = wost.Scene(sc, leaf_size=leaf)
+    depth = S.info()["stack_depth"]
+    dev = torch.from_numpy(pts).cuda()
+    got = [wost.solve(S, dev, walks, 1e-3, 1e-3, cap, seed=3, kernel=kernel, sigma=sigma, stack_depth=d, **kw)
+           for d in (0, depth)]
+    S.close()
+    a, b = got
+    assert a["done"] == b["done"] == 1 and a["guard_flags"] == b["guard_flags"] == 0
+    assert np.array_equal(a["walks"], b["walks"])
+    assert (a["total_steps"], a["capped_walks"], a["steps_run"]) == (b["total_steps"], b["capped_walks"],
+                                                                     b["steps_run"])
+    np.testing.assert_allclose(a["mean"], b["mean"], rtol=1e-9, atol=1e-12)
+    return a
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+@pytest.mark.parametrize("n,walks,kernel", [(1, 1, "plain"), (61, 33, "persistent"), (257, 96, "persistent"),
+                                            (257, 96, "resumable")])
+def test_warp_walks_are_the_one_lane_walks(wost, name, n, walks, kernel):
+    make, leaf, sigma = CASES[name]
+    sc = make()
+    _both(wost, sc, leaf, sigma, _points(sc, n, np.random.default_rng(7)), walks, kernel)
+
+
+def test_warp_walks_from_boundary_points(wost):
+    for sc in (scenes.config1(), scenes.box_sphere_scene(data="analytic")):
+        sel = np.flatnonzero(sc["flags"] == 1)
+        sel = sel[:: max(1, len(sel) // 48)]
+        V, P = sc["vertices"], sc["prims"][sel]
+        w = np.array([0.3, 0.7]) if sc["dim"] == 2 else np.array([0.2, 0.3, 0.5])
+        pts = np.einsum("k,nkd->nd", w, V[P].astype(np.float64)).astype(np.float32)
+        nrm = torch.from_numpy(scenes.prim_normals(sc)[sel].astype(np.float32)).cuda()
+        on = torch.ones(len(sel), dtype=torch.uint8, device="cuda")
+        _both(wost, sc, 0, 0.0, pts, 40, "persistent", normals=nrm, on_neumann=on)
