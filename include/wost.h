@@ -268,8 +268,9 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *desc, wost_solv
  * solve must run in order (one stream, or ordered by the caller).  No
  * launch waits for the longest walks of the solve, which is what keeps
  * the GPU full on workloads whose walk lengths have a long tail.  wost_wait
- * on a resumable solve issues launches of 2048 iterations itself until
- * every walk has finished.  The walks and estimates are those of the other
+ * on a resumable solve issues the launches itself until every walk has
+ * finished: of 2048 iterations each while a solve already advanced has walks
+ * left to draw, else to the walks' ends.  The walks and estimates are those of the other
  * kernels for the same seed.  Errors: INVALID_ARG (not a resumable solve,
  * iterations < 1), CUDA. */
 wost_status wost_solve_advance(wost_solve_handle *solve, int32_t iterations, void *stream);
@@ -341,7 +342,7 @@ wost_status wost_screened_kernels(int32_t dim, int64_t n, const float *rho, cons
  * normals), mean_out and stderr_out (device, n_points floats) belong to the
  * caller and must stay valid until the stream has passed this call.
  * The call allocates nothing: the FP64 accumulators and counters live in one
- * fixed device array of the library (about 2 MiB, held by every device that
+ * fixed device array of the library (about 3.7 MiB, held by every device that
  * loads the library until the process exits), which the call clears on
  * `stream` before use.  Hence:
  *   - n_points > WOST_STATIC_MAX_POINTS is rejected with INVALID_ARG;

@@ -26,14 +26,6 @@ wost_status cuda_fail(cudaError_t e, const char *what);
         if (_e != cudaSuccess) return wost::cuda_fail(_e, what); \
     } while (0)
 
-// A solve of at most this many walks runs them one per warp from the start,
-// and a larger one hands its last walks over when so many are left: that is
-// where the two forms run equally many steps per second (Koch workload: 4,864
-// walks one per warp 2.4e8 steps/s; 12,288 of them left over in 4,864 warps of
-// one-lane walks ~2e8, each step of such a warp taking 60 us).
-constexpr uint64_t kWarpWalks = 12288;
-constexpr unsigned kTailWalks = 12288;
-
 // device allocation owned by a scene or solve
 struct DevBuf {
     void *p = nullptr;
@@ -68,9 +60,34 @@ cudaError_t upload(DevBuf &b, const std::vector<T> &v) {
     return e;
 }
 
+// Words (u64) of a batched launch's counters.
+constexpr size_t kBatchCounters = 4 + 2 * kMaxStages;
+// The chain buffers of dimension di (0: 2D, 1: 3D) of a batched launch,
+// allocated for its grid.
+inline cudaError_t batch_chain_buffers(DevBuf chain[2], unsigned long long *counters, int di, int block, int blocks,
+                                       ChainBuffers *cb) {
+    for (int i = 0; i < 2; ++i) {
+        const size_t cap = (size_t)batch_chain_capacity(block, blocks, i), bytes = cap * 3 * sizeof(float4);
+        if (chain[i].p && chain[i].bytes < bytes) {
+            cudaFree(chain[i].p);
+            chain[i].p = nullptr;
+        }
+        if (!chain[i].p) {
+            cudaError_t e = chain[i].alloc(bytes);
+            if (e != cudaSuccess) return e;
+        }
+        cb->cap[i] = (unsigned)cap;
+        cb->slots[i] = (float4 *)chain[i].p;
+    }
+    cb->counters = (unsigned int *)(counters + 4 + di * kMaxStages);
+    return cudaSuccess;
+}
+
 // resources shared by the solves of one batched launch
 struct BatchShared {
-    DevBuf jobs[2], counters;  // counters: next walk (2D), next walk (3D), guard
+    // counters: next walk (2D), next walk (3D), guard, -, then each
+    // dimension's hand-over counters; chain: its slot arrays
+    DevBuf jobs[2], counters, chain[2][2];
     unsigned long long total[2] = {0, 0};
     cudaEvent_t ev_start = nullptr, ev_done = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;  // the 3D launch's side stream
@@ -133,11 +150,12 @@ struct wost_solve_handle {
     wost::SolveParams sp{};
     wost::Accumulators acc{};
     wost::DevBuf points, normals, onN;
-    wost::DevBuf sum, sumsq, walks_done, steps, globals;  // globals: capped, next_walk, guard
+    wost::DevBuf sum, sumsq, walks_done, steps, globals;  // globals: capped, next_walk, guard, -, hand-over counters
     wost::DevBuf counts;                                   // counting kernel only
     // resumable solves: saved-walk slots of the fixed grid, launch counters
     // (steps_run u64, live u32), launches enqueued so far
     wost::DevBuf slots, rstate;
+    wost::DevBuf chain[2];  // slots of walks handed over between launches
     int resume_blocks = 0;
     uint64_t launches = 0;
     bool resumable() const { return kernel == WOST_KERNEL_RESUMABLE; }
@@ -186,6 +204,8 @@ void set_layout_info(wost_scene *s, int lanes);
 // both on streams of its own).
 wost_status prepare_solve(wost_scene *scene, const wost_solve_desc *d, cudaStream_t stream, wost_solve_handle *h,
                           bool fill = true);
+// u64 words of a solve's globals: 4, then the hand-over counters
+constexpr size_t kGlobals = 4 + kMaxStages;
 // Zeroes a solve's accumulators and counters on `stream`.
 cudaError_t clear_accumulators(wost_solve_handle *h, cudaStream_t stream);
 // Blocks until the work queued so far on `stream` (the input copies) is done.

@@ -8,18 +8,40 @@
 
 namespace wost {
 
+// the job that walk index `my` of a batched launch belongs to
+__device__ __forceinline__ int job_of(const BatchJob *jobs, int n_jobs, unsigned long long my) {
+    int lo = 0, hi = n_jobs - 1;
+    while (lo < hi) {
+        int mid = (lo + hi + 1) >> 1;
+        if (jobs[mid].walk_begin <= my) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+template <int D>
+__device__ __forceinline__ void init_job_walk(const BatchJob &J, unsigned long long my, Walk &w) {
+    const SolveParams &sp = J.sp;
+    unsigned long long local = my - J.walk_begin;
+    int64_t pt = sp.point_begin + (int64_t)(local / (uint64_t)sp.walks_per_point);
+    uint32_t j = (uint32_t)(local % (uint64_t)sp.walks_per_point) + sp.first_walk;
+    walk_init<D>(sp, w, pt, j);
+}
+
 // Batched persistent kernel: many solves (scenes, point sets, walk counts,
 // parameters) in one launch.  The walk index space is the concatenation of
 // the jobs' walks; a team maps its next index to a job by binary search over
 // the jobs' first indices and runs that job's walk on that job's scene.
 // steps_out (may be null) receives the walk steps of the finished walks.
+// src, ho: walks taken up from, and handed over to, another launch (a saved
+// walk keeps its job index).
 template <int D, bool SCR>
 __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hdr,
                                                     const BatchJob *__restrict__ jobs, unsigned long long *counter,
                                                     unsigned int *guard, int stack_depth, const int *cancel,
-                                                    unsigned long long *steps_out) {
+                                                    unsigned long long *steps_out, const SavedWalks src,
+                                                    const HandOver ho) {
     const int n_jobs = hdr->n_jobs;
-    const unsigned long long total = hdr->total;
+    const unsigned long long total = src.slots ? (unsigned long long)*src.count : hdr->total;
     if (n_jobs <= 0) return;
     Cnt<false> cnt;
     auto q = make_q<D, false>(stack_depth, guard, cnt);
@@ -38,35 +60,39 @@ __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hd
             int lead = __ffs(need) - 1;
             unsigned long long base = 0;
             if (lane == lead) {
-                bool stop = cancel && *(volatile const int *)cancel != 0;
-                base = stop ? total : atomicAdd(counter, (unsigned long long)__popc(need));
+                if (src.slots) {
+                    base = atomicAdd(src.next, (unsigned)__popc(need));
+                } else {
+                    bool stop = cancel && *(volatile const int *)cancel != 0;
+                    base = stop ? total : atomicAdd(counter, (unsigned long long)__popc(need));
+                }
             }
             base = __shfl_sync(FULL, base, lead);
             if ((need >> g.base) & 1u) {
                 unsigned long long my = base + __popc(need & ((1u << g.base) - 1u));
                 if (my >= total) {
                     drained = true;
+                } else if (src.slots) {
+                    load_walk(src.slots + 3 * (size_t)my, w, &job);
                 } else {
-                    int lo = 0, hi = n_jobs - 1;
-                    while (lo < hi) {
-                        int mid = (lo + hi + 1) >> 1;
-                        if (jobs[mid].walk_begin <= my) lo = mid;
-                        else hi = mid - 1;
-                    }
+                    const int lo = job_of(jobs, n_jobs, my);
                     // a cancelled solve's remaining walks are skipped: the
                     // team takes another index at the next iteration
                     if (!team_flag(g, jobs[lo].acc.cancel)) {
                         job = lo;
-                        const SolveParams &sp = jobs[job].sp;
-                        unsigned long long local = my - jobs[job].walk_begin;
-                        int64_t pt = sp.point_begin + (int64_t)(local / (uint64_t)sp.walks_per_point);
-                        uint32_t j = (uint32_t)(local % (uint64_t)sp.walks_per_point) + sp.first_walk;
-                        walk_init<D>(sp, w, pt, j);
+                        init_job_walk<D>(jobs[job], my, w);
                     }
                 }
             }
         }
-        if (!__any_sync(FULL, job >= 0 || !drained)) break;
+        const unsigned held = __ballot_sync(FULL, job >= 0);
+        if (!held) {
+            if (__any_sync(FULL, !drained)) continue;
+            break;
+        }
+        if (ho.slots && (src.slots ? hand_over(ho, src.next, total, lane, w, job >= 0, held, job)
+                                   : hand_over(ho, counter, total, lane, w, job >= 0, held, job)))
+            break;
         // lanes without a job step a dummy reference to job 0 (inactive)
         const BatchJob &J = jobs[job >= 0 ? job : 0];
         if (walk_step<D, SCR>(*J.scene, J.sp, w, q, job >= 0)) {

@@ -241,7 +241,7 @@ cudaError_t wost::clear_accumulators(wost_solve_handle *h, cudaStream_t stream) 
     cudaError_t e = cudaSuccess;
     for (DevBuf *b : {&h->sum, &h->sumsq, &h->walks_done, &h->steps})
         if (e == cudaSuccess) e = cudaMemsetAsync(b->p, 0, n * 8, stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(h->globals.p, 0, 4 * 8, stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(h->globals.p, 0, kGlobals * 8, stream);
     return e;
 }
 
@@ -314,7 +314,7 @@ wost_status wost::prepare_solve(wost_scene *scene, const wost_solve_desc *d, cud
     CK(alloc(h->sumsq, n * 8), "cudaMalloc accumulators");
     CK(alloc(h->walks_done, n * 8), "cudaMalloc accumulators");
     CK(alloc(h->steps, n * 8), "cudaMalloc accumulators");
-    CK(alloc(h->globals, 4 * 8), "cudaMalloc accumulators");
+    CK(alloc(h->globals, kGlobals * 8), "cudaMalloc accumulators");
     if (fill) CK(clear_accumulators(h, stream), "memset");
     if (!h->cancel_host) {
         CK(cudaHostAlloc((void **)&h->cancel_host, sizeof(int), cudaHostAllocMapped), "cudaHostAlloc");
@@ -367,6 +367,21 @@ wost_status wost::wait_for_copies(cudaStream_t stream) {
     return WOST_OK;
 }
 
+// The slot arrays of a solve's chain of launches (allocated once) and its
+// counters in the solve's globals (still zero: a solve runs one chain).
+static cudaError_t chain_buffers(wost_solve_handle *h, uint64_t walks, int blocks, ChainBuffers *cb) {
+    for (int i = 0; i < 2; ++i) {
+        cb->cap[i] = (unsigned)chain_capacity(walks, h->block, blocks, i);
+        if (!h->chain[i].p) {
+            cudaError_t e = h->chain[i].alloc((size_t)cb->cap[i] * 3 * sizeof(float4));
+            if (e != cudaSuccess) return e;
+        }
+        cb->slots[i] = (float4 *)h->chain[i].p;
+    }
+    cb->counters = (unsigned int *)((unsigned long long *)h->globals.p + 4);
+    return cudaSuccess;
+}
+
 extern "C" {
 
 wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_handle **out) {
@@ -411,8 +426,8 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
         // (few of them) or the last walks (of many) run one per warp
         const uint64_t total = (uint64_t)d->n_points * (uint64_t)d->walks_per_point;
         const bool warp_ok = h->lanes == 1 && h->warp_ok;
-        if (warp_ok && total <= kWarpWalks && d->kernel != WOST_KERNEL_COUNTING) {
-            le = launch_walk_warp(scene->view, sp, acc, TailWalks{}, total, stream);
+        if (warp_ok && total <= kTailWalks && d->kernel != WOST_KERNEL_COUNTING) {
+            le = launch_walk_warp(scene->view, sp, acc, SavedWalks{}, total, stream);
         } else if (d->kernel == WOST_KERNEL_PLAIN) {
             le = launch_walk_plain(scene->view, sp, acc, h->block, stream);
         } else if (d->kernel == WOST_KERNEL_COUNTING) {
@@ -423,17 +438,14 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
         } else {
             int blocks = 0;
             le = persistent_grid(h->dim, h->block, sp.stack_depth, &blocks, h->lanes);
-            HandOver ho{};
-            TailWalks tw{};
             if (le == cudaSuccess && warp_ok) {
-                le = h->slots.alloc((size_t)kTailWalks * 3 * sizeof(float4));
-                unsigned int *ctr = (unsigned int *)((unsigned long long *)h->globals.p + 3);
-                ho = HandOver{(float4 *)h->slots.p, ctr, kTailWalks, 0};
-                tw = TailWalks{(float4 *)h->slots.p, nullptr, ctr, ctr + 1, nullptr};
+                ChainBuffers cb{};
+                le = chain_buffers(h.get(), total, blocks, &cb);
+                if (le == cudaSuccess)
+                    le = launch_walk_chain(scene->view, sp, acc, SavedWalks{}, total, cb, h->block, blocks, stream);
+            } else if (le == cudaSuccess) {
+                le = launch_walk_persistent(scene->view, sp, acc, h->block, blocks, stream, h->lanes);
             }
-            if (le == cudaSuccess)
-                le = launch_walk_persistent(scene->view, sp, acc, h->block, blocks, stream, h->lanes, ho);
-            if (le == cudaSuccess && warp_ok) le = launch_walk_warp(scene->view, sp, acc, tw, kTailWalks, stream);
         }
         if (le != cudaSuccess) return cuda_fail(le, "kernel launch");
         CK(cudaEventRecord(h->ev_done, stream), "cudaEventRecord");
@@ -504,8 +516,16 @@ wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_so
             CK(cudaMemcpyAsync(shared->jobs[di].p, staging[di].data(), staging[di].size(), cudaMemcpyHostToDevice,
                                stream), "copy jobs");
         }
-        CK(shared->counters.alloc(4 * 8), "cudaMalloc counters");
-        CK(cudaMemsetAsync(shared->counters.p, 0, 4 * 8, stream), "memset");
+        CK(shared->counters.alloc(kBatchCounters * 8), "cudaMalloc counters");
+        CK(cudaMemsetAsync(shared->counters.p, 0, kBatchCounters * 8, stream), "memset");
+        int blocks[2] = {0, 0};
+        ChainBuffers chain[2];
+        for (int di = 0; di < 2; ++di) {
+            if (jobs[di].empty()) continue;
+            CK(batch_grid(di + 2, block, depth[di], &blocks[di]), "occupancy");
+            CK(batch_chain_buffers(shared->chain[di], (unsigned long long *)shared->counters.p, di, block, blocks[di],
+                                   &chain[di]), "cudaMalloc slots");
+        }
         CK(cudaEventCreate(&shared->ev_start), "cudaEventCreate");
         CK(cudaEventCreate(&shared->ev_done), "cudaEventCreate");
         wost_status st = wait_for_copies(stream);
@@ -527,15 +547,13 @@ wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_so
         }
         for (int di = 0; di < 2; ++di) {
             if (jobs[di].empty()) continue;
-            int blocks = 0;
-            CK(batch_grid(di + 2, block, depth[di], &blocks), "occupancy");
             const unsigned char *base = (const unsigned char *)shared->jobs[di].p;
             cudaStream_t ls = (both && di == 1) ? shared->side : stream;
             const bool scr = std::any_of(jobs[di].begin(), jobs[di].end(),
                                          [](const BatchJob &j) { return j.sp.sigma > 0.f; });
             CK(launch_walk_batch(di + 2, (const BatchHeader *)base, (const BatchJob *)(base + sizeof(BatchHeader)),
-                                 ctr + di, (unsigned int *)(ctr + 2), depth[di], nullptr, block, blocks, ls, nullptr,
-                                 scr),
+                                 ctr + di, (unsigned int *)(ctr + 2), depth[di], nullptr, block, blocks[di], chain[di],
+                                 ls, nullptr, scr),
                "kernel launch");
         }
         if (both) {
@@ -687,26 +705,35 @@ static wost_status advance_locked(wost_solve_handle *h, int iters, cudaStream_t 
 }
 
 // The next launch of a resumable solve while its caller waits: bounded as
-// wost_solve_advance's, or, once the last walks are few, one walk per warp to
-// their ends (caller holds h->mu; the previous launch has completed).
+// wost_solve_advance's or, when every remaining walk is still to be drawn or
+// none is, the chain of launches that runs them all to their ends (caller
+// holds h->mu; the previous launch has completed).
 static wost_status advance_waiting(wost_solve_handle *h) {
-    const bool warp_ok = h->lanes == 1 && h->warp_ok;
-    if (warp_ok && h->launches > 0) {
+    if (h->lanes != 1 || !h->warp_ok) return advance_locked(h, 2048, h->stream);
+    unsigned long long *steps_run = (unsigned long long *)h->rstate.p;
+    unsigned int *ctr = (unsigned int *)((char *)h->rstate.p + 8);
+    SavedWalks src{nullptr, nullptr, nullptr, nullptr, steps_run};
+    uint64_t walks = (uint64_t)h->n_points * (uint64_t)h->walks;
+    if (h->launches > 0) {
         bool fin = false, drained = false;
         unsigned int live = 0;
         wost_status st = resumable_finished(h, &fin, &drained, &live);
-        if (st != WOST_OK) return st;
-        if (drained && live > 0 && live <= kTailWalks) {
-            unsigned int *ctr = (unsigned int *)((char *)h->rstate.p + 8);
-            TailWalks tw{(float4 *)h->slots.p, ctr + 2, ctr, ctr + 1, (unsigned long long *)h->rstate.p};
-            CK(launch_walk_warp(h->scene->view, h->sp, h->acc, tw, live, h->stream), "kernel launch");
-            CK(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned int), h->stream), "memset");
-            CK(cudaEventRecord(h->ev_done, h->stream), "cudaEventRecord");
-            h->launches++;
-            return WOST_OK;
-        }
+        if (st != WOST_OK || fin) return st;
+        if (!drained) return advance_locked(h, 2048, h->stream);
+        src = SavedWalks{(float4 *)h->slots.p, ctr + 2, ctr, ctr + 1, steps_run};
+        walks = live;
+    } else {
+        h->t_launch = std::chrono::steady_clock::now();
+        CK(cudaEventRecord(h->ev_start, h->stream), "cudaEventRecord");
     }
-    return advance_locked(h, 2048, h->stream);
+    ChainBuffers cb{};
+    CK(chain_buffers(h, walks, h->resume_blocks, &cb), "cudaMalloc slots");
+    CK(launch_walk_chain(h->scene->view, h->sp, h->acc, src, walks, cb, h->block, h->resume_blocks, h->stream),
+       "kernel launch");
+    CK(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned int), h->stream), "memset");
+    CK(cudaEventRecord(h->ev_done, h->stream), "cudaEventRecord");
+    h->launches++;
+    return WOST_OK;
 }
 
 wost_status wost_solve_advance(wost_solve_handle *h, int32_t iterations, void *stream) {

@@ -70,7 +70,8 @@ struct Slot {
     size_t cap[2] = {0, 0};    // jobs per table
     int depth[2] = {0, 0};     // stack entries the graph was captured with
     bool scr[2] = {true, true};  // the kernels' form: screened, or Poisson only
-    DevBuf counters;           // next walk 2D, next walk 3D, guard, walk steps run
+    DevBuf counters;           // next walk 2D, next walk 3D, guard, walk steps run, hand-over counters
+    DevBuf chain[2][2];        // slots of walks handed over between the round's launches
     unsigned long long *steps_host = nullptr;  // pinned copy of the walk-step count
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -476,7 +477,7 @@ cudaError_t ensure_graph(wost_engine *e, Slot &sl, const size_t cnt[2], const in
         }
     }
     if (!sl.counters.p) {
-        if ((er = sl.counters.alloc(4 * 8)) != cudaSuccess) return er;
+        if ((er = sl.counters.alloc(kBatchCounters * 8)) != cudaSuccess) return er;
         if ((er = cudaMallocHost((void **)&sl.steps_host, 8)) != cudaSuccess) return er;
         *sl.steps_host = 0;
         rebuild = true;
@@ -490,8 +491,12 @@ cudaError_t ensure_graph(wost_engine *e, Slot &sl, const size_t cnt[2], const in
     for (int di = 0; di < 2; ++di)
         if ((er = batch_grid(di + 2, e->block, sl.depth[di], &blocks[di])) != cudaSuccess) return er;
     unsigned long long *ctr = (unsigned long long *)sl.counters.p;
+    ChainBuffers chain[2];
+    for (int di = 0; di < 2; ++di)
+        if ((er = batch_chain_buffers(sl.chain[di], ctr, di, e->block, blocks[di], &chain[di])) != cudaSuccess)
+            return er;
     if ((er = cudaStreamBeginCapture(sl.stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return er;
-    cudaMemsetAsync(sl.counters.p, 0, 4 * 8, sl.stream);
+    cudaMemsetAsync(sl.counters.p, 0, kBatchCounters * 8, sl.stream);
     for (int di = 0; di < 2; ++di)
         cudaMemcpyAsync(sl.jobs[di].p, sl.host[di], table_bytes(sl.cap[di]), cudaMemcpyHostToDevice, sl.stream);
     // the 2D and 3D kernels are parallel branches of the graph (the 3D one
@@ -503,7 +508,7 @@ cudaError_t ensure_graph(wost_engine *e, Slot &sl, const size_t cnt[2], const in
         const unsigned char *base = (const unsigned char *)sl.jobs[di].p;
         launch_walk_batch(di + 2, (const BatchHeader *)base, (const BatchJob *)(base + sizeof(BatchHeader)), ctr + di,
                           (unsigned int *)(ctr + 2), sl.depth[di], nullptr, e->block, blocks[di],
-                          di == 0 ? sl.stream : sl.side, ctr + 3, sl.scr[di]);
+                          chain[di], di == 0 ? sl.stream : sl.side, ctr + 3, sl.scr[di]);
     }
     cudaEventRecord(sl.join, sl.side);
     cudaStreamWaitEvent(sl.stream, sl.join, 0);

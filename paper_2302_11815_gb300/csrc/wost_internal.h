@@ -124,25 +124,34 @@ struct ResumeState {
     uint32_t *list;                 // slots of those walks (one entry per slot; null with 8-lane teams)
 };
 
-// Where a one-lane kernel hands its last walks over (slots as in
-// ResumeState, filled from the front; null: it keeps them): once the solve's
-// counter is exhausted and at most `most` walks are left, every warp saves
-// the walks it holds and ends.
-struct HandOver {
-    float4 *slots;
-    unsigned int *count;  // [1] walks saved
-    unsigned int most;    // capacity of `slots`
-    unsigned int lanes;   // walks the launch can hold at once
-};
-
-// The saved walks a one-walk-per-warp kernel runs to their ends (slots null:
-// none saved, it draws the solve's own walks).
-struct TailWalks {
+// Saved walks (slots as in ResumeState; in a batch, a walk's job index is in
+// bits 8.. of its flags) that a launch takes up; slots null: none, it draws
+// the solve's own walks.
+struct SavedWalks {
     float4 *slots;
     const uint32_t *list;           // their slots (null: slots 0, 1, ...)
     const unsigned int *count;      // [1] how many
     unsigned int *next;             // [1] work counter
     unsigned long long *steps_run;  // [1] receives the steps run (may be null)
+};
+
+// Where a one-lane kernel hands its last walks over (slots filled from the
+// front; null: it keeps them): once nothing is left to draw and at most
+// `most` walks are left, every warp saves the walks it holds and ends.
+struct HandOver {
+    float4 *slots;
+    unsigned int *count;  // [1] walks saved
+    unsigned int most;    // at most the capacity of `slots`
+    unsigned int lanes;   // walks the launch can hold at once
+};
+
+// Buffers of a chain of launches that hand walks over: two slot arrays used
+// in turn, and a (count, work counter) pair per hand-over, zeroed beforehand.
+constexpr int kMaxStages = 8;
+struct ChainBuffers {
+    float4 *slots[2];
+    unsigned int cap[2];
+    unsigned int *counters;  // [2 * kMaxStages]
 };
 
 // Accumulators of one solve, for the per-solve summary kernel.

@@ -154,12 +154,40 @@ cudaError_t persistent_grid(int dim, int block, int depth, int *blocks_out, int 
 }
 
 cudaError_t launch_walk_persistent(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, int block,
-                                   int blocks, cudaStream_t s, int lanes, const HandOver &ho) {
+                                   int blocks, cudaStream_t s, int lanes, const SavedWalks &src, const HandOver &ho) {
     if (lanes == WOST_WIDE) return launch_walk_persistent_team(sc, sp, acc, block, blocks, s);
     HandOver h = ho;
     h.lanes = (unsigned)blocks * (unsigned)block;
-    if (sp.sigma > 0.f) return launch_walk_persistent_scr(sc, sp, acc, h, block, blocks, s);
-    return walk_persistent_launch<false, 1>(sc, sp, acc, h, block, blocks, s);
+    if (sp.sigma > 0.f) return launch_walk_persistent_scr(sc, sp, acc, src, h, block, blocks, s);
+    return walk_persistent_launch<false, 1>(sc, sp, acc, src, h, block, blocks, s);
+}
+
+// Lane kernels that pass the remaining walks on to one another, then the
+// warp kernel.  A warp of one-lane walks takes 35 us per step (Koch) whether
+// 32 or 8 of its lanes still hold a walk, so once half of the walks of a
+// launch have ended the rest is packed into half as many warps.
+cudaError_t launch_walk_chain(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, SavedWalks src,
+                              uint64_t walks, const ChainBuffers &cb, int block, int blocks, cudaStream_t s) {
+    const uint64_t resident = (uint64_t)blocks * (uint64_t)block;
+    for (int stage = 0; stage < kMaxStages && walks > kTailWalks; ++stage) {
+        const int b = stage & 1;
+        const uint64_t held = std::min(walks, resident);
+        uint64_t most = held / 2 < kTailWalks * 3 / 2 ? kTailWalks : held / 2;
+        most = std::min<uint64_t>(most, cb.cap[b]);
+        unsigned int *ctr = cb.counters + 2 * stage;
+        const HandOver ho{cb.slots[b], ctr, (unsigned)most, 0u};
+        const int grid = (int)std::min<uint64_t>((uint64_t)blocks, (walks + block - 1) / block);
+        cudaError_t e = launch_walk_persistent(sc, sp, acc, block, grid, s, 1, src, ho);
+        if (e != cudaSuccess) return e;
+        src = SavedWalks{cb.slots[b], nullptr, ctr, ctr + 1, src.steps_run};
+        walks = most;
+    }
+    return launch_walk_warp(sc, sp, acc, src, walks, s);
+}
+
+uint64_t chain_capacity(uint64_t walks, int block, int blocks, int which) {
+    const uint64_t held = std::min<uint64_t>(walks, (uint64_t)blocks * (uint64_t)block);
+    return walks <= kTailWalks ? 0 : std::max<uint64_t>(kTailWalks, held >> (which + 1));
 }
 
 // the resumable kernels share the persistent ones' occupancy (same body)

@@ -7,6 +7,14 @@
 
 namespace wost {
 
+// A solve of at most this many walks runs them one per warp from the start,
+// and a larger one hands its last walks over when so many are left.  Measured
+// with 4,096 / 8,192 / 16,384 / 32,768 / 65,536: 8,192 keyhole walks 74 / 40 /
+// 40 / 39 / 40 ms, 64,000 box-sphere walks 19 / 16 / 13 / 12 / 13 ms, 48,000
+// torus walks 80 / 59 / 50 / 44 / 49 ms, 131,072 flower walks (short ones)
+// 2.6 / 2.4 / 2.3 / 2.6 / 3.1 ms.
+constexpr unsigned kTailWalks = 16384;
+
 cudaError_t launch_walk_plain(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, int block,
                               cudaStream_t s);
 cudaError_t launch_walk_count(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
@@ -18,14 +26,29 @@ cudaError_t launch_request_stats(const StatJob *jobs, int n_jobs, int64_t max_po
                                  unsigned long long *walks_sum, cudaStream_t s);
 cudaError_t launch_walk_batch(int dim, const BatchHeader *hdr, const BatchJob *jobs, unsigned long long *counter,
                               unsigned int *guard, int depth, const int *cancel, int block, int blocks,
-                              cudaStream_t s, unsigned long long *steps_out = nullptr, bool screened = true);
+                              const ChainBuffers &cb, cudaStream_t s, unsigned long long *steps_out = nullptr,
+                              bool screened = true);
+cudaError_t prepare_walk_warp_batch(int dim, int depth, bool screened);
+// slots that slot array `which` (0, 1) of a batch's chain has to hold
+uint64_t batch_chain_capacity(int block, int blocks, int which);
+cudaError_t launch_walk_warp_batch(int dim, const BatchHeader *hdr, const BatchJob *jobs, unsigned int *guard, int depth,
+                                   const SavedWalks &src, unsigned long long *steps_out, bool screened,
+                                   cudaStream_t s);
 // lanes: lanes per walk, 1 (binary trees) or 8 (8-lane teams over the 8-wide
 // trees; Poisson solves)
 cudaError_t launch_walk_persistent(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, int block,
-                                   int blocks, cudaStream_t s, int lanes = 1, const HandOver &ho = HandOver{});
+                                   int blocks, cudaStream_t s, int lanes = 1, const SavedWalks &src = SavedWalks{},
+                                   const HandOver &ho = HandOver{});
 // one walk per warp: `walks` walks (an upper bound), saved ones or the solve's own
-cudaError_t launch_walk_warp(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, const TailWalks &tw,
-                             uint64_t walks, cudaStream_t s);
+cudaError_t launch_walk_warp(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
+                             const SavedWalks &src, uint64_t walks, cudaStream_t s);
+// all of a solve's walks (src.slots null), or `walks` saved ones at most, to
+// their ends: launches that hand the remaining walks over to one another
+// (block, blocks: the persistent kernel's resident grid)
+cudaError_t launch_walk_chain(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, SavedWalks src,
+                              uint64_t walks, const ChainBuffers &cb, int block, int blocks, cudaStream_t s);
+// slots that the chain's slot array `which` (0, 1) has to hold
+uint64_t chain_capacity(uint64_t walks, int block, int blocks, int which);
 // resumable solves: grid of the fixed launch, its walk slots, one launch
 cudaError_t resume_grid(int dim, int block, int depth, int *blocks_out, int lanes = 1);
 int64_t resume_slots(int block, int blocks, int lanes = 1);

@@ -36,26 +36,61 @@ cudaError_t batch_grid(int dim, int block, int depth, int *blocks_out) {
         e = dim == 2 ? occupancy<2, false>(block, sm, &per_sm_p) : occupancy<3, false>(block, sm, &per_sm_p);
     if (e != cudaSuccess) return e;
     per_sm = std::min(per_sm, per_sm_p);
+    // the warp kernels that end a batch are loaded now, not while a graph is captured
+    for (int scr = 0; scr < 2 && e == cudaSuccess; ++scr) e = prepare_walk_warp_batch(dim, depth, scr != 0);
+    if (e != cudaSuccess) return e;
     *blocks_out = sms * (per_sm > 0 ? per_sm : 1);
     return cudaSuccess;
 }
 
+namespace {
+
+template <int D, bool SCR>
+cudaError_t launch(const BatchHeader *hdr, const BatchJob *jobs, unsigned long long *counter, unsigned int *guard,
+                   int depth, const int *cancel, int block, int blocks, cudaStream_t s, unsigned long long *steps_out,
+                   const SavedWalks &src, const HandOver &ho) {
+    k_walk_batch<D, SCR><<<blocks, block, smem_bytes(depth, block), s>>>(hdr, jobs, counter, guard, depth, cancel,
+                                                                         steps_out, src, ho);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+uint64_t batch_chain_capacity(int block, int blocks, int which) {
+    return std::max<uint64_t>(kTailWalks, ((uint64_t)blocks * (uint64_t)block) >> (which + 1));
+}
+
+// As launch_walk_chain, without knowing how many walks the launch will hold
+// (a captured graph is replayed over other tables): a launch that begins
+// with fewer walks than it would hand over hands them over at once.
 cudaError_t launch_walk_batch(int dim, const BatchHeader *hdr, const BatchJob *jobs, unsigned long long *counter,
                               unsigned int *guard, int depth, const int *cancel, int block, int blocks,
-                              cudaStream_t s, unsigned long long *steps_out, bool screened) {
-    const size_t sm = smem_bytes(depth, block);
-    if (dim == 2) {
-        if (screened)
-            k_walk_batch<2, true><<<blocks, block, sm, s>>>(hdr, jobs, counter, guard, depth, cancel, steps_out);
-        else
-            k_walk_batch<2, false><<<blocks, block, sm, s>>>(hdr, jobs, counter, guard, depth, cancel, steps_out);
-    } else {
-        if (screened)
-            k_walk_batch<3, true><<<blocks, block, sm, s>>>(hdr, jobs, counter, guard, depth, cancel, steps_out);
-        else
-            k_walk_batch<3, false><<<blocks, block, sm, s>>>(hdr, jobs, counter, guard, depth, cancel, steps_out);
+                              const ChainBuffers &cb, cudaStream_t s, unsigned long long *steps_out, bool screened) {
+    SavedWalks src{};
+    const uint64_t resident = (uint64_t)blocks * (uint64_t)block;
+    uint64_t walks = ~0ull;
+    for (int stage = 0; stage < kMaxStages && walks > kTailWalks; ++stage) {
+        const int b = stage & 1;
+        const uint64_t held = std::min(walks, resident);
+        uint64_t most = held / 2 < kTailWalks * 3 / 2 ? kTailWalks : held / 2;
+        most = std::min<uint64_t>(most, cb.cap[b]);
+        unsigned int *ctr = cb.counters + 2 * stage;
+        const int grid = walks == ~0ull ? blocks : (int)std::min<uint64_t>((uint64_t)blocks, (walks + block - 1) / block);
+        const HandOver ho{cb.slots[b], ctr, (unsigned)most, (unsigned)grid * (unsigned)block};
+        cudaError_t e =
+            dim == 2 ? (screened ? launch<2, true>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
+                                                   src, ho)
+                                 : launch<2, false>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
+                                                    src, ho))
+                     : (screened ? launch<3, true>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
+                                                   src, ho)
+                                 : launch<3, false>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
+                                                    src, ho));
+        if (e != cudaSuccess) return e;
+        src = SavedWalks{cb.slots[b], nullptr, ctr, ctr + 1, nullptr};
+        walks = most;
     }
-    return cudaGetLastError();
+    return launch_walk_warp_batch(dim, hdr, jobs, guard, depth, src, steps_out, screened, s);
 }
 
 }  // namespace wost

@@ -41,8 +41,9 @@ cudaError_t launch_walk_count_scr(const SceneView &sc, const SolveParams &sp, co
     return walk_count_launch<true>(sc, sp, acc, stats, block, s);
 }
 cudaError_t launch_walk_persistent_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
-                                       const HandOver &ho, int block, int blocks, cudaStream_t s) {
-    return walk_persistent_launch<true, 1>(sc, sp, acc, ho, block, blocks, s);
+                                       const SavedWalks &src, const HandOver &ho, int block, int blocks,
+                                       cudaStream_t s) {
+    return walk_persistent_launch<true, 1>(sc, sp, acc, src, ho, block, blocks, s);
 }
 cudaError_t launch_walk_resume_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                    const ResumeState &rs, int iters, int block, int blocks, cudaStream_t s) {

@@ -16,7 +16,7 @@ cudaError_t persistent_grid_team(int dim, int block, int depth, int *blocks_out)
 
 cudaError_t launch_walk_persistent_team(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                         int block, int blocks, cudaStream_t s) {
-    return walk_persistent_launch<false, WOST_WIDE>(sc, sp, acc, HandOver{}, block, blocks, s);
+    return walk_persistent_launch<false, WOST_WIDE>(sc, sp, acc, SavedWalks{}, HandOver{}, block, blocks, s);
 }
 
 cudaError_t launch_walk_resume_team(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,

@@ -7,8 +7,21 @@
 namespace wost {
 
 cudaError_t launch_walk_warp_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
-                                 const TailWalks &tw, uint64_t walks, cudaStream_t s) {
-    return walk_warp_launch<true>(sc, sp, acc, tw, walks, s);
+                                 const SavedWalks &src, uint64_t walks, cudaStream_t s) {
+    return walk_warp_launch<true>(sc, sp, acc, src, walks, s);
+}
+
+cudaError_t launch_walk_warp_batch_scr(int dim, const BatchHeader *hdr, const BatchJob *jobs, unsigned int *guard,
+                                       int depth, const SavedWalks &src, unsigned long long *steps_out,
+                                       cudaStream_t s) {
+    return dim == 2 ? warp_batch_launch<2, true>(hdr, jobs, guard, depth, src, steps_out, s)
+                    : warp_batch_launch<3, true>(hdr, jobs, guard, depth, src, steps_out, s);
+}
+
+cudaError_t prepare_walk_warp_batch_scr(int dim, int depth) {
+    size_t sm = 0;
+    int blocks = 0;
+    return dim == 2 ? warp_batch_grid<2, true>(depth, 64, &sm, &blocks) : warp_batch_grid<3, true>(depth, 64, &sm, &blocks);
 }
 
 }  // namespace wost

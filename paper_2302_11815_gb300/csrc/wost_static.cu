@@ -9,7 +9,7 @@
 // kernel, but its FP64 accumulators and work counters live in one fixed
 // device array of this library, g_static_scratch, sized for
 // WOST_STATIC_MAX_POINTS points; every device that loads the library holds
-// that array (about 2 MiB) until the process exits.
+// that array (about 3.7 MiB) until the process exits.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -23,11 +23,16 @@ namespace wost {
 //   [8, 16)   next-walk counter of the persistent kernel (u64)
 //   [16, 20)  guard flags (u32)
 //   [20, 24)  cancel flag (i32, never set by this entry point)
+//   [32, 96)  hand-over counters of the chain of launches (u32 pairs)
 //   [256, ..) per point: walk-sum, sum of squares (f64), walk count, step
-//             count (u64), four arrays of WOST_STATIC_MAX_POINTS entries
+//             count (u64), four arrays of WOST_STATIC_MAX_POINTS entries;
+//             then the chain's two slot arrays (48 bytes a slot)
 constexpr size_t kHeader = 256;
 constexpr size_t kArray = 8 * (size_t)WOST_STATIC_MAX_POINTS;
-constexpr size_t kScratchBytes = kHeader + 4 * kArray;
+constexpr unsigned kSlots0 = 20480, kSlots1 = kTailWalks;
+constexpr size_t kSlotBytes = 3 * sizeof(float4);
+constexpr size_t kScratchBytes = kHeader + 4 * kArray + (kSlots0 + kSlots1) * kSlotBytes;
+static_assert(32 + 2 * kMaxStages * sizeof(unsigned int) <= kHeader, "hand-over counters fit the header");
 
 static __device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
 
@@ -116,7 +121,13 @@ extern "C" wost_status wost_solve_static(wost_scene *scene, int64_t n_points, co
     const int block = scene->tuned_block ? scene->tuned_block : 128;
     int blocks = 0;
     CK(persistent_grid(scene->view.dim, block, sp.stack_depth, &blocks), "occupancy");
-    CK(launch_walk_persistent(scene->view, sp, acc, block, blocks, stream), "kernel launch");
+    unsigned char *slots = s + kHeader + 4 * kArray;
+    const ChainBuffers cb{{(float4 *)slots, (float4 *)(slots + kSlots0 * kSlotBytes)},
+                          {kSlots0, kSlots1},
+                          (unsigned int *)(s + 32)};
+    CK(launch_walk_chain(scene->view, sp, acc, SavedWalks{}, (uint64_t)n_points * (uint64_t)walks_per_point, cb, block,
+                         blocks, stream),
+       "kernel launch");
     k_static_finish<<<(unsigned)((n + 255) / 256), 256, 0, stream>>>(s, n_points, mean_out, stderr_out);
     CK(cudaGetLastError(), "kernel launch");
     return WOST_OK;

@@ -102,11 +102,13 @@ __device__ __forceinline__ void accumulate(const Accumulators &acc, const Walk &
     if (w.capped) atomicAdd(acc.capped, 1ull);
 }
 
-// saved walks (layout: ResumeState)
-__device__ __forceinline__ bool load_walk(const float4 *slot, Walk &w) {
+// saved walks (layout: ResumeState); taking one empties its slot
+__device__ __forceinline__ bool load_walk(float4 *slot, Walk &w, int *job = nullptr, bool empty_it = true) {
     const float4 c = slot[2];
     const uint32_t flags = __float_as_uint(c.w);
     if (!(flags & 1u)) return false;
+    if (empty_it) slot[2] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (job) *job = (int)(flags >> 8);
     const float4 a = slot[0], b = slot[1];
     w.x = mk(a.x, a.y, a.z);
     w.acc = a.w;
@@ -119,8 +121,8 @@ __device__ __forceinline__ bool load_walk(const float4 *slot, Walk &w) {
     w.capped = (flags & 4u) != 0;
     return true;
 }
-__device__ __forceinline__ void save_walk(float4 *slot, const Walk &w) {
-    const uint32_t flags = 1u | (w.onN ? 2u : 0u) | (w.capped ? 4u : 0u);
+__device__ __forceinline__ void save_walk(float4 *slot, const Walk &w, int job = 0) {
+    const uint32_t flags = 1u | (w.onN ? 2u : 0u) | (w.capped ? 4u : 0u) | ((uint32_t)job << 8);
     slot[0] = make_float4(w.x.x, w.x.y, w.x.z, w.acc);
     slot[1] = make_float4(w.n.x, w.n.y, w.n.z, w.dbound);
     slot[2] = make_float4(__uint_as_float((uint32_t)w.steps), __uint_as_float(w.point), __uint_as_float(w.index),
@@ -176,13 +178,34 @@ __global__ void WOST_WALK_BOUNDS k_walk_plain(const SceneView sc, const SolvePar
     }
 }
 
+// Hands the walks of this warp over (true) once nothing is left to draw and
+// at most ho.most walks are left.  Every lane that finds nothing to draw has
+// added 1 to the counter, once, so the counter tells how many hold a walk.
+template <class CTR>
+__device__ __forceinline__ bool hand_over(const HandOver &ho, const CTR *counter, unsigned long long total, int lane,
+                                          const Walk &w, bool have, unsigned held, int job) {
+    const unsigned FULL = 0xffffffffu;
+    unsigned first = 0xffffffffu;
+    if (lane == 0) {
+        const unsigned long long drawn = *(volatile const CTR *)counter;
+        if (drawn >= total && ho.lanes - (unsigned)(drawn - total) <= ho.most)
+            first = atomicAdd(ho.count, (unsigned)__popc(held));
+    }
+    first = __shfl_sync(FULL, first, 0);
+    if (first == 0xffffffffu) return false;
+    if (have) save_walk(ho.slots + 3 * (size_t)(first + __popc(held & ((1u << lane) - 1u))), w, job);
+    return true;
+}
+
 template <int D, bool SCR, int T>
 __global__ void WOST_WALK_BOUNDS k_walk_persistent(const SceneView sc, const SolveParams sp,
-                                                         const Accumulators acc, const HandOver ho) {
+                                                         const Accumulators acc, const SavedWalks src,
+                                                         const HandOver ho) {
     Cnt<false> cnt;
     auto q = make_q<D, false, T>(sp.stack_depth, acc.guard, cnt, sp.visit_limit);
     const Group g = make_team<T>();
-    const uint64_t total = (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
+    const uint64_t total =
+        src.slots ? (uint64_t)*src.count : (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
     Walk w{};
@@ -201,42 +224,39 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const SceneView sc, const Sol
             int lead = __ffs(need) - 1;
             unsigned long long base = 0;
             if (lane == lead) {
-                bool stop = *(volatile int *)acc.cancel != 0;
-                base = stop ? total : atomicAdd(acc.next_walk, (unsigned long long)__popc(need));
+                if (src.slots) {
+                    base = atomicAdd(src.next, (unsigned)__popc(need));
+                } else {
+                    bool stop = *(volatile int *)acc.cancel != 0;
+                    base = stop ? total : atomicAdd(acc.next_walk, (unsigned long long)__popc(need));
+                }
             }
             base = __shfl_sync(FULL, base, lead);
             if ((need >> g.base) & 1u) {
                 unsigned long long my = base + __popc(need & ((1u << g.base) - 1u));
-                if (my < total) {
+                if (my >= total) {
+                    drained = true;
+                } else if (src.slots) {
+                    have = load_walk(src.slots + 3 * (size_t)(src.list ? src.list[my] : (uint32_t)my), w);
+                } else {
                     int64_t pt = (int64_t)(my / (uint64_t)sp.walks_per_point);
                     uint32_t j = (uint32_t)(my % (uint64_t)sp.walks_per_point) + sp.first_walk;
                     walk_init<D>(sp, w, pt, j);
                     have = true;
-                } else {
-                    drained = true;
                 }
             }
         }
         const unsigned held = __ballot_sync(FULL, have);
-        if (!held) break;
-        if constexpr (T == 1) {
-            // Once this warp has found the counter exhausted: every lane of
-            // the launch has failed once to draw (adding 1 to the counter)
-            // or holds a walk, so the counter tells how many are left.
-            if (ho.slots && held != FULL) {
-                unsigned first = 0xffffffffu;
-                if (lane == 0) {
-                    const unsigned long long drawn = *(volatile unsigned long long *)acc.next_walk;
-                    if (drawn >= total && ho.lanes - (unsigned)(drawn - total) <= ho.most)
-                        first = atomicAdd(ho.count, (unsigned)__popc(held));
-                }
-                first = __shfl_sync(FULL, first, 0);
-                if (first != 0xffffffffu) {
-                    if (have) save_walk(ho.slots + 3 * (size_t)(first + __popc(held & ((1u << lane) - 1u))), w);
-                    break;
-                }
-            }
+        if (!held) {
+            if (__any_sync(FULL, !drained)) continue;
+            break;
         }
+        if constexpr (T == 1) {
+            if (ho.slots && (src.slots ? hand_over(ho, src.next, total, lane, w, have, held, 0)
+                                       : hand_over(ho, acc.next_walk, total, lane, w, have, held, 0)))
+                break;
+        }
+        if (src.steps_run && lane == 0) atomicAdd(src.steps_run, (unsigned long long)__popc(held));
         if (walk_step<D, SCR>(sc, sp, w, q, have)) {
             if (g.leader()) accumulate(acc, w);
             have = false;
@@ -263,7 +283,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_resume(const SceneView sc, const SolvePa
     float4 *slot = rs.slots + 3 * (((size_t)blockIdx.x * blockDim.x + threadIdx.x) / T);
     Walk w{};
     bool have = false, drained = false;  // uniform within a team
-    have = load_walk(slot, w);
+    have = load_walk(slot, w, nullptr, false);
     unsigned long long ran = 0;
     for (int it = 0; it < iters; ++it) {
         unsigned need = __ballot_sync(FULL, g.leader() && !have && !drained);
@@ -407,16 +427,16 @@ static cudaError_t resident_grid(const void *k, int block, int depth, int *block
 
 template <bool SCR, int T>
 static cudaError_t walk_persistent_launch(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
-                                          const HandOver &ho, int block, int blocks, cudaStream_t s) {
+                                          const SavedWalks &src, const HandOver &ho, int block, int blocks, cudaStream_t s) {
     size_t sm = smem_bytes(sp.stack_depth, block, T);
     const void *k =
         sc.dim == 2 ? (const void *)k_walk_persistent<2, SCR, T> : (const void *)k_walk_persistent<3, SCR, T>;
     cudaError_t e = smem_limit(k, sm);
     if (e != cudaSuccess) return e;
     if (sc.dim == 2)
-        k_walk_persistent<2, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc, ho);
+        k_walk_persistent<2, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc, src, ho);
     else
-        k_walk_persistent<3, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc, ho);
+        k_walk_persistent<3, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc, src, ho);
     return cudaGetLastError();
 }
 
@@ -440,11 +460,15 @@ cudaError_t launch_walk_plain_scr(const SceneView &sc, const SolveParams &sp, co
 cudaError_t launch_walk_count_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                   unsigned long long *stats, int block, cudaStream_t s);
 cudaError_t launch_walk_persistent_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
-                                       const HandOver &ho, int block, int blocks, cudaStream_t s);
+                                       const SavedWalks &src, const HandOver &ho, int block, int blocks, cudaStream_t s);
 cudaError_t launch_walk_warp_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
-                                 const TailWalks &tw, uint64_t walks, cudaStream_t s);
+                                 const SavedWalks &src, uint64_t walks, cudaStream_t s);
 cudaError_t launch_walk_resume_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                    const ResumeState &rs, int iters, int block, int blocks, cudaStream_t s);
+cudaError_t launch_walk_warp_batch_scr(int dim, const BatchHeader *hdr, const BatchJob *jobs, unsigned int *guard,
+                                       int depth, const SavedWalks &src, unsigned long long *steps_out,
+                                       cudaStream_t s);
+cudaError_t prepare_walk_warp_batch_scr(int dim, int depth);
 // 8-lane team instantiations (Poisson), defined in wost_kernels_team.cu
 cudaError_t persistent_grid_team(int dim, int block, int depth, int *blocks_out);
 cudaError_t launch_walk_persistent_team(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,

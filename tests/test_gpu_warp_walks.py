@@ -109,3 +109,38 @@ def test_warp_walks_from_boundary_points(wost):
         nrm = torch.from_numpy(scenes.prim_normals(sc)[sel].astype(np.float32)).cuda()
         on = torch.ones(len(sel), dtype=torch.uint8, device="cuda")
         _both(wost, sc, 0, 0.0, pts, 40, "persistent", normals=nrm, on_neumann=on)
+
+
+@pytest.mark.parametrize("n,walks", [(300, 64), (900, 400), (3000, 160)])
+def test_handed_over_walks_are_the_one_lane_walks(wost, n, walks):
+    """Solves larger than one warp per walk: their last walks pass through one
+    or more hand-overs (a few thousand walks to more than the GPU's lanes)."""
+    for name in ("flower", "koch3", "disk_screened", "box_sphere"):
+        make, leaf, sigma = CASES[name]
+        sc = make()
+        for kernel in ("persistent", "resumable"):
+            _both(wost, sc, leaf, sigma, _points(sc, n, np.random.default_rng(11)), walks, kernel, cap=600)
+
+
+def test_static_solve_and_batch_hand_over_to_warps(wost):
+    specs = [CASES[k][0]() for k in ("flower", "koch3", "box_sphere", "cube_torus")]
+    S = [wost.Scene(sc) for sc in specs]
+    n, walks = [700, 300, 900, 200], [64, 96, 48, 80]
+    pts = [torch.from_numpy(_points(sc, k, np.random.default_rng(5))).cuda() for sc, k in zip(specs, n)]
+    ref = [wost.solve(s, p, w, 1e-3, 1e-3, 1024, seed=9 + i, kernel="persistent",
+                      stack_depth=s.info()["stack_depth"]) for i, (s, p, w) in enumerate(zip(S, pts, walks))]
+    hs = wost.wost_solve_batch([s.handle for s in S],
+                               [dict(points=p, walks_per_point=w, epsilon=1e-3, r_min=1e-3, max_steps=1024, seed=9 + i)
+                                for i, (p, w) in enumerate(zip(pts, walks))])
+    for h, r, k in zip(hs, ref, n):
+        wost.wost_wait(h, 120)
+        mean, _, wd, pr = wost.wost_poll(h, k)
+        wost.wost_solve_destroy(h)
+        assert np.array_equal(wd, r["walks"]) and pr["total_steps"] == r["total_steps"]
+        np.testing.assert_allclose(mean, r["mean"], rtol=1e-9, atol=1e-12)
+    for i, (s, p, w, r) in enumerate(zip(S, pts, walks, ref)):
+        mean = torch.empty(len(p), device="cuda")
+        for _ in range(2):  # the scratch array keeps the first call's contents
+            wost.wost_solve_static(s.handle, p, w, 1e-3, 1e-3, 1024, 9 + i, 0, mean)
+        np.testing.assert_array_equal(mean.cpu().numpy(), r["mean"].astype(np.float32))
+        s.close()
