@@ -390,10 +390,89 @@ struct WideFlattener {
     }
 };
 
+// The top of the wide tree as up to 32 subtrees: the root's children, the
+// largest inner ones replaced by their own children while they fit (build
+// nodes; every one is a wide node or a wide leaf).
+std::vector<int> open_top(const std::vector<BNode> &bn, const WideFlattener &wf, int root, int dim) {
+    if (wf.is_wide_leaf(root)) return {root};
+    std::vector<int> top = wf.slots[0];
+    for (;;) {
+        int best = -1;
+        float area = -1;
+        for (size_t i = 0; i < top.size(); ++i) {
+            if (wf.is_wide_leaf(top[i])) continue;
+            if (top.size() - 1 + wf.slots[wf.wide_of[top[i]]].size() > 32) continue;
+            float a = area_measure(bn[top[i]].lo, bn[top[i]].hi, dim);
+            if (a > area) {
+                area = a;
+                best = (int)i;
+            }
+        }
+        if (best < 0) return top;
+        const std::vector<int> ch = wf.slots[wf.wide_of[top[best]]];
+        top[best] = ch[0];
+        top.insert(top.end(), ch.begin() + 1, ch.end());
+    }
+}
+
+// the two child references of a flattened binary node
+void child_refs(const std::vector<float4> &nodes, int dim, uint32_t i, uint32_t r[2]) {
+    const float4 &q = nodes[4 * (size_t)i + (dim == 2 ? 2 : 3)];
+    std::memcpy(&r[0], &q.x, 4);
+    std::memcpy(&r[1], &q.y, 4);
+}
+
+// Five-level treelets of a binary tree (layout: wost_internal.h).
+void make_treelets(HostTree &t, int dim) {
+    t.treelets.clear();
+    if (t.root == WOST_EMPTY_REF || (t.root & WOST_LEAF_BIT)) return;
+    std::vector<uint32_t> roots{t.root};
+    for (size_t k = 0; k < roots.size(); ++k) {
+        uint32_t heap[63];
+        std::fill(heap, heap + 63, WOST_EMPTY_REF);
+        heap[0] = roots[k];
+        const size_t base = t.treelets.size();
+        t.treelets.resize(base + 64, WOST_EMPTY_REF);
+        for (int j = 0; j < 31; ++j) {
+            if (heap[j] == WOST_EMPTY_REF) continue;
+            t.treelets[base + j] = heap[j];
+            uint32_t r[2];
+            child_refs(t.nodes, dim, heap[j], r);
+            for (int c = 0; c < 2; ++c)
+                if (!(r[c] & WOST_LEAF_BIT)) heap[2 * j + 1 + c] = r[c];
+        }
+        for (int j = 31; j < 63; ++j)
+            if (heap[j] != WOST_EMPTY_REF) {
+                t.treelets[base + 32 + (j - 31)] = (uint32_t)roots.size();
+                roots.push_back(heap[j]);
+            }
+    }
+}
+
+// Where every binary node and every record's leaf hangs.
+void make_parents(HostTree &t, int dim) {
+    t.parents.assign(std::max(t.n_nodes, 1), WOST_EMPTY_REF);
+    t.leaf_parents.assign(std::max(t.n_prims, 1), WOST_EMPTY_REF);
+    for (int i = 0; i < t.n_nodes; ++i) {
+        uint32_t r[2];
+        child_refs(t.nodes, dim, (uint32_t)i, r);
+        for (uint32_t c = 0; c < 2; ++c) {
+            const uint32_t at = (uint32_t)i * 2u + c;
+            if (!(r[c] & WOST_LEAF_BIT)) {
+                t.parents[r[c]] = at;
+            } else {
+                const uint32_t first = (r[c] & 0x7FFFFFFFu) >> 4, count = (r[c] & 15u) + 1u;
+                for (uint32_t k = first; k < first + count; ++k) t.leaf_parents[k] = at;
+            }
+        }
+    }
+}
+
 // Builds one tree over `items` (records 0..n-1) and returns the leaf order of
 // the records (perm[k] = record stored at position k).
 std::vector<int> build_tree(std::vector<Item> &items, int dim, int leaf, HostTree &t,
-                            std::vector<BNode> *keep_nodes, int *root_out, const std::vector<OCone> *cones = nullptr) {
+                            std::vector<BNode> *keep_nodes, int *root_out, const std::vector<OCone> *cones = nullptr,
+                            std::vector<int> *top_out = nullptr) {
     t.n_prims = (int)items.size();
     std::vector<int> perm(items.size());
     if (items.empty()) {
@@ -417,6 +496,16 @@ std::vector<int> build_tree(std::vector<Item> &items, int dim, int leaf, HostTre
     t.wdepth = wf.depth + 1;
     t.wslots = wf.slots;
     t.wide_of = wf.wide_of;
+    const std::vector<int> top = open_top(b.nodes_, wf, root, dim);
+    t.wtop.assign(64, f4(INFINITY, INFINITY, INFINITY, ibits(WOST_EMPTY_REF)));
+    for (size_t c = 0; c < 32; ++c) {
+        t.wtop[2 * c + 1] = f4(-INFINITY, -INFINITY, -INFINITY, 0);
+        if (c >= top.size()) continue;
+        const BNode &n = b.nodes_[top[c]];
+        t.wtop[2 * c] = f4(n.lo[0], n.lo[1], n.lo[2], ibits(wf.ref_of(top[c])));
+        t.wtop[2 * c + 1] = f4(n.hi[0], n.hi[1], n.hi[2], 0);
+    }
+    if (top_out) *top_out = top;
     for (int a = 0; a < 3; ++a) {
         t.root_lo[a] = b.nodes_[root].lo[a];
         t.root_hi[a] = b.nodes_[root].hi[a];
@@ -604,6 +693,8 @@ std::string build_scene(const wost_scene_desc &d, HostScene &S) {
         for (size_t i = 0; i < Dl.size(); ++i) items[i] = prim_item(Dl[i], (int)i);
         auto perm = build_tree(items, dim, leaf, S.D, nullptr, nullptr);
         fill_prims(Dl, perm, d.g, d.g_minus, false, S.D);
+        make_parents(S.D, dim);
+        S.D.parents.clear();
     }
     // --- Neumann BVH ---
     {
@@ -611,6 +702,7 @@ std::string build_scene(const wost_scene_desc &d, HostScene &S) {
         for (size_t i = 0; i < Nl.size(); ++i) items[i] = prim_item(Nl[i], (int)i);
         auto perm = build_tree(items, dim, leaf, S.N, nullptr, nullptr);
         fill_prims(Nl, perm, d.h, d.h_minus, true, S.N);
+        make_treelets(S.N, dim);
     }
     // --- silhouette candidates and their cone hierarchy ---
     struct Sil {
@@ -686,13 +778,20 @@ std::string build_scene(const wost_scene_desc &d, HostScene &S) {
         }
         std::vector<BNode> bn;
         int root = -1;
-        auto perm = build_tree(items, dim, leaf, S.S, &bn, &root, d.silhouette_split == 1 ? nullptr : &icones);
+        std::vector<int> top;
+        auto perm = build_tree(items, dim, leaf, S.S, &bn, &root, d.silhouette_split == 1 ? nullptr : &icones, &top);
+        make_parents(S.S, dim);
         size_t n = sil.size();
+        std::vector<int32_t> n_rec(np, -1);  // N record of each primitive
+        for (size_t k = 0; k < S.N.ids.size(); ++k) n_rec[S.N.ids[k]] = (int32_t)k;
+        S.N.hints.assign(std::max<size_t>(S.N.ids.size(), 1), 0);
         S.S.prims.assign(n * (dim == 2 ? 2 : 3), f4(0, 0, 0, 0));
         S.S.ids.resize(n);
         for (size_t k = 0; k < n; ++k) {
             const Sil &s = sil[perm[k]];
             S.S.ids[k] = (int32_t)s.a;
+            S.N.hints[n_rec[s.f0]] = (uint32_t)k;
+            if (s.f1 >= 0) S.N.hints[n_rec[s.f1]] = (uint32_t)k;
             V3 n0 = nrm[s.f0];
             V3 n1 = s.f1 >= 0 ? nrm[s.f1] : V3{0, 0, 0};
             V3 pa = V(s.a);
@@ -740,6 +839,8 @@ std::string build_scene(const wost_scene_desc &d, HostScene &S) {
                 const std::vector<int> &ch = S.S.wslots[i];
                 for (size_t c = 0; c < ch.size(); ++c) S.S.wcones[i * WOST_WIDE + c] = cf(cones[ch[c]]);
             }
+            S.S.wtopcones.assign(32, f4(0, 0, 1, -1));
+            for (size_t c = 0; c < top.size(); ++c) S.S.wtopcones[c] = cf(cones[top[c]]);
         } else {
             S.S.root_cone = f4(0, 0, 1, -1);
         }

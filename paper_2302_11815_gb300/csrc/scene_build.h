@@ -26,6 +26,13 @@ struct HostTree {
     int wn_nodes = 0, wdepth = 0;
     std::vector<std::vector<int>> wslots;  // build-time only: binary children of each wide node
     std::vector<int> wide_of;
+    // one-walk-per-warp searches: the top of the wide tree as up to 32
+    // subtrees (child layout of a wide node; unused entries: the empty
+    // reference), their cones (S); the parents of S's binary nodes
+    // and of D's and S's leaves; the five-level treelets and the silhouette hints of N
+    // (wost_internal.h)
+    std::vector<float4> wtop, wtopcones;
+    std::vector<uint32_t> parents, leaf_parents, treelets, hints;
 };
 
 struct HostScene {

@@ -87,6 +87,20 @@ wost_status wost_scene_create(const wost_scene_desc *desc, wost_scene **out) {
             CK(upload(w[0], T.wnodes), "upload wide nodes");
             CK(upload(w[1], T.wcones), "upload wide cones");
             bytes += (int64_t)(w[0].bytes + w[1].bytes);
+            DevBuf *x = &s->xbufs[6 * t];
+            CK(upload(x[0], T.wtop), "upload wide top");
+            CK(upload(x[1], T.wtopcones), "upload wide top");
+            CK(upload(x[2], T.parents), "upload parents");
+            CK(upload(x[3], T.leaf_parents), "upload parents");
+            CK(upload(x[4], T.treelets), "upload treelets");
+            CK(upload(x[5], T.hints), "upload hints");
+            for (int k = 0; k < 6; ++k) bytes += (int64_t)x[k].bytes;
+            V.hints = (const uint32_t *)x[5].p;
+            V.wtop = (const float4 *)x[0].p;
+            V.wtopcones = (const float4 *)x[1].p;
+            V.parents = (const uint32_t *)x[2].p;
+            V.leaf_parents = (const uint32_t *)x[3].p;
+            V.treelets = (const uint32_t *)x[4].p;
             V.wnodes = (const float4 *)w[0].p;
             V.wcones = (const float4 *)w[1].p;
             V.wroot = T.wroot;
@@ -123,6 +137,11 @@ wost_status wost_scene_create(const wost_scene_desc *desc, wost_scene **out) {
                 if (a < H.dim) d2 += (H.hi[a] - H.lo[a]) * (H.hi[a] - H.lo[a]);
             }
             s->view.rmax = std::sqrt(d2);
+            float c = 0.f;
+            for (const TreeView *V : {&s->view.D, &s->view.N})
+                for (int a = 0; a < 3; ++a) c = std::max(c, std::max(std::fabs(V->root_lo[a]), std::fabs(V->root_hi[a])));
+            s->view.scale = c;
+            s->view.tau = 6e-7f * c;
         }
         // binary trees: one pending subtree per level
         s->stack_depth = std::max(H.D.depth, std::max(H.N.depth, H.S.depth)) + 2;
@@ -719,7 +738,8 @@ static wost_status advance_waiting(wost_solve_handle *h) {
         unsigned int live = 0;
         wost_status st = resumable_finished(h, &fin, &drained, &live);
         if (st != WOST_OK || fin) return st;
-        if (!drained) return advance_locked(h, 2048, h->stream);
+        if (!drained || live > (uint64_t)resume_slots(h->block, h->resume_blocks, 1))
+            return advance_locked(h, 2048, h->stream);
         src = SavedWalks{(float4 *)h->slots.p, ctr + 2, ctr, ctr + 1, steps_run};
         walks = live;
     } else {

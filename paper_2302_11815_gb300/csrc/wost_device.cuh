@@ -389,6 +389,15 @@ __device__ __forceinline__ bool prim_ray(const Prim<D> &p, P3 o, P3 v, float tma
     }
 }
 
+// squared distance of record k (out of line: a second opinion, not a hot loop)
+template <int D>
+__device__ __noinline__ float prim_dist2(const float4 *prims, uint32_t k, P3 x) {
+    const Prim<D> p = load_prim<D>(prims, k);
+    float s0, s1;
+    const P3 dq = prim_closest<D>(p, x, s0, s1) - x;
+    return dotp<D>(dq, dq);
+}
+
 // ---------------------------------------------------------------------------
 // Q.1 closest point on the Dirichlet boundary
 // ---------------------------------------------------------------------------
@@ -420,6 +429,7 @@ __device__ Closest q_closest(const TreeView &T, P3 x, const Stack &st, Cnt<CN> &
         if (over_visit_limit(visits, T.n_nodes, st.guard, st.visit_limit)) break;
         if (is_leaf(ref)) {
             uint32_t f = leaf_first(ref), c = leaf_count(ref);
+#pragma unroll 1
             for (uint32_t k = f; k < f + c; ++k) {
                 cnt.prim(C_Q1);
                 Prim<D> p = load_prim<D>(T.prims, k);
@@ -521,21 +531,62 @@ __device__ __forceinline__ float sil_test(const float4 *prims, uint32_t k, P3 x,
     return INFINITY;
 }
 
+// Rounding of a distance.  A computed closest point lies within ~3 ulp of the
+// largest coordinate of its primitive's box, so a box's computed distance
+// exceeds that of a primitive in it by at most tau1, and a traversal can miss
+// a primitive only in favour of one less than tau1 farther.  With tau = 4
+// tau1 (SceneView::tau): beyond(d2) is a bound (on squared distances) above
+// the square of distance + 2 tau (4 tau d <= d^2 / 1000 + 4000 tau^2).  A
+// traversal that starts with beyond(the distance of some record it reaches)
+// instead of its own bound gives the same bits: what it no longer visits lies
+// farther than the answer by more than can prune, or be pruned by, any record
+// that ties with the answer.
+__device__ __forceinline__ float beyond(float d2, float tau) { return fmaf(d2, 1.002f, 4200.f * tau * tau); }
+
+// Squared distance of silhouette candidate k if it is one from x for certain:
+// not grazing, i.e. the view direction farther from both normals' planes than
+// the cone test's padding can lose in single precision (a cone's half angle
+// of 3.4e-4 or less rounds to 0), so that no cone that holds them is culled.
+// A boundary candidate (n1 = 0) is never culled.  Else +inf.
+template <int D>
+__device__ __noinline__ float sil_certain(const float4 *prims, uint32_t k, P3 x) {
+    P3 pe, n0, n1;
+    if constexpr (D == 2) {
+        const float4 q0 = __ldg(prims + 2 * (size_t)k), q1 = __ldg(prims + 2 * (size_t)k + 1);
+        pe = mk(q0.x, q0.y, 0.f);
+        n0 = mk(q1.x, q1.y, 0.f);
+        n1 = mk(q1.z, q1.w, 0.f);
+    } else {
+        const float4 q0 = __ldg(prims + 3 * (size_t)k), q1 = __ldg(prims + 3 * (size_t)k + 1),
+                     q2 = __ldg(prims + 3 * (size_t)k + 2);
+        const P3 a = mk(q0.x, q0.y, q0.z), b = mk(q1.x, q1.y, q1.z);
+        n0 = mk(q0.w, q1.w, q2.x);
+        n1 = mk(q2.y, q2.z, q2.w);
+        pe = a + (b - a) * seg_param(a, b, x, 1);
+    }
+    const P3 v = pe - x;
+    const float d2 = dotp<D>(v, v), a0 = dotp<D>(v, n0), a1 = dotp<D>(v, n1);
+    if (n1.x == 0.f && n1.y == 0.f && n1.z == 0.f) return d2;
+    const float lim2 = 1.6e-7f * d2;
+    return a0 * a1 <= 0.f && a0 * a0 > lim2 && a1 * a1 > lim2 ? d2 : INFINITY;
+}
+
 template <int D, bool CN = false>
 __device__ float q_silhouette(const TreeView &T, P3 x, float rmax, const Stack &st, Cnt<CN> &cnt) {
+    bool found = false;
     float r2 = rmax * rmax;
     if (T.root == WOST_EMPTY_REF) return rmax;
     int sp = 0;
     float d0 = box_dist2<D>(T.root_lo, T.root_hi, x);
     if (d0 >= r2) return rmax;
     if (d0 > 0.f && !has_silhouette<D>(T.root_lo, T.root_hi, T.root_cone, x)) return rmax;
-    bool found = false;
     uint32_t ref = T.root;
     unsigned visits = 0;
     for (;;) {
         if (over_visit_limit(visits, T.n_nodes, st.guard, st.visit_limit)) break;
         if (is_leaf(ref)) {
             uint32_t f = leaf_first(ref), c = leaf_count(ref);
+#pragma unroll 1
             for (uint32_t k = f; k < f + c; ++k) {
                 cnt.prim(C_Q2);
                 float d2 = sil_test<D>(T.prims, k, x, r2);
@@ -596,6 +647,7 @@ __device__ __noinline__ int q_ray(const TreeView &T, P3 o, P3 v, float tmax, int
         if (over_visit_limit(visits, T.n_nodes, st.guard, st.visit_limit)) break;
         if (is_leaf(ref)) {
             uint32_t f = leaf_first(ref), c = leaf_count(ref);
+#pragma unroll 1
             for (uint32_t k = f; k < f + c; ++k) {
                 if ((int)k == skip) continue;
                 cnt.prim(cq);
@@ -673,6 +725,7 @@ __device__ __noinline__ int q_ray2(const TreeView &T, P3 o, P3 va, float tmaxA, 
         if (over_visit_limit(visits, T.n_nodes, st.guard, st.visit_limit)) break;
         if (is_leaf(ref)) {
             uint32_t f = leaf_first(ref), c = leaf_count(ref);
+#pragma unroll 1
             for (uint32_t k = f; k < f + c; ++k) {
                 Prim<D> p = load_prim<D>(T.prims, k);
                 float t;
@@ -812,6 +865,7 @@ struct ClosestVisitor {  // Q.1
         h1 = k1 < best.d2;
     }
     __device__ __forceinline__ void leaf(uint32_t f, uint32_t c) {
+#pragma unroll 1
         for (uint32_t k = f; k < f + c; ++k) {
             cnt.prim(C_Q1);
             Prim<D> p = load_prim<D>(T.prims, k);
@@ -861,6 +915,7 @@ struct SilhouetteVisitor {  // Q.2
         if (h1 && k1 > 0.f) h1 = has_silhouette<D>(n.lo1, n.hi1, load_cone<D>(T.cones, ref, 1), x);
     }
     __device__ __forceinline__ void leaf(uint32_t f, uint32_t c) {
+#pragma unroll 1
         for (uint32_t k = f; k < f + c; ++k) {
             cnt.prim(C_Q2);
             float d2 = sil_test<D>(T.prims, k, x, r2);
@@ -905,6 +960,7 @@ struct Ray2Visitor {  // Q.3 (ray A) and the visibility of the Neumann sample (r
         k1 = key_with_b(a1, b1);
     }
     __device__ __forceinline__ void leaf(uint32_t f, uint32_t c) {
+#pragma unroll 1
         for (uint32_t k = f; k < f + c; ++k) {
             Prim<D> p = load_prim<D>(T.prims, k);
             float t;
@@ -952,6 +1008,63 @@ struct NSample {
     float s0, s1;  // interpolation weights of z on the primitive
 };
 
+// Alg. 6's weight of a child: proximity of its box centre if its box meets
+// the ball, else 0
+template <int D>
+__device__ __forceinline__ float child_weight(const float lo[3], const float hi[3], P3 x, float r2) {
+    if (!(box_dist2<D>(lo, hi, x) <= r2)) return 0.f;
+    P3 c = mk(0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]));
+    P3 dc = c - x;
+    return rsqrtf(fmaxf(dotp<D>(dc, dc), 1e-24f));
+}
+
+// Alg. 6's leaf and Alg. 5: a primitive of the leaf, a point on it
+template <int D, bool CN, class RNG>
+__device__ __forceinline__ void sample_leaf(const TreeView &T, P3 x, float r2, uint32_t ref, float pdf, RNG &rng,
+                                            Cnt<CN> &cnt, NSample &out) {
+    // reservoir choice proportional to area among primitives meeting the ball
+    uint32_t f = leaf_first(ref), c = leaf_count(ref);
+    float total = 0.f;
+    int chosen = -1;
+    Prim<D> cp;
+#pragma unroll 1
+    for (uint32_t k = f; k < f + c; ++k) {
+        cnt.prim(C_Q4);
+        Prim<D> p = load_prim<D>(T.prims, k);
+        float s0, s1;
+        P3 q = prim_closest<D>(p, x, s0, s1);
+        P3 dq = q - x;
+        if (dotp<D>(dq, dq) <= r2) {
+            float A = prim_area<D>(p);
+            total += A;
+            if (rng.next() * total < A) {
+                chosen = (int)k;
+                cp = p;
+            }
+        }
+    }
+    if (chosen < 0) return;
+    // uniform point on the chosen primitive
+    if constexpr (D == 2) {
+        float u = rng.next();
+        out.z = cp.a + (cp.b - cp.a) * u;
+        out.s0 = u;
+        out.s1 = 0.f;
+        out.pdf = pdf / total;
+    } else {
+        float u1 = rng.next(), u2 = rng.next();
+        float su = sqrtf(u1);
+        // rounded products: fused into a use (1 - s0), they would depend on
+        // which kernel this is compiled into
+        float wb = __fmul_rn(su, 1.f - u2), wc = __fmul_rn(su, u2);
+        out.z = cp.a * (1.f - su) + cp.b * wb + cp.c * wc;
+        out.s0 = wb;
+        out.s1 = wc;
+        out.pdf = pdf / total;
+    }
+    out.rec = chosen;
+}
+
 template <int D, bool CN = false, class RNG>
 __device__ NSample q_sample(const TreeView &T, P3 x, float r, RNG &rng, Cnt<CN> &cnt) {
     NSample out;
@@ -971,17 +1084,7 @@ __device__ NSample q_sample(const TreeView &T, P3 x, float r, RNG &rng, Cnt<CN> 
         if (level > WOST_MAX_DEPTH) return out;
         cnt.node(C_Q4);
         Node<D> n = load_node<D>(T.nodes, ref);
-        float w0 = 0.f, w1 = 0.f;
-        if (box_dist2<D>(n.lo0, n.hi0, x) <= r2) {
-            P3 c = mk(0.5f * (n.lo0[0] + n.hi0[0]), 0.5f * (n.lo0[1] + n.hi0[1]), 0.5f * (n.lo0[2] + n.hi0[2]));
-            P3 dc = c - x;
-            w0 = rsqrtf(fmaxf(dotp<D>(dc, dc), 1e-24f));
-        }
-        if (box_dist2<D>(n.lo1, n.hi1, x) <= r2) {
-            P3 c = mk(0.5f * (n.lo1[0] + n.hi1[0]), 0.5f * (n.lo1[1] + n.hi1[1]), 0.5f * (n.lo1[2] + n.hi1[2]));
-            P3 dc = c - x;
-            w1 = rsqrtf(fmaxf(dotp<D>(dc, dc), 1e-24f));
-        }
+        float w0 = child_weight<D>(n.lo0, n.hi0, x, r2), w1 = child_weight<D>(n.lo1, n.hi1, x, r2);
         float tot = w0 + w1;
         if (!(tot > 0.f)) return out;
         float p0 = __fdividef(w0, tot);  // the decision and the pdf use this same p0
@@ -993,45 +1096,7 @@ __device__ NSample q_sample(const TreeView &T, P3 x, float r, RNG &rng, Cnt<CN> 
             ref = n.r1;
         }
     }
-    // Alg. 6 leaf: reservoir choice proportional to area among primitives
-    // meeting the ball
-    uint32_t f = leaf_first(ref), c = leaf_count(ref);
-    float total = 0.f;
-    int chosen = -1;
-    Prim<D> cp;
-    for (uint32_t k = f; k < f + c; ++k) {
-        cnt.prim(C_Q4);
-        Prim<D> p = load_prim<D>(T.prims, k);
-        float s0, s1;
-        P3 q = prim_closest<D>(p, x, s0, s1);
-        P3 dq = q - x;
-        if (dotp<D>(dq, dq) <= r2) {
-            float A = prim_area<D>(p);
-            total += A;
-            if (rng.next() * total < A) {
-                chosen = (int)k;
-                cp = p;
-            }
-        }
-    }
-    if (chosen < 0) return out;
-    // Alg. 5: uniform point on the chosen primitive
-    if constexpr (D == 2) {
-        float u = rng.next();
-        out.z = cp.a + (cp.b - cp.a) * u;
-        out.s0 = u;
-        out.s1 = 0.f;
-        out.pdf = pdf / total;
-    } else {
-        float u1 = rng.next(), u2 = rng.next();
-        float su = sqrtf(u1);
-        float wb = su * (1.f - u2), wc = su * u2;
-        out.z = cp.a * (1.f - su) + cp.b * wb + cp.c * wc;
-        out.s0 = wb;
-        out.s1 = wc;
-        out.pdf = pdf / total;
-    }
-    out.rec = chosen;
+    sample_leaf<D, CN>(T, x, r2, ref, pdf, rng, cnt, out);
     return out;
 }
 
@@ -1163,6 +1228,7 @@ struct LaneQ {
     static constexpr bool kWarp = false;
     Stack st;
     Cnt<CN> &cnt;
+    __device__ __forceinline__ void hit(const TreeView &, int) {}
     __device__ Closest closest(const TreeView &T, P3 x, float bound2) { return q_closest<D, CN>(T, x, st, cnt, bound2); }
     __device__ float silhouette(const TreeView &T, P3 x, float rmax) { return q_silhouette<D, CN>(T, x, rmax, st, cnt); }
     __device__ int ray(const TreeView &T, P3 o, P3 v, float tmax, int skip, bool any, float &t) {
@@ -1356,6 +1422,7 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
     if (!act) return ended;
     P3 p, np = mk(0.f, 0.f, 0.f);
     if (hrec >= 0) {
+        q.hit(sc.N, hrec);
         p = xq + v * th;
         np = prim_normal<D>(load_prim<D>(sc.N.prims, (uint32_t)hrec));
         // App. B: a double-sided sheet is hit from the side the walk is on;

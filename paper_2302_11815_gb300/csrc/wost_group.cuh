@@ -359,6 +359,7 @@ struct GroupQ {
 
     // warp-wide forms (every lane of the warp calls them; act is uniform
     // within a team)
+    __device__ __forceinline__ void hit(const TreeView &, int) {}
     __device__ Closest closest_w(const TreeView &T, P3 x, float bound2, bool act) {
         Closest c;
         c.d2 = bound2;

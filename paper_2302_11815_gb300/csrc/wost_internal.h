@@ -72,6 +72,19 @@ struct TreeView {
     const float4 *wcones;
     uint32_t wroot;
     int32_t wn_nodes, wdepth;
+    // One walk per warp: the top of the wide tree opened to up to 32 subtrees,
+    // one per lane (as wnodes' and wcones' child records).
+    const float4 *wtop;
+    const float4 *wtopcones;  // S only
+    // Where the binary nodes (S only) and the leaf of every record (D and S)
+    // hang, parent node * 2 + side (the root: WOST_EMPTY_REF)
+    const uint32_t *parents, *leaf_parents;
+    // N only: the binary tree cut into treelets of five levels, 64 words
+    // each: word j < 31 the node at heap position j (children of j: 2j + 1,
+    // 2j + 2; WOST_EMPTY_REF: none), word 32 + j the treelet below exit j
+    const uint32_t *treelets;
+    // N only: a silhouette candidate (S record) of every record
+    const uint32_t *hints;
 };
 
 struct SceneView {
@@ -81,6 +94,8 @@ struct SceneView {
     // the boundary's bounding box grown by its largest side on every side: a
     // walk outside it has left the domain (through a rounding gap)
     float out_lo[3], out_hi[3];
+    float tau;   // four times the rounding of a distance (Near, wost_device.cuh)
+    float scale; // largest coordinate of the boundary
     float rmax;  // diagonal of the boundary's bounding box: bound on the star radius
 };
 

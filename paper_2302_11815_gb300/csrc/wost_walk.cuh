@@ -330,7 +330,9 @@ __global__ void WOST_WALK_BOUNDS k_walk_resume(const SceneView sc, const SolvePa
         if (lane == 0) first = atomicAdd(rs.live, (unsigned)__popc(saved));
         if constexpr (T == 1) {
             first = __shfl_sync(FULL, first, 0);
-            if (have) rs.list[first + __popc(saved & ((1u << lane) - 1u))] = blockIdx.x * blockDim.x + threadIdx.x;
+            // (launches of one solve that the caller let overlap could count past the list)
+            const unsigned at = first + __popc(saved & ((1u << lane) - 1u));
+            if (have && at < gridDim.x * blockDim.x) rs.list[at] = blockIdx.x * blockDim.x + threadIdx.x;
         }
     }
 }

@@ -15,17 +15,6 @@ namespace wost {
 
 constexpr int kWarpFrontier = 192;  // frontier entries per warp (an overflow falls back to the binary trees)
 
-// largest coordinate of the boundary
-__device__ __forceinline__ float scene_scale(const SceneView &sc) {
-    float m = 0.f;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        m = fmaxf(m, fmaxf(fabsf(sc.D.root_lo[a]), fabsf(sc.D.root_hi[a])));
-        m = fmaxf(m, fmaxf(fabsf(sc.N.root_lo[a]), fabsf(sc.N.root_hi[a])));
-    }
-    return m;
-}
-
 template <int D>
 __device__ __forceinline__ WarpQ<D> make_warp_q(int depth, unsigned int *guard) {
     extern __shared__ int2 smem_stack[];
@@ -40,17 +29,20 @@ __device__ __forceinline__ WarpQ<D> make_warp_q(int depth, unsigned int *guard) 
 }
 
 // Walks drawn from the solve's counter, or saved ones (src.slots).  Bound by
-// the latency of its dependent rounds: a step takes 10 us alone (Koch; one
-// lane 20 us, a full warp of one-lane walks 35 us).  Whole solves, before ->
-// after: 976 Koch walks 1,348 -> 426 ms, 6,144 keyhole walks 164 -> 36 ms, 768
-// walks by a crack 5.5 -> 1.7 ms, 544,096 torus walks (tail only) 391 -> 234 ms.
+// the latency of dependent instructions (~3,000 of them per step, 6 cycles
+// each when a warp runs alone): a step takes 9.7 us alone on the Koch workload
+// (one lane 20 us, a full warp of one-lane walks 35 us) and 14 us with 4,864
+// walks resident, 3.4e8 steps/s.  Whole solves, one-lane kernels -> this one:
+// 976 Koch walks 1,348 -> 390 ms, 6,144 keyhole walks 179 -> 22 ms, 768 walks
+// by a crack 8.8 -> 2.1 ms.  Cap of 96 registers: 64 to 128 are within 5%.
 template <int D, bool SCR>
 __global__ void __maxnreg__(WOST_WARP_REGS) k_walk_warp(const __grid_constant__ SceneView sc,
                                                         const __grid_constant__ SolveParams sp,
                                                         const Accumulators acc, const SavedWalks src) {
     WarpQ<D> q = make_warp_q<D>(sp.stack_depth, acc.guard);
-    q.scale = scene_scale(sc);
-    q.eps = sp.epsilon;
+    q.scale = sc.scale;
+    q.tau = sc.tau;
+    q.eps2 = sp.epsilon * sp.epsilon * 1.00001f;
     const uint64_t total = (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
     const unsigned n_saved = src.slots ? *src.count : 0u;
     for (;;) {
@@ -104,8 +96,9 @@ __global__ void __maxnreg__(WOST_WARP_REGS) k_walk_warp_batch(const BatchHeader 
         int job = 0;
         load_walk(src.slots + 3 * (size_t)my, w, &job, false);
         const BatchJob &J = jobs[job];
-        q.scale = scene_scale(*J.scene);
-        q.eps = J.sp.epsilon;
+        q.scale = J.scene->scale;
+        q.tau = J.scene->tau;
+        q.eps2 = J.sp.epsilon * J.sp.epsilon * 1.00001f;
         q.new_walk();
         while (!walk_step<D, SCR>(*J.scene, J.sp, w, q, true)) {
         }

@@ -11,12 +11,11 @@
 //
 // The answers are, bit for bit, those of the one-lane traversals over the
 // binary trees, so that a walk does not depend on which kernel runs it.  The
-// wide search tests every primitive the binary one can reach and also keeps
-// what decides whether the binary one returns the same value: its answer is
-// taken when no other candidate lies within rounding of the best one (or
-// when it has the same bits) and the best one is not itself on the edge of a
-// rounded test; otherwise (a few percent of the queries) lane 0 repeats the
-// query over the binary tree.  The reasons are stated at each query.
+// wide search tests every primitive the binary one can reach, so its best
+// value is at most the binary one's; it is the binary one's unless rounding
+// keeps that search from the record that has it, which is checked (the
+// reasons are stated at each query).  Where the check fails, lane 0 repeats
+// the query over the binary tree (about 1% of the queries).
 #pragma once
 
 #include "wost_device.cuh"
@@ -55,19 +54,50 @@ __device__ __forceinline__ float warp_min(float v) {  // non-negative floats (an
 }
 
 // Uniforms of slots 1, 2, ... computed one slot per lane; every lane of the
-// warp draws the same sequence.
+// warp draws the same sequence.  `mine` of lane j: slot j; `u`: draw j of the
+// first 32.
 struct WarpStream {
-    uint4 mine;  // lane j holds slot j
-    int i;
+    uint4 mine;
+    float u;
+    int i, lane;
+    __device__ __forceinline__ float at(int n, int src) const {
+        const uint32_t x = __shfl_sync(0xffffffffu, mine.x, src), y = __shfl_sync(0xffffffffu, mine.y, src),
+                       z = __shfl_sync(0xffffffffu, mine.z, src), w = __shfl_sync(0xffffffffu, mine.w, src);
+        return u01(n & 2 ? (n & 1 ? w : z) : (n & 1 ? y : x));
+    }
+    __device__ __forceinline__ WarpStream(uint4 m, int l) : mine(m), u(0.f), i(0), lane(l) { u = at(l, 1 + (l >> 2)); }
     __device__ __forceinline__ float next() {
-        const int src = 1 + (i >> 2), c = i & 3;
-        const uint32_t w = c == 0 ? mine.x : (c == 1 ? mine.y : (c == 2 ? mine.z : mine.w));
-        ++i;
-        return u01(__shfl_sync(0xffffffffu, w, src));
+        const int n = i++;
+        return n < 32 ? __shfl_sync(0xffffffffu, u, n) : at(n, 1 + (n >> 2));
     }
 };
 // draws of one sample: at most one per level, one per leaf primitive, two for the point
 static_assert(4 * 31 >= WOST_MAX_DEPTH + 2 + WOST_MAX_LEAF + 2, "slots 1..31 hold every draw of a Neumann sample");
+
+__device__ __forceinline__ float sqrt_fast(float a) {
+    float r;
+    asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(a));
+    return r;
+}
+
+// has_silhouette (the cone test of the one-lane search) with fast square
+// roots and the slack that covers them: true wherever that one is.  (An ulp
+// of sv moves cv, at least 0.014 here, by 1.3e-5.)
+template <int D>
+__device__ __forceinline__ bool may_have_silhouette(const float lo[3], const float hi[3], float4 cone, P3 x) {
+    const float ct = cone.w;
+    const P3 c = mk(0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]));
+    const P3 av = c - x;
+    const float l2 = dotp<D>(av, av);
+    const P3 ext = mk(hi[0] - lo[0], hi[1] - lo[1], hi[2] - lo[2]);
+    const float rb2 = 0.25f * dotp<D>(ext, ext);
+    const float il = rsqrtf(l2);
+    const float sv = sqrt_fast(rb2) * il, cv = sqrt_fast(fmaxf(0.f, 1.f - sv * sv));
+    const float st = sqrt_fast(fmaxf(0.f, 1.f - ct * ct));
+    const float cphi = (cone.x * av.x + cone.y * av.y + (D == 3 ? cone.z * av.z : 0.f)) * il;
+    return ct <= 0.f || l2 <= rb2 * 1.0002f || ct * cv - st * sv <= 3e-5f ||
+           fabsf(cphi) <= st * cv + ct * sv + 3e-5f;
+}
 
 // Is the accepted hit of ray o + t v on primitive p clear of every rounded
 // decision: inside the primitive by more than the rounding of its
@@ -76,8 +106,11 @@ static_assert(4 * 31 >= WOST_MAX_DEPTH + 2 + WOST_MAX_LEAF + 2, "slots 1..31 hol
 // The error terms: u is a quotient of cross products over the determinant,
 // so its rounding grows with 1 / |determinant| (grazing rays); margin kEdgeTol
 // of the hit test doubled.  te: the rounding of t.
+// Returns te, negative if the hit is not clear (out of line: two call sites).
 template <int D>
-__device__ __forceinline__ bool hit_clear(const Prim<D> &p, P3 o, P3 v, float t, float tmax, float scale, float &te) {
+__device__ __noinline__ float hit_clear(const float4 *prims, uint32_t k, P3 o, P3 v, float t, float tmax, float scale) {
+    const Prim<D> p = load_prim<D>(prims, k);
+    float te;
     const float vl = rsqrtf(dotp<D>(v, v));
     if constexpr (D == 2) {
         const P3 e = p.b - p.a, ao = p.a - o;
@@ -87,7 +120,7 @@ __device__ __forceinline__ bool hit_clear(const Prim<D> &p, P3 o, P3 v, float t,
         const float ue = ai * (fabsf(v.x) + fabsf(v.y)) + 2.f * kEdgeTol +
                          4e-6f * scale * rsqrtf(fmaxf(dotp<D>(e, e), 1e-30f));
         te = ai * (fabsf(e.x) + fabsf(e.y)) + 4e-6f * scale * vl;
-        return u > ue && u < 1.f - ue && t > te && t < tmax - te;
+        return u > ue && u < 1.f - ue && t > te && t < tmax - te ? te : -1.f;
     } else {
         const P3 e1 = p.b - p.a, e2 = p.c - p.a, pv = crossp(v, e2), tv = o - p.a;
         const float inv = __fdividef(1.f, dotp<D>(e1, pv));
@@ -100,7 +133,7 @@ __device__ __forceinline__ bool hit_clear(const Prim<D> &p, P3 o, P3 v, float t,
         const P3 nn = crossp(e1, e2);
         const float ue = ai * lv + 2.f * kEdgeTol + 4e-6f * scale * 2.f * l1 * rsqrtf(fmaxf(dotp<D>(nn, nn), 1e-30f));
         te = ai * l1 + 4e-6f * scale * vl;
-        return u > ue && w > ue && u + w < 1.f - ue && t > te && t < tmax - te;
+        return u > ue && w > ue && u + w < 1.f - ue && t > te && t < tmax - te ? te : -1.f;
     }
 }
 
@@ -165,6 +198,24 @@ __device__ __noinline__ RayAnswer ray2_binary(const TreeView &T, P3 o, P3 va, fl
     return a;
 }
 
+// lim, lim2: the squares of distance + tau and + 2 tau (tau: see beyond)
+struct Near {
+    float lim, lim2;
+    __device__ __forceinline__ Near(float d2, float tau) {
+        const float s = sqrt_fast(d2) * 1.000002f + tau;
+        lim = s * s;
+        lim2 = (s + tau) * (s + tau);
+    }
+};
+
+// the box of the child at `at` (parent node * 2 + side)
+template <int D>
+__device__ __forceinline__ float box_dist2_at(const TreeView &T, uint32_t at, P3 x) {
+    if (at == WOST_EMPTY_REF) return box_dist2<D>(T.root_lo, T.root_hi, x);
+    const Node<D> n = load_node<D>(T.nodes, at >> 1);
+    return at & 1u ? box_dist2<D>(n.lo1, n.hi1, x) : box_dist2<D>(n.lo0, n.hi0, x);
+}
+
 // Query policy: the whole warp answers the queries of its one walk.
 template <int D>
 struct WarpQ {
@@ -177,8 +228,8 @@ struct WarpQ {
     int2 *fr;      // frontier (shared memory): (node reference, key)
     int fcap;
     Stack st;      // lane 0's stack for the binary trees
-    float scale;   // largest coordinate of the scene
-    float eps;
+    float scale, tau;  // of the scene
+    float eps2;    // square of epsilon, rounded up
     int lane;
     // per step
     bool want_rec;  // the closest record itself will be used, not only the distance
@@ -186,8 +237,10 @@ struct WarpQ {
     // the previous step's answers: their distance from the new position
     // bounds the new answer (it is found again if it is still the best)
     int last_d, last_s;
+    int hit_s;  // a candidate on the Neumann primitive hit last
 
-    __device__ __forceinline__ void new_walk() { last_d = last_s = -1; }
+    __device__ __forceinline__ void new_walk() { last_d = last_s = hit_s = -1; }
+    __device__ __forceinline__ void hit(const TreeView &N, int rec) { hit_s = (int)__ldg(N.hints + rec); }
     __device__ __forceinline__ void begin_step(const SolveParams &sp, const Walk &w, bool lost) {
         want_rec = lost || w.steps + 1 >= sp.max_steps;
         rb = philox10(make_uint4(w.index, w.point, (uint32_t)w.steps, (uint32_t)lane), sp.key0, sp.key1);
@@ -197,79 +250,130 @@ struct WarpQ {
                           __shfl_sync(FULL, rb.w, 0));
     }
 
-    // Rounding of a distance.  A computed closest point lies within ~3 ulp of
-    // the largest coordinate of its primitive's box, so a box's computed
-    // distance exceeds that of a primitive in it by at most tau1, and the
-    // one-lane traversal can miss a primitive only in favour of one less than
-    // tau1 farther.  near2(d2): the square of (distance + 4 tau1).
-    __device__ __forceinline__ float near2(float d2) const {
-        const float tau = 6e-7f * scale;
-        const float s = sqrtf(d2) * 1.000001f + tau;
-        return s * s;
-    }
-
-    // One frontier search.  box(child, node ref, c, key) decides whether a
-    // child is kept (key orders the visits), prim(k) tests record k, bound()
-    // is the current pruning key (entries beyond it are dropped), after()
-    // runs, for the whole warp, after a round that tested records.  Returns
-    // false when the frontier overflows.
+    // One frontier search over tree T.  box(child, cone, key) decides whether
+    // a child is kept (cone: its record; key orders the visits), prim(k)
+    // tests record k, bound() is the current pruning key (entries beyond it
+    // are dropped), after() runs, for the whole warp, after a round that
+    // tested records.  A list of at most `brute` records is tested outright.
+    // Else the first round tests the tree's top, one subtree per lane; a
+    // later one takes the up to four nearest entries still within the bound
+    // (of the top 32, looked at together, so that a bound that tightens late
+    // costs no rounds of its own).  Returns false when the frontier overflows.
+    // (One call site each for box and prim: the code is walked through once
+    // per query, so its size is latency.)
     template <class BOX, class PRIM, class BOUND, class AFTER>
-    __device__ __forceinline__ bool search(const float4 *wnodes, uint32_t root, BOX box, PRIM prim, BOUND bound,
-                                           AFTER after) {
+    __device__ __forceinline__ bool search(const TreeView &T, int brute, BOX box, PRIM prim, BOUND bound, AFTER after) {
         const int g = lane >> 3, c = lane & 7;
-        int sp = 1;
-        if (lane == 0) fr[0] = make_int2((int)root, 0);
-        __syncwarp();
-#pragma unroll 1
-        while (sp > 0) {
-            int n = min(sp, 4);
-            if (sp - n + 8 * n > fcap) n = 1;
-            if (sp - 1 + 8 > fcap) return false;
-            bool on = g < n, leaf = false, hit = false;
-            uint32_t ref = 0, cref = 0;
-            float key = 0.f;
-            if (on) {
-                const int2 e = fr[sp - 1 - g];
-                ref = (uint32_t)e.x;
-                on = __int_as_float(e.y) <= bound();
-            }
-            sp -= n;
-            if (on) {
-                leaf = is_leaf(ref);
-                if (leaf) {
-                    const uint32_t f = leaf_first(ref), cnt = leaf_count(ref);
-#pragma unroll 1
-                    for (uint32_t j = c; j < cnt; j += 8) prim(f + j);
-                } else {
-                    const WChild ch = load_wchild(wnodes, ref, c);
-                    cref = ch.ref;
-                    hit = !ref_empty(ch.ref) && box(ch, ref, c, key);
-                }
-            }
-            if (__any_sync(FULL, leaf)) after();  // (a barrier too: the popped entries are read)
-            const unsigned hits = __ballot_sync(FULL, hit);
-            if (hits) {
-                // the nearest child on top, the others below it in any order
-                const unsigned kb = hit ? __float_as_uint(key) : 0xffffffffu;
-                const unsigned near = __reduce_min_sync(FULL, kb);
-                const int top = __ffs(__ballot_sync(FULL, hit && kb == near)) - 1;
-                const int cnt = __popc(hits);
-                if (hit) {
-                    int pos = __popc(hits & ((1u << lane) - 1u)) - (lane > top ? 1 : 0);
-                    if (lane == top) pos = cnt - 1;
-                    fr[sp + pos] = make_int2((int)cref, __float_as_int(key));
-                }
-                sp += cnt;
-            }
-            __syncwarp();
+        int sp = 0;
+        // this round's work of the lane: a child record, or records j0, j0 + js, ... < j1
+        const float4 *child = T.wtop + 2 * lane, *cone = T.wtopcones + lane;
+        uint32_t j0 = 0, j1 = 0, js = 8;
+        if (T.n_prims <= brute) {
+            child = nullptr;
+            j0 = (uint32_t)lane;
+            j1 = (uint32_t)T.n_prims;
+            js = 32;
         }
-        return true;
+#pragma unroll 1
+        for (;;) {
+            uint32_t cref = 0;
+            float key = 0.f;
+            bool hit = false;
+            if (child) {
+                const WChild ch = load_wchild(child, 0, 0);
+                cref = ch.ref;
+                hit = !ref_empty(cref) && box(ch, cone, key);
+            }
+            const bool tests = __any_sync(FULL, j0 < j1);
+            if (tests) {
+#pragma unroll 1
+                for (uint32_t j = j0; j < j1; j += js) prim(j);
+                __syncwarp();
+                after();
+            }
+            const unsigned hits = __ballot_sync(FULL, hit);
+            unsigned m = hits, m1, m2, m3;
+            uint32_t from = cref;  // this lane's entry of the candidates in m
+            if (sp == 0 && __popc(hits) <= 4) {
+                // few enough: visited at once, without the frontier
+                if (!hits) return true;
+                m1 = m & (m - 1u);
+                m2 = m1 & (m1 - 1u);
+                m3 = m2 & (m2 - 1u);
+            } else {
+                if (hit) fr[sp + __popc(hits & ((1u << lane) - 1u))] = make_int2((int)cref, __float_as_int(key));
+                sp += __popc(hits);
+                __syncwarp();
+                // entries to visit: the four nearest within the bound
+                float ekey = 0.f;
+                m = 0;
+                while (sp > 0) {
+                    const int n = min(sp, 32);
+                    bool alive = false;
+                    if (lane < n) {
+                        const int2 e = fr[sp - 1 - lane];
+                        from = (uint32_t)e.x;
+                        ekey = __int_as_float(e.y);
+                        alive = ekey <= bound();
+                    }
+                    m = __ballot_sync(FULL, alive);
+                    if (m) break;
+                    sp -= n;
+                }
+                if (!m) return true;
+                const int n = min(sp, 32);
+                unsigned rest = 0u;
+                if (__popc(m) > 4) {
+                    // the four nearest of them; the others stay
+                    unsigned kb = (m >> lane) & 1u ? __float_as_uint(ekey) : 0xffffffffu, sel = 0u;
+#pragma unroll 1
+                    for (int i = 0; i < 4; ++i) {
+                        const unsigned at = __ballot_sync(FULL, kb == __reduce_min_sync(FULL, kb));
+                        const unsigned one = at & (0u - at);
+                        sel |= one;
+                        if ((one >> lane) & 1u) kb = 0xffffffffu;
+                    }
+                    rest = m & ~sel;
+                    m = sel;
+                }
+                m1 = m & (m - 1u);
+                m2 = m1 & (m1 - 1u);
+                m3 = m2 & (m2 - 1u);
+                const int kept = __popc(rest);
+                if (sp - n + kept + 32 > fcap) {  // one at a time while space is short
+                    rest |= m1;
+                    m &= ~m1;
+                    m1 = m2 = m3 = 0u;
+                    if (sp - n + __popc(rest) + 8 > fcap) return false;
+                }
+                __syncwarp();
+                if ((rest >> lane) & 1u)
+                    fr[sp - n + __popc(rest >> lane >> 1)] = make_int2((int)from, __float_as_int(ekey));
+                sp += __popc(rest) - n;
+            }
+            const unsigned mine = g == 0 ? m : (g == 1 ? m1 : (g == 2 ? m2 : m3));
+            const uint32_t ref = __shfl_sync(FULL, from, mine ? __ffs(mine) - 1 : 0);
+            child = nullptr;
+            j0 = j1 = 0;
+            js = 8;
+            if (mine && is_leaf(ref)) {
+                j0 = leaf_first(ref) + c;
+                j1 = leaf_first(ref) + leaf_count(ref);
+            } else if (mine) {
+                child = T.wnodes + (size_t)ref * (2 * WOST_WIDE) + 2 * c;
+                cone = T.wcones + (size_t)ref * WOST_WIDE + c;
+            }
+        }
     }
 
-    // Q.1.  Certain when every record within near2 of the best has the
-    // best's bits (the one-lane search then returns those bits, whatever
-    // order it meets the records in), and, if the record itself is used, when
-    // there is only one.
+    // Q.1.  The one-lane search prunes a box whose computed distance is not
+    // below the best value so far.  It reaches the record with the smallest
+    // value m, in whatever order it goes, if the box of that record's leaf is
+    // computed no farther than m (those above it are no farther either:
+    // rounding is monotonic): m is then its answer.  Where rounding puts the
+    // box beyond m (a vertex computed just outside it), m is still the answer
+    // if no record with other bits lies within rounding.  Which of several
+    // records with the bits of m it returns depends on its order.
     __device__ __forceinline__ Closest closest_w(const TreeView &T, P3 x, float bound2, bool act) {
         Closest best;
         best.d2 = bound2;
@@ -293,37 +397,34 @@ struct WarpQ {
             }
         };
         bool ok = T.root != WOST_EMPTY_REF;
-        if (T.n_prims <= kBrute) {
-#pragma unroll 1
-            for (uint32_t k = lane; k < (uint32_t)T.n_prims; k += 32) test(k);
-        } else {
-            if (last_d >= 0) {
-                const Prim<D> p = load_prim<D>(T.prims, (uint32_t)last_d);
-                float t0, t1;
-                const P3 dq = prim_closest<D>(p, x, t0, t1) - x;
-                B = fminf(B, near2(near2(dotp<D>(dq, dq))));
-            }
+        // the records around the last answer (neighbours in leaf order are
+        // neighbours in space) bound the new one
+        if (last_d >= 0 && T.n_prims > kBrute) {
+            const int k = min(max(last_d - 16 + lane, 0), T.n_prims - 1);
+            B = fminf(B, beyond(warp_min(prim_dist2<D>(T.prims, (uint32_t)k, x)), tau));
+        }
+        if (ok)
             ok = search(
-                T.wnodes, T.wroot,
-                [&](const WChild &ch, uint32_t, int, float &key) {
+                T, kBrute,
+                [&](const WChild &ch, const float4 *, float &key) {
                     key = box_dist2<D>(ch.lo, ch.hi, x);
                     return key < B;
                 },
-                test, [&] { return B; }, [&] { B = fminf(B, near2(near2(warp_min(lb.d2)))); });
-        }
+                test, [&] { return B; }, [&] { B = fminf(B, beyond(warp_min(lb.d2), tau)); });
         const float m = warp_min(lb.d2);
-        const float lim = near2(m);
+        const Near nr(m, tau);
         const unsigned at = __ballot_sync(FULL, lb.d2 == m);
-        bool amb = (lb.d2 != m && lb.d2 <= lim) || lb.alt <= lim;
-        const bool rec_used = want_rec || !(sqrtf(m) >= eps);
-        if (rec_used) amb = amb || (lb.d2 == m && lb.dup) || __popc(at) != 1;
-        // (a bound that comes near the answer, no answer, NaN: not certain)
-        if (!ok || __any_sync(FULL, amb) || !(near2(lim) < bound2)) {
-            best = closest_binary<D>(T, x, st, D == 3 && m < INFINITY ? fminf(bound2, near2(lim)) : bound2);
+        const bool tie = __any_sync(FULL, (lb.d2 != m && lb.d2 <= nr.lim) || lb.alt <= nr.lim);
+        const int src = at ? __ffs(at) - 1 : 0, k = __shfl_sync(FULL, lb.rec, src);
+        bool certain = ok && m < bound2;  // (no answer, NaN: not certain)
+        if (want_rec || !(m >= eps2))  // the record is used
+            certain = certain && __popc(at) == 1 && !__any_sync(FULL, lb.d2 == m && lb.dup);
+        if (certain && (tie || !(nr.lim2 < bound2))) certain = box_dist2_at<D>(T, __ldg(T.leaf_parents + k), x) <= m;
+        if (!certain) {
+            best = closest_binary<D>(T, x, st, D == 3 && m < INFINITY ? fminf(bound2, nr.lim2) : bound2);
         } else {
-            const int src = __ffs(at) - 1;
             best.d2 = m;
-            best.rec = __shfl_sync(FULL, lb.rec, src);
+            best.rec = k;
             best.s0 = __shfl_sync(FULL, s0, src);
             best.s1 = __shfl_sync(FULL, s1, src);
             best.p.x = __shfl_sync(FULL, q.x, src);
@@ -334,78 +435,147 @@ struct WarpQ {
         return best;
     }
 
-    // Q.2.  Certain, beside the near ties of Q.1, when the best candidate is
-    // not grazing: the normals on both sides of the view direction by more
-    // than the cone test's padding can lose in single precision (a cone's
-    // half angle of 3.4e-4 or less rounds to 0), so that no cone that holds
-    // them is culled.  A boundary candidate (n1 = 0) is never culled.
+    // Q.2.  As Q.1 (only the distance is used), and the best candidate must
+    // not be culled: one that is not grazing (sil_certain) never is.  Of a
+    // grazing one (common on flat walls, where rounding decides the signs)
+    // the cone tests above it decide: a candidate whose leaf is culled is
+    // none, and the best one's whole path is tested.
     __device__ __forceinline__ float silhouette_w(const TreeView &T, P3 x, float rmax, bool act) {
         if (!act || T.root == WOST_EMPTY_REF) return rmax;
         const float r2 = rmax * rmax;
         LaneBest lb;
         lb.clear();
+        bool clear = false;
         float B = r2;
-        auto test = [&](uint32_t k) { lb.add(sil_test<D>(T.prims, k, x, r2), (int)k); };
-        bool ok = true;
-        if (T.n_prims <= 3 * kBrute) {
-#pragma unroll 2
-            for (uint32_t k = lane; k < (uint32_t)T.n_prims; k += 32) test(k);
-        } else {
-            if (last_s >= 0) {
-                const float d2 = sil_test<D>(T.prims, (uint32_t)last_s, x, r2);
-                if (d2 < r2) B = fminf(B, near2(near2(d2)));
+        auto test = [&](uint32_t k) {
+            const float d2 = sil_test<D>(T.prims, k, x, r2);
+            if (d2 < INFINITY && d2 <= B) {
+                const bool cl = sil_certain<D>(T.prims, k, x) < INFINITY;
+                if (!cl && !reached(T, T.leaf_parents[k], x)) return;
+                if (lb.add(d2, (int)k)) clear = cl;
             }
-            ok = search(
-                T.wnodes, T.wroot,
-                [&](const WChild &ch, uint32_t ref, int c, float &key) {
+        };
+        // the candidates around the last answer and around the last hit bound
+        // the new one
+        if ((last_s >= 0 || hit_s >= 0) && T.n_prims > 3 * kBrute) {
+            const int mid = (lane < 16 && last_s >= 0) || hit_s < 0 ? last_s : hit_s;
+            const int k = min(max(mid - 8 + (lane & 15), 0), T.n_prims - 1);
+            B = fminf(B, beyond(warp_min(sil_certain<D>(T.prims, (uint32_t)k, x)), tau));
+        }
+        const bool ok = search(
+                T, 3 * kBrute,
+                [&](const WChild &ch, const float4 *cone, float &key) {
+                    const float4 cn = __ldg(cone);
                     key = box_dist2<D>(ch.lo, ch.hi, x);
                     bool keep = key < B;
-                    if (keep && key > 0.f)
-                        keep = has_silhouette<D>(ch.lo, ch.hi, __ldg(T.wcones + (size_t)ref * WOST_WIDE + c), x);
+                    if (keep && key > 0.f) keep = may_have_silhouette<D>(ch.lo, ch.hi, cn, x);
                     return keep;
                 },
-                test, [&] { return B; }, [&] { B = fminf(B, near2(near2(warp_min(lb.d2)))); });
-        }
+                test, [&] { return B; }, [&] { B = fminf(B, beyond(warp_min(lb.d2), tau)); });
         const float m = warp_min(lb.d2);
         if (ok && m == INFINITY) return rmax;
-        const float lim = near2(m);
+        const Near nr(m, tau);
         const unsigned at = __ballot_sync(FULL, lb.d2 == m);
-        bool amb = (lb.d2 != m && lb.d2 <= lim) || lb.alt <= lim;
-        const int k = __shfl_sync(FULL, lb.rec, at ? __ffs(at) - 1 : 0);
-        bool certain = ok && !__any_sync(FULL, amb) && near2(lim) < r2;
-        if (certain) certain = sil_clear<D>(T.prims, (uint32_t)k, x);
+        const bool tie = __any_sync(FULL, (lb.d2 != m && lb.d2 <= nr.lim) || lb.alt <= nr.lim);
+        const int src = at ? __ffs(at) - 1 : 0;
+        const int k = __shfl_sync(FULL, lb.rec, src);
+        bool certain = ok;
+        if (certain && (tie || !(nr.lim2 < r2))) certain = box_dist2_at<D>(T, __ldg(T.leaf_parents + k), x) <= m;
+        if (certain && !__shfl_sync(FULL, (int)clear, src)) certain = path_reached(T, (uint32_t)k, x);
         last_s = k;
-        return certain ? sqrtf(m) : silhouette_binary<D>(T, x, rmax, st);
-    }
-
-    template <int DD>
-    __device__ __forceinline__ static bool sil_clear(const float4 *prims, uint32_t k, P3 x) {
-        P3 pe, n0, n1;
-        if constexpr (DD == 2) {
-            const float4 q0 = __ldg(prims + 2 * (size_t)k), q1 = __ldg(prims + 2 * (size_t)k + 1);
-            pe = mk(q0.x, q0.y, 0.f);
-            n0 = mk(q1.x, q1.y, 0.f);
-            n1 = mk(q1.z, q1.w, 0.f);
-        } else {
-            const float4 q0 = __ldg(prims + 3 * (size_t)k), q1 = __ldg(prims + 3 * (size_t)k + 1),
-                         q2 = __ldg(prims + 3 * (size_t)k + 2);
-            const P3 a = mk(q0.x, q0.y, q0.z), b = mk(q1.x, q1.y, q1.z);
-            n0 = mk(q0.w, q1.w, q2.x);
-            n1 = mk(q2.y, q2.z, q2.w);
-            pe = a + (b - a) * seg_param(a, b, x, 1);
+        if (certain) return sqrtf(m);
+        if (ok) {
+            // the one-lane search among the candidates near the best one, if
+            // it finds one there (culled candidates can leave none)
+            const float rn = sqrtf(nr.lim2) * 1.000001f;
+            if (rn < rmax) {
+                const float s = silhouette_binary<D>(T, x, rn, st);
+                if (s * s <= nr.lim) return s;
+            }
         }
-        const P3 v = pe - x;
-        if (n1.x == 0.f && n1.y == 0.f && n1.z == 0.f) return true;
-        const float lim = 4e-4f * sqrtf(dotp<DD>(v, v));
-        return fabsf(dotp<DD>(v, n0)) > lim && fabsf(dotp<DD>(v, n1)) > lim;
+        return silhouette_binary<D>(T, x, rmax, st);
     }
 
-    // Q.4 over the binary tree, every lane alike; the uniforms come from the
-    // lanes' slots.
+    // does the binary search enter the child at `at` (parent * 2 + side)?
+    __device__ __noinline__ static bool reached(const TreeView &T, uint32_t at, P3 x) {
+        if (at == WOST_EMPTY_REF)
+            return !(box_dist2<D>(T.root_lo, T.root_hi, x) > 0.f) ||
+                   has_silhouette<D>(T.root_lo, T.root_hi, T.root_cone, x);
+        const Node<D> n = load_node<D>(T.nodes, at >> 1);
+        float lo[3], hi[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            lo[a] = at & 1u ? n.lo1[a] : n.lo0[a];
+            hi[a] = at & 1u ? n.hi1[a] : n.hi0[a];
+        }
+        return !(box_dist2<D>(lo, hi, x) > 0.f) ||
+               has_silhouette<D>(lo, hi, load_cone<D>(T.cones, at >> 1, (int)(at & 1u)), x);
+    }
+    // ... and every one above record k?  (lane i tests the i-th from below)
+    __device__ __forceinline__ bool path_reached(const TreeView &T, uint32_t k, P3 x) const {
+        uint32_t at = __ldg(T.leaf_parents + k), mine = WOST_EMPTY_REF;
+        for (int i = 0; at != WOST_EMPTY_REF; ++i) {
+            if (i == 31) return false;  // deeper than the warp is wide: undecided
+            if (lane == i) mine = at;
+            at = __ldg(T.parents + (at >> 1));
+        }
+        return __all_sync(FULL, reached(T, mine, x));  // (a lane without an entry tests the root)
+    }
+
+    // Q.4 over the binary tree; the uniforms come from the lanes' slots.  The
+    // descent is a chain of one decision per level, each on the two children's
+    // weights: the lanes compute the decisions of a five-level treelet at
+    // once, so a level costs a shuffle and a comparison instead of a node
+    // fetch and two weights (480 cycles).
     __device__ __forceinline__ NSample sample(const TreeView &T, P3 x, float r) {
-        WarpStream rng{rb, 0};
         Cnt<false> cnt;
-        return q_sample<D, false>(T, x, r, rng, cnt);
+        NSample out;
+        out.rec = -1;
+        out.pdf = 0.f;
+        out.z = x;
+        out.s0 = out.s1 = 0.f;
+        const float r2 = r * r;
+        if (T.root == WOST_EMPTY_REF || box_dist2<D>(T.root_lo, T.root_hi, x) > r2) return out;
+        WarpStream rng(rb, lane);
+        uint32_t ref = T.root, t = 0;
+        float pdf = 1.f;
+        const int depth = 31 - __clz(lane + 1);  // of heap position `lane` in a treelet
+#pragma unroll 1
+        for (int level = 0; !is_leaf(ref); level += 5) {
+            if (level > WOST_MAX_DEPTH) return out;
+            const uint32_t *tl = T.treelets + 64 * (size_t)t;
+            const uint32_t node = lane < 31 ? __ldg(tl + lane) : WOST_EMPTY_REF, exit = __ldg(tl + 32 + lane);
+            uint32_t next = WOST_EMPTY_REF;
+            bool live = false, first = false;
+            float f = 0.f;
+            // the draw that a walk arriving at this position takes
+            const int n = rng.i + depth;
+            const float u = __shfl_sync(FULL, rng.u, n & 31);
+            const float ub = rng.i + 4 >= 32 ? rng.at(n, min(1 + (n >> 2), 31)) : u;
+            if (node != WOST_EMPTY_REF) {
+                const Node<D> nd = load_node<D>(T.nodes, node);
+                const float w0 = child_weight<D>(nd.lo0, nd.hi0, x, r2), w1 = child_weight<D>(nd.lo1, nd.hi1, x, r2);
+                const float tot = w0 + w1, p0 = __fdividef(w0, tot);
+                live = tot > 0.f;
+                first = (n < 32 ? u : ub) < p0;  // the decision and the pdf use this same p0
+                f = first ? p0 : 1.f - p0;
+                next = first ? nd.r0 : nd.r1;
+            }
+            const unsigned lives = __ballot_sync(FULL, live), firsts = __ballot_sync(FULL, first),
+                           ends = __ballot_sync(FULL, is_leaf(next));
+            int pos = 0, last;
+            do {
+                if (!((lives >> pos) & 1u)) return out;
+                pdf *= __shfl_sync(FULL, f, pos);
+                last = pos;
+                pos = 2 * pos + 2 - (int)((firsts >> pos) & 1u);
+                ++rng.i;
+            } while (pos < 31 && !((ends >> last) & 1u));
+            ref = __shfl_sync(FULL, next, last);
+            if (!is_leaf(ref)) t = __shfl_sync(FULL, exit, pos - 31);
+        }
+        sample_leaf<D, false>(T, x, r2, ref, pdf, rng, cnt, out);
+        return out;
     }
 
     // Q.3 and the visibility ray.  Every primitive of every wide leaf that
@@ -419,44 +589,44 @@ struct WarpQ {
         t_out = tmaxA;
         occB = false;
         if (!act || T.root == WOST_EMPTY_REF) return -1;
-        const P3 ia = mk(1.f / va.x, 1.f / va.y, D == 3 ? 1.f / va.z : 0.f);
+        // fast reciprocals: the boxes are widened by more than they, and the
+        // rounding of the one-lane slab test, can move its planes
+        const P3 ia = mk(__fdividef(1.f, va.x), __fdividef(1.f, va.y), D == 3 ? __fdividef(1.f, va.z) : 0.f);
         P3 ib = mk(0.f, 0.f, 0.f);
-        if (wantB) ib = mk(1.f / vb.x, 1.f / vb.y, D == 3 ? 1.f / vb.z : 0.f);
+        if (wantB) ib = mk(__fdividef(1.f, vb.x), __fdividef(1.f, vb.y), D == 3 ? __fdividef(1.f, vb.z) : 0.f);
+        const float pad = 8e-6f * scale;
         // a zero component makes the slab test drop boxes that touch the ray
         // (0 x inf): such a ray is lane 0's
-        const bool axis = va.x == 0.f || va.y == 0.f || (D == 3 && va.z == 0.f) ||
-                          (wantB && (vb.x == 0.f || vb.y == 0.f || (D == 3 && vb.z == 0.f)));
+        auto flat = [](P3 v) {
+            return fminf(fminf(fabsf(v.x), fabsf(v.y)), D == 3 ? fabsf(v.z) : INFINITY) < 1e-30f;
+        };
+        const bool axis = flat(va) || (wantB && flat(vb));
         LaneBest lb;
         lb.clear();
-        bool clearA = false, occ = false, occ_maybe = false;
-        float teA = 0.f;
+        bool occ = false, occ_maybe = false;
+        float teA = -1.f;
         auto test = [&](uint32_t k) {
             const Prim<D> p = load_prim<D>(T.prims, k);
-            float t, te;
-            if (prim_ray<D>(p, o, va, tmaxA, t, kEdgeTol) && lb.add(t, (int)k)) {
-                clearA = hit_clear<D>(p, o, va, t, tmaxA, scale, te);
-                teA = te;
-            }
+            float t;
+            if (prim_ray<D>(p, o, va, tmaxA, t, kEdgeTol) && lb.add(t, (int)k))
+                teA = hit_clear<D>(T.prims, k, o, va, t, tmaxA, scale);
             if (wantB && (int)k != skipB && prim_ray<D>(p, o, vb, tmaxB, t, 0.f)) {
-                if (hit_clear<D>(p, o, vb, t, tmaxB, scale, te)) occ = true;
+                if (hit_clear<D>(T.prims, k, o, vb, t, tmaxB, scale) >= 0.f) occ = true;
                 else occ_maybe = true;
             }
         };
         bool ok = !axis;
-        if (!ok) {
-        } else if (T.n_prims <= kBrute) {
-#pragma unroll 1
-            for (uint32_t k = lane; k < (uint32_t)T.n_prims; k += 32) test(k);
-        } else {
+        if (ok)
             ok = search(
-                T.wnodes, T.wroot,
-                [&](const WChild &ch, uint32_t, int, float &key) {
+                T, kBrute,
+                [&](const WChild &ch, const float4 *, float &key) {
                     key = 0.f;
-                    return box_ray<D>(ch.lo, ch.hi, o, ia, tmaxA) != INFINITY ||
-                           (wantB && box_ray<D>(ch.lo, ch.hi, o, ib, tmaxB) != INFINITY);
+                    const float lo[3] = {ch.lo[0] - pad, ch.lo[1] - pad, ch.lo[2] - pad};
+                    const float hi[3] = {ch.hi[0] + pad, ch.hi[1] + pad, ch.hi[2] + pad};
+                    return box_ray<D>(lo, hi, o, ia, tmaxA) != INFINITY ||
+                           (wantB && box_ray<D>(lo, hi, o, ib, tmaxB) != INFINITY);
                 },
                 test, [&] { return 0.f; }, [&] {});
-        }
         const float m = warp_min(lb.d2);
         bool certain = ok;
         int hit = -1;
@@ -464,7 +634,7 @@ struct WarpQ {
             const unsigned at = __ballot_sync(FULL, lb.d2 == m);
             const int src = __ffs(at) - 1;
             const float lim = m + __shfl_sync(FULL, teA, src);
-            const bool bad = lane == src ? (!clearA || lb.dup || lb.alt <= lim) : lb.d2 <= lim;
+            const bool bad = lane == src ? (!(teA >= 0.f) || lb.dup || lb.alt <= lim) : lb.d2 <= lim;
             certain = certain && !__any_sync(FULL, bad);
             hit = __shfl_sync(FULL, lb.rec, src);
             t_out = m;
