@@ -44,7 +44,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hd
     const unsigned long long total = src.slots ? (unsigned long long)*src.count : hdr->total;
     if (n_jobs <= 0) return;
     Cnt<false> cnt;
-    auto q = make_q<D, false>(stack_depth, guard, cnt);
+    auto q = make_q<D, false>(stack_depth, guard, cnt, 0u, true);
     const Group g = make_team<1>();
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;

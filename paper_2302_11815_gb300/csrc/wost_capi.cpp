@@ -358,6 +358,7 @@ wost_status wost::prepare_solve(wost_scene *scene, const wost_solve_desc *d, cud
     sp.stack_depth = d->stack_depth ? d->stack_depth : (lanes == 1 ? scene->stack_depth : scene->stack_depth_team);
     sp.visit_limit = (uint32_t)d->visit_limit;
     h->warp_ok = !d->stack_depth && !d->visit_limit;
+    sp.coop = h->warp_ok ? 1 : 0;
     sp.sigma = d->sigma;
     sp.sqrt_sigma = std::sqrt(d->sigma);
     sp.screen_after = d->screen_after;

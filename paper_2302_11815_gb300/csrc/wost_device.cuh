@@ -573,13 +573,13 @@ __device__ __noinline__ float sil_certain(const float4 *prims, uint32_t k, P3 x)
 
 template <int D, bool CN = false>
 __device__ float q_silhouette(const TreeView &T, P3 x, float rmax, const Stack &st, Cnt<CN> &cnt) {
-    bool found = false;
     float r2 = rmax * rmax;
     if (T.root == WOST_EMPTY_REF) return rmax;
     int sp = 0;
     float d0 = box_dist2<D>(T.root_lo, T.root_hi, x);
     if (d0 >= r2) return rmax;
     if (d0 > 0.f && !has_silhouette<D>(T.root_lo, T.root_hi, T.root_cone, x)) return rmax;
+    bool found = false;
     uint32_t ref = T.root;
     unsigned visits = 0;
     for (;;) {
@@ -621,6 +621,80 @@ __device__ float q_silhouette(const TreeView &T, P3 x, float rmax, const Stack &
         if (!(key < r2)) break;
     }
     return found ? sqrtf(r2) : rmax;
+}
+
+// One lane's search in slices (3D): the whole warp calls it (act: the lane has
+// a query).  After every slice of visits the lanes meet; once at most `few` of
+// them have not finished, those are left open (returns true; found2: the
+// squared distance found so far, or +inf).  r: the answer of a lane that
+// finished.
+constexpr unsigned kSilSlice = 8;
+constexpr int kSilFew = 24;
+
+template <int D, bool CN = false>
+__device__ __forceinline__ bool q_silhouette_sliced(const TreeView &T, P3 x, float rmax, const Stack &st, Cnt<CN> &cnt,
+                                                    bool act, int few, float &r, float &found2) {
+    bool found = false;
+    float r2 = rmax * rmax;
+    r = rmax;
+    bool open = act && T.root != WOST_EMPTY_REF;
+    if (open) {
+        const float d0 = box_dist2<D>(T.root_lo, T.root_hi, x);
+        open = d0 < r2 && (!(d0 > 0.f) || has_silhouette<D>(T.root_lo, T.root_hi, T.root_cone, x));
+    }
+    int sp = 0;
+    uint32_t ref = T.root;
+    unsigned visits = 0, slice = 0;
+    for (;;) {
+        const unsigned m = __ballot_sync(0xffffffffu, open);
+        if (__popc(m) <= few) break;
+        slice += kSilSlice;
+        while (open && visits < slice) {
+            if (over_visit_limit(visits, T.n_nodes, st.guard, st.visit_limit)) {
+                open = false;
+                break;
+            }
+            if (is_leaf(ref)) {
+                uint32_t f = leaf_first(ref), c = leaf_count(ref);
+#pragma unroll 1
+                for (uint32_t k = f; k < f + c; ++k) {
+                    cnt.prim(C_Q2);
+                    float d2 = sil_test<D>(T.prims, k, x, r2);
+                    if (d2 < r2) {
+                        r2 = d2;
+                        found = true;
+                    }
+                }
+            } else {
+                cnt.node(C_Q2);
+                Node<D> n = load_node<D>(T.nodes, ref);
+                float e0 = box_dist2<D>(n.lo0, n.hi0, x), e1 = box_dist2<D>(n.lo1, n.hi1, x);
+                bool v0 = e0 < r2, v1 = e1 < r2;
+                if (v0 && e0 > 0.f) v0 = has_silhouette<D>(n.lo0, n.hi0, load_cone<D>(T.cones, ref, 0), x);
+                if (v1 && e1 > 0.f) v1 = has_silhouette<D>(n.lo1, n.hi1, load_cone<D>(T.cones, ref, 1), x);
+                if (v0 && v1) {
+                    bool first0 = e0 <= e1;
+                    spush(st, sp, first0 ? n.r1 : n.r0, first0 ? e1 : e0);
+                    ref = first0 ? n.r0 : n.r1;
+                    continue;
+                }
+                if (v0 || v1) {
+                    ref = v0 ? n.r0 : n.r1;
+                    continue;
+                }
+            }
+            float key = INFINITY;
+            while (sp > 0) {
+                spop(st, sp, ref, key);
+                if (key < r2) break;
+            }
+            if (!(key < r2)) open = false;
+        }
+        __syncwarp();
+    }
+    found2 = found ? r2 : INFINITY;
+    if (found && !open) r = sqrtf(r2);
+    return open;
 }
 
 // ---------------------------------------------------------------------------
@@ -1221,6 +1295,11 @@ struct Walk {
 
 __device__ __forceinline__ float maxabs3(P3 a) { return fmaxf(fabsf(a.x), fmaxf(fabsf(a.y), fabsf(a.z))); }
 
+// Q.2 by the whole warp (wost_warp.cuh)
+template <int D>
+__device__ __noinline__ float2 coop_silhouette(const TreeView &T, P3 x, float rmax, float bound2, float tau, int2 *fr,
+                                               int frs, int fcap);
+
 // Query policy over the binary trees: each lane answers its own walk's
 // queries with its own shared-memory stack.
 template <int D, bool CN>
@@ -1231,6 +1310,7 @@ struct LaneQ {
     __device__ __forceinline__ void hit(const TreeView &, int) {}
     __device__ Closest closest(const TreeView &T, P3 x, float bound2) { return q_closest<D, CN>(T, x, st, cnt, bound2); }
     __device__ float silhouette(const TreeView &T, P3 x, float rmax) { return q_silhouette<D, CN>(T, x, rmax, st, cnt); }
+    bool coop = false;  // long silhouette searches are the whole warp's (walk kernels under the scene's limits)
     __device__ int ray(const TreeView &T, P3 o, P3 v, float tmax, int skip, bool any, float &t) {
         return q_ray<D, CN>(T, o, v, tmax, skip, any, t, st, cnt);
     }
@@ -1257,11 +1337,53 @@ struct LaneQ {
             return c;
         }
     }
-    __device__ float silhouette_w(const TreeView &T, P3 x, float rmax, bool act) {
+    __device__ float silhouette_w(const TreeView &T, P3 x, float rmax, bool act, float tau) {
         if constexpr (kPostpone) {
             return q_silhouette_w<D, CN>(T, x, rmax, st, cnt, act);
         } else {
-            return act ? silhouette(T, x, rmax) : rmax;
+            // The searches are heavy-tailed (110 visits on the mean around
+            // the noisy torus, thousands at worst) and the warp waits for its
+            // longest, while the 32 lanes together need ~4,000 instructions
+            // for any of them.  So once at most kSilFew lanes are open, the
+            // warp finishes their searches one after the other.  Million walk
+            // steps/s with kSilFew 0 / 3 / 10 / 24 / 32: torus (212k
+            // triangles) 60 / 66 / 87 / 105 / 105, (15k) 180 / 175 / 193 /
+            // 215 / 211, box around a sphere 270 / 284 / 359 / 382 / 384;
+            // a cube of 192 triangles, whose searches are short, 1,020 (24:
+            // 1,210, 32: 1,030).
+            float r = rmax, found2 = INFINITY;
+            bool need = act;
+            int few = coop ? kSilFew : 0;
+#pragma unroll 1
+            for (;;) {
+                float rr;
+                const bool asked = need;
+                need = q_silhouette_sliced<D, CN>(T, x, rmax, st, cnt, need, few, rr, found2);
+                if (asked && !need) r = rr;
+                if constexpr (CN) return r;
+                unsigned m = __ballot_sync(0xffffffffu, need);
+                if (!m) return r;
+                const int lane = threadIdx.x & 31;
+#pragma unroll 1
+                for (; m; m &= m - 1u) {
+                    const int src = __ffs(m) - 1;
+                    // (in a batch every lane has a scene of its own)
+                    const TreeView *Ts = (const TreeView *)__shfl_sync(0xffffffffu, (unsigned long long)&T, src);
+                    const P3 xs = mk(__shfl_sync(0xffffffffu, x.x, src), __shfl_sync(0xffffffffu, x.y, src),
+                                     __shfl_sync(0xffffffffu, x.z, src));
+                    const float rs = __shfl_sync(0xffffffffu, rmax, src), ts = __shfl_sync(0xffffffffu, tau, src),
+                                fs = __shfl_sync(0xffffffffu, found2, src);
+                    const float2 a =
+                        coop_silhouette<D>(*Ts, xs, rs, beyond(fs, ts), ts, st.base - lane, st.stride, 32 * st.cap);
+                    if (lane == src && a.y != 0.f) {
+                        r = a.x;
+                        need = false;
+                    }
+                    __syncwarp();
+                }
+                if (!__any_sync(0xffffffffu, need)) return r;
+                few = 0;  // uncertain: that lane's search, to its end
+            }
         }
     }
     __device__ int ray2_w(const TreeView &T, P3 o, P3 va, float tmaxA, float &t, bool wantB, P3 vb, int skipB,
@@ -1355,7 +1477,7 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
     const float delta = sp.offset * (1.f + maxabs3(w.x));
     const P3 xq = w.onN ? w.x - w.n * delta : w.x;
     // distance to the visibility silhouette (Q.2) within d_D, star radius (R3)
-    float dsil = q.silhouette_w(sc.S, xq, dD, act);
+    float dsil = q.silhouette_w(sc.S, xq, dD, act, sc.tau);
     if (!act) dsil = dD;
     __syncwarp();
     float r = fminf(dD, fmaxf(sp.r_min, dsil));

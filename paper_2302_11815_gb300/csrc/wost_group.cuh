@@ -369,7 +369,7 @@ struct GroupQ {
         if (act) c = closest(T, x, bound2);
         return c;
     }
-    __device__ float silhouette_w(const TreeView &T, P3 x, float rmax, bool act) {
+    __device__ float silhouette_w(const TreeView &T, P3 x, float rmax, bool act, float) {
         return act ? silhouette(T, x, rmax) : rmax;
     }
     __device__ int ray2_w(const TreeView &T, P3 o, P3 va, float tmaxA, float &t, bool wantB, P3 vb, int skipB,

@@ -114,6 +114,7 @@ struct SolveParams {
     float vis_tmax;             // visibility ray end for the Neumann sample
     int32_t stack_depth;        // shared-memory stack entries per walk (thread or team)
     uint32_t visit_limit;       // node visits allowed per traversal (0: 2 n_nodes + 8)
+    int32_t coop;               // the scene's own limits: a warp may finish a lane's search together
     float sigma;                // screening coefficient (0: Poisson)
     float sqrt_sigma;
     int32_t screen_after;       // steps k >= screen_after are screened (Tikhonov switch)

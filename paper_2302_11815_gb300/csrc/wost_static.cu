@@ -109,6 +109,7 @@ extern "C" wost_status wost_solve_static(wost_scene *scene, int64_t n_points, co
     sp.offset = 1e-6f;
     sp.vis_tmax = 1.f - 1e-4f;
     sp.stack_depth = scene->stack_depth;
+    sp.coop = 1;
     Accumulators acc{};
     acc.sum = (double *)(s + kHeader);
     acc.sumsq = (double *)(s + kHeader + kArray);

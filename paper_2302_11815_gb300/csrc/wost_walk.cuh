@@ -31,6 +31,7 @@
 
 #include "wost_device.cuh"
 #include "wost_group.cuh"
+#include "wost_warp.cuh"
 #include "wost_kernels.h"
 
 // Register caps of the walk kernels (2D and 3D instantiations).  They are
@@ -75,11 +76,11 @@ struct PolicyOf<D, CN, WOST_WIDE> {
 // the query policy of this thread's team, with its shared-memory stack
 template <int D, bool CN, int T = 1>
 __device__ __forceinline__ typename PolicyOf<D, CN, T>::type make_q(int depth, unsigned int *guard, Cnt<CN> &cnt,
-                                                                    uint32_t visit_limit = 0u) {
+                                                                    uint32_t visit_limit = 0u, bool coop = false) {
     extern __shared__ int2 smem_stack[];
     if constexpr (T == 1) {
         Stack s{smem_stack + threadIdx.x, (int)blockDim.x, depth, guard, visit_limit};
-        return LaneQ<D, CN>{s, cnt};
+        return LaneQ<D, CN>{s, cnt, coop};
     } else {
         GStack s{smem_stack + (threadIdx.x / T) * depth, depth, guard};
         return GroupQ<D, CN>{make_team<T>(), s, cnt};
@@ -130,10 +131,10 @@ __device__ __forceinline__ void save_walk(float4 *slot, const Walk &w, int job =
 }
 
 template <int D, bool SCR>
-__global__ void WOST_WALK_BOUNDS k_walk_plain(const SceneView sc, const SolveParams sp, const Accumulators acc,
+__global__ void WOST_WALK_BOUNDS k_walk_plain(const __grid_constant__ SceneView sc, const SolveParams sp, const Accumulators acc,
                                                     int warp_uniform_points) {
     Cnt<false> cnt;
-    auto q = make_q<D, false>(sp.stack_depth, acc.guard, cnt, sp.visit_limit);
+    auto q = make_q<D, false>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, sp.coop != 0);
     const Group g = make_team<1>();
     const uint64_t total = (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -198,11 +199,11 @@ __device__ __forceinline__ bool hand_over(const HandOver &ho, const CTR *counter
 }
 
 template <int D, bool SCR, int T>
-__global__ void WOST_WALK_BOUNDS k_walk_persistent(const SceneView sc, const SolveParams sp,
+__global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ SceneView sc, const SolveParams sp,
                                                          const Accumulators acc, const SavedWalks src,
                                                          const HandOver ho) {
     Cnt<false> cnt;
-    auto q = make_q<D, false, T>(sp.stack_depth, acc.guard, cnt, sp.visit_limit);
+    auto q = make_q<D, false, T>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, sp.coop != 0);
     const Group g = make_team<T>();
     const uint64_t total =
         src.slots ? (uint64_t)*src.count : (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
@@ -272,10 +273,10 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const SceneView sc, const Sol
 // the longest walks of the solve: their steps spill into later launches
 // while the rest of the grid keeps drawing new walks.
 template <int D, bool SCR, int T>
-__global__ void WOST_WALK_BOUNDS k_walk_resume(const SceneView sc, const SolveParams sp,
+__global__ void WOST_WALK_BOUNDS k_walk_resume(const __grid_constant__ SceneView sc, const SolveParams sp,
                                                      const Accumulators acc, const ResumeState rs, int iters) {
     Cnt<false> cnt;
-    auto q = make_q<D, false, T>(sp.stack_depth, acc.guard, cnt, sp.visit_limit);
+    auto q = make_q<D, false, T>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, sp.coop != 0);
     const Group g = make_team<T>();
     const uint64_t total = (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
     const int lane = threadIdx.x & 31;
@@ -340,10 +341,10 @@ __global__ void WOST_WALK_BOUNDS k_walk_resume(const SceneView sc, const SolvePa
 // Counting variant of the plain kernel: same walks, plus per-query node
 // visits and primitive tests summed into stats[2 * C_NQ] (nodes then prims).
 template <int D, bool SCR>
-__global__ void __launch_bounds__(256) k_walk_count(const SceneView sc, const SolveParams sp, const Accumulators acc,
+__global__ void __launch_bounds__(256) k_walk_count(const __grid_constant__ SceneView sc, const SolveParams sp, const Accumulators acc,
                                                     unsigned long long *stats) {
     Cnt<true> cnt;
-    auto q = make_q<D, true>(sp.stack_depth, acc.guard, cnt, sp.visit_limit);
+    auto q = make_q<D, true>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, sp.coop != 0);
     const Group g = make_team<1>();
     const uint64_t total = (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;

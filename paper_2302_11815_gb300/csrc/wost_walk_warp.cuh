@@ -21,6 +21,7 @@ __device__ __forceinline__ WarpQ<D> make_warp_q(int depth, unsigned int *guard) 
     WarpQ<D> q;
     int2 *mine = smem_stack + (threadIdx.x >> 5) * (kWarpFrontier + depth);
     q.fr = mine;
+    q.frs = 32;
     q.fcap = kWarpFrontier;
     q.st = Stack{mine + kWarpFrontier, 1, depth, guard, 0u};
     q.lane = threadIdx.x & 31;

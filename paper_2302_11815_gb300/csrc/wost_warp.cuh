@@ -225,8 +225,10 @@ struct WarpQ {
     // round of tests costs less than a round of nodes, and four rounds of
     // them less than the tree's two levels of nodes and one of leaves.
     static constexpr int kBrute = 128;
-    int2 *fr;      // frontier (shared memory): (node reference, key)
-    int fcap;
+    // frontier (shared memory): entry j, (node reference, key), at
+    // fr[(j / 32) * frs + j % 32]
+    int2 *fr;
+    int frs, fcap;
     Stack st;      // lane 0's stack for the binary trees
     float scale, tau;  // of the scene
     float eps2;    // square of epsilon, rounded up
@@ -249,6 +251,8 @@ struct WarpQ {
         return make_uint4(__shfl_sync(FULL, rb.x, 0), __shfl_sync(FULL, rb.y, 0), __shfl_sync(FULL, rb.z, 0),
                           __shfl_sync(FULL, rb.w, 0));
     }
+
+    __device__ __forceinline__ int2 &entry(int j) const { return fr[(j >> 5) * frs + (j & 31)]; }
 
     // One frontier search over tree T.  box(child, cone, key) decides whether
     // a child is kept (cone: its record; key orders the visits), prim(k)
@@ -301,7 +305,7 @@ struct WarpQ {
                 m2 = m1 & (m1 - 1u);
                 m3 = m2 & (m2 - 1u);
             } else {
-                if (hit) fr[sp + __popc(hits & ((1u << lane) - 1u))] = make_int2((int)cref, __float_as_int(key));
+                if (hit) entry(sp + __popc(hits & ((1u << lane) - 1u))) = make_int2((int)cref, __float_as_int(key));
                 sp += __popc(hits);
                 __syncwarp();
                 // entries to visit: the four nearest within the bound
@@ -311,7 +315,7 @@ struct WarpQ {
                     const int n = min(sp, 32);
                     bool alive = false;
                     if (lane < n) {
-                        const int2 e = fr[sp - 1 - lane];
+                        const int2 e = entry(sp - 1 - lane);
                         from = (uint32_t)e.x;
                         ekey = __int_as_float(e.y);
                         alive = ekey <= bound();
@@ -348,7 +352,7 @@ struct WarpQ {
                 }
                 __syncwarp();
                 if ((rest >> lane) & 1u)
-                    fr[sp - n + __popc(rest >> lane >> 1)] = make_int2((int)from, __float_as_int(ekey));
+                    entry(sp - n + __popc(rest >> lane >> 1)) = make_int2((int)from, __float_as_int(ekey));
                 sp += __popc(rest) - n;
             }
             const unsigned mine = g == 0 ? m : (g == 1 ? m1 : (g == 2 ? m2 : m3));
@@ -440,13 +444,15 @@ struct WarpQ {
     // grazing one (common on flat walls, where rounding decides the signs)
     // the cone tests above it decide: a candidate whose leaf is culled is
     // none, and the best one's whole path is tested.
-    __device__ __forceinline__ float silhouette_w(const TreeView &T, P3 x, float rmax, bool act) {
-        if (!act || T.root == WOST_EMPTY_REF) return rmax;
+    // B: a bound on the squared distance (beyond that of a certain candidate,
+    // or rmax^2).  certain: the value returned is the one-lane search's.  nr:
+    // around the best distance found.
+    __device__ __forceinline__ float silhouette_search(const TreeView &T, P3 x, float rmax, float B, bool &certain,
+                                                       Near &nr) {
         const float r2 = rmax * rmax;
         LaneBest lb;
         lb.clear();
         bool clear = false;
-        float B = r2;
         auto test = [&](uint32_t k) {
             const float d2 = sil_test<D>(T.prims, k, x, r2);
             if (d2 < INFINITY && d2 <= B) {
@@ -455,6 +461,33 @@ struct WarpQ {
                 if (lb.add(d2, (int)k)) clear = cl;
             }
         };
+        const bool ok = search(
+            T, 3 * kBrute,
+            [&](const WChild &ch, const float4 *cone, float &key) {
+                const float4 cn = __ldg(cone);
+                key = box_dist2<D>(ch.lo, ch.hi, x);
+                bool keep = key < B;
+                if (keep && key > 0.f) keep = may_have_silhouette<D>(ch.lo, ch.hi, cn, x);
+                return keep;
+            },
+            test, [&] { return B; }, [&] { B = fminf(B, beyond(warp_min(lb.d2), tau)); });
+        const float m = warp_min(lb.d2);
+        nr = Near(m, tau);
+        certain = ok;
+        if (m == INFINITY) return rmax;
+        const unsigned at = __ballot_sync(FULL, lb.d2 == m);
+        const bool tie = __any_sync(FULL, (lb.d2 != m && lb.d2 <= nr.lim) || lb.alt <= nr.lim);
+        const int src = __ffs(at) - 1;
+        const int k = __shfl_sync(FULL, lb.rec, src);
+        if (certain && (tie || !(nr.lim2 < r2))) certain = box_dist2_at<D>(T, __ldg(T.leaf_parents + k), x) <= m;
+        if (certain && !__shfl_sync(FULL, (int)clear, src)) certain = path_reached(T, (uint32_t)k, x);
+        if (ok) last_s = k;
+        return sqrtf(m);
+    }
+
+    __device__ __forceinline__ float silhouette_w(const TreeView &T, P3 x, float rmax, bool act, float) {
+        if (!act || T.root == WOST_EMPTY_REF) return rmax;
+        float B = rmax * rmax;
         // the candidates around the last answer and around the last hit bound
         // the new one
         if ((last_s >= 0 || hit_s >= 0) && T.n_prims > 3 * kBrute) {
@@ -462,36 +495,16 @@ struct WarpQ {
             const int k = min(max(mid - 8 + (lane & 15), 0), T.n_prims - 1);
             B = fminf(B, beyond(warp_min(sil_certain<D>(T.prims, (uint32_t)k, x)), tau));
         }
-        const bool ok = search(
-                T, 3 * kBrute,
-                [&](const WChild &ch, const float4 *cone, float &key) {
-                    const float4 cn = __ldg(cone);
-                    key = box_dist2<D>(ch.lo, ch.hi, x);
-                    bool keep = key < B;
-                    if (keep && key > 0.f) keep = may_have_silhouette<D>(ch.lo, ch.hi, cn, x);
-                    return keep;
-                },
-                test, [&] { return B; }, [&] { B = fminf(B, beyond(warp_min(lb.d2), tau)); });
-        const float m = warp_min(lb.d2);
-        if (ok && m == INFINITY) return rmax;
-        const Near nr(m, tau);
-        const unsigned at = __ballot_sync(FULL, lb.d2 == m);
-        const bool tie = __any_sync(FULL, (lb.d2 != m && lb.d2 <= nr.lim) || lb.alt <= nr.lim);
-        const int src = at ? __ffs(at) - 1 : 0;
-        const int k = __shfl_sync(FULL, lb.rec, src);
-        bool certain = ok;
-        if (certain && (tie || !(nr.lim2 < r2))) certain = box_dist2_at<D>(T, __ldg(T.leaf_parents + k), x) <= m;
-        if (certain && !__shfl_sync(FULL, (int)clear, src)) certain = path_reached(T, (uint32_t)k, x);
-        last_s = k;
-        if (certain) return sqrtf(m);
-        if (ok) {
-            // the one-lane search among the candidates near the best one, if
-            // it finds one there (culled candidates can leave none)
-            const float rn = sqrtf(nr.lim2) * 1.000001f;
-            if (rn < rmax) {
-                const float s = silhouette_binary<D>(T, x, rn, st);
-                if (s * s <= nr.lim) return s;
-            }
+        bool certain;
+        Near nr(0.f, tau);
+        const float s = silhouette_search(T, x, rmax, B, certain, nr);
+        if (certain) return s;
+        // the one-lane search among the candidates near the best one, if
+        // it finds one there (culled candidates can leave none)
+        const float rn = sqrtf(nr.lim2) * 1.000001f;
+        if (rn < rmax) {
+            const float t = silhouette_binary<D>(T, x, rn, st);
+            if (t * t <= nr.lim) return t;
         }
         return silhouette_binary<D>(T, x, rmax, st);
     }
@@ -652,5 +665,24 @@ struct WarpQ {
         return hit;
     }
 };
+
+// Q.2 of one lane's walk by its whole warp (every lane calls it with that
+// walk's x, rmax and bound2): for the one-lane kernels, whose warps would
+// otherwise wait for the lane with the longest search.  (answer, 1), or
+// (-, 0) where the binary search has to decide.
+template <int D>
+__device__ __noinline__ float2 coop_silhouette(const TreeView &T, P3 x, float rmax, float bound2, float tau, int2 *fr,
+                                               int frs, int fcap) {
+    WarpQ<D> q;
+    q.fr = fr;
+    q.frs = frs;
+    q.fcap = fcap;
+    q.lane = threadIdx.x & 31;
+    q.tau = tau;
+    bool certain;
+    Near nr(0.f, tau);
+    const float s = q.silhouette_search(T, x, rmax, fminf(rmax * rmax, bound2), certain, nr);
+    return make_float2(s, certain ? 1.f : 0.f);
+}
 
 }  // namespace wost
