@@ -5,10 +5,12 @@
 #include <cuda_runtime.h>
 
 #include <chrono>
+#include <cstring>
 #include <memory>
 #include <atomic>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/wost.h"
@@ -26,19 +28,36 @@ wost_status cuda_fail(cudaError_t e, const char *what);
         if (_e != cudaSuccess) return wost::cuda_fail(_e, what); \
     } while (0)
 
-// device allocation owned by a scene or solve
+// device allocation owned by a scene or solve, or a part of one (view)
 struct DevBuf {
     void *p = nullptr;
     size_t bytes = 0;
+    bool owned = true;
     DevBuf() = default;
     DevBuf(const DevBuf &) = delete;
     DevBuf &operator=(const DevBuf &) = delete;
-    ~DevBuf() {
-        if (p) cudaFree(p);
+    ~DevBuf() { release(); }
+    void release() {
+        if (p && owned) cudaFree(p);
+        p = nullptr;
+        bytes = 0;
+        owned = true;
     }
     cudaError_t alloc(size_t n) {
         bytes = n;
         return n ? cudaMalloc(&p, n) : cudaSuccess;
+    }
+    // at least n bytes (contents lost when it grows)
+    cudaError_t ensure(size_t n) {
+        if (bytes >= n) return cudaSuccess;
+        release();
+        return alloc((n + 65535) & ~(size_t)65535);
+    }
+    void view(void *base, size_t n) {
+        release();
+        p = n ? base : nullptr;
+        bytes = n;
+        owned = false;
     }
     // stream-ordered allocation / release: neither waits for the device,
     // unlike cudaMalloc / cudaFree, which synchronise with all work in flight
@@ -53,12 +72,96 @@ struct DevBuf {
     }
 };
 
-template <class T>
-cudaError_t upload(DevBuf &b, const std::vector<T> &v) {
-    cudaError_t e = b.alloc(v.size() * sizeof(T));
-    if (e == cudaSuccess && !v.empty()) e = cudaMemcpy(b.p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
-    return e;
-}
+// One device allocation for many arrays, filled by one copy: arrays are added
+// to a host image, placed (their buffers become views of the allocation) and
+// uploaded.
+struct DevImage {
+    std::vector<unsigned char> host;
+    std::vector<std::pair<DevBuf *, std::pair<size_t, size_t>>> parts;
+    size_t reserve(size_t n) {
+        const size_t at = (host.size() + 255) & ~(size_t)255;
+        host.resize(at + n);
+        return at;
+    }
+    template <class T>
+    void add(DevBuf &b, const std::vector<T> &v) {
+        const size_t n = v.size() * sizeof(T), at = reserve(n);
+        if (n) std::memcpy(host.data() + at, v.data(), n);
+        parts.push_back({&b, {at, n}});
+    }
+    cudaError_t place(DevBuf &dev) {
+        cudaError_t e = dev.alloc(host.size());
+        if (e != cudaSuccess) return e;
+        for (auto &q : parts) q.first->view((unsigned char *)dev.p + q.second.first, q.second.second);
+        return cudaSuccess;
+    }
+    cudaError_t upload(const DevBuf &dev) const {
+        return cudaMemcpy(dev.p, host.data(), host.size(), cudaMemcpyHostToDevice);
+    }
+};
+
+// What a solve needs beside its results' memory: streams, events, pinned host
+// memory and device buffers.  Setting these up and giving them back took 0.5
+// ms per solve, so a scene keeps those of its last finished solves.
+struct SolveRes {
+    DevBuf main, chain, resume;  // inputs and accumulators; hand-over slots; saved walks
+    unsigned char *host = nullptr;  // pinned, mapped: the cancel flag, then kStaging bytes for results
+    unsigned char *host_dev = nullptr;
+    cudaStream_t stream = nullptr, poll = nullptr;
+    cudaEvent_t ev_start = nullptr, ev_done = nullptr, ev_copy = nullptr;
+    static constexpr size_t kStagingAt = 256, kStaging = 64u << 10;
+    cudaError_t init() {
+        cudaError_t e = cudaHostAlloc((void **)&host, kStagingAt + kStaging, cudaHostAllocMapped);
+        if (e == cudaSuccess) e = cudaHostGetDevicePointer((void **)&host_dev, host, 0);
+        if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&poll, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreate(&ev_start);
+        if (e == cudaSuccess) e = cudaEventCreate(&ev_done);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev_copy, cudaEventDisableTiming);
+        return e;
+    }
+    size_t bytes() const { return main.bytes + chain.bytes + resume.bytes; }
+    ~SolveRes() {
+        for (cudaEvent_t e : {ev_start, ev_done, ev_copy})
+            if (e) cudaEventDestroy(e);
+        for (cudaStream_t s : {stream, poll})
+            if (s) cudaStreamDestroy(s);
+        if (host) cudaFreeHost(host);
+    }
+};
+
+// The idle resources of a scene: at most kIdle sets, kIdleBytes of device
+// memory each; freed with the scene (a set given back later is freed then).
+struct SolvePool {
+    static constexpr size_t kIdle = 4, kIdleBytes = 64u << 20;
+    std::mutex mu;
+    std::vector<std::unique_ptr<SolveRes>> idle;
+    bool closed = false;
+    cudaError_t take(std::unique_ptr<SolveRes> &out) {
+        {
+            std::lock_guard<std::mutex> lk(mu);
+            if (!idle.empty()) {
+                out = std::move(idle.back());
+                idle.pop_back();
+                return cudaSuccess;
+            }
+        }
+        std::unique_ptr<SolveRes> r(new SolveRes);
+        const cudaError_t e = r->init();
+        if (e == cudaSuccess) out = std::move(r);
+        return e;
+    }
+    // (the device is no longer using the set)
+    void give(std::unique_ptr<SolveRes> r) {
+        if (r->bytes() > kIdleBytes) return;
+        std::lock_guard<std::mutex> lk(mu);
+        if (!closed && idle.size() < kIdle) idle.push_back(std::move(r));
+    }
+    void close() {
+        std::lock_guard<std::mutex> lk(mu);
+        closed = true;
+        idle.clear();
+    }
+};
 
 // Words (u64) of a batched launch's counters.
 constexpr size_t kBatchCounters = 4 + 2 * kMaxStages;
@@ -111,12 +214,15 @@ struct wost_scene {
     int device = 0;
     wost::HostScene host;
     wost::SceneView view{};
+    wost::DevBuf image;  // every array below, one allocation
     wost::DevBuf bufs[16];
     wost::DevBuf wbufs[6];  // wide layout: nodes and cones of the three trees
     wost::DevBuf xbufs[18];  // per tree: wide top and its cones, parents, leaf parents, treelets, hints
     wost::DevBuf sbufs[4];  // double-sided records (App. B): - side data and flags of D and N
     wost::DevBuf n_rec_of_id;
-    unsigned int *guard = nullptr;        // device guard word for query kernels
+    unsigned int *guard = nullptr;        // guard word of the query kernels (pinned host memory), its device address
+    unsigned int *guard_dev = nullptr;
+    std::shared_ptr<wost::SolvePool> pool = std::make_shared<wost::SolvePool>();
     wost::SceneView *view_dev = nullptr;  // device copy of `view` (batched launches)
     wost_scene_info info{};
     int stack_depth = 0;                  // traversal stack entries per walk, one lane per walk
@@ -125,8 +231,8 @@ struct wost_scene {
     int tuned_lanes = 1;                  // lanes per walk chosen by wost_scene_autotune
     std::mutex mu;
     ~wost_scene() {
-        if (guard) cudaFree(guard);
-        if (view_dev) cudaFree(view_dev);
+        pool->close();
+        if (guard) cudaFreeHost(guard);
     }
 };
 
@@ -140,14 +246,14 @@ struct wost_solve_handle {
     int lanes = 1;                        // lanes per walk (persistent / resumable kernels)
     bool warp_ok = false;                 // the scene's own traversal limits: walks may run one per warp
     cudaStream_t stream = nullptr;
-    bool own_stream = false;
     cudaStream_t poll_stream = nullptr;
-    bool own_poll_stream = true;  // engine requests share the engine's poll streams
+    bool own_poll_stream = false;  // an engine request whose engine is gone
     cudaEvent_t ev_start = nullptr, ev_done = nullptr;
-    bool own_events = false;
     std::shared_ptr<wost::BatchShared> batch;  // set for solves started by wost_solve_batch
     unsigned int *batch_guard = nullptr;
     wost_engine *engine = nullptr;             // set for solves submitted to an engine
+    std::unique_ptr<wost::SolveRes> res;       // streams, events, memory (not for engine requests)
+    std::shared_ptr<wost::SolvePool> res_pool;  // where they go back to
     wost::SolveParams sp{};
     wost::Accumulators acc{};
     wost::DevBuf points, normals, onN;
@@ -156,7 +262,6 @@ struct wost_solve_handle {
     // resumable solves: saved-walk slots of the fixed grid, launch counters
     // (steps_run u64, live u32), launches enqueued so far
     wost::DevBuf slots, rstate;
-    wost::DevBuf chain[2];  // slots of walks handed over between launches
     int resume_blocks = 0;
     uint64_t launches = 0;
     bool resumable() const { return kernel == WOST_KERNEL_RESUMABLE; }
@@ -179,19 +284,18 @@ struct wost_solve_handle {
     wost_status final_status = WOST_OK;                    // engine requests
     std::mutex mu;
     ~wost_solve_handle() {
-        if (ev_done) cudaEventSynchronize(ev_done);
-        else if (stream) cudaStreamSynchronize(stream);
-        if (own_events && ev_start) cudaEventDestroy(ev_start);
-        if (own_events && ev_done) cudaEventDestroy(ev_done);
+        if (ev_done && launches) cudaEventSynchronize(ev_done);
+        else if (stream) cudaStreamSynchronize(stream);  // nothing launched: its copies
+        if (res) {
+            res_pool->give(std::move(res));
+            return;
+        }
         if (engine_buffers) {
             for (wost::DevBuf *b : {&points, &normals, &onN, &sum, &sumsq, &walks_done, &steps, &globals})
                 b->release_async(poll_stream);
             delete cancel_host;
-        } else if (cancel_host) {
-            cudaFreeHost(cancel_host);
         }
         if (poll_stream && own_poll_stream) cudaStreamDestroy(poll_stream);
-        if (own_stream && stream) cudaStreamDestroy(stream);
     }
 };
 
@@ -210,7 +314,7 @@ constexpr size_t kGlobals = 4 + kMaxStages;
 // Zeroes a solve's accumulators and counters on `stream`.
 cudaError_t clear_accumulators(wost_solve_handle *h, cudaStream_t stream);
 // Blocks until the work queued so far on `stream` (the input copies) is done.
-wost_status wait_for_copies(cudaStream_t stream);
+wost_status wait_for_copies(cudaStream_t stream, cudaEvent_t ev);
 // Engine side of wost_solve_destroy / wost_cancel for engine requests.
 void engine_detach(wost_engine *e, wost_solve_handle *h);
 }  // namespace wost

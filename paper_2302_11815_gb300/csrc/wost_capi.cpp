@@ -59,15 +59,41 @@ wost_status wost_scene_create(const wost_scene_desc *desc, wost_scene **out) {
         HostTree *trees[3] = {&H.D, &H.N, &H.S};
         TreeView *views[3] = {&s->view.D, &s->view.N, &s->view.S};
         int64_t bytes = 0;
+        // all arrays in one allocation and one copy
+        DevImage img;
         for (int t = 0; t < 3; ++t) {
             HostTree &T = *trees[t];
-            DevBuf *b = &s->bufs[5 * t];
-            CK(upload(b[0], T.nodes), "upload nodes");
-            CK(upload(b[1], T.cones), "upload cones");
-            CK(upload(b[2], T.prims), "upload prims");
-            CK(upload(b[3], T.data), "upload data");
-            CK(upload(b[4], T.ids), "upload ids");
-            for (int k = 0; k < 5; ++k) bytes += (int64_t)b[k].bytes;
+            DevBuf *b = &s->bufs[5 * t], *w = &s->wbufs[2 * t], *x = &s->xbufs[6 * t];
+            img.add(b[0], T.nodes);
+            img.add(b[1], T.cones);
+            img.add(b[2], T.prims);
+            img.add(b[3], T.data);
+            img.add(b[4], T.ids);
+            img.add(w[0], T.wnodes);
+            img.add(w[1], T.wcones);
+            img.add(x[0], T.wtop);
+            img.add(x[1], T.wtopcones);
+            img.add(x[2], T.parents);
+            img.add(x[3], T.leaf_parents);
+            img.add(x[4], T.treelets);
+            img.add(x[5], T.hints);
+        }
+        for (int t = 0; t < 2; ++t) {  // double-sided records of D and N
+            img.add(s->sbufs[2 * t], trees[t]->data_minus);
+            img.add(s->sbufs[2 * t + 1], trees[t]->sided);
+        }
+        img.add(s->bufs[15], H.grid);
+        std::vector<int32_t> rec_of_id((size_t)desc->n_prims, -1);
+        for (size_t k = 0; k < H.N.ids.size(); ++k) rec_of_id[H.N.ids[k]] = (int32_t)k;
+        img.add(s->n_rec_of_id, rec_of_id);
+        const size_t view_at = img.reserve(sizeof(SceneView));
+        CK(img.place(s->image), "cudaMalloc scene");
+        s->view_dev = (SceneView *)((unsigned char *)s->image.p + view_at);
+        for (auto &q : img.parts)
+            if (q.first != &s->n_rec_of_id) bytes += (int64_t)q.first->bytes;
+        for (int t = 0; t < 3; ++t) {
+            HostTree &T = *trees[t];
+            DevBuf *b = &s->bufs[5 * t], *w = &s->wbufs[2 * t], *x = &s->xbufs[6 * t];
             TreeView &V = *views[t];
             V.nodes = (const float4 *)b[0].p;
             V.cones = (const float4 *)b[1].p;
@@ -83,18 +109,6 @@ wost_status wost_scene_create(const wost_scene_desc *desc, wost_scene **out) {
             V.n_prims = T.n_prims;
             V.n_nodes = T.n_nodes;
             V.depth = T.depth;
-            DevBuf *w = &s->wbufs[2 * t];
-            CK(upload(w[0], T.wnodes), "upload wide nodes");
-            CK(upload(w[1], T.wcones), "upload wide cones");
-            bytes += (int64_t)(w[0].bytes + w[1].bytes);
-            DevBuf *x = &s->xbufs[6 * t];
-            CK(upload(x[0], T.wtop), "upload wide top");
-            CK(upload(x[1], T.wtopcones), "upload wide top");
-            CK(upload(x[2], T.parents), "upload parents");
-            CK(upload(x[3], T.leaf_parents), "upload parents");
-            CK(upload(x[4], T.treelets), "upload treelets");
-            CK(upload(x[5], T.hints), "upload hints");
-            for (int k = 0; k < 6; ++k) bytes += (int64_t)x[k].bytes;
             V.hints = (const uint32_t *)x[5].p;
             V.wtop = (const float4 *)x[0].p;
             V.wtopcones = (const float4 *)x[1].p;
@@ -107,21 +121,13 @@ wost_status wost_scene_create(const wost_scene_desc *desc, wost_scene **out) {
             V.wn_nodes = T.wn_nodes;
             V.wdepth = T.wdepth;
         }
-        for (int t = 0; t < 2; ++t) {  // double-sided records of D and N
-            HostTree &T = *trees[t];
-            CK(upload(s->sbufs[2 * t], T.data_minus), "upload data");
-            CK(upload(s->sbufs[2 * t + 1], T.sided), "upload flags");
-            bytes += (int64_t)(s->sbufs[2 * t].bytes + s->sbufs[2 * t + 1].bytes);
+        for (int t = 0; t < 2; ++t) {
             views[t]->data_minus = (const float4 *)s->sbufs[2 * t].p;
             views[t]->sided = (const uint8_t *)s->sbufs[2 * t + 1].p;
         }
-        CK(upload(s->bufs[15], H.grid), "upload grid");
-        bytes += (int64_t)s->bufs[15].bytes;
-        std::vector<int32_t> rec_of_id((size_t)desc->n_prims, -1);
-        for (size_t k = 0; k < H.N.ids.size(); ++k) rec_of_id[H.N.ids[k]] = (int32_t)k;
-        CK(upload(s->n_rec_of_id, rec_of_id), "upload map");
-        CK(cudaMalloc(&s->guard, sizeof(unsigned int)), "cudaMalloc guard");
-        CK(cudaMemset(s->guard, 0, sizeof(unsigned int)), "cudaMemset guard");
+        CK(cudaHostAlloc((void **)&s->guard, sizeof(unsigned int), cudaHostAllocMapped), "cudaHostAlloc guard");
+        *s->guard = 0;
+        CK(cudaHostGetDevicePointer((void **)&s->guard_dev, s->guard, 0), "cudaHostGetDevicePointer");
         s->view.dim = H.dim;
         s->view.g = H.g;
         s->view.h = H.h;
@@ -148,8 +154,8 @@ wost_status wost_scene_create(const wost_scene_desc *desc, wost_scene **out) {
         // 8-wide trees: at most 7 pending subtrees per level; odd, so that
         // the teams of a warp start in different shared-memory banks
         s->stack_depth_team = ((WOST_WIDE - 1) * std::max(H.D.wdepth, std::max(H.N.wdepth, H.S.wdepth)) + 1) | 1;
-        CK(cudaMalloc(&s->view_dev, sizeof(SceneView)), "cudaMalloc view");
-        CK(cudaMemcpy(s->view_dev, &s->view, sizeof(SceneView), cudaMemcpyHostToDevice), "copy view");
+        std::memcpy(img.host.data() + view_at, &s->view, sizeof(SceneView));
+        CK(img.upload(s->image), "upload scene");
         wost_scene_info &I = s->info;
         I.dim = H.dim;
         I.n_dirichlet = H.n_dirichlet;
@@ -258,6 +264,7 @@ void wost::set_layout_info(wost_scene *s, int lanes) {
 cudaError_t wost::clear_accumulators(wost_solve_handle *h, cudaStream_t stream) {
     const size_t n = (size_t)h->n_points;
     cudaError_t e = cudaSuccess;
+    if (h->res) return cudaMemsetAsync(h->globals.p, 0, h->globals.bytes + 4 * n * 8, stream);  // (one after the other)
     for (DevBuf *b : {&h->sum, &h->sumsq, &h->walks_done, &h->steps})
         if (e == cudaSuccess) e = cudaMemsetAsync(b->p, 0, n * 8, stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(h->globals.p, 0, kGlobals * 8, stream);
@@ -309,36 +316,64 @@ wost_status wost::prepare_solve(wost_scene *scene, const wost_solve_desc *d, cud
     h->lanes = lanes;
     h->stream = stream;
     const int dim = h->dim;
-    if (!h->poll_stream) {  // (the serving engine assigns one of its own)
-        CK(cudaStreamCreateWithFlags(&h->poll_stream, cudaStreamNonBlocking), "cudaStreamCreate");
-        h->own_poll_stream = true;
-    }
-    const size_t n = (size_t)d->n_points;
-    // engine requests allocate on the engine's stream without waiting for it
-    auto alloc = [&](DevBuf &b, size_t bytes) {
-        return h->engine_buffers ? b.alloc_async(bytes, stream, h->pool) : b.alloc(bytes);
-    };
-    CK(alloc(h->points, n * dim * sizeof(float)), "cudaMalloc points");
-    cudaMemcpyKind kind = d->memory == WOST_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
-    if (fill) CK(cudaMemcpyAsync(h->points.p, d->points, n * dim * sizeof(float), kind, stream), "copy points");
-    if (d->normals && d->on_neumann) {
-        CK(alloc(h->normals, n * dim * sizeof(float)), "cudaMalloc normals");
-        CK(alloc(h->onN, n), "cudaMalloc on_neumann");
-        if (fill) {
-            CK(cudaMemcpyAsync(h->normals.p, d->normals, n * dim * sizeof(float), kind, stream), "copy normals");
-            CK(cudaMemcpyAsync(h->onN.p, d->on_neumann, n, kind, stream), "copy on_neumann");
+    const size_t n = (size_t)d->n_points, pb = n * dim * sizeof(float);
+    const bool has_n = d->normals && d->on_neumann;
+    if (h->engine_buffers) {
+        // engine requests allocate on the engine's stream without waiting for it
+        auto alloc = [&](DevBuf &b, size_t bytes) { return b.alloc_async(bytes, stream, h->pool); };
+        CK(alloc(h->points, pb), "cudaMalloc points");
+        if (has_n) {
+            CK(alloc(h->normals, pb), "cudaMalloc normals");
+            CK(alloc(h->onN, n), "cudaMalloc on_neumann");
+        }
+        CK(alloc(h->sum, n * 8), "cudaMalloc accumulators");
+        CK(alloc(h->sumsq, n * 8), "cudaMalloc accumulators");
+        CK(alloc(h->walks_done, n * 8), "cudaMalloc accumulators");
+        CK(alloc(h->steps, n * 8), "cudaMalloc accumulators");
+        CK(alloc(h->globals, kGlobals * 8), "cudaMalloc accumulators");
+    } else {
+        h->res_pool = scene->pool;
+        CK(scene->pool->take(h->res), "streams, events and pinned memory of a solve");
+        SolveRes &R = *h->res;
+        if (!stream) {  // no stream given: the set's own
+            if (!R.stream) CK(cudaStreamCreateWithFlags(&R.stream, cudaStreamNonBlocking), "cudaStreamCreate");
+            stream = R.stream;
+        }
+        h->stream = stream;
+        h->poll_stream = R.poll;
+        h->cancel_host = (int *)R.host;
+        h->cancel_dev = (int *)R.host_dev;
+        *h->cancel_host = 0;
+        // globals, sum, sumsq, walks, steps one after the other (one memset,
+        // one copy per poll), then the inputs
+        const size_t need = kGlobals * 8 + 4 * n * 8 + 2 * pb + n + 64;
+        CK(R.main.ensure(need), "cudaMalloc accumulators");
+        unsigned char *p = (unsigned char *)R.main.p;
+        auto part = [&](DevBuf &b, size_t bytes) {
+            b.view(p, bytes);
+            p += (bytes + 15) & ~(size_t)15;
+        };
+        static_assert(kGlobals % 2 == 0, "no gap before the sums");
+        part(h->globals, kGlobals * 8);
+        h->sum.view(p, n * 8);
+        h->sumsq.view(p + n * 8, n * 8);
+        h->walks_done.view(p + 2 * n * 8, n * 8);
+        h->steps.view(p + 3 * n * 8, n * 8);
+        p += 4 * n * 8;
+        part(h->points, pb);
+        if (has_n) {
+            part(h->normals, pb);
+            part(h->onN, n);
         }
     }
-    CK(alloc(h->sum, n * 8), "cudaMalloc accumulators");
-    CK(alloc(h->sumsq, n * 8), "cudaMalloc accumulators");
-    CK(alloc(h->walks_done, n * 8), "cudaMalloc accumulators");
-    CK(alloc(h->steps, n * 8), "cudaMalloc accumulators");
-    CK(alloc(h->globals, kGlobals * 8), "cudaMalloc accumulators");
-    if (fill) CK(clear_accumulators(h, stream), "memset");
-    if (!h->cancel_host) {
-        CK(cudaHostAlloc((void **)&h->cancel_host, sizeof(int), cudaHostAllocMapped), "cudaHostAlloc");
-        *h->cancel_host = 0;
-        CK(cudaHostGetDevicePointer((void **)&h->cancel_dev, h->cancel_host, 0), "cudaHostGetDevicePointer");
+    cudaMemcpyKind kind = d->memory == WOST_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+    if (fill) {
+        CK(cudaMemcpyAsync(h->points.p, d->points, pb, kind, stream), "copy points");
+        if (has_n) {
+            CK(cudaMemcpyAsync(h->normals.p, d->normals, pb, kind, stream), "copy normals");
+            CK(cudaMemcpyAsync(h->onN.p, d->on_neumann, n, kind, stream), "copy on_neumann");
+        }
+        CK(clear_accumulators(h, stream), "memset");
     }
     SolveParams &sp = h->sp;
     sp = SolveParams{};
@@ -377,27 +412,24 @@ wost_status wost::prepare_solve(wost_scene *scene, const wost_solve_desc *d, cud
 }
 
 // The caller's arrays may be released once a solve call returns.
-wost_status wost::wait_for_copies(cudaStream_t stream) {
-    cudaEvent_t copied;
-    CK(cudaEventCreateWithFlags(&copied, cudaEventDisableTiming), "cudaEventCreate");
-    cudaEventRecord(copied, stream);
-    cudaError_t ce = cudaEventSynchronize(copied);
-    cudaEventDestroy(copied);
-    if (ce != cudaSuccess) return cuda_fail(ce, "input copy");
+wost_status wost::wait_for_copies(cudaStream_t stream, cudaEvent_t ev) {
+    CK(cudaEventRecord(ev, stream), "cudaEventRecord");
+    CK(cudaEventSynchronize(ev), "input copy");
     return WOST_OK;
 }
 
 // The slot arrays of a solve's chain of launches (allocated once) and its
 // counters in the solve's globals (still zero: a solve runs one chain).
 static cudaError_t chain_buffers(wost_solve_handle *h, uint64_t walks, int blocks, ChainBuffers *cb) {
+    size_t bytes[2];
     for (int i = 0; i < 2; ++i) {
         cb->cap[i] = (unsigned)chain_capacity(walks, h->block, blocks, i);
-        if (!h->chain[i].p) {
-            cudaError_t e = h->chain[i].alloc((size_t)cb->cap[i] * 3 * sizeof(float4));
-            if (e != cudaSuccess) return e;
-        }
-        cb->slots[i] = (float4 *)h->chain[i].p;
+        bytes[i] = (size_t)cb->cap[i] * 3 * sizeof(float4);
     }
+    cudaError_t e = h->res->chain.ensure(bytes[0] + bytes[1]);
+    if (e != cudaSuccess) return e;
+    cb->slots[0] = (float4 *)h->res->chain.p;
+    cb->slots[1] = (float4 *)((unsigned char *)h->res->chain.p + bytes[0]);
     cb->counters = (unsigned int *)((unsigned long long *)h->globals.p + 4);
     return cudaSuccess;
 }
@@ -410,33 +442,28 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
         *out = nullptr;
         CK(cudaSetDevice(scene->device), "cudaSetDevice");
         std::unique_ptr<wost_solve_handle> h(new wost_solve_handle);
-        cudaStream_t stream = (cudaStream_t)d->stream;
-        if (!stream) {
-            CK(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking), "cudaStreamCreate");
-            h->own_stream = true;
-            h->stream = stream;
-        }
-        wost_status st = prepare_solve(scene, d, stream, h.get());
+        wost_status st = prepare_solve(scene, d, (cudaStream_t)d->stream, h.get());
         if (st != WOST_OK) return st;
-        CK(cudaEventCreate(&h->ev_start), "cudaEventCreate");
-        CK(cudaEventCreate(&h->ev_done), "cudaEventCreate");
-        h->own_events = true;
+        const cudaStream_t stream = h->stream;
+        h->ev_start = h->res->ev_start;
+        h->ev_done = h->res->ev_done;
         if (d->kernel == WOST_KERNEL_RESUMABLE) {
             // state only; the launches come from wost_solve_advance
             CK(resume_grid(h->dim, h->block, h->sp.stack_depth, &h->resume_blocks, h->lanes), "occupancy");
-            CK(h->slots.alloc((size_t)resume_slots(h->block, h->resume_blocks, h->lanes) * 3 * sizeof(float4)),
-               "cudaMalloc slots");
-            // counters (steps_run u64; live u32; the tail's work counter u32),
-            // then the list of the saved walks' slots
+            // slots; counters (steps_run u64; live u32; the tail's work
+            // counter u32); the list of the saved walks' slots
             const size_t n_slots = (size_t)resume_slots(h->block, h->resume_blocks, h->lanes);
-            CK(h->rstate.alloc(16 + n_slots * sizeof(uint32_t)), "cudaMalloc counters");
+            const size_t slot_bytes = n_slots * 3 * sizeof(float4), state_bytes = 16 + n_slots * sizeof(uint32_t);
+            CK(h->res->resume.ensure(slot_bytes + state_bytes), "cudaMalloc slots");
+            h->slots.view(h->res->resume.p, slot_bytes);
+            h->rstate.view((unsigned char *)h->res->resume.p + slot_bytes, state_bytes);
             CK(cudaMemsetAsync(h->slots.p, 0, h->slots.bytes, stream), "memset");
             CK(cudaMemsetAsync(h->rstate.p, 0, 16, stream), "memset");
-            if ((st = wait_for_copies(stream)) != WOST_OK) return st;
+            if ((st = wait_for_copies(stream, h->res->ev_copy)) != WOST_OK) return st;
             *out = h.release();
             return WOST_OK;
         }
-        if ((st = wait_for_copies(stream)) != WOST_OK) return st;
+        if ((st = wait_for_copies(stream, h->res->ev_copy)) != WOST_OK) return st;
         const SolveParams &sp = h->sp;
         const Accumulators &acc = h->acc;
         h->t_launch = std::chrono::steady_clock::now();
@@ -548,7 +575,7 @@ wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_so
         }
         CK(cudaEventCreate(&shared->ev_start), "cudaEventCreate");
         CK(cudaEventCreate(&shared->ev_done), "cudaEventCreate");
-        wost_status st = wait_for_copies(stream);
+        wost_status st = wait_for_copies(stream, hs[0]->res->ev_copy);
         if (st != WOST_OK) return st;
         auto t0 = std::chrono::steady_clock::now();
         CK(cudaEventRecord(shared->ev_start, stream), "cudaEventRecord");
@@ -661,13 +688,29 @@ wost_status wost_poll(wost_solve_handle *h, double *mean, double *se, uint64_t *
             }
             return WOST_OK;
         }
-        std::vector<double> s(n), q(n);
-        std::vector<unsigned long long> w(n), stp(n), glob(4);
-        CK(cudaMemcpyAsync(s.data(), h->sum.p, n * 8, cudaMemcpyDeviceToHost, h->poll_stream), "poll copy");
-        CK(cudaMemcpyAsync(q.data(), h->sumsq.p, n * 8, cudaMemcpyDeviceToHost, h->poll_stream), "poll copy");
-        CK(cudaMemcpyAsync(w.data(), h->walks_done.p, n * 8, cudaMemcpyDeviceToHost, h->poll_stream), "poll copy");
-        if (pr) CK(cudaMemcpyAsync(stp.data(), h->steps.p, n * 8, cudaMemcpyDeviceToHost, h->poll_stream), "poll copy");
-        CK(cudaMemcpyAsync(glob.data(), h->globals.p, 4 * 8, cudaMemcpyDeviceToHost, h->poll_stream), "poll copy");
+        // globals, sums, walks and steps: one block on the device, copied
+        // through the solve's pinned staging when it fits (engine requests:
+        // one by one)
+        const size_t gw = kGlobals, words = gw + 4 * n;
+        std::vector<unsigned long long> store;
+        unsigned long long *blk = nullptr;
+        if (h->res && words * 8 <= SolveRes::kStaging) {
+            blk = (unsigned long long *)(h->res->host + SolveRes::kStagingAt);
+        } else {
+            store.resize(words);
+            blk = store.data();
+        }
+        if (h->res) {
+            CK(cudaMemcpyAsync(blk, h->globals.p, (pr ? words : words - n) * 8, cudaMemcpyDeviceToHost, h->poll_stream),
+               "poll copy");
+        } else {
+            const DevBuf *src[5] = {&h->globals, &h->sum, &h->sumsq, &h->walks_done, &h->steps};
+            for (int i = 0; i < (pr ? 5 : 4); ++i)
+                CK(cudaMemcpyAsync(i ? blk + gw + (i - 1) * n : blk, src[i]->p, (i ? n : gw) * 8,
+                                   cudaMemcpyDeviceToHost, h->poll_stream), "poll copy");
+        }
+        const unsigned long long *glob = blk, *w = blk + gw + 2 * n, *stp = blk + gw + 3 * n;
+        const double *s = (const double *)(blk + gw), *q = (const double *)(blk + gw + n);
         unsigned int bg = 0;
         if (h->batch_guard)
             CK(cudaMemcpyAsync(&bg, h->batch_guard, sizeof bg, cudaMemcpyDeviceToHost, h->poll_stream), "poll copy");
@@ -788,7 +831,9 @@ wost_status wost_wait(wost_solve_handle *h, double timeout_s) {
         }
         double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         if (timeout_s >= 0 && el >= timeout_s) return fail(WOST_ERR_TIMEOUT, "solve not finished");
-        std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 20 : 500));
+        // (a sleep takes ~70 us at least: short solves are polled)
+        if (el < 0.001) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds(el < 0.01 ? 20 : 500));
     }
     if (h->engine || !h->ev_done) {  // engine request: its outcome was recorded by the engine
         if (h->final_status == WOST_ERR_CANCELLED) return fail(WOST_ERR_CANCELLED, "solve was cancelled");
@@ -796,9 +841,19 @@ wost_status wost_wait(wost_solve_handle *h, double timeout_s) {
         return WOST_OK;
     }
     unsigned long long glob[4];
-    CK(cudaMemcpy(glob, h->globals.p, sizeof glob, cudaMemcpyDeviceToHost), "copy guard");
     unsigned int bg = 0;
-    if (h->batch_guard) CK(cudaMemcpy(&bg, h->batch_guard, sizeof bg, cudaMemcpyDeviceToHost), "copy guard");
+    {
+        // (pinned words beside the cancel flag, under the lock as poll's staging)
+        std::lock_guard<std::mutex> lk(h->mu);
+        unsigned char *pin = h->res->host + 64;
+        CK(cudaMemcpyAsync(pin, h->globals.p, sizeof glob, cudaMemcpyDeviceToHost, h->poll_stream), "copy guard");
+        if (h->batch_guard)
+            CK(cudaMemcpyAsync(pin + sizeof glob, h->batch_guard, sizeof bg, cudaMemcpyDeviceToHost, h->poll_stream),
+               "copy guard");
+        CK(cudaStreamSynchronize(h->poll_stream), "copy guard");
+        std::memcpy(glob, pin, sizeof glob);
+        if (h->batch_guard) std::memcpy(&bg, pin + sizeof glob, sizeof bg);
+    }
     if ((uint32_t)glob[2] | bg) return fail(WOST_ERR_INTERNAL, "device guard fired (traversal stack overflow or visit limit)");
     if (*(volatile int *)h->cancel_host) return fail(WOST_ERR_CANCELLED, "solve was cancelled");
     return WOST_OK;
@@ -855,10 +910,8 @@ static wost_status query_prologue(wost_scene *s, int64_t n) {
 }
 static wost_status query_epilogue(wost_scene *s, cudaError_t e, cudaStream_t st) {
     if (e != cudaSuccess) return cuda_fail(e, "query launch");
-    unsigned int g = 0;
-    CK(cudaMemcpyAsync(&g, s->guard, sizeof g, cudaMemcpyDeviceToHost, st), "copy guard");
     CK(cudaStreamSynchronize(st), "query sync");
-    if (g) return fail(WOST_ERR_INTERNAL, "device guard fired (traversal stack overflow or visit limit)");
+    if (*(volatile unsigned int *)s->guard) return fail(WOST_ERR_INTERNAL, "device guard fired (traversal stack overflow or visit limit)");
     return WOST_OK;
 }
 
@@ -869,7 +922,7 @@ wost_status wost_query_closest_dirichlet(wost_scene *s, int64_t n, const float *
     if (!n) return WOST_OK;
     if (!pts || !dist || !closest || !prim) return fail(WOST_ERR_INVALID_ARG, "null array");
     std::lock_guard<std::mutex> lk(s->mu);
-    cudaError_t e = launch_query_closest(s->view, n, pts, dist, closest, prim, s->stack_depth, s->guard,
+    cudaError_t e = launch_query_closest(s->view, n, pts, dist, closest, prim, s->stack_depth, s->guard_dev,
                                          (cudaStream_t)stream);
     return query_epilogue(s, e, (cudaStream_t)stream);
 }
@@ -881,7 +934,7 @@ wost_status wost_query_silhouette(wost_scene *s, int64_t n, const float *pts, co
     if (!n) return WOST_OK;
     if (!pts || !rmax || !dist) return fail(WOST_ERR_INVALID_ARG, "null array");
     std::lock_guard<std::mutex> lk(s->mu);
-    cudaError_t e = launch_query_silhouette(s->view, n, pts, rmax, dist, s->stack_depth, s->guard, (cudaStream_t)stream);
+    cudaError_t e = launch_query_silhouette(s->view, n, pts, rmax, dist, s->stack_depth, s->guard_dev, (cudaStream_t)stream);
     return query_epilogue(s, e, (cudaStream_t)stream);
 }
 
@@ -894,7 +947,7 @@ wost_status wost_query_intersect_neumann(wost_scene *s, int64_t n, const float *
     std::lock_guard<std::mutex> lk(s->mu);
     cudaError_t e = launch_query_ray(s->view, n, o, v, tmax, skip, (const int32_t *)s->n_rec_of_id.p,
                                      (int64_t)(s->n_rec_of_id.bytes / sizeof(int32_t)), hit, t, prim, s->stack_depth,
-                                     s->guard, (cudaStream_t)stream);
+                                     s->guard_dev, (cudaStream_t)stream);
     return query_epilogue(s, e, (cudaStream_t)stream);
 }
 
