@@ -51,7 +51,8 @@ __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hd
     Walk w{};
     int job = -1;
     unsigned int ran = 0;  // steps of this lane's finished walks
-    bool drained = false;  // the launch's counter has run past `total`
+    // the launch's counter has run past `total`, or the lane holds no walks
+    bool drained = src.per_warp && lane >= (int)src.per_warp;
     // as in k_walk_persistent: the whole warp stays in the loop and
     // reconverges after every step
     for (;;) {

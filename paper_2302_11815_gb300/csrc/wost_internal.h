@@ -149,6 +149,7 @@ struct SavedWalks {
     const unsigned int *count;      // [1] how many
     unsigned int *next;             // [1] work counter
     unsigned long long *steps_run;  // [1] receives the steps run (may be null)
+    unsigned int per_warp;          // one-lane kernels: walks a warp holds at most (0: 32)
 };
 
 // Where a one-lane kernel hands its last walks over (slots filled from the

@@ -157,7 +157,7 @@ cudaError_t launch_walk_persistent(const SceneView &sc, const SolveParams &sp, c
                                    int blocks, cudaStream_t s, int lanes, const SavedWalks &src, const HandOver &ho) {
     if (lanes == WOST_WIDE) return launch_walk_persistent_team(sc, sp, acc, block, blocks, s);
     HandOver h = ho;
-    h.lanes = (unsigned)blocks * (unsigned)block;
+    h.lanes = (unsigned)blocks * (unsigned)(block / 32) * (src.per_warp ? src.per_warp : 32u);
     if (sp.sigma > 0.f) return launch_walk_persistent_scr(sc, sp, acc, src, h, block, blocks, s);
     return walk_persistent_launch<false, 1>(sc, sp, acc, src, h, block, blocks, s);
 }
@@ -176,10 +176,11 @@ cudaError_t launch_walk_chain(const SceneView &sc, const SolveParams &sp, const 
         most = std::min<uint64_t>(most, cb.cap[b]);
         unsigned int *ctr = cb.counters + 2 * stage;
         const HandOver ho{cb.slots[b], ctr, (unsigned)most, 0u};
-        const int grid = (int)std::min<uint64_t>((uint64_t)blocks, (walks + block - 1) / block);
+        const uint64_t per_block = (uint64_t)(block / 32) * (src.per_warp ? src.per_warp : 32u);
+        const int grid = (int)std::min<uint64_t>((uint64_t)blocks, (walks + per_block - 1) / per_block);
         cudaError_t e = launch_walk_persistent(sc, sp, acc, block, grid, s, 1, src, ho);
         if (e != cudaSuccess) return e;
-        src = SavedWalks{cb.slots[b], nullptr, ctr, ctr + 1, src.steps_run};
+        src = SavedWalks{cb.slots[b], nullptr, ctr, ctr + 1, src.steps_run, spread_walks(sc.dim, most)};
         walks = most;
     }
     return launch_walk_warp(sc, sp, acc, src, walks, s);

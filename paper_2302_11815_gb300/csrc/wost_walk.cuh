@@ -210,7 +210,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ Scene
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
     Walk w{};
-    bool have = false, drained = false;  // uniform within a team
+    bool have = false, drained = T == 1 && src.per_warp && lane >= (int)src.per_warp;  // uniform within a team
     // All 32 lanes stay in this loop until the warp runs out of work, call
     // the warp-synchronous walk_step together (lanes without a walk take part
     // in its meetings only) and meet at __syncwarp() after every walk step,
