@@ -63,7 +63,16 @@ cudaError_t launch_request_stats(const StatJob *jobs, int n_jobs, int64_t max_po
 }
 
 // ------------------------------- queries ---------------------------------
-// one team per query; the team's leader writes the answer
+// one lane per query.  Few queries run one per warp instead
+// (wost_kernels_query.cu): one lane's chain of node visits takes 30 to 1,400
+// us however few there are.  One lane / one warp per query, us per call of
+// 4,000 / 16,000 / 65,000 / 250,000 queries:
+//   Q.1  torus 45 43 43 53 / 49 64 128 369; Koch (1,000: 56 / 46) 54 58 / 47 70
+//   Q.2  torus 843 1110 1116 1440 / 84 111 192 540; box-sphere 314 345 365 660
+//        / 45 48 91 245 (3D: always one per warp); Koch 111 122 / 29 39
+//   Q.3  torus 81 81 111 136 / 49 61 83 179; box-sphere 43 46 46 60 / 35 41 64
+//        138; Koch 51 50 / 36 46
+//   Q.4  torus 36 38 39 56 / 32 38 70 191; Koch 35 34 / 31 39
 template <int D>
 __global__ void k_query_closest(const SceneView sc, int64_t n, const float *pts, float *dist, float *closest,
                                 int32_t *prim, int depth, unsigned int *guard) {
@@ -214,6 +223,7 @@ static cudaError_t query_smem(const void *fn, size_t bytes) {
 
 cudaError_t launch_query_closest(const SceneView &sc, int64_t n, const float *pts, float *dist, float *closest,
                                  int32_t *prim, int depth, unsigned int *guard, cudaStream_t s) {
+    if (n <= kWarpClosest) return launch_query_closest_warp(sc, n, pts, dist, closest, prim, depth, guard, s);
     const int block = 128;
     unsigned grid = (unsigned)((n + block - 1) / block);
     size_t sm = smem_bytes(depth, block);
@@ -231,24 +241,22 @@ cudaError_t launch_query_closest(const SceneView &sc, int64_t n, const float *pt
 
 cudaError_t launch_query_silhouette(const SceneView &sc, int64_t n, const float *pts, const float *rmax, float *dist,
                                     int depth, unsigned int *guard, cudaStream_t s) {
+    if (sc.dim == 3 || n <= kWarpSilhouette2D)
+        return launch_query_silhouette_warp(sc, n, pts, rmax, dist, depth, guard, s);
     const int block = 128;
     unsigned grid = (unsigned)((n + block - 1) / block);
     size_t sm = smem_bytes(depth, block);
-    if (sc.dim == 2) {
-        cudaError_t e = query_smem((const void *)k_query_silhouette<2>, sm);
-        if (e != cudaSuccess) return e;
-        k_query_silhouette<2><<<grid, block, sm, s>>>(sc, n, pts, rmax, dist, depth, guard);
-    } else {
-        cudaError_t e = query_smem((const void *)k_query_silhouette<3>, sm);
-        if (e != cudaSuccess) return e;
-        k_query_silhouette<3><<<grid, block, sm, s>>>(sc, n, pts, rmax, dist, depth, guard);
-    }
+    cudaError_t e = query_smem((const void *)k_query_silhouette<2>, sm);
+    if (e != cudaSuccess) return e;
+    k_query_silhouette<2><<<grid, block, sm, s>>>(sc, n, pts, rmax, dist, depth, guard);
     return cudaGetLastError();
 }
 
 cudaError_t launch_query_ray(const SceneView &sc, int64_t n, const float *o, const float *v, const float *tmax,
                              const int32_t *skip, const int32_t *rec_of_id, int64_t n_ids, int32_t *hit, float *t,
                              int32_t *prim, int depth, unsigned int *guard, cudaStream_t s) {
+    if (n <= (sc.dim == 2 ? kWarpRay2D : kWarpRay3D))
+        return launch_query_ray_warp(sc, n, o, v, tmax, skip, rec_of_id, n_ids, hit, t, prim, depth, guard, s);
     const int block = 128;
     unsigned grid = (unsigned)((n + block - 1) / block);
     size_t sm = smem_bytes(depth, block);
@@ -267,6 +275,7 @@ cudaError_t launch_query_ray(const SceneView &sc, int64_t n, const float *o, con
 cudaError_t launch_query_sample(const SceneView &sc, int64_t n, const float *pts, const float *r, uint32_t k0,
                                 uint32_t k1, uint32_t c1, uint32_t c2, float *z, float *pdf, int32_t *prim,
                                 cudaStream_t s) {
+    if (n <= kWarpSample) return launch_query_sample_warp(sc, n, pts, r, k0, k1, c1, c2, z, pdf, prim, s);
     const int block = 128;
     unsigned grid = (unsigned)((n + block - 1) / block);
     if (sc.dim == 2)

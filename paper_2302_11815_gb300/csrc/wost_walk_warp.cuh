@@ -15,10 +15,10 @@ namespace wost {
 
 constexpr int kWarpFrontier = 192;  // frontier entries per warp (an overflow falls back to the binary trees)
 
-template <int D>
-__device__ __forceinline__ WarpQ<D> make_warp_q(int depth, unsigned int *guard) {
+template <int D, bool WALK = true>
+__device__ __forceinline__ WarpQ<D, WALK> make_warp_q(int depth, unsigned int *guard) {
     extern __shared__ int2 smem_stack[];
-    WarpQ<D> q;
+    WarpQ<D, WALK> q;
     int2 *mine = smem_stack + (threadIdx.x >> 5) * (kWarpFrontier + depth);
     q.fr = mine;
     q.frs = 32;

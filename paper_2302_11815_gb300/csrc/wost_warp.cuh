@@ -139,7 +139,9 @@ __device__ __noinline__ float hit_clear(const float4 *prims, uint32_t k, P3 o, P
 
 // The binary-tree queries, out of line: lane 0's second opinion.  All lanes
 // call them (the 2D ones are warp-wide) and get lane 0's answer.
-template <int D>
+// WALK: as the walk kernels search (2D: postponed leaves), or as the query
+// kernels do; their order differs, and with it the answer among ties.
+template <int D, bool WALK>
 __device__ __noinline__ Closest closest_binary(const TreeView &T, P3 x, Stack st, float bound2) {
     Cnt<false> cnt;
     const bool first = (threadIdx.x & 31) == 0;
@@ -148,7 +150,7 @@ __device__ __noinline__ Closest closest_binary(const TreeView &T, P3 x, Stack st
     c.rec = -1;
     c.s0 = c.s1 = 0.f;
     c.p = x;
-    if constexpr (WOST_POSTPONE_LEAVES && D == 2) {
+    if constexpr (WOST_POSTPONE_LEAVES && D == 2 && WALK) {
         c = q_closest_w<D, false>(T, x, st, cnt, bound2, first);
     } else {
         if (first) c = q_closest<D, false>(T, x, st, cnt, bound2);
@@ -216,8 +218,9 @@ __device__ __forceinline__ float box_dist2_at(const TreeView &T, uint32_t at, P3
     return at & 1u ? box_dist2<D>(n.lo1, n.hi1, x) : box_dist2<D>(n.lo0, n.hi0, x);
 }
 
-// Query policy: the whole warp answers the queries of its one walk.
-template <int D>
+// Query policy: the whole warp answers the queries of its one walk (WALK), or
+// one query of an array of queries.
+template <int D, bool WALK = true>
 struct WarpQ {
     static constexpr bool kWarp = true;
     static constexpr unsigned FULL = 0xffffffffu;
@@ -425,7 +428,7 @@ struct WarpQ {
             certain = certain && __popc(at) == 1 && !__any_sync(FULL, lb.d2 == m && lb.dup);
         if (certain && (tie || !(nr.lim2 < bound2))) certain = box_dist2_at<D>(T, __ldg(T.leaf_parents + k), x) <= m;
         if (!certain) {
-            best = closest_binary<D>(T, x, st, D == 3 && m < INFINITY ? fminf(bound2, nr.lim2) : bound2);
+            best = closest_binary<D, WALK>(T, x, st, D == 3 && m < INFINITY ? fminf(bound2, nr.lim2) : bound2);
         } else {
             best.d2 = m;
             best.rec = k;
@@ -597,11 +600,11 @@ struct WarpQ {
     // Certain: no hit at all; or the nearest hit clear of rounding (hit_clear)
     // and the next one farther by more than its rounding.  An occluder that is
     // clear of rounding occludes; none accepted, no occlusion.
-    __device__ __forceinline__ int ray2_w(const TreeView &T, P3 o, P3 va, float tmaxA, float &t_out, bool wantB, P3 vb,
-                                          int skipB, float tmaxB, bool &occB, bool act) {
+    // skipA: a record ray A does not meet (-1: none).
+    __device__ __forceinline__ int ray2_search(const TreeView &T, P3 o, P3 va, float tmaxA, int skipA, float &t_out,
+                                               bool wantB, P3 vb, int skipB, float tmaxB, bool &occB, bool &certain) {
         t_out = tmaxA;
         occB = false;
-        if (!act || T.root == WOST_EMPTY_REF) return -1;
         // fast reciprocals: the boxes are widened by more than they, and the
         // rounding of the one-lane slab test, can move its planes
         const P3 ia = mk(__fdividef(1.f, va.x), __fdividef(1.f, va.y), D == 3 ? __fdividef(1.f, va.z) : 0.f);
@@ -621,7 +624,7 @@ struct WarpQ {
         auto test = [&](uint32_t k) {
             const Prim<D> p = load_prim<D>(T.prims, k);
             float t;
-            if (prim_ray<D>(p, o, va, tmaxA, t, kEdgeTol) && lb.add(t, (int)k))
+            if ((int)k != skipA && prim_ray<D>(p, o, va, tmaxA, t, kEdgeTol) && lb.add(t, (int)k))
                 teA = hit_clear<D>(T.prims, k, o, va, t, tmaxA, scale);
             if (wantB && (int)k != skipB && prim_ray<D>(p, o, vb, tmaxB, t, 0.f)) {
                 if (hit_clear<D>(T.prims, k, o, vb, t, tmaxB, scale) >= 0.f) occ = true;
@@ -641,7 +644,7 @@ struct WarpQ {
                 },
                 test, [&] { return 0.f; }, [&] {});
         const float m = warp_min(lb.d2);
-        bool certain = ok;
+        certain = ok;
         int hit = -1;
         if (m < INFINITY) {
             const unsigned at = __ballot_sync(FULL, lb.d2 == m);
@@ -656,6 +659,16 @@ struct WarpQ {
             occB = __any_sync(FULL, occ);
             certain = certain && (occB || !__any_sync(FULL, occ_maybe));
         }
+        return hit;
+    }
+
+    __device__ __forceinline__ int ray2_w(const TreeView &T, P3 o, P3 va, float tmaxA, float &t_out, bool wantB, P3 vb,
+                                          int skipB, float tmaxB, bool &occB, bool act) {
+        t_out = tmaxA;
+        occB = false;
+        if (!act || T.root == WOST_EMPTY_REF) return -1;
+        bool certain;
+        int hit = ray2_search(T, o, va, tmaxA, -1, t_out, wantB, vb, skipB, tmaxB, occB, certain);
         if (!certain) {
             const RayAnswer a = ray2_binary<D>(T, o, va, tmaxA, wantB, vb, skipB, tmaxB, st);
             t_out = a.t;

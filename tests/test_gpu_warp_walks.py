@@ -144,3 +144,47 @@ def test_static_solve_and_batch_hand_over_to_warps(wost):
             wost.wost_solve_static(s.handle, p, w, 1e-3, 1e-3, 1024, 9 + i, 0, mean)
         np.testing.assert_array_equal(mean.cpu().numpy(), r["mean"].astype(np.float32))
         s.close()
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_small_query_arrays_get_the_answers_of_large_ones(wost, name):
+    """Arrays of few queries (at most 16,384, by query) run one query per warp,
+    larger ones one per lane (Q.2 in 3D: always one per warp, checked against
+    the oracle elsewhere): the same distances, points, records, hits and samples, bit for
+    bit, also for points on vertices and midway between primitives (ties),
+    far outside, and not finite."""
+    make, leaf, _ = CASES[name]
+    sc = make()
+    dim = sc["dim"]
+    rng = np.random.default_rng(13)
+    V = sc["vertices"].astype(np.float64)
+    lo, hi = V.min(0), V.max(0)
+    k = rng.integers(len(V), size=900)
+    P = sc["prims"][rng.integers(len(sc["prims"]), size=900)]
+    pts = np.concatenate([lo + (hi - lo) * rng.random((14000, dim)), V[k], V[P].mean(1), 0.5 * (V[P[:, 0]] + V[P[:, 1]]),
+                          np.round(lo + (hi - lo) * rng.random((300, dim)), 1), V[k[:100]] * 30.0,
+                          np.full((1, dim), np.nan), np.zeros((1, dim))])
+    n = len(pts)
+    d = rng.normal(size=(n, dim))
+    d[::7] = np.eye(dim)[rng.integers(dim, size=len(d[::7]))]  # along an axis
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a, np.float32)).cuda()  # noqa: E731
+    x, v, t, r = dev(pts), dev(d), dev(rng.uniform(0.05, 2.0, n)), dev(rng.uniform(0.02, 1.5, n))
+    skip = torch.from_numpy(rng.integers(-1, len(sc["prims"]), n).astype(np.int32)).cuda()
+    S = wost.Scene(sc, leaf_size=leaf)
+
+    def ask(s):
+        m = s.stop - s.start
+        return [*wost.wost_query_closest_dirichlet(S.handle, x[s]), wost.wost_query_silhouette(S.handle, x[s], r[s]),
+                *wost.wost_query_intersect_neumann(S.handle, x[s], v[s], t[s]),
+                *wost.wost_query_intersect_neumann(S.handle, x[s], v[s], t[s], skip=skip[s]),
+                *[o[: min(m, 1111)] for o in wost.wost_query_neumann_sample(S.handle, x[s], r[s], 5, 1, 2)]]
+
+    assert n > 16384
+    whole = ask(slice(0, n))
+    parts = [ask(slice(a, min(a + 1111, n))) for a in range(0, n, 1111)]
+    for i, w in enumerate(whole):
+        # (a sample's random numbers are keyed by its index in the array: the first part only)
+        got = parts[0][i] if i >= len(whole) - 3 else torch.cat([p[i] for p in parts])
+        np.testing.assert_array_equal(got.cpu().numpy(), w.cpu().numpy(), err_msg=f"{name}: output {i}")
+    S.close()
