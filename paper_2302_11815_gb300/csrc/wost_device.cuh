@@ -1295,10 +1295,16 @@ struct Walk {
 
 __device__ __forceinline__ float maxabs3(P3 a) { return fmaxf(fabsf(a.x), fmaxf(fabsf(a.y), fabsf(a.z))); }
 
-// Q.2 by the whole warp (wost_warp.cuh)
+// Q.2 by the whole warp (wost_warp.cuh): the distance found (rec < 0: none
+// within rmax); certain: it is the one-lane search's answer
+struct SilAnswer {
+    float d;
+    int rec;
+    bool certain;
+};
 template <int D>
-__device__ __noinline__ float2 coop_silhouette(const TreeView &T, P3 x, float rmax, float bound2, float tau, int2 *fr,
-                                               int frs, int fcap);
+__device__ __noinline__ SilAnswer coop_silhouette(const TreeView &T, P3 x, float rmax, float bound2, float tau,
+                                                  int2 *fr, int frs, int fcap);
 
 // Query policy over the binary trees: each lane answers its own walk's
 // queries with its own shared-memory stack.
@@ -1373,10 +1379,10 @@ struct LaneQ {
                                      __shfl_sync(0xffffffffu, x.z, src));
                     const float rs = __shfl_sync(0xffffffffu, rmax, src), ts = __shfl_sync(0xffffffffu, tau, src),
                                 fs = __shfl_sync(0xffffffffu, found2, src);
-                    const float2 a =
+                    const SilAnswer a =
                         coop_silhouette<D>(*Ts, xs, rs, beyond(fs, ts), ts, st.base - lane, st.stride, 32 * st.cap);
-                    if (lane == src && a.y != 0.f) {
-                        r = a.x;
+                    if (lane == src && a.certain) {
+                        r = a.d;
                         need = false;
                     }
                     __syncwarp();
@@ -1430,6 +1436,15 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
     // domain through a rounding gap; it ends like a capped walk (R5)
     const bool lost = act && !in_bounds<D>(sc, w.x);
     if constexpr (Q::kWarp) q.begin_step(sp, w, lost);  // the whole warp holds this walk
+    // R4: query origin off the Neumann boundary
+    const float delta = sp.offset * (1.f + maxabs3(w.x));
+    const P3 xq = w.onN ? w.x - w.n * delta : w.x;
+    // A walk that hugs the Neumann boundary far from the Dirichlet one does
+    // not need its distance: with a silhouette nearer than a lower bound of
+    // that distance, the star radius is the silhouette's.
+    bool skip1 = false;
+    float dsil0 = 0.f;
+    if constexpr (Q::kWarp) skip1 = q.near_silhouette(sc.S, xq, sp.epsilon, dsil0);
     // distance to the Dirichlet boundary (Q.1).  The closest point of the
     // previous step is at most dbound away (triangle inequality), which
     // prunes the search; the result is the exact closest point either way,
@@ -1440,7 +1455,7 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
     cl.rec = -1;
     cl.s0 = cl.s1 = 0.f;
     cl.p = w.x;
-    bool need = act;
+    bool need = act && !skip1;
 #pragma unroll 1
     for (int pass = 0; pass < 2; ++pass) {  // one call site keeps the code small
         if (!__any_sync(FULL, need)) break;
@@ -1452,7 +1467,7 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
         __syncwarp();
     }
     bool ended = false;
-    const float dD = sqrtf(cl.d2);
+    const float dD = skip1 ? w.dbound : sqrtf(cl.d2);
     if (act) {
         w.steps += 1;
         if (dD < sp.epsilon || w.steps >= sp.max_steps || lost) {
@@ -1473,11 +1488,9 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
         }
     }
     act = act && !ended;
-    // R4: query origin off the Neumann boundary
-    const float delta = sp.offset * (1.f + maxabs3(w.x));
-    const P3 xq = w.onN ? w.x - w.n * delta : w.x;
     // distance to the visibility silhouette (Q.2) within d_D, star radius (R3)
-    float dsil = q.silhouette_w(sc.S, xq, dD, act, sc.tau);
+    float dsil = dsil0;
+    if (!skip1) dsil = q.silhouette_w(sc.S, xq, dD, act, sc.tau);
     if (!act) dsil = dD;
     __syncwarp();
     float r = fminf(dD, fmaxf(sp.r_min, dsil));
@@ -1607,6 +1620,7 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
     if constexpr (SCR) {
         if (sqs > 0.f && u01(rb.w) >= screened_q<D>(moved, r, sqs)) return true;
     }
+    if constexpr (Q::kWarp) q.moved_on(w.x, dD, moved, dsil, skip1);
     w.dbound = dD + moved;
     w.x = p;
     w.n = np;

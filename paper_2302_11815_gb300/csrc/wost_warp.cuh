@@ -218,6 +218,9 @@ __device__ __forceinline__ float box_dist2_at(const TreeView &T, uint32_t at, P3
     return at & 1u ? box_dist2<D>(n.lo1, n.hi1, x) : box_dist2<D>(n.lo0, n.hi0, x);
 }
 
+template <int D>
+__device__ __noinline__ float coop_distance(const TreeView &T, P3 x, float tau, int2 *fr, int frs, int fcap);
+
 // Query policy: the whole warp answers the queries of its one walk (WALK), or
 // one query of an array of queries.
 template <int D, bool WALK = true>
@@ -243,8 +246,42 @@ struct WarpQ {
     // bounds the new answer (it is found again if it is still the best)
     int last_d, last_s;
     int hit_s;  // a candidate on the Neumann primitive hit last
+    // The walk's distance to the Dirichlet boundary is at least dlow (less
+    // than 0: not known) and at most its dbound; they are of the previous
+    // step's position px plus or minus the length of its move, `moved`, except
+    // after steps that skipped Q.1 (skipped), when they have grown apart.
+    // hug: the previous step's silhouette was near against dlow.
+    float dlow, moved;
+    P3 px;
+    bool skipped, hug;
 
-    __device__ __forceinline__ void new_walk() { last_d = last_s = hit_s = -1; }
+    __device__ __forceinline__ void new_walk() {
+        last_d = last_s = hit_s = -1;
+        dlow = -1.f;
+        skipped = hug = false;
+    }
+    // After a step from x: Q.1's answer dD there (or, skipped, an upper bound),
+    // the length of the move, the silhouette distance.
+    __device__ __forceinline__ void moved_on(P3 x, float dD, float len, float dsil, bool skip) {
+        dlow = (skip ? dlow : dD) * 0.999999f - len - tau;
+        px = x;
+        moved = len;
+        skipped = skip;
+        hug = dsil < 0.5f * dlow;
+    }
+    // Q.2 ahead of Q.1: true if a silhouette lies nearer than the Dirichlet
+    // boundary can (then d is Q.2's answer whatever Q.1's is, and the step is
+    // no epsilon-shell hit), and Q.1's record is not needed.
+    __device__ __forceinline__ bool near_silhouette(const TreeView &S, P3 xq, float epsilon, float &d) {
+        if (!hug || want_rec || !(dlow > 1.001f * epsilon + tau) || S.root == WOST_EMPTY_REF) return false;
+        const float lim = dlow * 0.9999f - tau;
+        if (!(lim > 0.f)) return false;
+        const SilAnswer a = coop_silhouette<D>(S, xq, lim, hint_bound(S, xq, lim * lim), tau, fr, frs, fcap);
+        if (a.rec >= 0) last_s = a.rec;
+        d = a.d;
+        return a.certain && a.rec >= 0;
+    }
+
     __device__ __forceinline__ void hit(const TreeView &N, int rec) { hit_s = (int)__ldg(N.hints + rec); }
     __device__ __forceinline__ void begin_step(const SolveParams &sp, const Walk &w, bool lost) {
         want_rec = lost || w.steps + 1 >= sp.max_steps;
@@ -428,6 +465,12 @@ struct WarpQ {
             certain = certain && __popc(at) == 1 && !__any_sync(FULL, lb.d2 == m && lb.dup);
         if (certain && (tie || !(nr.lim2 < bound2))) certain = box_dist2_at<D>(T, __ldg(T.leaf_parents + k), x) <= m;
         if (!certain) {
+            if (WALK && skipped && bound2 < INFINITY) {
+                // the bound the one-lane walk has here: Q.1's answer at the
+                // previous position, which was skipped
+                const float b = (coop_distance<D>(T, px, tau, fr, frs, fcap) + moved) * 1.0001f + 1e-6f;
+                bound2 = b * b;
+            }
             best = closest_binary<D, WALK>(T, x, st, D == 3 && m < INFINITY ? fminf(bound2, nr.lim2) : bound2);
         } else {
             best.d2 = m;
@@ -448,10 +491,8 @@ struct WarpQ {
     // the cone tests above it decide: a candidate whose leaf is culled is
     // none, and the best one's whole path is tested.
     // B: a bound on the squared distance (beyond that of a certain candidate,
-    // or rmax^2).  certain: the value returned is the one-lane search's.  nr:
-    // around the best distance found.
-    __device__ __forceinline__ float silhouette_search(const TreeView &T, P3 x, float rmax, float B, bool &certain,
-                                                       Near &nr) {
+    // or rmax^2).
+    __device__ __forceinline__ SilAnswer silhouette_search(const TreeView &T, P3 x, float rmax, float B) {
         const float r2 = rmax * rmax;
         LaneBest lb;
         lb.clear();
@@ -475,35 +516,35 @@ struct WarpQ {
             },
             test, [&] { return B; }, [&] { B = fminf(B, beyond(warp_min(lb.d2), tau)); });
         const float m = warp_min(lb.d2);
-        nr = Near(m, tau);
-        certain = ok;
-        if (m == INFINITY) return rmax;
+        const Near nr(m, tau);
+        bool certain = ok;
+        if (m == INFINITY) return SilAnswer{rmax, -1, ok};
         const unsigned at = __ballot_sync(FULL, lb.d2 == m);
         const bool tie = __any_sync(FULL, (lb.d2 != m && lb.d2 <= nr.lim) || lb.alt <= nr.lim);
         const int src = __ffs(at) - 1;
         const int k = __shfl_sync(FULL, lb.rec, src);
         if (certain && (tie || !(nr.lim2 < r2))) certain = box_dist2_at<D>(T, __ldg(T.leaf_parents + k), x) <= m;
         if (certain && !__shfl_sync(FULL, (int)clear, src)) certain = path_reached(T, (uint32_t)k, x);
-        if (ok) last_s = k;
-        return sqrtf(m);
+        return SilAnswer{sqrtf(m), k, certain};
+    }
+
+    // the candidates around the last answer and around the last hit bound the
+    // new one
+    __device__ __forceinline__ float hint_bound(const TreeView &T, P3 x, float B) const {
+        if ((last_s < 0 && hit_s < 0) || T.n_prims <= 3 * kBrute) return B;
+        const int mid = (lane < 16 && last_s >= 0) || hit_s < 0 ? last_s : hit_s;
+        const int k = min(max(mid - 8 + (lane & 15), 0), T.n_prims - 1);
+        return fminf(B, beyond(warp_min(sil_certain<D>(T.prims, (uint32_t)k, x)), tau));
     }
 
     __device__ __forceinline__ float silhouette_w(const TreeView &T, P3 x, float rmax, bool act, float) {
         if (!act || T.root == WOST_EMPTY_REF) return rmax;
-        float B = rmax * rmax;
-        // the candidates around the last answer and around the last hit bound
-        // the new one
-        if ((last_s >= 0 || hit_s >= 0) && T.n_prims > 3 * kBrute) {
-            const int mid = (lane < 16 && last_s >= 0) || hit_s < 0 ? last_s : hit_s;
-            const int k = min(max(mid - 8 + (lane & 15), 0), T.n_prims - 1);
-            B = fminf(B, beyond(warp_min(sil_certain<D>(T.prims, (uint32_t)k, x)), tau));
-        }
-        bool certain;
-        Near nr(0.f, tau);
-        const float s = silhouette_search(T, x, rmax, B, certain, nr);
-        if (certain) return s;
+        const SilAnswer a = coop_silhouette<D>(T, x, rmax, hint_bound(T, x, rmax * rmax), tau, fr, frs, fcap);
+        if (a.rec >= 0) last_s = a.rec;
+        if (a.certain) return a.d;
         // the one-lane search among the candidates near the best one, if
         // it finds one there (culled candidates can leave none)
+        const Near nr(a.d * a.d, tau);
         const float rn = sqrtf(nr.lim2) * 1.000001f;
         if (rn < rmax) {
             const float t = silhouette_binary<D>(T, x, rn, st);
@@ -679,23 +720,40 @@ struct WarpQ {
     }
 };
 
-// Q.2 of one lane's walk by its whole warp (every lane calls it with that
-// walk's x, rmax and bound2): for the one-lane kernels, whose warps would
-// otherwise wait for the lane with the longest search.  (answer, 1), or
-// (-, 0) where the binary search has to decide.
+// the distance alone (to within the ties that only a one-lane search decides)
 template <int D>
-__device__ __noinline__ float2 coop_silhouette(const TreeView &T, P3 x, float rmax, float bound2, float tau, int2 *fr,
-                                               int frs, int fcap) {
+__device__ __noinline__ float coop_distance(const TreeView &T, P3 x, float tau, int2 *fr, int frs, int fcap) {
     WarpQ<D> q;
     q.fr = fr;
     q.frs = frs;
     q.fcap = fcap;
     q.lane = threadIdx.x & 31;
     q.tau = tau;
-    bool certain;
-    Near nr(0.f, tau);
-    const float s = q.silhouette_search(T, x, rmax, fminf(rmax * rmax, bound2), certain, nr);
-    return make_float2(s, certain ? 1.f : 0.f);
+    float B = INFINITY, best = INFINITY;
+    q.search(
+        T, WarpQ<D>::kBrute,
+        [&](const WChild &ch, const float4 *, float &key) {
+            key = box_dist2<D>(ch.lo, ch.hi, x);
+            return key < B;
+        },
+        [&](uint32_t k) { best = fminf(best, prim_dist2<D>(T.prims, k, x)); }, [&] { return B; },
+        [&] { B = fminf(B, beyond(warp_min(best), tau)); });
+    return sqrtf(warp_min(best));
+}
+
+// One copy of the silhouette search for every caller, and for the one-lane
+// kernels, whose warps would otherwise wait for the lane with the longest
+// search (every lane calls it with the same arguments).
+template <int D>
+__device__ __noinline__ SilAnswer coop_silhouette(const TreeView &T, P3 x, float rmax, float bound2, float tau,
+                                                  int2 *fr, int frs, int fcap) {
+    WarpQ<D> q;
+    q.fr = fr;
+    q.frs = frs;
+    q.fcap = fcap;
+    q.lane = threadIdx.x & 31;
+    q.tau = tau;
+    return q.silhouette_search(T, x, rmax, fminf(rmax * rmax, bound2));
 }
 
 }  // namespace wost
