@@ -44,8 +44,10 @@ struct DevBuf {
         owned = true;
     }
     cudaError_t alloc(size_t n) {
-        bytes = n;
-        return n ? cudaMalloc(&p, n) : cudaSuccess;
+        const cudaError_t e = n ? cudaMalloc(&p, n) : cudaSuccess;
+        if (e != cudaSuccess) p = nullptr;
+        bytes = p ? n : 0;
+        return e;
     }
     // at least n bytes (contents lost when it grows)
     cudaError_t ensure(size_t n) {
@@ -157,26 +159,43 @@ struct SolvePool {
         if (!closed && idle.size() < kIdle) idle.push_back(std::move(r));
     }
     void close() {
+        drop();
         std::lock_guard<std::mutex> lk(mu);
         closed = true;
+    }
+    // frees the idle sets (also when an allocation finds no memory)
+    void drop() {
+        std::lock_guard<std::mutex> lk(mu);
         idle.clear();
+    }
+    // b.ensure(n), once more without the idle sets if memory is short
+    cudaError_t ensure(DevBuf &b, size_t n) {
+        cudaError_t e = b.ensure(n);
+        if (e != cudaErrorMemoryAllocation) return e;
+        cudaGetLastError();
+        drop();
+        return b.ensure(n);
     }
 };
 
 // Words (u64) of a batched launch's counters.
 constexpr size_t kBatchCounters = 4 + 2 * kMaxStages;
 // The chain buffers of dimension di (0: 2D, 1: 3D) of a batched launch,
-// allocated for its grid.
+// allocated for its grid; without memory for them, none (the launch then keeps
+// its walks to their ends).
 inline cudaError_t batch_chain_buffers(DevBuf chain[2], unsigned long long *counters, int di, int block, int blocks,
                                        ChainBuffers *cb) {
     for (int i = 0; i < 2; ++i) {
         const size_t cap = (size_t)batch_chain_capacity(block, blocks, i), bytes = cap * 3 * sizeof(float4);
-        if (chain[i].p && chain[i].bytes < bytes) {
-            cudaFree(chain[i].p);
-            chain[i].p = nullptr;
-        }
+        if (chain[i].bytes < bytes) chain[i].release();
         if (!chain[i].p) {
             cudaError_t e = chain[i].alloc(bytes);
+            if (e == cudaErrorMemoryAllocation) {
+                cudaGetLastError();
+                chain[i].release();
+                *cb = ChainBuffers{};
+                return cudaSuccess;
+            }
             if (e != cudaSuccess) return e;
         }
         cb->cap[i] = (unsigned)cap;

@@ -347,7 +347,7 @@ wost_status wost::prepare_solve(wost_scene *scene, const wost_solve_desc *d, cud
         // globals, sum, sumsq, walks, steps one after the other (one memset,
         // one copy per poll), then the inputs
         const size_t need = kGlobals * 8 + 4 * n * 8 + 2 * pb + n + 64;
-        CK(R.main.ensure(need), "cudaMalloc accumulators");
+        CK(scene->pool->ensure(R.main, need), "cudaMalloc accumulators");
         unsigned char *p = (unsigned char *)R.main.p;
         auto part = [&](DevBuf &b, size_t bytes) {
             b.view(p, bytes);
@@ -426,7 +426,7 @@ static cudaError_t chain_buffers(wost_solve_handle *h, uint64_t walks, int block
         cb->cap[i] = (unsigned)chain_capacity(walks, h->block, blocks, i);
         bytes[i] = (size_t)cb->cap[i] * 3 * sizeof(float4);
     }
-    cudaError_t e = h->res->chain.ensure(bytes[0] + bytes[1]);
+    cudaError_t e = h->res_pool->ensure(h->res->chain, bytes[0] + bytes[1]);
     if (e != cudaSuccess) return e;
     cb->slots[0] = (float4 *)h->res->chain.p;
     cb->slots[1] = (float4 *)((unsigned char *)h->res->chain.p + bytes[0]);
@@ -454,7 +454,7 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
             // counter u32); the list of the saved walks' slots
             const size_t n_slots = (size_t)resume_slots(h->block, h->resume_blocks, h->lanes);
             const size_t slot_bytes = n_slots * 3 * sizeof(float4), state_bytes = 16 + n_slots * sizeof(uint32_t);
-            CK(h->res->resume.ensure(slot_bytes + state_bytes), "cudaMalloc slots");
+            CK(scene->pool->ensure(h->res->resume, slot_bytes + state_bytes), "cudaMalloc slots");
             h->slots.view(h->res->resume.p, slot_bytes);
             h->rstate.view((unsigned char *)h->res->resume.p + slot_bytes, state_bytes);
             CK(cudaMemsetAsync(h->slots.p, 0, h->slots.bytes, stream), "memset");
@@ -488,8 +488,12 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
             if (le == cudaSuccess && warp_ok) {
                 ChainBuffers cb{};
                 le = chain_buffers(h.get(), total, blocks, &cb);
-                if (le == cudaSuccess)
+                if (le == cudaSuccess) {
                     le = launch_walk_chain(scene->view, sp, acc, SavedWalks{}, total, cb, h->block, blocks, stream);
+                } else if (le == cudaErrorMemoryAllocation) {  // no memory to hand walks over in
+                    cudaGetLastError();
+                    le = launch_walk_persistent(scene->view, sp, acc, h->block, blocks, stream, h->lanes);
+                }
             } else if (le == cudaSuccess) {
                 le = launch_walk_persistent(scene->view, sp, acc, h->block, blocks, stream, h->lanes);
             }
@@ -775,7 +779,7 @@ static wost_status advance_waiting(wost_solve_handle *h) {
     if (h->lanes != 1 || !h->warp_ok) return advance_locked(h, 2048, h->stream);
     unsigned long long *steps_run = (unsigned long long *)h->rstate.p;
     unsigned int *ctr = (unsigned int *)((char *)h->rstate.p + 8);
-    SavedWalks src{nullptr, nullptr, nullptr, nullptr, steps_run};
+    SavedWalks src{nullptr, nullptr, nullptr, nullptr, steps_run, 0};
     uint64_t walks = (uint64_t)h->n_points * (uint64_t)h->walks;
     if (h->launches > 0) {
         bool fin = false, drained = false;
@@ -784,14 +788,20 @@ static wost_status advance_waiting(wost_solve_handle *h) {
         if (st != WOST_OK || fin) return st;
         if (!drained || live > (uint64_t)resume_slots(h->block, h->resume_blocks, 1))
             return advance_locked(h, 2048, h->stream);
-        src = SavedWalks{(float4 *)h->slots.p, ctr + 2, ctr, ctr + 1, steps_run};
+        src = SavedWalks{(float4 *)h->slots.p, ctr + 2, ctr, ctr + 1, steps_run, 0};
         walks = live;
-    } else {
+    }
+    ChainBuffers cb{};
+    const cudaError_t ce = chain_buffers(h, walks, h->resume_blocks, &cb);
+    if (ce == cudaErrorMemoryAllocation) {  // no memory to hand walks over in
+        cudaGetLastError();
+        return advance_locked(h, 2048, h->stream);
+    }
+    CK(ce, "cudaMalloc slots");
+    if (h->launches == 0) {
         h->t_launch = std::chrono::steady_clock::now();
         CK(cudaEventRecord(h->ev_start, h->stream), "cudaEventRecord");
     }
-    ChainBuffers cb{};
-    CK(chain_buffers(h, walks, h->resume_blocks, &cb), "cudaMalloc slots");
     CK(launch_walk_chain(h->scene->view, h->sp, h->acc, src, walks, cb, h->block, h->resume_blocks, h->stream),
        "kernel launch");
     CK(cudaMemsetAsync(ctr, 0, 2 * sizeof(unsigned int), h->stream), "memset");

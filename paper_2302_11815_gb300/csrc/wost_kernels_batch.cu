@@ -74,11 +74,12 @@ cudaError_t launch_walk_batch(int dim, const BatchHeader *hdr, const BatchJob *j
         const uint64_t held = std::min(walks, resident);
         uint64_t most = held / 2 < kTailWalks * 3 / 2 ? kTailWalks : held / 2;
         most = std::min<uint64_t>(most, cb.cap[b]);
-        unsigned int *ctr = cb.counters + 2 * stage;
+        unsigned int *ctr = cb.slots[b] ? cb.counters + 2 * stage : nullptr;
         const unsigned per_warp = src.per_warp ? src.per_warp : 32u;
         const uint64_t per_block = (uint64_t)(block / 32) * per_warp;
         const int grid =
             walks == ~0ull ? blocks : (int)std::min<uint64_t>((uint64_t)blocks, (walks + per_block - 1) / per_block);
+        if (!cb.slots[b]) most = 0;  // (no memory: this launch runs its walks to their ends)
         const HandOver ho{cb.slots[b], ctr, (unsigned)most, (unsigned)grid * (unsigned)per_block};
         cudaError_t e =
             dim == 2 ? (screened ? launch<2, true>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
@@ -89,7 +90,7 @@ cudaError_t launch_walk_batch(int dim, const BatchHeader *hdr, const BatchJob *j
                                                    src, ho)
                                  : launch<3, false>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
                                                     src, ho));
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess || !cb.slots[b]) return e;
         src = SavedWalks{cb.slots[b], nullptr, ctr, ctr + 1, nullptr, spread_walks(dim, most)};
         walks = most;
     }

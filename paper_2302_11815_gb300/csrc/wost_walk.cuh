@@ -15,7 +15,11 @@
 //   k_walk_persistent  one resident grid; each team runs one walk step per
 //                      iteration and, when its walk ends, takes the next walk
 //                      from a global counter (warp ballot + one atomicAdd per
-//                      warp), so finished teams are refilled at once.
+//                      warp), so finished teams are refilled at once.  Once
+//                      nothing is left to draw and few enough walks are left,
+//                      it hands them over to the next launch of a chain
+//                      (launch_walk_chain), the last of which runs one walk
+//                      per warp (wost_walk_warp.cuh).
 //   k_walk_resume      the persistent loop for a bounded number of steps,
 //                      unfinished walks saved for the next launch.
 //   k_walk_batch       the persistent kernel over many solves (wost_batch.cuh).
