@@ -1359,7 +1359,9 @@ struct LaneQ {
             // 1,210, 32: 1,030).
             float r = rmax, found2 = INFINITY;
             bool need = act;
-            int few = coop ? kSilFew : 0;
+            // (work counters are per lane and of the binary tree: each of their
+            // searches is the lane's own, to its end)
+            int few = !CN && coop ? kSilFew : 0;
 #pragma unroll 1
             for (;;) {
                 float rr;

@@ -348,7 +348,7 @@ template <int D, bool SCR>
 __global__ void __launch_bounds__(256) k_walk_count(const __grid_constant__ SceneView sc, const SolveParams sp, const Accumulators acc,
                                                     unsigned long long *stats) {
     Cnt<true> cnt;
-    auto q = make_q<D, true>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, sp.coop != 0);
+    auto q = make_q<D, true>(sp.stack_depth, acc.guard, cnt, sp.visit_limit);
     const Group g = make_team<1>();
     const uint64_t total = (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;

@@ -99,6 +99,24 @@ def test_warp_walks_are_the_one_lane_walks(wost, name, n, walks, kernel):
     _both(wost, sc, leaf, sigma, _points(sc, n, np.random.default_rng(7)), walks, kernel)
 
 
+@pytest.mark.parametrize("name", ["koch3", "box_sphere", "cube_faces_leaf16", "cube_torus"])
+@pytest.mark.parametrize("n,walks", [(1, 1), (61, 33), (257, 96)])
+def test_counting_kernel_runs_the_same_walks_and_counts_all_of_them(wost, name, n, walks):
+    """Its searches are the lane's own to their end, whatever the limits."""
+    make, leaf, sigma = CASES[name]
+    sc = make()
+    pts = _points(sc, n, np.random.default_rng(7))
+    own = _both(wost, sc, leaf, sigma, pts, walks, "counting")
+    ref = _both(wost, sc, leaf, sigma, pts, walks, "persistent")
+    assert own["total_steps"] == ref["total_steps"]
+    np.testing.assert_allclose(own["mean"], ref["mean"], rtol=1e-9, atol=1e-12)
+    S = wost.Scene(sc, leaf_size=leaf)
+    given = wost.solve(S, torch.from_numpy(pts).cuda(), walks, 1e-3, 1e-3, 2048, seed=3, kernel="counting",
+                       sigma=sigma, stack_depth=S.info()["stack_depth"])
+    S.close()
+    assert own["counts"] == given["counts"]
+
+
 def test_warp_walks_from_boundary_points(wost):
     for sc in (scenes.config1(), scenes.box_sphere_scene(data="analytic")):
         sel = np.flatnonzero(sc["flags"] == 1)
