@@ -157,9 +157,17 @@ cudaError_t launch_walk_count(const SceneView &sc, const SolveParams &sp, const 
 // screened solves and the other kernels use one lane per walk)
 cudaError_t persistent_grid(int dim, int block, int depth, int *blocks_out, int lanes) {
     if (lanes == WOST_WIDE) return persistent_grid_team(dim, block, depth, blocks_out);
-    return resident_grid(dim == 2 ? (const void *)k_walk_persistent<2, false, 1>
-                                  : (const void *)k_walk_persistent<3, false, 1>,
-                         block, depth, blocks_out);
+    // both forms run on the grid (and both are loaded before a capture)
+    int saved = 0;
+    cudaError_t e = resident_grid(dim == 2 ? (const void *)k_walk_persistent<2, false, 1, true>
+                                           : (const void *)k_walk_persistent<3, false, 1, true>,
+                                  block, depth, &saved);
+    if (e != cudaSuccess) return e;
+    e = resident_grid(dim == 2 ? (const void *)k_walk_persistent<2, false, 1, false>
+                               : (const void *)k_walk_persistent<3, false, 1, false>,
+                      block, depth, blocks_out);
+    if (e == cudaSuccess && saved < *blocks_out) *blocks_out = saved;
+    return e;
 }
 
 cudaError_t launch_walk_persistent(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, int block,

@@ -183,26 +183,37 @@ __global__ void WOST_WALK_BOUNDS k_walk_plain(const __grid_constant__ SceneView 
     }
 }
 
-// Hands the walks of this warp over (true) once nothing is left to draw and
-// at most ho.most walks are left.  Every lane that finds nothing to draw has
-// added 1 to the counter, once, so the counter tells how many hold a walk.
+// Where the walks of this warp are to be saved: a value once nothing is left
+// to draw and at most ho.most walks are left (else ~0).  Every lane that finds
+// nothing to draw has added 1 to the counter, once, so the counter tells how
+// many hold a walk.  hand_over saves them as well, and tells if it did.
 template <class CTR>
-__device__ __forceinline__ bool hand_over(const HandOver &ho, const CTR *counter, unsigned long long total, int lane,
-                                          const Walk &w, bool have, unsigned held, int job) {
-    const unsigned FULL = 0xffffffffu;
+__device__ __forceinline__ unsigned hand_over_at(const HandOver &ho, const CTR *counter, unsigned long long total,
+                                                 int lane, unsigned held) {
     unsigned first = 0xffffffffu;
     if (lane == 0) {
         const unsigned long long drawn = *(volatile const CTR *)counter;
         if (drawn >= total && ho.lanes - (unsigned)(drawn - total) <= ho.most)
             first = atomicAdd(ho.count, (unsigned)__popc(held));
     }
-    first = __shfl_sync(FULL, first, 0);
+    return __shfl_sync(0xffffffffu, first, 0);
+}
+
+template <class CTR>
+__device__ __forceinline__ bool hand_over(const HandOver &ho, const CTR *counter, unsigned long long total, int lane,
+                                          const Walk &w, bool have, unsigned held, int job) {
+    const unsigned first = hand_over_at(ho, counter, total, lane, held);
     if (first == 0xffffffffu) return false;
     if (have) save_walk(ho.slots + 3 * (size_t)(first + __popc(held & ((1u << lane) - 1u))), w, job);
     return true;
 }
 
-template <int D, bool SCR, int T>
+// SAVED: the walks are those of src.slots.  A parameter of the template, and
+// the stores of a hand-over behind the loop, because the loop is bound by its
+// instruction supply: 1,824,000 walks in a disk of 356 segments take
+// 24.6 ms, 27.7 with both inside (25.2 without hand-over); Koch level 3, 380,000
+// walks: 162, 177 (172).
+template <int D, bool SCR, int T, bool SAVED>
 __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ SceneView sc, const SolveParams sp,
                                                          const Accumulators acc, const SavedWalks src,
                                                          const HandOver ho) {
@@ -210,17 +221,18 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ Scene
     auto q = make_q<D, false, T>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, sp.coop != 0);
     const Group g = make_team<T>();
     const uint64_t total =
-        src.slots ? (uint64_t)*src.count : (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
+        SAVED ? (uint64_t)*src.count : (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
     const int lane = threadIdx.x & 31;
     const unsigned FULL = 0xffffffffu;
     Walk w{};
-    bool have = false, drained = T == 1 && src.per_warp && lane >= (int)src.per_warp;  // uniform within a team
+    bool have = false, drained = SAVED && src.per_warp && lane >= (int)src.per_warp;  // uniform within a team
     // All 32 lanes stay in this loop until the warp runs out of work, call
     // the warp-synchronous walk_step together (lanes without a walk take part
     // in its meetings only) and meet at __syncwarp() after every walk step,
     // so the warp starts each step and each query converged (without it,
     // independent thread scheduling lets the lanes drift apart and issue
     // alone).
+    unsigned first = 0xffffffffu, held;
     for (;;) {
         // regeneration: teams without a walk take the next ones (one ballot
         // bit per team, on its leader)
@@ -229,7 +241,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ Scene
             int lead = __ffs(need) - 1;
             unsigned long long base = 0;
             if (lane == lead) {
-                if (src.slots) {
+                if constexpr (SAVED) {
                     base = atomicAdd(src.next, (unsigned)__popc(need));
                 } else {
                     bool stop = *(volatile int *)acc.cancel != 0;
@@ -241,7 +253,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ Scene
                 unsigned long long my = base + __popc(need & ((1u << g.base) - 1u));
                 if (my >= total) {
                     drained = true;
-                } else if (src.slots) {
+                } else if constexpr (SAVED) {
                     have = load_walk(src.slots + 3 * (size_t)(src.list ? src.list[my] : (uint32_t)my), w);
                 } else {
                     int64_t pt = (int64_t)(my / (uint64_t)sp.walks_per_point);
@@ -251,15 +263,17 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ Scene
                 }
             }
         }
-        const unsigned held = __ballot_sync(FULL, have);
+        held = __ballot_sync(FULL, have);
         if (!held) {
             if (__any_sync(FULL, !drained)) continue;
             break;
         }
         if constexpr (T == 1) {
-            if (ho.slots && (src.slots ? hand_over(ho, src.next, total, lane, w, have, held, 0)
-                                       : hand_over(ho, acc.next_walk, total, lane, w, have, held, 0)))
-                break;
+            if (ho.slots) {
+                if constexpr (SAVED) first = hand_over_at(ho, src.next, total, lane, held);
+                else first = hand_over_at(ho, acc.next_walk, total, lane, held);
+                if (first != 0xffffffffu) break;
+            }
         }
         if (src.steps_run && lane == 0) atomicAdd(src.steps_run, (unsigned long long)__popc(held));
         if (walk_step<D, SCR>(sc, sp, w, q, have)) {
@@ -267,6 +281,10 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ Scene
             have = false;
         }
         __syncwarp();
+    }
+    if constexpr (T == 1) {
+        if (first != 0xffffffffu && have)
+            save_walk(ho.slots + 3 * (size_t)(first + __popc(held & ((1u << lane) - 1u))), w, 0);
     }
 }
 
@@ -432,19 +450,28 @@ static cudaError_t resident_grid(const void *k, int block, int depth, int *block
     return resident_blocks(k, block, smem_bytes(depth, block, lanes), blocks_out);
 }
 
-template <bool SCR, int T>
-static cudaError_t walk_persistent_launch(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
-                                          const SavedWalks &src, const HandOver &ho, int block, int blocks, cudaStream_t s) {
+template <bool SCR, int T, bool SAVED>
+static cudaError_t walk_persistent_form(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
+                                        const SavedWalks &src, const HandOver &ho, int block, int blocks, cudaStream_t s) {
     size_t sm = smem_bytes(sp.stack_depth, block, T);
     const void *k =
-        sc.dim == 2 ? (const void *)k_walk_persistent<2, SCR, T> : (const void *)k_walk_persistent<3, SCR, T>;
+        sc.dim == 2 ? (const void *)k_walk_persistent<2, SCR, T, SAVED> : (const void *)k_walk_persistent<3, SCR, T, SAVED>;
     cudaError_t e = smem_limit(k, sm);
     if (e != cudaSuccess) return e;
     if (sc.dim == 2)
-        k_walk_persistent<2, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc, src, ho);
+        k_walk_persistent<2, SCR, T, SAVED><<<blocks, block, sm, s>>>(sc, sp, acc, src, ho);
     else
-        k_walk_persistent<3, SCR, T><<<blocks, block, sm, s>>>(sc, sp, acc, src, ho);
+        k_walk_persistent<3, SCR, T, SAVED><<<blocks, block, sm, s>>>(sc, sp, acc, src, ho);
     return cudaGetLastError();
+}
+
+template <bool SCR, int T>
+static cudaError_t walk_persistent_launch(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
+                                          const SavedWalks &src, const HandOver &ho, int block, int blocks, cudaStream_t s) {
+    if constexpr (T == 1) {
+        if (src.slots) return walk_persistent_form<SCR, T, true>(sc, sp, acc, src, ho, block, blocks, s);
+    }
+    return walk_persistent_form<SCR, T, false>(sc, sp, acc, src, ho, block, blocks, s);
 }
 
 template <bool SCR, int T>
