@@ -227,7 +227,8 @@ def measure_read_gbs(torch, wost, stream, nbytes, passes, reps=5):
     return best
 
 
-KERNEL_SOURCES = ("wost_device.cuh", "wost_walk.cuh", "wost_kernels.cu", "wost_internal.h")
+KERNEL_SOURCES = ("wost_device.cuh", "wost_walk.cuh", "wost_kernels.cu", "wost_internal.h", "wost_group.cuh",
+                  "wost_warp.cuh")
 
 
 def kernel_source_hash():
