@@ -30,12 +30,12 @@ __device__ __forceinline__ WarpQ<D, WALK> make_warp_q(int depth, unsigned int *g
 }
 
 // Walks drawn from the solve's counter, or saved ones (src.slots).  Bound by
-// the latency of dependent instructions (~3,000 of them per step, 6 cycles
-// each when a warp runs alone): a step takes 9.7 us alone on the Koch workload
-// (one lane 20 us, a full warp of one-lane walks 35 us) and 14 us with 4,864
-// walks resident, 3.4e8 steps/s.  Whole solves, one-lane kernels -> this one:
-// 976 Koch walks 1,348 -> 390 ms, 6,144 keyhole walks 179 -> 22 ms, 768 walks
-// by a crack 8.8 -> 2.1 ms.  Cap of 96 registers: 64 to 128 are within 5%.
+// the latency of dependent instructions (2,450 of them per step, 5.8 cycles
+// each when a warp runs alone): a step takes 7.1 us alone on the Koch workload
+// (one lane 20 us, a full warp of one-lane walks 35 us), and 4,864 walks of 200
+// steps run at 1.6e8 steps/s (4.07 ms).  Whole solves, one-lane kernels -> this
+// one: 976 Koch walks 1,501 -> 420 ms, 6,144 keyhole walks 173 -> 26 ms, 768
+// walks by a crack 6.8 -> 1.1 ms.  Cap of 96 registers: 64 to 128 within 5%.
 template <int D, bool SCR>
 __global__ void __maxnreg__(WOST_WARP_REGS) k_walk_warp(const __grid_constant__ SceneView sc,
                                                         const __grid_constant__ SolveParams sp,

@@ -15,7 +15,7 @@
 // value is at most the binary one's; it is the binary one's unless rounding
 // keeps that search from the record that has it, which is checked (the
 // reasons are stated at each query).  Where the check fails, lane 0 repeats
-// the query over the binary tree (about 1% of the queries).
+// the query over the binary tree (at most 1.7% of the searches on seven scenes).
 #pragma once
 
 #include "wost_device.cuh"
