@@ -283,6 +283,7 @@ struct wost_solve_handle {
     wost::DevBuf slots, rstate;
     int resume_blocks = 0;
     uint64_t launches = 0;
+    bool idle = false;  // nothing of it is in flight though no event tells: a resumable solve until its first launch
     bool resumable() const { return kernel == WOST_KERNEL_RESUMABLE; }
     int kernel = 0;
     int *cancel_host = nullptr;                            // mapped pinned (engine requests: plain host)
@@ -303,8 +304,10 @@ struct wost_solve_handle {
     wost_status final_status = WOST_OK;                    // engine requests
     std::mutex mu;
     ~wost_solve_handle() {
+        // (a stream of the caller's is used only by a call that failed before
+        // its event was recorded: the caller may have destroyed it since)
         if (ev_done && launches) cudaEventSynchronize(ev_done);
-        else if (stream) cudaStreamSynchronize(stream);  // nothing launched: its copies
+        else if (stream && !idle) cudaStreamSynchronize(stream);
         if (res) {
             res_pool->give(std::move(res));
             return;

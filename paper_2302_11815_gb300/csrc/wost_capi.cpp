@@ -460,6 +460,7 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
             CK(cudaMemsetAsync(h->slots.p, 0, h->slots.bytes, stream), "memset");
             CK(cudaMemsetAsync(h->rstate.p, 0, 16, stream), "memset");
             if ((st = wait_for_copies(stream, h->res->ev_copy)) != WOST_OK) return st;
+            h->idle = true;
             *out = h.release();
             return WOST_OK;
         }
@@ -756,6 +757,7 @@ wost_status wost_poll(wost_solve_handle *h, double *mean, double *se, uint64_t *
 
 // One launch of a resumable solve (caller holds h->mu).
 static wost_status advance_locked(wost_solve_handle *h, int iters, cudaStream_t s) {
+    h->idle = false;
     if (h->launches == 0) {
         h->t_launch = std::chrono::steady_clock::now();
         CK(cudaEventRecord(h->ev_start, s), "cudaEventRecord");
@@ -798,6 +800,7 @@ static wost_status advance_waiting(wost_solve_handle *h) {
         return advance_locked(h, 2048, h->stream);
     }
     CK(ce, "cudaMalloc slots");
+    h->idle = false;
     if (h->launches == 0) {
         h->t_launch = std::chrono::steady_clock::now();
         CK(cudaEventRecord(h->ev_start, h->stream), "cudaEventRecord");

@@ -1,0 +1,82 @@
+"""The host side of the C ABI without a device: wost_capi.cpp linked against
+hostsim.cpp, which stands in for the CUDA runtime and the kernel launchers
+and records how streams, memory and launches are used."""
+import ctypes as C
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2302_11815_gb300 import build as libbuild
+from paper_2302_11815_gb300 import scenes, wost
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def simlib(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
+    if not os.path.exists(os.path.join(inc, "cuda_runtime.h")):
+        pytest.skip("no CUDA headers")
+    out = tmp_path_factory.mktemp("hostsim")
+    objs = []
+    src = [os.path.join(libbuild.CSRC, f) for f in ("wost_capi.cpp", "scene_build.cpp", "scene_check.cpp")]
+    for s in [*src, os.path.join(HERE, "hostsim.cpp")]:
+        objs.append((s, str(out / (os.path.basename(s) + ".o"))))
+    procs = [subprocess.Popen(["g++", "-O1", "-std=c++17", "-fPIC", "-w", "-I" + inc, "-I" + libbuild.CSRC, "-I" +
+                               os.path.join(libbuild.ROOT, "include"), "-c", s, "-o", o]) for s, o in objs]
+    assert all(p.wait() == 0 for p in procs)
+    path = str(out / "libhostsim.so")
+    # (its own cuda* functions, whatever else the process has loaded)
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-o", path, *[o for _, o in objs], "-lpthread"], check=True)
+    lib = C.CDLL(path)
+    for name, argt in wost._SIGS.items():
+        if hasattr(lib, name):
+            getattr(lib, name).argtypes = argt
+            getattr(lib, name).restype = C.c_int
+    lib.wost_last_error.restype = C.c_char_p
+    lib.sim_log.restype = C.c_char_p
+    lib.sim_used.restype = C.c_size_t
+    lib.sim_reset.argtypes = lib.sim_limit.argtypes = [C.c_size_t]
+    return lib
+
+
+@pytest.fixture
+def sim(simlib, monkeypatch):
+    """The stand-in in place of the library."""
+    monkeypatch.setattr(wost, "_lib", simlib)
+    simlib.sim_reset(1 << 40)
+    return simlib
+
+
+def _log(sim):
+    return sim.sim_log().decode().split("\n")[:-1]
+
+
+def _stream(sim):
+    s = C.c_void_p()
+    assert sim.cudaStreamCreateWithFlags(C.byref(s), 0) == 0
+    return s.value
+
+
+def _solve(scene, n=64, walks=4, kernel="persistent", **kw):
+    return wost.wost_solve(scene.handle, np.zeros((n, scene.dim), np.float32), walks, 1e-3, 1e-3, 256, 1, 0, kernel,
+                           **kw)
+
+
+def test_destroy_leaves_a_stream_alone_that_the_caller_has_destroyed(sim):
+    """A handle whose work has completed touches its stream no more: a
+    resumable solve that was never advanced, and a finished one."""
+    S = wost.Scene(scenes.config1(n_points=1))
+    for kernel in ("resumable", "persistent", "plain"):
+        s = _stream(sim)
+        h = _solve(S, kernel=kernel, stream=s)
+        if kernel != "resumable":
+            wost.wost_wait(h)
+        sim.cudaStreamDestroy(C.c_void_p(s))
+        wost.wost_solve_destroy(h)
+        assert sim.sim_bad() == 0, kernel
+    S.close()
