@@ -300,9 +300,10 @@ wost_status wost_wait(wost_solve_handle *solve, double timeout_s);
 wost_status wost_cancel(wost_solve_handle *solve);
 wost_status wost_solve_destroy(wost_solve_handle *solve);
 
-/* Device pointers to the per-point FP64 accumulators of a solve (valid until
- * destroy): sum and sum of squares of the walk estimates, walk and step
- * counts. */
+/* Device pointers to the per-point FP64 accumulators of a solve: sum and sum
+ * of squares of the walk estimates, walk and step counts.  Valid until
+ * destroy, which (engine requests aside) waits for the reads enqueued on the
+ * device by then. */
 wost_status wost_solve_device_accumulators(wost_solve_handle *solve, const double **sum,
                                            const double **sumsq, const uint64_t **walks,
                                            const uint64_t **steps);

@@ -284,6 +284,7 @@ struct wost_solve_handle {
     int resume_blocks = 0;
     uint64_t launches = 0;
     bool idle = false;  // nothing of it is in flight though no event tells: a resumable solve until its first launch
+    std::atomic<bool> handed_out{false};  // the caller has device pointers to the accumulators
     bool resumable() const { return kernel == WOST_KERNEL_RESUMABLE; }
     int kernel = 0;
     int *cancel_host = nullptr;                            // mapped pinned (engine requests: plain host)
@@ -309,6 +310,9 @@ struct wost_solve_handle {
         if (ev_done && launches) cudaEventSynchronize(ev_done);
         else if (stream && !idle) cudaStreamSynchronize(stream);
         if (res) {
+            // reads that the caller enqueued on its own streams, before the
+            // memory is another solve's
+            if (handed_out) cudaDeviceSynchronize();
             res_pool->give(std::move(res));
             return;
         }

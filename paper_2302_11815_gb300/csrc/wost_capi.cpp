@@ -889,6 +889,7 @@ wost_status wost_solve_destroy(wost_solve_handle *h) {
 wost_status wost_solve_device_accumulators(wost_solve_handle *h, const double **sum, const double **sumsq,
                                            const uint64_t **walks, const uint64_t **steps) {
     if (!h) return fail(WOST_ERR_INVALID_ARG, "null solve");
+    h->handed_out = true;
     if (sum) *sum = (const double *)h->sum.p;
     if (sumsq) *sumsq = (const double *)h->sumsq.p;
     if (walks) *walks = (const uint64_t *)h->walks_done.p;

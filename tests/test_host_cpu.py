@@ -80,3 +80,20 @@ def test_destroy_leaves_a_stream_alone_that_the_caller_has_destroyed(sim):
         wost.wost_solve_destroy(h)
         assert sim.sim_bad() == 0, kernel
     S.close()
+
+
+@pytest.mark.parametrize("kernel", ["persistent", "resumable"])
+def test_destroy_waits_for_reads_of_accumulators_handed_out(sim, kernel):
+    """A solve's memory goes to the next solve of its scene at once: reads that
+    the caller enqueued through the pointers it was given must be over."""
+    S = wost.Scene(scenes.config1(n_points=1))
+    h = _solve(S, kernel=kernel)
+    wost.wost_wait(h)
+    wost.wost_solve_destroy(h)
+    assert "device synchronised" not in _log(sim)
+    h = _solve(S, kernel=kernel)
+    wost.wost_wait(h)
+    assert all(wost.wost_solve_device_accumulators(h))
+    wost.wost_solve_destroy(h)
+    assert _log(sim)[-1] == "device synchronised"
+    S.close()
