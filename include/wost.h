@@ -298,6 +298,11 @@ wost_status wost_wait(wost_solve_handle *solve, double timeout_s);
 
 /* Stops a solve at the next walk boundary (walks already accumulated stay). */
 wost_status wost_cancel(wost_solve_handle *solve);
+
+/* Ends a solve.  Its device memory stays with its scene for the next solve, up
+ * to 64 MiB per solve, 4 solves per scene and 256 MiB per device (the oldest
+ * is freed first), until the scene is destroyed or an allocation of the
+ * library on that device finds no memory. */
 wost_status wost_solve_destroy(wost_solve_handle *solve);
 
 /* Device pointers to the per-point FP64 accumulators of a solve: sum and sum

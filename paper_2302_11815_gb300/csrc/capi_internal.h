@@ -131,68 +131,47 @@ struct SolveRes {
     }
 };
 
-// The idle resources of a scene: at most kIdle sets, kIdleBytes of device
-// memory each; freed with the scene (a set given back later is freed then).
+// The resources that a scene's finished solves left for its next ones.  All
+// scenes' idle sets are in one list (idle_sets, in the order they were given
+// back): a device keeps kAllBytes of them in all, a scene kIdle sets of
+// kIdleBytes each at most; the oldest go first, all of a device's when an
+// allocation of the library finds no memory there, a scene's with the scene
+// (a set given back later is freed then).
 struct SolvePool {
-    static constexpr size_t kIdle = 4, kIdleBytes = 64u << 20;
-    std::mutex mu;
-    std::vector<std::unique_ptr<SolveRes>> idle;
-    bool closed = false;
-    cudaError_t take(std::unique_ptr<SolveRes> &out) {
-        {
-            std::lock_guard<std::mutex> lk(mu);
-            if (!idle.empty()) {
-                out = std::move(idle.back());
-                idle.pop_back();
-                return cudaSuccess;
-            }
-        }
-        std::unique_ptr<SolveRes> r(new SolveRes);
-        const cudaError_t e = r->init();
-        if (e == cudaSuccess) out = std::move(r);
-        return e;
-    }
-    // (the device is no longer using the set)
-    void give(std::unique_ptr<SolveRes> r) {
-        if (r->bytes() > kIdleBytes) return;
-        std::lock_guard<std::mutex> lk(mu);
-        if (!closed && idle.size() < kIdle) idle.push_back(std::move(r));
-    }
-    void close() {
-        drop();
-        std::lock_guard<std::mutex> lk(mu);
-        closed = true;
-    }
-    // frees the idle sets (also when an allocation finds no memory)
-    void drop() {
-        std::lock_guard<std::mutex> lk(mu);
-        idle.clear();
-    }
-    // b.ensure(n), once more without the idle sets if memory is short
-    cudaError_t ensure(DevBuf &b, size_t n) {
-        cudaError_t e = b.ensure(n);
-        if (e != cudaErrorMemoryAllocation) return e;
-        cudaGetLastError();
-        drop();
-        return b.ensure(n);
-    }
+    static constexpr size_t kIdle = 4, kIdleBytes = 64u << 20, kAllBytes = 256u << 20;
+    int device = 0;
+    bool closed = false;  // (guarded by the list's mutex)
+    cudaError_t take(std::unique_ptr<SolveRes> &out);
+    void give(std::unique_ptr<SolveRes> r);  // (the device is no longer using the set)
+    void close();
 };
+// frees the idle sets of `device`; returns how many
+size_t drop_idle(int device);
+// alloc(), once more without the device's idle sets if memory is short
+template <class F>
+inline cudaError_t with_memory(int device, F alloc) {
+    const cudaError_t e = alloc();
+    if (e != cudaErrorMemoryAllocation) return e;
+    cudaGetLastError();
+    return drop_idle(device) ? alloc() : e;
+}
 
 // Words (u64) of a batched launch's counters.
 constexpr size_t kBatchCounters = 4 + 2 * kMaxStages;
 // The chain buffers of dimension di (0: 2D, 1: 3D) of a batched launch,
 // allocated for its grid; without memory for them, none (the launch then keeps
 // its walks to their ends).
-inline cudaError_t batch_chain_buffers(DevBuf chain[2], unsigned long long *counters, int di, int block, int blocks,
-                                       ChainBuffers *cb) {
+inline cudaError_t batch_chain_buffers(int device, DevBuf chain[2], unsigned long long *counters, int di, int block,
+                                       int blocks, ChainBuffers *cb) {
     for (int i = 0; i < 2; ++i) {
         const size_t cap = (size_t)batch_chain_capacity(block, blocks, i), bytes = cap * 3 * sizeof(float4);
         if (chain[i].bytes < bytes) chain[i].release();
         if (!chain[i].p) {
-            cudaError_t e = chain[i].alloc(bytes);
+            cudaError_t e = with_memory(device, [&] { return chain[i].alloc(bytes); });
             if (e == cudaErrorMemoryAllocation) {
                 cudaGetLastError();
-                chain[i].release();
+                chain[0].release();
+                chain[1].release();
                 *cb = ChainBuffers{};
                 return cudaSuccess;
             }

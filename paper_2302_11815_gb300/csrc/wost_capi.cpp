@@ -33,6 +33,90 @@ wost_status cuda_fail(cudaError_t e, const char *what) {
                 std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+namespace {
+struct IdleSet {
+    SolvePool *pool;
+    std::unique_ptr<SolveRes> res;
+};
+struct IdleSets {
+    std::mutex mu;
+    std::vector<IdleSet> sets;  // oldest first
+    // moves the sets that `which` names to `out` (to be freed without the lock)
+    template <class F>
+    void move_out(F which, std::vector<IdleSet> &out) {
+        size_t kept = 0;
+        for (IdleSet &q : sets) {
+            if (which(q)) out.push_back(std::move(q));
+            else if (IdleSet &to = sets[kept++]; &to != &q) to = std::move(q);
+        }
+        sets.erase(sets.begin() + (std::ptrdiff_t)kept, sets.end());
+    }
+};
+// (never destroyed: at exit the CUDA runtime may be gone before it)
+IdleSets &idle_sets() {
+    static IdleSets *all = new IdleSets;
+    return *all;
+}
+}  // namespace
+
+cudaError_t SolvePool::take(std::unique_ptr<SolveRes> &out) {
+    {
+        IdleSets &all = idle_sets();
+        std::lock_guard<std::mutex> lk(all.mu);
+        for (size_t i = all.sets.size(); i-- > 0;) {
+            if (all.sets[i].pool != this) continue;
+            out = std::move(all.sets[i].res);
+            all.sets.erase(all.sets.begin() + (std::ptrdiff_t)i);
+            return cudaSuccess;
+        }
+    }
+    return with_memory(device, [&] {
+        out.reset(new SolveRes);
+        const cudaError_t e = out->init();
+        if (e != cudaSuccess) out.reset();
+        return e;
+    });
+}
+
+void SolvePool::give(std::unique_ptr<SolveRes> r) {
+    if (r->bytes() > kIdleBytes) return;
+    std::vector<IdleSet> gone;
+    IdleSets &all = idle_sets();
+    std::lock_guard<std::mutex> lk(all.mu);
+    size_t mine = 0, bytes = r->bytes();
+    for (const IdleSet &q : all.sets) {
+        mine += q.pool == this;
+        if (q.pool->device == device) bytes += q.res->bytes();
+    }
+    if (closed || mine >= kIdle) return;
+    all.move_out(
+        [&](const IdleSet &q) {
+            if (q.pool->device != device || bytes <= kAllBytes) return false;
+            bytes -= q.res->bytes();
+            return true;
+        },
+        gone);
+    all.sets.push_back(IdleSet{this, std::move(r)});
+}
+
+void SolvePool::close() {
+    std::vector<IdleSet> gone;
+    IdleSets &all = idle_sets();
+    std::lock_guard<std::mutex> lk(all.mu);
+    closed = true;
+    all.move_out([&](const IdleSet &q) { return q.pool == this; }, gone);
+}
+
+size_t drop_idle(int device) {
+    std::vector<IdleSet> gone;
+    {
+        IdleSets &all = idle_sets();
+        std::lock_guard<std::mutex> lk(all.mu);
+        all.move_out([&](const IdleSet &q) { return q.pool->device == device; }, gone);
+    }
+    return gone.size();
+}
+
 }  // namespace wost
 
 extern "C" {
@@ -87,7 +171,8 @@ wost_status wost_scene_create(const wost_scene_desc *desc, wost_scene **out) {
         for (size_t k = 0; k < H.N.ids.size(); ++k) rec_of_id[H.N.ids[k]] = (int32_t)k;
         img.add(s->n_rec_of_id, rec_of_id);
         const size_t view_at = img.reserve(sizeof(SceneView));
-        CK(img.place(s->image), "cudaMalloc scene");
+        s->pool->device = s->device;
+        CK(with_memory(s->device, [&] { return img.place(s->image); }), "cudaMalloc scene");
         s->view_dev = (SceneView *)((unsigned char *)s->image.p + view_at);
         for (auto &q : img.parts)
             if (q.first != &s->n_rec_of_id) bytes += (int64_t)q.first->bytes;
@@ -320,7 +405,9 @@ wost_status wost::prepare_solve(wost_scene *scene, const wost_solve_desc *d, cud
     const bool has_n = d->normals && d->on_neumann;
     if (h->engine_buffers) {
         // engine requests allocate on the engine's stream without waiting for it
-        auto alloc = [&](DevBuf &b, size_t bytes) { return b.alloc_async(bytes, stream, h->pool); };
+        auto alloc = [&](DevBuf &b, size_t bytes) {
+            return with_memory(h->device, [&] { return b.alloc_async(bytes, stream, h->pool); });
+        };
         CK(alloc(h->points, pb), "cudaMalloc points");
         if (has_n) {
             CK(alloc(h->normals, pb), "cudaMalloc normals");
@@ -347,7 +434,7 @@ wost_status wost::prepare_solve(wost_scene *scene, const wost_solve_desc *d, cud
         // globals, sum, sumsq, walks, steps one after the other (one memset,
         // one copy per poll), then the inputs
         const size_t need = kGlobals * 8 + 4 * n * 8 + 2 * pb + n + 64;
-        CK(scene->pool->ensure(R.main, need), "cudaMalloc accumulators");
+        CK(with_memory(h->device, [&] { return R.main.ensure(need); }), "cudaMalloc accumulators");
         unsigned char *p = (unsigned char *)R.main.p;
         auto part = [&](DevBuf &b, size_t bytes) {
             b.view(p, bytes);
@@ -426,7 +513,7 @@ static cudaError_t chain_buffers(wost_solve_handle *h, uint64_t walks, int block
         cb->cap[i] = (unsigned)chain_capacity(walks, h->block, blocks, i);
         bytes[i] = (size_t)cb->cap[i] * 3 * sizeof(float4);
     }
-    cudaError_t e = h->res_pool->ensure(h->res->chain, bytes[0] + bytes[1]);
+    cudaError_t e = with_memory(h->device, [&] { return h->res->chain.ensure(bytes[0] + bytes[1]); });
     if (e != cudaSuccess) return e;
     cb->slots[0] = (float4 *)h->res->chain.p;
     cb->slots[1] = (float4 *)((unsigned char *)h->res->chain.p + bytes[0]);
@@ -454,7 +541,8 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
             // counter u32); the list of the saved walks' slots
             const size_t n_slots = (size_t)resume_slots(h->block, h->resume_blocks, h->lanes);
             const size_t slot_bytes = n_slots * 3 * sizeof(float4), state_bytes = 16 + n_slots * sizeof(uint32_t);
-            CK(scene->pool->ensure(h->res->resume, slot_bytes + state_bytes), "cudaMalloc slots");
+            CK(with_memory(h->device, [&] { return h->res->resume.ensure(slot_bytes + state_bytes); }),
+               "cudaMalloc slots");
             h->slots.view(h->res->resume.p, slot_bytes);
             h->rstate.view((unsigned char *)h->res->resume.p + slot_bytes, state_bytes);
             CK(cudaMemsetAsync(h->slots.p, 0, h->slots.bytes, stream), "memset");
@@ -479,7 +567,7 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *d, wost_solve_h
         } else if (d->kernel == WOST_KERNEL_PLAIN) {
             le = launch_walk_plain(scene->view, sp, acc, h->block, stream);
         } else if (d->kernel == WOST_KERNEL_COUNTING) {
-            le = h->counts.alloc(10 * 8);
+            le = with_memory(h->device, [&] { return h->counts.alloc(10 * 8); });
             if (le == cudaSuccess) le = cudaMemsetAsync(h->counts.p, 0, 10 * 8, stream);
             if (le == cudaSuccess)
                 le = launch_walk_count(scene->view, sp, acc, (unsigned long long *)h->counts.p, h->block, stream);
@@ -564,19 +652,21 @@ wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_so
             std::memcpy(staging[di].data(), &hd, sizeof hd);
             if (!jobs[di].empty())
                 std::memcpy(staging[di].data() + sizeof hd, jobs[di].data(), jobs[di].size() * sizeof(BatchJob));
-            CK(shared->jobs[di].alloc(staging[di].size()), "cudaMalloc jobs");
+            CK(with_memory(scenes[0]->device, [&] { return shared->jobs[di].alloc(staging[di].size()); }),
+               "cudaMalloc jobs");
             CK(cudaMemcpyAsync(shared->jobs[di].p, staging[di].data(), staging[di].size(), cudaMemcpyHostToDevice,
                                stream), "copy jobs");
         }
-        CK(shared->counters.alloc(kBatchCounters * 8), "cudaMalloc counters");
+        CK(with_memory(scenes[0]->device, [&] { return shared->counters.alloc(kBatchCounters * 8); }),
+           "cudaMalloc counters");
         CK(cudaMemsetAsync(shared->counters.p, 0, kBatchCounters * 8, stream), "memset");
         int blocks[2] = {0, 0};
         ChainBuffers chain[2];
         for (int di = 0; di < 2; ++di) {
             if (jobs[di].empty()) continue;
             CK(batch_grid(di + 2, block, depth[di], &blocks[di]), "occupancy");
-            CK(batch_chain_buffers(shared->chain[di], (unsigned long long *)shared->counters.p, di, block, blocks[di],
-                                   &chain[di]), "cudaMalloc slots");
+            CK(batch_chain_buffers(scenes[0]->device, shared->chain[di], (unsigned long long *)shared->counters.p, di,
+                                   block, blocks[di], &chain[di]), "cudaMalloc slots");
         }
         CK(cudaEventCreate(&shared->ev_start), "cudaEventCreate");
         CK(cudaEventCreate(&shared->ev_done), "cudaEventCreate");
@@ -990,7 +1080,7 @@ wost_status wost_scene_autotune(wost_scene *scene, const float *points, int64_t 
         const int dim = scene->view.dim;
         const int64_t m = std::min<int64_t>(n, 65536), stride = n / m;
         DevBuf sample;
-        CK(sample.alloc((size_t)m * dim * sizeof(float)), "cudaMalloc");
+        CK(with_memory(scene->device, [&] { return sample.alloc((size_t)m * dim * sizeof(float)); }), "cudaMalloc");
         CK(cudaMemcpy2D(sample.p, dim * sizeof(float), points, (size_t)stride * dim * sizeof(float),
                         dim * sizeof(float), (size_t)m, cudaMemcpyDeviceToDevice),
            "sample copy");

@@ -377,8 +377,11 @@ void issue_check(wost_engine *e, std::vector<Request *> &ready) {
         cs.out.release_async(e->check_stream);
         if ((err = cudaMallocHost((void **)&cs.host_jobs, nc * sizeof(StatJob))) == cudaSuccess &&
             (err = cudaMallocHost((void **)&cs.host_out, nc * 32)) == cudaSuccess &&
-            (err = cs.jobs.alloc_async(nc * sizeof(StatJob), e->check_stream, e->pool)) == cudaSuccess &&
-            (err = cs.out.alloc_async(nc * 32, e->check_stream, e->pool)) == cudaSuccess)
+            (err = with_memory(e->device, [&] {
+                 return cs.jobs.alloc_async(nc * sizeof(StatJob), e->check_stream, e->pool);
+             })) == cudaSuccess &&
+            (err = with_memory(e->device, [&] { return cs.out.alloc_async(nc * 32, e->check_stream, e->pool); })) ==
+                cudaSuccess)
             cs.cap = nc;
     }
     if (err == cudaSuccess && !cs.ev) err = cudaEventCreateWithFlags(&cs.ev, cudaEventDisableTiming);
@@ -462,7 +465,8 @@ cudaError_t ensure_graph(wost_engine *e, Slot &sl, const size_t cnt[2], const in
             std::memset(sl.host[di], 0, sizeof(BatchHeader));
             sl.jobs[di].~DevBuf();
             new (&sl.jobs[di]) DevBuf();
-            if ((er = sl.jobs[di].alloc(table_bytes(nc))) != cudaSuccess) return er;
+            if ((er = with_memory(e->device, [&] { return sl.jobs[di].alloc(table_bytes(nc)); })) != cudaSuccess)
+                return er;
             sl.cap[di] = nc;
             rebuild = true;
         }
@@ -477,7 +481,8 @@ cudaError_t ensure_graph(wost_engine *e, Slot &sl, const size_t cnt[2], const in
         }
     }
     if (!sl.counters.p) {
-        if ((er = sl.counters.alloc(kBatchCounters * 8)) != cudaSuccess) return er;
+        if ((er = with_memory(e->device, [&] { return sl.counters.alloc(kBatchCounters * 8); })) != cudaSuccess)
+            return er;
         if ((er = cudaMallocHost((void **)&sl.steps_host, 8)) != cudaSuccess) return er;
         *sl.steps_host = 0;
         rebuild = true;
@@ -493,7 +498,8 @@ cudaError_t ensure_graph(wost_engine *e, Slot &sl, const size_t cnt[2], const in
     unsigned long long *ctr = (unsigned long long *)sl.counters.p;
     ChainBuffers chain[2];
     for (int di = 0; di < 2; ++di)
-        if ((er = batch_chain_buffers(sl.chain[di], ctr, di, e->block, blocks[di], &chain[di])) != cudaSuccess)
+        if ((er = batch_chain_buffers(e->device, sl.chain[di], ctr, di, e->block, blocks[di], &chain[di])) !=
+            cudaSuccess)
             return er;
     if ((er = cudaStreamBeginCapture(sl.stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess) return er;
     cudaMemsetAsync(sl.counters.p, 0, kBatchCounters * 8, sl.stream);

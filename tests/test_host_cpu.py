@@ -97,3 +97,65 @@ def test_destroy_waits_for_reads_of_accumulators_handed_out(sim, kernel):
     wost.wost_solve_destroy(h)
     assert _log(sim)[-1] == "device synchronised"
     S.close()
+
+
+def _finished(S, n, walks=4, kernel="persistent"):
+    h = _solve(S, n, walks, kernel)
+    wost.wost_wait(h)
+    wost.wost_solve_destroy(h)
+
+
+def _batch(S, n, walks):
+    hs = wost.wost_solve_batch([S.handle], [dict(points=np.zeros((n, S.dim), np.float32), walks_per_point=walks,
+                                                 epsilon=1e-3, r_min=1e-3, max_steps=256, seed=1)])
+    for h in hs:
+        wost.wost_wait(h)
+        wost.wost_solve_destroy(h)
+
+
+@pytest.mark.parametrize("what", ["scene", "solve", "counting", "resumable", "batch"])
+def test_memory_that_is_short_comes_from_other_scenes_idle_sets(sim, what):
+    """A finished solve's memory stays with its scene for the next solve, until
+    an allocation of the library finds none: whichever scene's it is."""
+    spec = scenes.config1(n_points=1)
+    A, B = wost.Scene(spec), wost.Scene(spec)
+    _finished(A, 200000)
+    sim.sim_limit(sim.sim_used())  # nothing is left but A's idle set
+    if what == "scene":
+        wost.Scene(spec).close()
+    elif what == "batch":
+        _batch(B, 1000, 4)
+    else:
+        _finished(B, 1000, kernel="persistent" if what == "solve" else what)
+    A.close()
+    B.close()
+
+
+def test_idle_memory_of_all_scenes_is_bounded(sim):
+    spec = scenes.config1(n_points=1)
+    before = sim.sim_used()
+    S = [wost.Scene(spec) for _ in range(12)]
+    held = sim.sim_used()
+    for s in S:
+        _finished(s, 600000, 1)  # some 40 MB each, 480 in all
+    assert sim.sim_used() - held <= 256 << 20
+    # the last scenes' sets are those that are left
+    used = sim.sim_used()
+    _finished(S[-1], 600000, 1)
+    assert sim.sim_used() == used
+    for s in S:
+        s.close()
+    assert sim.sim_used() == before
+
+
+@pytest.mark.parametrize("kernel,want", [("persistent", ["persistent"]), ("resumable", ["resume 2048"] * 4),
+                                         ("batch", ["batch 2d without slots"])])
+def test_without_memory_for_hand_overs_the_walks_stay(sim, kernel, want):
+    S = wost.Scene(scenes.config1(n_points=1))
+    sim.sim_limit(sim.sim_used() + (1 << 20))  # (the stand-in's slots take 6 MB)
+    if kernel == "batch":
+        _batch(S, 64, 400)
+    else:
+        _finished(S, 64, 400, kernel)
+    assert _log(sim) == want
+    S.close()
