@@ -106,6 +106,7 @@ __device__ __forceinline__ bool may_have_silhouette(const float lo[3], const flo
 // The error terms: u is a quotient of cross products over the determinant,
 // so its rounding grows with 1 / |determinant| (grazing rays); margin kEdgeTol
 // of the hit test doubled.  te: the rounding of t.
+// scale: the largest coordinate of the boundary and of o.
 // Returns te, negative if the hit is not clear (out of line: two call sites).
 template <int D>
 __device__ __noinline__ float hit_clear(const float4 *prims, uint32_t k, P3 o, P3 v, float t, float tmax, float scale) {
@@ -647,11 +648,14 @@ struct WarpQ {
         t_out = tmaxA;
         occB = false;
         // fast reciprocals: the boxes are widened by more than they, and the
-        // rounding of the one-lane slab test, can move its planes
+        // rounding of the one-lane slab test, can move its planes: that grows
+        // with |plane - o|, so with the largest coordinate in play (a walk's
+        // origin is near the boundary, a query's anywhere)
+        const float reach = fmaxf(scale, maxabs3(o));
         const P3 ia = mk(__fdividef(1.f, va.x), __fdividef(1.f, va.y), D == 3 ? __fdividef(1.f, va.z) : 0.f);
         P3 ib = mk(0.f, 0.f, 0.f);
         if (wantB) ib = mk(__fdividef(1.f, vb.x), __fdividef(1.f, vb.y), D == 3 ? __fdividef(1.f, vb.z) : 0.f);
-        const float pad = 8e-6f * scale;
+        const float pad = 8e-6f * reach;
         // a zero component makes the slab test drop boxes that touch the ray
         // (0 x inf): such a ray is lane 0's
         auto flat = [](P3 v) {
@@ -666,13 +670,13 @@ struct WarpQ {
             const Prim<D> p = load_prim<D>(T.prims, k);
             float t;
             if ((int)k != skipA && prim_ray<D>(p, o, va, tmaxA, t, kEdgeTol) && lb.add(t, (int)k))
-                teA = hit_clear<D>(T.prims, k, o, va, t, tmaxA, scale);
+                teA = hit_clear<D>(T.prims, k, o, va, t, tmaxA, reach);
             if (wantB && (int)k != skipB && prim_ray<D>(p, o, vb, tmaxB, t, 0.f)) {
-                if (hit_clear<D>(T.prims, k, o, vb, t, tmaxB, scale) >= 0.f) occ = true;
+                if (hit_clear<D>(T.prims, k, o, vb, t, tmaxB, reach) >= 0.f) occ = true;
                 else occ_maybe = true;
             }
         };
-        bool ok = !axis;
+        bool ok = !axis && reach < INFINITY;
         if (ok)
             ok = search(
                 T, kBrute,
