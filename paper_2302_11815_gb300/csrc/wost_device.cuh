@@ -631,9 +631,9 @@ __device__ float q_silhouette(const TreeView &T, P3 x, float rmax, const Stack &
 constexpr unsigned kSilSlice = 8;
 constexpr int kSilFew = 24;
 
-template <int D, bool CN = false>
-__device__ __forceinline__ bool q_silhouette_sliced(const TreeView &T, P3 x, float rmax, const Stack &st, Cnt<CN> &cnt,
-                                                    bool act, int few, float &r, float &found2) {
+template <int D>
+__device__ __forceinline__ bool q_silhouette_sliced(const TreeView &T, P3 x, float rmax, const Stack &st, bool act,
+                                                    int few, float &r, float &found2) {
     bool found = false;
     float r2 = rmax * rmax;
     r = rmax;
@@ -658,7 +658,6 @@ __device__ __forceinline__ bool q_silhouette_sliced(const TreeView &T, P3 x, flo
                 uint32_t f = leaf_first(ref), c = leaf_count(ref);
 #pragma unroll 1
                 for (uint32_t k = f; k < f + c; ++k) {
-                    cnt.prim(C_Q2);
                     float d2 = sil_test<D>(T.prims, k, x, r2);
                     if (d2 < r2) {
                         r2 = d2;
@@ -666,7 +665,6 @@ __device__ __forceinline__ bool q_silhouette_sliced(const TreeView &T, P3 x, flo
                     }
                 }
             } else {
-                cnt.node(C_Q2);
                 Node<D> n = load_node<D>(T.nodes, ref);
                 float e0 = box_dist2<D>(n.lo0, n.hi0, x), e1 = box_dist2<D>(n.lo1, n.hi1, x);
                 bool v0 = e0 < r2, v1 = e1 < r2;
@@ -1307,8 +1305,11 @@ __device__ __noinline__ SilAnswer coop_silhouette(const TreeView &T, P3 x, float
                                                   int2 *fr, int frs, int fcap);
 
 // Query policy over the binary trees: each lane answers its own walk's
-// queries with its own shared-memory stack.
-template <int D, bool CN>
+// queries with its own shared-memory stack.  COOP: long silhouette searches in
+// 3D may be the whole warp's (where `coop` says so: under the scene's limits).
+// Without it every search is the lane's own and uninterrupted: the slices cost
+// a search that stays its lane's own 5 to 8% (plain kernel, torus, box).
+template <int D, bool CN, bool COOP = false>
 struct LaneQ {
     static constexpr bool kWarp = false;
     Stack st;
@@ -1316,7 +1317,7 @@ struct LaneQ {
     __device__ __forceinline__ void hit(const TreeView &, int) {}
     __device__ Closest closest(const TreeView &T, P3 x, float bound2) { return q_closest<D, CN>(T, x, st, cnt, bound2); }
     __device__ float silhouette(const TreeView &T, P3 x, float rmax) { return q_silhouette<D, CN>(T, x, rmax, st, cnt); }
-    bool coop = false;  // long silhouette searches are the whole warp's (walk kernels under the scene's limits)
+    bool coop = false;
     __device__ int ray(const TreeView &T, P3 o, P3 v, float tmax, int skip, bool any, float &t) {
         return q_ray<D, CN>(T, o, v, tmax, skip, any, t, st, cnt);
     }
@@ -1346,6 +1347,9 @@ struct LaneQ {
     __device__ float silhouette_w(const TreeView &T, P3 x, float rmax, bool act, float tau) {
         if constexpr (kPostpone) {
             return q_silhouette_w<D, CN>(T, x, rmax, st, cnt, act);
+        } else if constexpr (!COOP || CN) {
+            // (work counters are per lane and of the binary tree)
+            return act ? silhouette(T, x, rmax) : rmax;
         } else {
             // The searches are heavy-tailed (110 visits on the mean around
             // the noisy torus, thousands at worst) and the warp waits for its
@@ -1359,16 +1363,13 @@ struct LaneQ {
             // 1,210, 32: 1,030).
             float r = rmax, found2 = INFINITY;
             bool need = act;
-            // (work counters are per lane and of the binary tree: each of their
-            // searches is the lane's own, to its end)
-            int few = !CN && coop ? kSilFew : 0;
+            int few = coop ? kSilFew : 0;
 #pragma unroll 1
             for (;;) {
                 float rr;
                 const bool asked = need;
-                need = q_silhouette_sliced<D, CN>(T, x, rmax, st, cnt, need, few, rr, found2);
+                need = q_silhouette_sliced<D>(T, x, rmax, st, need, few, rr, found2);
                 if (asked && !need) r = rr;
-                if constexpr (CN) return r;
                 unsigned m = __ballot_sync(0xffffffffu, need);
                 if (!m) return r;
                 const int lane = threadIdx.x & 31;

@@ -66,25 +66,26 @@ __device__ __forceinline__ Group make_team() {
     return g;
 }
 
-template <int D, bool CN, int T>
+template <int D, bool CN, int T, bool COOP>
 struct PolicyOf;
-template <int D, bool CN>
-struct PolicyOf<D, CN, 1> {
-    using type = LaneQ<D, CN>;
+template <int D, bool CN, bool COOP>
+struct PolicyOf<D, CN, 1, COOP> {
+    using type = LaneQ<D, CN, COOP>;
 };
-template <int D, bool CN>
-struct PolicyOf<D, CN, WOST_WIDE> {
+template <int D, bool CN, bool COOP>
+struct PolicyOf<D, CN, WOST_WIDE, COOP> {
     using type = GroupQ<D, CN>;
 };
 
 // the query policy of this thread's team, with its shared-memory stack
-template <int D, bool CN, int T = 1>
-__device__ __forceinline__ typename PolicyOf<D, CN, T>::type make_q(int depth, unsigned int *guard, Cnt<CN> &cnt,
-                                                                    uint32_t visit_limit = 0u, bool coop = false) {
+template <int D, bool CN, int T = 1, bool COOP = true>
+__device__ __forceinline__ typename PolicyOf<D, CN, T, COOP>::type make_q(int depth, unsigned int *guard, Cnt<CN> &cnt,
+                                                                          uint32_t visit_limit = 0u,
+                                                                          bool coop = false) {
     extern __shared__ int2 smem_stack[];
     if constexpr (T == 1) {
         Stack s{smem_stack + threadIdx.x, (int)blockDim.x, depth, guard, visit_limit};
-        return LaneQ<D, CN>{s, cnt, coop};
+        return LaneQ<D, CN, COOP>{s, cnt, coop};
     } else {
         GStack s{smem_stack + (threadIdx.x / T) * depth, depth, guard};
         return GroupQ<D, CN>{make_team<T>(), s, cnt};
@@ -134,11 +135,12 @@ __device__ __forceinline__ void save_walk(float4 *slot, const Walk &w, int job =
                           __uint_as_float(flags));
 }
 
-template <int D, bool SCR>
+// COOP: joint silhouette searches (3D)
+template <int D, bool SCR, bool COOP>
 __global__ void WOST_WALK_BOUNDS k_walk_plain(const __grid_constant__ SceneView sc, const SolveParams sp, const Accumulators acc,
                                                     int warp_uniform_points) {
     Cnt<false> cnt;
-    auto q = make_q<D, false>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, sp.coop != 0);
+    auto q = make_q<D, false, 1, COOP>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, COOP);
     const Group g = make_team<1>();
     const uint64_t total = (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
     const uint64_t gid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -399,6 +401,14 @@ static cudaError_t smem_limit(const void *k, size_t bytes) {
                              : cudaSuccess;
 }
 
+// Silhouette candidates from which the plain kernel's warps search jointly in
+// 3D.  Its lanes run dry one by one, so most steps have few open searches and
+// would be the warp's, one after the other, however short.  Lane's own / joint,
+// ms: 65,000 points x 32 walks in a cube of 108 candidates 48 / 70, x 16 in one
+// of 1,584 61 / 80, x 8 around a sphere of 1,440 63 / 70; 17,003 x 32 around
+// a torus of 4,320 144 / 174, of 18,750 243 / 216.
+constexpr int kPlainCoop = 8192;
+
 template <bool SCR>
 static cudaError_t walk_plain_launch(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, int block,
                                      cudaStream_t s) {
@@ -407,14 +417,15 @@ static cudaError_t walk_plain_launch(const SceneView &sc, const SolveParams &sp,
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
     size_t sm = smem_bytes(sp.stack_depth, block);
     int uniform = (sp.walks_per_point % 32 == 0) && (block % 32 == 0);
-    const void *k = sc.dim == 2 ? (const void *)k_walk_plain<2, SCR> : (const void *)k_walk_plain<3, SCR>;
-    cudaError_t e = smem_limit(k, sm);
-    if (e != cudaSuccess) return e;
-    if (sc.dim == 2)
-        k_walk_plain<2, SCR><<<(unsigned)grid, block, sm, s>>>(sc, sp, acc, uniform);
-    else
-        k_walk_plain<3, SCR><<<(unsigned)grid, block, sm, s>>>(sc, sp, acc, uniform);
-    return cudaGetLastError();
+    auto launch = [&](auto *k) {
+        cudaError_t e = smem_limit((const void *)k, sm);
+        if (e != cudaSuccess) return e;
+        k<<<(unsigned)grid, block, sm, s>>>(sc, sp, acc, uniform);
+        return cudaGetLastError();
+    };
+    if (sc.dim == 2) return launch(k_walk_plain<2, SCR, false>);
+    return sp.coop && sc.S.n_prims >= kPlainCoop ? launch(k_walk_plain<3, SCR, true>)
+                                                 : launch(k_walk_plain<3, SCR, false>);
 }
 
 template <bool SCR>
