@@ -1432,7 +1432,14 @@ __device__ __forceinline__ bool in_bounds(const SceneView &sc, P3 x) {
 //
 // SCR: compiled with the screened-equation terms (R15); the Poisson-only
 // instantiation keeps them, and their registers, out of the hot loop.
-template <int D, bool SCR, class Q>
+// EARLY (one lane per walk): the query origin, which Q.2 needs first, is
+// formed before Q.1 instead of after it, and takes registers there.  Before /
+// after, 2D, 3,800 points x 480 walks (Koch level 3: x 100), ms: plain kernel,
+// flower 23.0 / 21.9, disk 42.0 / 40.8, crack 70.5 / 68.7, Koch 673 / 664; the
+// persistent kernel that hands its walks over, disk of 356 segments 25.2 /
+// 25.8, of 128 17.9 / 18.5, but crack 18.5 / 18.0, Koch 306 / 300: it stays
+// before Q.1 there.
+template <int D, bool SCR, bool EARLY = false, class Q>
 __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q &q, bool act) {
     constexpr unsigned FULL = 0xffffffffu;
     // R13: a walk outside the grown bounding box of the boundary has left the
@@ -1440,8 +1447,13 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
     const bool lost = act && !in_bounds<D>(sc, w.x);
     if constexpr (Q::kWarp) q.begin_step(sp, w, lost);  // the whole warp holds this walk
     // R4: query origin off the Neumann boundary
-    const float delta = sp.offset * (1.f + maxabs3(w.x));
-    const P3 xq = w.onN ? w.x - w.n * delta : w.x;
+    float delta = 0.f;
+    P3 xq = w.x;
+    const auto off_boundary = [&] {
+        delta = sp.offset * (1.f + maxabs3(w.x));
+        xq = w.onN ? w.x - w.n * delta : w.x;
+    };
+    if constexpr (Q::kWarp || EARLY) off_boundary();
     // A walk that hugs the Neumann boundary far from the Dirichlet one does
     // not need its distance: with a silhouette nearer than a lower bound of
     // that distance, the star radius is the silhouette's.
@@ -1491,6 +1503,7 @@ __device__ bool walk_step(const SceneView &sc, const SolveParams &sp, Walk &w, Q
         }
     }
     act = act && !ended;
+    if constexpr (!(Q::kWarp || EARLY)) off_boundary();
     // distance to the visibility silhouette (Q.2) within d_D, star radius (R3)
     float dsil = dsil0;
     if (!skip1) dsil = q.silhouette_w(sc.S, xq, dD, act, sc.tau);

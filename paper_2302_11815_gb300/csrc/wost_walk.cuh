@@ -278,7 +278,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ Scene
             }
         }
         if (src.steps_run && lane == 0) atomicAdd(src.steps_run, (unsigned long long)__popc(held));
-        if (walk_step<D, SCR>(sc, sp, w, q, have)) {
+        if (walk_step<D, SCR, T == 1>(sc, sp, w, q, have)) {
             if (g.leader()) accumulate(acc, w);
             have = false;
         }
