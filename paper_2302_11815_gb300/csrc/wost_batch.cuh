@@ -32,16 +32,25 @@ __device__ __forceinline__ void init_job_walk(const BatchJob &J, unsigned long l
 // the jobs' walks; a team maps its next index to a job by binary search over
 // the jobs' first indices and runs that job's walk on that job's scene.
 // steps_out (may be null) receives the walk steps of the finished walks.
-// src, ho: walks taken up from, and handed over to, another launch (a saved
-// walk keeps its job index).
-template <int D, bool SCR>
+// src, ho: walks taken up from (SAVED), and handed over to, another launch (a
+// saved walk keeps its job index).  As in k_walk_persistent, the loop is bound
+// by its instruction supply, so SAVED is a parameter of the template and the
+// stores of a hand-over are behind the loop, and the counter is read by a warp
+// that has itself found nothing to draw, and else every eighth step of lane 0's
+// walk.  Device time of one scene of 3,800 points x 480 walks (Koch level 3: x
+// 100; torus of 18,750 candidates: 17,003 x 32), ms, without hand-over / all of
+// it in the loop, every step / as it is: disk of 356 segments 27.9 / 30.2 / 28.2,
+// flower 9.75 / 10.5 / 10.1, annulus 37.2 / 32.2 / 30.3, crack 26.8 / 18.1 /
+// 17.4, Koch 356 / 341 / 334, torus 146 / 83 / 80.  Read only after a failed
+// draw, 12 mixed scenes with long walks take 358 ms instead of 255.
+template <int D, bool SCR, bool SAVED>
 __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hdr,
                                                     const BatchJob *__restrict__ jobs, unsigned long long *counter,
                                                     unsigned int *guard, int stack_depth, const int *cancel,
                                                     unsigned long long *steps_out, const SavedWalks src,
                                                     const HandOver ho) {
     const int n_jobs = hdr->n_jobs;
-    const unsigned long long total = src.slots ? (unsigned long long)*src.count : hdr->total;
+    const unsigned long long total = SAVED ? (unsigned long long)*src.count : hdr->total;
     if (n_jobs <= 0) return;
     Cnt<false> cnt;
     auto q = make_q<D, false>(stack_depth, guard, cnt, 0u, true);
@@ -52,7 +61,8 @@ __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hd
     int job = -1;
     unsigned int ran = 0;  // steps of this lane's finished walks
     // the launch's counter has run past `total`, or the lane holds no walks
-    bool drained = src.per_warp && lane >= (int)src.per_warp;
+    bool drained = SAVED && src.per_warp && lane >= (int)src.per_warp;
+    unsigned first = 0xffffffffu, held;
     // as in k_walk_persistent: the whole warp stays in the loop and
     // reconverges after every step
     for (;;) {
@@ -61,7 +71,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hd
             int lead = __ffs(need) - 1;
             unsigned long long base = 0;
             if (lane == lead) {
-                if (src.slots) {
+                if constexpr (SAVED) {
                     base = atomicAdd(src.next, (unsigned)__popc(need));
                 } else {
                     bool stop = cancel && *(volatile const int *)cancel != 0;
@@ -73,7 +83,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hd
                 unsigned long long my = base + __popc(need & ((1u << g.base) - 1u));
                 if (my >= total) {
                     drained = true;
-                } else if (src.slots) {
+                } else if constexpr (SAVED) {
                     load_walk(src.slots + 3 * (size_t)my, w, &job);
                 } else {
                     const int lo = job_of(jobs, n_jobs, my);
@@ -86,14 +96,17 @@ __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hd
                 }
             }
         }
-        const unsigned held = __ballot_sync(FULL, job >= 0);
+        held = __ballot_sync(FULL, job >= 0);
         if (!held) {
             if (__any_sync(FULL, !drained)) continue;
             break;
         }
-        if (ho.slots && (src.slots ? hand_over(ho, src.next, total, lane, w, job >= 0, held, job)
-                                   : hand_over(ho, counter, total, lane, w, job >= 0, held, job)))
-            break;
+        // (a warp whose walks are all long finds nothing to draw late)
+        if (ho.slots && __any_sync(FULL, drained || (lane == 0 && (w.steps & 7) == 0))) {
+            if constexpr (SAVED) first = hand_over_at(ho, src.next, total, lane, held);
+            else first = hand_over_at(ho, counter, total, lane, held);
+            if (first != 0xffffffffu) break;
+        }
         // lanes without a job step a dummy reference to job 0 (inactive)
         const BatchJob &J = jobs[job >= 0 ? job : 0];
         if (walk_step<D, SCR>(*J.scene, J.sp, w, q, job >= 0)) {
@@ -105,6 +118,8 @@ __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hd
         }
         __syncwarp();
     }
+    if (first != 0xffffffffu && job >= 0)
+        save_walk(ho.slots + 3 * (size_t)(first + __popc(held & ((1u << lane) - 1u))), w, job);
     if (steps_out) {
         unsigned long long r = ran;
 #pragma unroll

@@ -14,28 +14,30 @@ namespace wost {
 
 namespace {
 
-template <int D, bool SCR>
+// the fewest resident blocks per SM of a dimension's forms (their shared
+// memory size is set for all of them)
+template <int D>
 cudaError_t occupancy(int block, size_t sm, int *per_sm) {
-    cudaError_t e = cudaSuccess;
-    if (sm > 48 * 1024) e = cudaFuncSetAttribute(k_walk_batch<D, SCR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k_walk_batch<D, SCR>, block, sm);
-    return e;
+    *per_sm = 0;
+    for (const void *k : {(const void *)k_walk_batch<D, false, false>, (const void *)k_walk_batch<D, false, true>,
+                          (const void *)k_walk_batch<D, true, false>, (const void *)k_walk_batch<D, true, true>}) {
+        int n = 0;
+        cudaError_t e = smem_limit(k, sm);
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, block, sm);
+        if (e != cudaSuccess) return e;
+        if (!*per_sm || n < *per_sm) *per_sm = n;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
 
 cudaError_t batch_grid(int dim, int block, int depth, int *blocks_out) {
-    int dev = 0, sms = 0, per_sm = 0, per_sm_p = 0;
+    int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const size_t sm = smem_bytes(depth, block);
-    // both forms get the grid of the one with fewer resident blocks (the
-    // shared memory size is set for both)
-    if (e == cudaSuccess) e = dim == 2 ? occupancy<2, true>(block, sm, &per_sm) : occupancy<3, true>(block, sm, &per_sm);
-    if (e == cudaSuccess)
-        e = dim == 2 ? occupancy<2, false>(block, sm, &per_sm_p) : occupancy<3, false>(block, sm, &per_sm_p);
-    if (e != cudaSuccess) return e;
-    per_sm = std::min(per_sm, per_sm_p);
+    if (e == cudaSuccess) e = dim == 2 ? occupancy<2>(block, sm, &per_sm) : occupancy<3>(block, sm, &per_sm);
     // the warp kernels that end a batch are loaded now, not while a graph is captured
     for (int scr = 0; scr < 2 && e == cudaSuccess; ++scr) e = prepare_walk_warp_batch(dim, depth, scr != 0);
     if (e != cudaSuccess) return e;
@@ -49,8 +51,8 @@ template <int D, bool SCR>
 cudaError_t launch(const BatchHeader *hdr, const BatchJob *jobs, unsigned long long *counter, unsigned int *guard,
                    int depth, const int *cancel, int block, int blocks, cudaStream_t s, unsigned long long *steps_out,
                    const SavedWalks &src, const HandOver &ho) {
-    k_walk_batch<D, SCR><<<blocks, block, smem_bytes(depth, block), s>>>(hdr, jobs, counter, guard, depth, cancel,
-                                                                         steps_out, src, ho);
+    const auto k = src.slots ? k_walk_batch<D, SCR, true> : k_walk_batch<D, SCR, false>;
+    k<<<blocks, block, smem_bytes(depth, block), s>>>(hdr, jobs, counter, guard, depth, cancel, steps_out, src, ho);
     return cudaGetLastError();
 }
 
