@@ -158,28 +158,25 @@ inline cudaError_t with_memory(int device, F alloc) {
 
 // Words (u64) of a batched launch's counters.
 constexpr size_t kBatchCounters = 4 + 2 * kMaxStages;
-// The chain buffers of dimension di (0: 2D, 1: 3D) of a batched launch,
-// allocated for its grid; without memory for them, none (the launch then keeps
+// The chain buffers of dimension di (0: 2D, 1: 3D) of a batched launch, in
+// `chain`, for its grid; without memory for them, none (the launch then keeps
 // its walks to their ends).
-inline cudaError_t batch_chain_buffers(int device, DevBuf chain[2], unsigned long long *counters, int di, int block,
+inline cudaError_t batch_chain_buffers(int device, DevBuf &chain, unsigned long long *counters, int di, int block,
                                        int blocks, ChainBuffers *cb) {
+    size_t bytes[2];
     for (int i = 0; i < 2; ++i) {
-        const size_t cap = (size_t)batch_chain_capacity(block, blocks, i), bytes = cap * 3 * sizeof(float4);
-        if (chain[i].bytes < bytes) chain[i].release();
-        if (!chain[i].p) {
-            cudaError_t e = with_memory(device, [&] { return chain[i].alloc(bytes); });
-            if (e == cudaErrorMemoryAllocation) {
-                cudaGetLastError();
-                chain[0].release();
-                chain[1].release();
-                *cb = ChainBuffers{};
-                return cudaSuccess;
-            }
-            if (e != cudaSuccess) return e;
-        }
-        cb->cap[i] = (unsigned)cap;
-        cb->slots[i] = (float4 *)chain[i].p;
+        cb->cap[i] = (unsigned)batch_chain_capacity(block, blocks, i);
+        bytes[i] = (size_t)cb->cap[i] * 3 * sizeof(float4);
     }
+    const cudaError_t e = with_memory(device, [&] { return chain.ensure(bytes[0] + bytes[1]); });
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        *cb = ChainBuffers{};
+        return cudaSuccess;
+    }
+    if (e != cudaSuccess) return e;
+    cb->slots[0] = (float4 *)chain.p;
+    cb->slots[1] = (float4 *)((unsigned char *)chain.p + bytes[0]);
     cb->counters = (unsigned int *)(counters + 4 + di * kMaxStages);
     return cudaSuccess;
 }
@@ -187,8 +184,8 @@ inline cudaError_t batch_chain_buffers(int device, DevBuf chain[2], unsigned lon
 // resources shared by the solves of one batched launch
 struct BatchShared {
     // counters: next walk (2D), next walk (3D), guard, -, then each
-    // dimension's hand-over counters; chain: its slot arrays
-    DevBuf jobs[2], counters, chain[2][2];
+    // dimension's hand-over counters
+    DevBuf jobs[2], counters;
     unsigned long long total[2] = {0, 0};
     cudaEvent_t ev_start = nullptr, ev_done = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;  // the 3D launch's side stream

@@ -631,9 +631,11 @@ wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_so
         // jobs per dimension, in the caller's order
         std::vector<BatchJob> jobs[2];
         int depth[2] = {0, 0};
+        int32_t first[2] = {0, 0};  // solve of each dimension's first job
         for (int32_t i = 0; i < n; ++i) {
             wost_solve_handle *h = hs[i].get();
             int di = h->dim - 2;
+            if (jobs[di].empty()) first[di] = i;
             BatchJob j;
             j.scene = scenes[i]->view_dev;
             j.sp = h->sp;
@@ -665,8 +667,13 @@ wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_so
         for (int di = 0; di < 2; ++di) {
             if (jobs[di].empty()) continue;
             CK(batch_grid(di + 2, block, depth[di], &blocks[di]), "occupancy");
-            CK(batch_chain_buffers(scenes[0]->device, shared->chain[di], (unsigned long long *)shared->counters.p, di,
-                                   block, blocks[di], &chain[di]), "cudaMalloc slots");
+            // the slots are in the resources of the dimension's first solve, which
+            // its scene keeps for the next one (allocated and freed with every
+            // batch they took 0.2 ms of it); no solve of the batch gives its
+            // resources back before the whole batch has ended
+            DevBuf &slots = hs[first[di]]->res->chain;
+            CK(batch_chain_buffers(scenes[0]->device, slots, (unsigned long long *)shared->counters.p, di, block,
+                                   blocks[di], &chain[di]), "cudaMalloc slots");
         }
         CK(cudaEventCreate(&shared->ev_start), "cudaEventCreate");
         CK(cudaEventCreate(&shared->ev_done), "cudaEventCreate");

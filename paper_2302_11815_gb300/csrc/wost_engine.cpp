@@ -71,7 +71,7 @@ struct Slot {
     int depth[2] = {0, 0};     // stack entries the graph was captured with
     bool scr[2] = {true, true};  // the kernels' form: screened, or Poisson only
     DevBuf counters;           // next walk 2D, next walk 3D, guard, walk steps run, hand-over counters
-    DevBuf chain[2][2];        // slots of walks handed over between the round's launches
+    DevBuf chain[2];           // slots of walks handed over between the round's launches
     unsigned long long *steps_host = nullptr;  // pinned copy of the walk-step count
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;

@@ -159,3 +159,28 @@ def test_without_memory_for_hand_overs_the_walks_stay(sim, kernel, want):
         _finished(S, 64, 400, kernel)
     assert _log(sim) == want
     S.close()
+
+
+def test_a_batch_keeps_its_slots_for_the_next_one(sim):
+    """The slots come from the resources that the scenes keep: a second batch
+    of the same size takes no more memory than the first left, its job tables
+    and counters aside."""
+    S = [wost.Scene(scenes.config1(n_points=1)), wost.Scene(scenes.cube_scene(2, neumann_faces=(0,)))]
+
+    def batch():
+        hs = wost.wost_solve_batch([s.handle for s in S],
+                                   [dict(points=np.zeros((64, s.dim), np.float32), walks_per_point=400, epsilon=1e-3,
+                                         r_min=1e-3, max_steps=256, seed=1) for s in S])
+        for h in hs:
+            wost.wost_wait(h)
+        used = sim.sim_used()
+        for h in hs:
+            wost.wost_solve_destroy(h)
+        return used
+
+    used = batch()
+    sim.sim_limit(sim.sim_used() + (1 << 16))  # (a dimension's slots take 6 MB in the stand-in)
+    assert batch() == used
+    assert _log(sim) == ["batch 2d", "batch 3d"] * 2
+    for s in S:
+        s.close()
