@@ -157,17 +157,21 @@ cudaError_t launch_walk_count(const SceneView &sc, const SolveParams &sp, const 
 // screened solves and the other kernels use one lane per walk)
 cudaError_t persistent_grid(int dim, int block, int depth, int *blocks_out, int lanes) {
     if (lanes == WOST_WIDE) return persistent_grid_team(dim, block, depth, blocks_out);
-    // both forms run on the grid (and both are loaded before a capture)
-    int saved = 0;
-    cudaError_t e = resident_grid(dim == 2 ? (const void *)k_walk_persistent<2, false, 1, true>
-                                           : (const void *)k_walk_persistent<3, false, 1, true>,
-                                  block, depth, &saved);
-    if (e != cudaSuccess) return e;
-    e = resident_grid(dim == 2 ? (const void *)k_walk_persistent<2, false, 1, false>
-                               : (const void *)k_walk_persistent<3, false, 1, false>,
-                      block, depth, blocks_out);
-    if (e == cudaSuccess && saved < *blocks_out) *blocks_out = saved;
-    return e;
+    // every form runs on the grid (and all are loaded before a capture)
+    auto fits = [&](auto *keep, auto *hand, auto *saved) {
+        cudaError_t e = cudaSuccess;
+        *blocks_out = 0;
+        for (const void *k : {(const void *)keep, (const void *)hand, (const void *)saved}) {
+            int b = 0;
+            if (e == cudaSuccess) e = resident_grid(k, block, depth, &b);
+            if (!*blocks_out || b < *blocks_out) *blocks_out = b;
+        }
+        return e;
+    };
+    return dim == 2 ? fits(k_walk_persistent<2, false, 1, WALKS_KEEP>, k_walk_persistent<2, false, 1, WALKS_HAND_OVER>,
+                           k_walk_persistent<2, false, 1, WALKS_SAVED>)
+                    : fits(k_walk_persistent<3, false, 1, WALKS_KEEP>, k_walk_persistent<3, false, 1, WALKS_HAND_OVER>,
+                           k_walk_persistent<3, false, 1, WALKS_SAVED>);
 }
 
 cudaError_t launch_walk_persistent(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, int block,

@@ -9,8 +9,8 @@
 namespace wost {
 
 cudaError_t persistent_grid_team(int dim, int block, int depth, int *blocks_out) {
-    return resident_grid(dim == 2 ? (const void *)k_walk_persistent<2, false, WOST_WIDE, false>
-                                  : (const void *)k_walk_persistent<3, false, WOST_WIDE, false>,
+    return resident_grid(dim == 2 ? (const void *)k_walk_persistent<2, false, WOST_WIDE, WALKS_KEEP>
+                                  : (const void *)k_walk_persistent<3, false, WOST_WIDE, WALKS_KEEP>,
                          block, depth, blocks_out, WOST_WIDE);
 }
 

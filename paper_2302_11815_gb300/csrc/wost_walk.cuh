@@ -188,7 +188,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_plain(const __grid_constant__ SceneView 
 // Where the walks of this warp are to be saved: a value once nothing is left
 // to draw and at most ho.most walks are left (else ~0).  Every lane that finds
 // nothing to draw has added 1 to the counter, once, so the counter tells how
-// many hold a walk.  hand_over saves them as well, and tells if it did.
+// many hold a walk.
 template <class CTR>
 __device__ __forceinline__ unsigned hand_over_at(const HandOver &ho, const CTR *counter, unsigned long long total,
                                                  int lane, unsigned held) {
@@ -201,26 +201,27 @@ __device__ __forceinline__ unsigned hand_over_at(const HandOver &ho, const CTR *
     return __shfl_sync(0xffffffffu, first, 0);
 }
 
-template <class CTR>
-__device__ __forceinline__ bool hand_over(const HandOver &ho, const CTR *counter, unsigned long long total, int lane,
-                                          const Walk &w, bool have, unsigned held, int job) {
-    const unsigned first = hand_over_at(ho, counter, total, lane, held);
-    if (first == 0xffffffffu) return false;
-    if (have) save_walk(ho.slots + 3 * (size_t)(first + __popc(held & ((1u << lane) - 1u))), w, job);
-    return true;
-}
+// What a one-lane launch does with its walks: draws the solve's own and runs
+// them to their ends, draws them and hands the last ones over (with slots), or
+// takes saved ones up and hands the last of those over.
+enum { WALKS_KEEP, WALKS_HAND_OVER, WALKS_SAVED };
 
-// SAVED: the walks are those of src.slots.  A parameter of the template, and
-// the stores of a hand-over behind the loop, because the loop is bound by its
-// instruction supply: 1,824,000 walks in a disk of 356 segments take
-// 24.6 ms, 27.7 with both inside (25.2 without hand-over); Koch level 3, 380,000
-// walks: 162, 177 (172).
-template <int D, bool SCR, int T, bool SAVED>
+// MODE is a parameter of the template, and the stores of a hand-over are
+// behind the loop, because the loop is bound by its instruction supply:
+// 1,824,000 walks in a disk of 356 segments take 24.6 ms, 27.7 with the saved
+// walks' loads and the stores inside (25.2 without hand-over); Koch level 3,
+// 380,000 walks: 162, 177 (172).  A launch that keeps its walks (a solve with
+// given traversal limits) has nothing of it in its loop: 1,824,000 walks by a
+// crack 26.5 ms, 29.7 with the counter's check inside, Koch 325, 349 (another
+// 380,000 walks, cap 2,048).
+template <int D, bool SCR, int T, int MODE>
 __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ SceneView sc, const SolveParams sp,
                                                          const Accumulators acc, const SavedWalks src,
                                                          const HandOver ho) {
+    static_assert(T == 1 || MODE == WALKS_KEEP, "teams keep their walks");
+    constexpr bool SAVED = MODE == WALKS_SAVED;
     Cnt<false> cnt;
-    auto q = make_q<D, false, T>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, sp.coop != 0);
+    auto q = make_q<D, false, T, MODE != WALKS_KEEP>(sp.stack_depth, acc.guard, cnt, sp.visit_limit, sp.coop != 0);
     const Group g = make_team<T>();
     const uint64_t total =
         SAVED ? (uint64_t)*src.count : (uint64_t)sp.n_points * (uint64_t)sp.walks_per_point;
@@ -265,26 +266,28 @@ __global__ void WOST_WALK_BOUNDS k_walk_persistent(const __grid_constant__ Scene
                 }
             }
         }
-        held = __ballot_sync(FULL, have);
-        if (!held) {
-            if (__any_sync(FULL, !drained)) continue;
-            break;
-        }
-        if constexpr (T == 1) {
+        if constexpr (MODE == WALKS_KEEP) {
+            if (!__any_sync(FULL, have)) break;
+        } else {
+            held = __ballot_sync(FULL, have);
+            if (!held) {
+                if (__any_sync(FULL, !drained)) continue;
+                break;
+            }
             if (ho.slots) {
                 if constexpr (SAVED) first = hand_over_at(ho, src.next, total, lane, held);
                 else first = hand_over_at(ho, acc.next_walk, total, lane, held);
                 if (first != 0xffffffffu) break;
             }
+            if (src.steps_run && lane == 0) atomicAdd(src.steps_run, (unsigned long long)__popc(held));
         }
-        if (src.steps_run && lane == 0) atomicAdd(src.steps_run, (unsigned long long)__popc(held));
-        if (walk_step<D, SCR, T == 1>(sc, sp, w, q, have)) {
+        if (walk_step<D, SCR, MODE != WALKS_KEEP>(sc, sp, w, q, have)) {
             if (g.leader()) accumulate(acc, w);
             have = false;
         }
         __syncwarp();
     }
-    if constexpr (T == 1) {
+    if constexpr (MODE != WALKS_KEEP) {
         if (first != 0xffffffffu && have)
             save_walk(ho.slots + 3 * (size_t)(first + __popc(held & ((1u << lane) - 1u))), w, 0);
     }
@@ -461,28 +464,29 @@ static cudaError_t resident_grid(const void *k, int block, int depth, int *block
     return resident_blocks(k, block, smem_bytes(depth, block, lanes), blocks_out);
 }
 
-template <bool SCR, int T, bool SAVED>
+template <bool SCR, int T, int MODE>
 static cudaError_t walk_persistent_form(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                         const SavedWalks &src, const HandOver &ho, int block, int blocks, cudaStream_t s) {
     size_t sm = smem_bytes(sp.stack_depth, block, T);
-    const void *k =
-        sc.dim == 2 ? (const void *)k_walk_persistent<2, SCR, T, SAVED> : (const void *)k_walk_persistent<3, SCR, T, SAVED>;
-    cudaError_t e = smem_limit(k, sm);
-    if (e != cudaSuccess) return e;
-    if (sc.dim == 2)
-        k_walk_persistent<2, SCR, T, SAVED><<<blocks, block, sm, s>>>(sc, sp, acc, src, ho);
-    else
-        k_walk_persistent<3, SCR, T, SAVED><<<blocks, block, sm, s>>>(sc, sp, acc, src, ho);
-    return cudaGetLastError();
+    auto launch = [&](auto *k) {
+        cudaError_t e = smem_limit((const void *)k, sm);
+        if (e != cudaSuccess) return e;
+        k<<<blocks, block, sm, s>>>(sc, sp, acc, src, ho);
+        return cudaGetLastError();
+    };
+    return sc.dim == 2 ? launch(k_walk_persistent<2, SCR, T, MODE>) : launch(k_walk_persistent<3, SCR, T, MODE>);
 }
 
 template <bool SCR, int T>
 static cudaError_t walk_persistent_launch(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                           const SavedWalks &src, const HandOver &ho, int block, int blocks, cudaStream_t s) {
     if constexpr (T == 1) {
-        if (src.slots) return walk_persistent_form<SCR, T, true>(sc, sp, acc, src, ho, block, blocks, s);
+        if (src.slots) return walk_persistent_form<SCR, T, WALKS_SAVED>(sc, sp, acc, src, ho, block, blocks, s);
+        // (without slots, a solve under the scene's limits still searches jointly)
+        if (ho.slots || sp.coop)
+            return walk_persistent_form<SCR, T, WALKS_HAND_OVER>(sc, sp, acc, src, ho, block, blocks, s);
     }
-    return walk_persistent_form<SCR, T, false>(sc, sp, acc, src, ho, block, blocks, s);
+    return walk_persistent_form<SCR, T, WALKS_KEEP>(sc, sp, acc, src, ho, block, blocks, s);
 }
 
 template <bool SCR, int T>
