@@ -649,9 +649,9 @@ struct WarpQ {
         occB = false;
         // fast reciprocals: the boxes are widened by more than they, and the
         // rounding of the one-lane slab test, can move its planes: that grows
-        // with |plane - o|, so with the largest coordinate in play (a walk's
-        // origin is near the boundary, a query's anywhere)
-        const float reach = fmaxf(scale, maxabs3(o));
+        // with |plane - o|.  A walk's origin is within 3 scale of zero (it ends
+        // outside the grown bounding box), a query's is anywhere.
+        const float reach = WALK ? scale : fmaxf(scale, maxabs3(o));
         const P3 ia = mk(__fdividef(1.f, va.x), __fdividef(1.f, va.y), D == 3 ? __fdividef(1.f, va.z) : 0.f);
         P3 ib = mk(0.f, 0.f, 0.f);
         if (wantB) ib = mk(__fdividef(1.f, vb.x), __fdividef(1.f, vb.y), D == 3 ? __fdividef(1.f, vb.z) : 0.f);
