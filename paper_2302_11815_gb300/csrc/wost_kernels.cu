@@ -69,7 +69,18 @@ cudaError_t launch_request_stats(const StatJob *jobs, int n_jobs, int64_t max_po
 // 4,000 / 16,000 / 65,000 / 250,000 queries:
 //   Q.1  torus 45 43 43 53 / 49 64 128 369; Koch (1,000: 56 / 46) 54 58 / 47 70
 //   Q.2  torus 843 1110 1116 1440 / 84 111 192 540; box-sphere 314 345 365 660
-//        / 45 48 91 245 (3D: always one per warp); Koch 111 122 / 29 39
+//        / 45 48 91 245; Koch 111 122 / 29 39.  In 3D a lane is the faster one
+//        only for many queries of few candidates, whose search is short: us
+//        per call, radii up to 0.6 / the same in raster order / radii beyond the
+//        scene, one lane : one warp
+//            candidates     131,072 queries          262,144                   2,000,000
+//             56  45:54  56:54  56:70    58:95  60:94  82:128     234:638  83:626  366:891
+//            108  53:64  59:63 105:100   84:115 63:114 180:186    404:784 140:768  976:1336
+//            315  98:101 116:101 203:192 156:188 119:185 347:370  790:1332 279:1313 1884:2722
+//            336 195:113 204:108 256:184 308:208 227:202 455:354 1614:1462 728:1435 2571:2593
+//            540 229:100 241:90 324:347  370:176 275:162 576:672 2002:1201 933:1118 3350:4992
+//        (beyond 384 candidates only radii beyond the scene favour the lane,
+//        which a call does not know)
 //   Q.3  torus 81 81 111 136 / 49 61 83 179; box-sphere 43 46 46 60 / 35 41 64
 //        138; Koch 51 50 / 36 46
 //   Q.4  torus 36 38 39 56 / 32 38 70 191; Koch 35 34 / 31 39
@@ -251,17 +262,28 @@ cudaError_t launch_query_closest(const SceneView &sc, int64_t n, const float *pt
     return cudaGetLastError();
 }
 
-cudaError_t launch_query_silhouette(const SceneView &sc, int64_t n, const float *pts, const float *rmax, float *dist,
-                                    int depth, unsigned int *guard, cudaStream_t s) {
-    if (sc.dim == 3 || n <= kWarpSilhouette2D)
-        return launch_query_silhouette_warp(sc, n, pts, rmax, dist, depth, guard, s);
+cudaError_t launch_query_silhouette_lane(const SceneView &sc, int64_t n, const float *pts, const float *rmax,
+                                         float *dist, int depth, unsigned int *guard, cudaStream_t s) {
     const int block = 128;
     unsigned grid = (unsigned)((n + block - 1) / block);
     size_t sm = smem_bytes(depth, block);
-    cudaError_t e = query_smem((const void *)k_query_silhouette<2>, sm);
-    if (e != cudaSuccess) return e;
-    k_query_silhouette<2><<<grid, block, sm, s>>>(sc, n, pts, rmax, dist, depth, guard);
+    if (sc.dim == 2) {
+        cudaError_t e = query_smem((const void *)k_query_silhouette<2>, sm);
+        if (e != cudaSuccess) return e;
+        k_query_silhouette<2><<<grid, block, sm, s>>>(sc, n, pts, rmax, dist, depth, guard);
+    } else {
+        cudaError_t e = query_smem((const void *)k_query_silhouette<3>, sm);
+        if (e != cudaSuccess) return e;
+        k_query_silhouette<3><<<grid, block, sm, s>>>(sc, n, pts, rmax, dist, depth, guard);
+    }
     return cudaGetLastError();
+}
+
+cudaError_t launch_query_silhouette(const SceneView &sc, int64_t n, const float *pts, const float *rmax, float *dist,
+                                    int depth, unsigned int *guard, cudaStream_t s) {
+    return n <= warp_silhouettes(sc.dim, sc.S.n_prims)
+               ? launch_query_silhouette_warp(sc, n, pts, rmax, dist, depth, guard, s)
+               : launch_query_silhouette_lane(sc, n, pts, rmax, dist, depth, guard, s);
 }
 
 cudaError_t launch_query_ray(const SceneView &sc, int64_t n, const float *o, const float *v, const float *tmax,

@@ -71,6 +71,8 @@ cudaError_t launch_query_closest(const SceneView &sc, int64_t n, const float *pt
                                  int32_t *prim, int depth, unsigned int *guard, cudaStream_t s);
 cudaError_t launch_query_silhouette(const SceneView &sc, int64_t n, const float *pts, const float *rmax, float *dist,
                                     int depth, unsigned int *guard, cudaStream_t s);
+cudaError_t launch_query_silhouette_lane(const SceneView &sc, int64_t n, const float *pts, const float *rmax,
+                                         float *dist, int depth, unsigned int *guard, cudaStream_t s);
 cudaError_t launch_query_ray(const SceneView &sc, int64_t n, const float *o, const float *v, const float *tmax,
                              const int32_t *skip, const int32_t *rec_of_id, int64_t n_ids, int32_t *hit, float *t,
                              int32_t *prim, int depth, unsigned int *guard, cudaStream_t s);
@@ -79,8 +81,11 @@ cudaError_t launch_query_sample(const SceneView &sc, int64_t n, const float *pts
                                 cudaStream_t s);
 // one query per warp (wost_kernels_query.cu): the lines of the dispatch in
 // wost_kernels.cu, which states their measurements
-constexpr int64_t kWarpClosest = 2048, kWarpSilhouette2D = 16384, kWarpRay2D = 4096, kWarpRay3D = 16384,
-                  kWarpSample = 4096;
+constexpr int64_t kWarpClosest = 2048, kWarpRay2D = 4096, kWarpRay3D = 16384, kWarpSample = 4096;
+inline int64_t warp_silhouettes(int dim, int64_t candidates) {
+    if (dim == 2) return 16384;
+    return candidates <= 256 ? 131072 : candidates <= 384 ? 1 << 20 : INT64_MAX;
+}
 cudaError_t launch_query_closest_warp(const SceneView &sc, int64_t n, const float *pts, float *dist, float *closest,
                                       int32_t *prim, int depth, unsigned int *guard, cudaStream_t s);
 cudaError_t launch_query_silhouette_warp(const SceneView &sc, int64_t n, const float *pts, const float *rmax,
