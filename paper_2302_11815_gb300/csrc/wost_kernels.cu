@@ -201,6 +201,9 @@ cudaError_t launch_walk_persistent(const SceneView &sc, const SolveParams &sp, c
 cudaError_t launch_walk_chain(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, SavedWalks src,
                               uint64_t walks, const ChainBuffers &cb, int block, int blocks, cudaStream_t s) {
     const uint64_t resident = (uint64_t)blocks * (uint64_t)block;
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
     for (int stage = 0; stage < kMaxStages && walks > kTailWalks; ++stage) {
         const int b = stage & 1;
         const uint64_t held = std::min(walks, resident);
@@ -210,9 +213,9 @@ cudaError_t launch_walk_chain(const SceneView &sc, const SolveParams &sp, const 
         const HandOver ho{cb.slots[b], ctr, (unsigned)most, 0u};
         const uint64_t per_block = (uint64_t)(block / 32) * (src.per_warp ? src.per_warp : 32u);
         const int grid = (int)std::min<uint64_t>((uint64_t)blocks, (walks + per_block - 1) / per_block);
-        cudaError_t e = launch_walk_persistent(sc, sp, acc, block, grid, s, 1, src, ho);
+        e = launch_walk_persistent(sc, sp, acc, block, grid, s, 1, src, ho);
         if (e != cudaSuccess) return e;
-        src = SavedWalks{cb.slots[b], nullptr, ctr, ctr + 1, src.steps_run, spread_walks(sc.dim, most)};
+        src = SavedWalks{cb.slots[b], nullptr, ctr, ctr + 1, src.steps_run, spread_walks(sc.dim, most, sms)};
         walks = most;
     }
     return launch_walk_warp(sc, sp, acc, src, walks, s);

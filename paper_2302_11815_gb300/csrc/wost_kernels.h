@@ -15,13 +15,13 @@ namespace wost {
 // 2.6 / 2.4 / 2.3 / 2.6 / 3.1 ms.
 constexpr unsigned kTailWalks = 16384;
 
-// Walks per warp of a one-lane launch over `walks` saved walks.  2D: full
-// warps (a warp's step takes as long with 8 walks as with 32).  3D: spread
-// over 6 warps per SM partition, as a warp's silhouette searches run one after
-// the other (544,096 torus walks 206 -> 185 ms).
-inline unsigned spread_walks(int dim, uint64_t walks) {
+// Walks per warp of a one-lane launch over `walks` saved walks on `sms` SMs.
+// 2D: full warps (a warp's step takes as long with 8 walks as with 32).  3D:
+// spread over 6 warps per SM partition, 24 per SM, as a warp's silhouette
+// searches run one after the other (544,096 torus walks 206 -> 185 ms).
+inline unsigned spread_walks(int dim, uint64_t walks, int sms) {
     if (dim == 2) return 32u;
-    const uint64_t w = (walks + 3647) / 3648;
+    const uint64_t warps = 24u * (uint64_t)(sms > 0 ? sms : 1), w = (walks + warps - 1) / warps;
     return (unsigned)(w < 1 ? 1 : (w > 32 ? 32 : w));
 }
 

@@ -33,9 +33,8 @@ cudaError_t occupancy(int block, size_t sm, int *per_sm) {
 }  // namespace
 
 cudaError_t batch_grid(int dim, int block, int depth, int *blocks_out) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0, per_sm = 0;
+    cudaError_t e = sm_count(&sms);
     const size_t sm = smem_bytes(depth, block);
     if (e == cudaSuccess) e = dim == 2 ? occupancy<2>(block, sm, &per_sm) : occupancy<3>(block, sm, &per_sm);
     // the warp kernels that end a batch are loaded now, not while a graph is captured
@@ -71,6 +70,9 @@ cudaError_t launch_walk_batch(int dim, const BatchHeader *hdr, const BatchJob *j
     SavedWalks src{};
     const uint64_t resident = (uint64_t)blocks * (uint64_t)block;
     uint64_t walks = ~0ull;
+    int sms = 0;
+    cudaError_t e = sm_count(&sms);
+    if (e != cudaSuccess) return e;
     for (int stage = 0; stage < kMaxStages && walks > kTailWalks; ++stage) {
         const int b = stage & 1;
         const uint64_t held = std::min(walks, resident);
@@ -83,8 +85,7 @@ cudaError_t launch_walk_batch(int dim, const BatchHeader *hdr, const BatchJob *j
             walks == ~0ull ? blocks : (int)std::min<uint64_t>((uint64_t)blocks, (walks + per_block - 1) / per_block);
         if (!cb.slots[b]) most = 0;  // (no memory: this launch runs its walks to their ends)
         const HandOver ho{cb.slots[b], ctr, (unsigned)most, (unsigned)grid * (unsigned)per_block};
-        cudaError_t e =
-            dim == 2 ? (screened ? launch<2, true>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
+        e = dim == 2 ? (screened ? launch<2, true>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
                                                    src, ho)
                                  : launch<2, false>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
                                                     src, ho))
@@ -93,7 +94,7 @@ cudaError_t launch_walk_batch(int dim, const BatchHeader *hdr, const BatchJob *j
                                  : launch<3, false>(hdr, jobs, counter, guard, depth, cancel, block, grid, s, steps_out,
                                                     src, ho));
         if (e != cudaSuccess || !cb.slots[b]) return e;
-        src = SavedWalks{cb.slots[b], nullptr, ctr, ctr + 1, nullptr, spread_walks(dim, most)};
+        src = SavedWalks{cb.slots[b], nullptr, ctr, ctr + 1, nullptr, spread_walks(dim, most, sms)};
         walks = most;
     }
     return launch_walk_warp_batch(dim, hdr, jobs, guard, depth, src, steps_out, screened, s);

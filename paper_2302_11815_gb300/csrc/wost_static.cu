@@ -29,7 +29,10 @@ namespace wost {
 //             then the chain's two slot arrays (48 bytes a slot)
 constexpr size_t kHeader = 256;
 constexpr size_t kArray = 8 * (size_t)WOST_STATIC_MAX_POINTS;
-constexpr unsigned kSlots0 = 20480, kSlots1 = kTailWalks;
+// The first array only has to hold more than one launch of one walk per warp
+// takes up (a chain's first hand-over waits until so many walks are left):
+// 1.7 MB for both, where wost_solve's slots, half the grid, take 5.6 MB.
+constexpr unsigned kSlots0 = kTailWalks + kTailWalks / 4, kSlots1 = kTailWalks;
 constexpr size_t kSlotBytes = 3 * sizeof(float4);
 constexpr size_t kScratchBytes = kHeader + 4 * kArray + (kSlots0 + kSlots1) * kSlotBytes;
 static_assert(32 + 2 * kMaxStages * sizeof(unsigned int) <= kHeader, "hand-over counters fit the header");

@@ -448,12 +448,18 @@ static cudaError_t walk_count_launch(const SceneView &sc, const SolveParams &sp,
     return cudaGetLastError();
 }
 
+// SMs of the current device
+static cudaError_t sm_count(int *sms) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    return e;
+}
 // resident blocks of kernel k per SM times the SM count, its shared-memory
 // limit set
 static cudaError_t resident_blocks(const void *k, int block, size_t sm, int *blocks_out) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int sms = 0, per_sm = 0;
+    cudaError_t e = sm_count(&sms);
     if (e == cudaSuccess) e = smem_limit(k, sm);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, sm);
     if (e != cudaSuccess) return e;
