@@ -86,6 +86,16 @@ inline int64_t warp_silhouettes(int dim, int64_t candidates) {
     if (dim == 2) return 16384;
     return candidates <= 256 ? 131072 : candidates <= 384 ? 1 << 20 : INT64_MAX;
 }
+// A launch of one warp per query takes this many at most (two warps per block:
+// its grid stays below 2^31 blocks); a larger array is asked in parts,
+// f(first query, how many).
+constexpr int64_t kWarpQueries = (int64_t)1 << 31;
+template <class F>
+inline cudaError_t in_parts(int64_t n, int64_t most, F f) {
+    cudaError_t e = cudaSuccess;
+    for (int64_t at = 0; at < n && e == cudaSuccess; at += most) e = f(at, n - at < most ? n - at : most);
+    return e;
+}
 cudaError_t launch_query_closest_warp(const SceneView &sc, int64_t n, const float *pts, float *dist, float *closest,
                                       int32_t *prim, int depth, unsigned int *guard, cudaStream_t s);
 cudaError_t launch_query_silhouette_warp(const SceneView &sc, int64_t n, const float *pts, const float *rmax,

@@ -109,15 +109,14 @@ cudaError_t launch_query_closest_warp(const SceneView &sc, int64_t n, const floa
     return cudaGetLastError();
 }
 
+// (the only one that large arrays take, in 3D)
 cudaError_t launch_query_silhouette_warp(const SceneView &sc, int64_t n, const float *pts, const float *rmax,
                                          float *dist, int depth, unsigned int *guard, cudaStream_t s) {
-    if (sc.dim == 2)
-        k_query_silhouette_warp<2><<<warps_grid(n), kBlock, warps_smem(depth), s>>>(sc, n, pts, rmax, dist, depth,
-                                                                                    guard);
-    else
-        k_query_silhouette_warp<3><<<warps_grid(n), kBlock, warps_smem(depth), s>>>(sc, n, pts, rmax, dist, depth,
-                                                                                    guard);
-    return cudaGetLastError();
+    return in_parts(n, kWarpQueries, [&](int64_t at, int64_t m) {
+        const auto k = sc.dim == 2 ? k_query_silhouette_warp<2> : k_query_silhouette_warp<3>;
+        k<<<warps_grid(m), kBlock, warps_smem(depth), s>>>(sc, m, pts + at * sc.dim, rmax + at, dist + at, depth, guard);
+        return cudaGetLastError();
+    });
 }
 
 cudaError_t launch_query_ray_warp(const SceneView &sc, int64_t n, const float *o, const float *v, const float *tmax,
