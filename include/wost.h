@@ -477,17 +477,19 @@ typedef struct {
     int32_t tried_lanes[8];
 } wost_tune_result;
 
-/* Times the walk loop in steady state -- the resumable kernel, one launch
- * of 256 steps per lane to fill the lanes, then two timed launches (walk
- * steps executed over device time) -- on an evenly strided sample of the
- * caller's points (device pointer, n points, at most 65,536 used) at
- * walks_per_point (0: 32), for each layout -- one lane per walk over the
- * binary trees, 8-lane teams over the 8-wide trees -- and block sizes
- * 64..256 (8 combinations), and keeps the fastest block size as the
- * scene's default for persistent, batched and engine launches whose
- * block_size is 0, and the fastest layout as its default for persistent and
- * resumable Poisson solves whose lanes_per_walk is 0 (wost_scene_info then
- * reports that layout).  Same validation as wost_solve. */
+/* Times the walk loop on an evenly strided sample of the caller's points
+ * (device pointer, n points, at most 65,536 used) at walks_per_point (0: 32),
+ * for each layout -- one lane per walk over the binary trees, 8-lane teams
+ * over the 8-wide trees -- and block sizes 64..256 (8 combinations): in steady
+ * state (the resumable kernel, one launch of 256 steps per lane to fill the
+ * lanes, then two timed launches: walk steps executed over device time) if
+ * the sample's walks last so long on one lane each, else as whole persistent
+ * solves of the sample.  Keeps the fastest block size as the scene's default
+ * for persistent, batched and engine launches whose block_size is 0, and the
+ * fastest layout as its default for persistent and resumable Poisson solves
+ * whose lanes_per_walk is 0 (wost_scene_info then reports that layout;
+ * persistent solves of at most 16,384 walks run one walk per warp whatever it
+ * is).  Same validation as wost_solve. */
 wost_status wost_scene_autotune(wost_scene *scene, const float *points, int64_t n, int32_t walks_per_point,
                                 float epsilon, float r_min, int32_t max_steps, wost_tune_result *out);
 

@@ -389,7 +389,11 @@ wost_status wost::prepare_solve(wost_scene *scene, const wost_solve_desc *d, cud
     const bool team_ok = (d->kernel == WOST_KERNEL_PERSISTENT || d->kernel == WOST_KERNEL_RESUMABLE) && !(d->sigma > 0);
     if (d->lanes_per_walk == WOST_WIDE && !team_ok)
         return fail(WOST_ERR_INVALID_ARG, "8 lanes per walk: persistent or resumable Poisson solves only");
-    const int lanes = d->lanes_per_walk ? d->lanes_per_walk : (team_ok ? scene->tuned_lanes : 1);
+    // (a persistent solve of so few walks runs one per warp, whatever layout
+    // was the fastest with the lanes full: 8 lanes take 2 to 3 times as long)
+    const bool small = d->kernel == WOST_KERNEL_PERSISTENT && !d->stack_depth && !d->visit_limit &&
+                       (uint64_t)d->n_points * (uint64_t)d->walks_per_point <= kTailWalks;
+    const int lanes = d->lanes_per_walk ? d->lanes_per_walk : (team_ok && !small ? scene->tuned_lanes : 1);
     CK(cudaSetDevice(scene->device), "cudaSetDevice");
     h->scene = scene;
     h->device = scene->device;
@@ -1097,8 +1101,26 @@ wost_status wost_scene_autotune(wost_scene *scene, const float *points, int64_t 
         std::unique_ptr<CUevent_st, cudaError_t (*)(cudaEvent_t)> k0(e0, cudaEventDestroy), k1(e1, cudaEventDestroy);
         const int blocks[4] = {64, 128, 192, 256};
         const int iters = 256;  // walk steps per lane per launch
-        double best = -1;
-        for (int ci = 0; ci < 8; ++ci) {
+        const uint64_t total = (uint64_t)m * (uint64_t)(walks > 0 ? walks : 32);
+        // Steady state first: one launch of the resumable kernel fills every
+        // lane with a walk, the next two are timed (walk steps executed over
+        // their device time).  A sample whose walks do not last that long on
+        // one lane each is timed again as the whole persistent solves that
+        // its user would run, every combination to its last walk: what the
+        // draining launches show is the longest walks' latency, where 8 lanes
+        // look fast and a solve, which ends in one walk per warp, does not
+        // need them (a keyhole, 64 x 96 walks: 3.6e7 against 9.8e6 steps/s
+        // while draining, 45 against 22 ms for the solve).
+        bool whole = false, drained = false;
+        for (int ci = 0; ci < 8 || (drained && !whole); ++ci) {
+            if (ci == 8) {
+                whole = true;
+                ci = 0;
+            }
+            if (ci == 0) {
+                out->n_tried = 0;
+                out->steps_per_second = -1;
+            }
             const int bi = ci % 4, lanes = ci < 4 ? 1 : WOST_WIDE;
             wost_solve_desc d{};
             d.lanes_per_walk = lanes;
@@ -1110,36 +1132,45 @@ wost_status wost_scene_autotune(wost_scene *scene, const float *points, int64_t 
             d.r_min = r_min;
             d.max_steps = max_steps;
             d.seed = 0x5EED0000u;
-            d.kernel = WOST_KERNEL_RESUMABLE;
+            d.kernel = whole ? WOST_KERNEL_PERSISTENT : WOST_KERNEL_RESUMABLE;
             d.block_size = blocks[bi];
-            // steady state of the resumable kernel: one launch fills every
-            // lane with a walk, the next two are timed (walk steps executed
-            // over their device time); a sample too small to keep the lanes
-            // busy is timed as it drains, which is then its real regime
             wost_solve_handle *h = nullptr;
             wost_status st = wost_solve(scene, &d, &h);
             if (st != WOST_OK) return st;
             std::unique_ptr<wost_solve_handle, wost_status (*)(wost_solve_handle *)> hk(h, wost_solve_destroy);
-            const cudaStream_t s = h->stream;
-            unsigned long long before = 0, after = 0;
-            if ((st = wost_solve_advance(h, iters, nullptr)) != WOST_OK) return st;
-            CK(cudaStreamSynchronize(s), "cudaStreamSynchronize");
-            CK(cudaMemcpy(&before, h->rstate.p, sizeof before, cudaMemcpyDeviceToHost), "copy steps");
-            CK(cudaEventRecord(e0, s), "cudaEventRecord");
-            for (int rep = 0; rep < 2; ++rep)
+            double steps = 0, seconds = 0;
+            if (whole) {
+                wost_progress pr;
+                if ((st = wost_wait(h, -1)) != WOST_OK) return st;
+                if ((st = wost_poll(h, nullptr, nullptr, nullptr, &pr)) != WOST_OK) return st;
+                steps = (double)pr.total_steps;
+                seconds = pr.elapsed_seconds;
+            } else {
+                const cudaStream_t s = h->stream;
+                unsigned long long before = 0, after = 0, drawn = 0;
                 if ((st = wost_solve_advance(h, iters, nullptr)) != WOST_OK) return st;
-            CK(cudaEventRecord(e1, s), "cudaEventRecord");
-            CK(cudaEventSynchronize(e1), "cudaEventSynchronize");
-            CK(cudaMemcpy(&after, h->rstate.p, sizeof after, cudaMemcpyDeviceToHost), "copy steps");
-            float ms = 0;
-            CK(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
-            const double rate = ms > 0 ? (double)(after - before) / (ms * 1e-3) : 0;
+                CK(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+                CK(cudaMemcpy(&before, h->rstate.p, sizeof before, cudaMemcpyDeviceToHost), "copy steps");
+                CK(cudaEventRecord(e0, s), "cudaEventRecord");
+                for (int rep = 0; rep < 2; ++rep)
+                    if ((st = wost_solve_advance(h, iters, nullptr)) != WOST_OK) return st;
+                CK(cudaEventRecord(e1, s), "cudaEventRecord");
+                CK(cudaEventSynchronize(e1), "cudaEventSynchronize");
+                CK(cudaMemcpy(&after, h->rstate.p, sizeof after, cudaMemcpyDeviceToHost), "copy steps");
+                CK(cudaMemcpy(&drawn, (unsigned long long *)h->globals.p + 1, sizeof drawn, cudaMemcpyDeviceToHost),
+                   "copy counter");
+                float ms = 0;
+                CK(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
+                steps = (double)(after - before);
+                seconds = ms * 1e-3;
+                drained = drained || (lanes == 1 && drawn >= total);
+            }
+            const double rate = seconds > 0 ? steps / seconds : 0;
             out->tried_block[out->n_tried] = blocks[bi];
             out->tried_lanes[out->n_tried] = lanes;
             out->tried_steps_per_second[out->n_tried] = rate;
             out->n_tried++;
-            if (rate > best) {
-                best = rate;
+            if (rate > out->steps_per_second) {
                 out->block_size = blocks[bi];
                 out->lanes_per_walk = lanes;
                 out->steps_per_second = rate;

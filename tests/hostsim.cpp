@@ -60,6 +60,7 @@ void sim_reset(size_t limit) {
     sim.log.clear();
 }
 void sim_limit(size_t n) { sim.limit = n; }
+void sim_to_go(int n) { sim.to_go = n; }
 void sim_hold(int on) { sim.hold = on != 0; }
 size_t sim_used(void) { return sim.used; }
 int sim_bad(void) { return sim.bad; }
@@ -183,21 +184,25 @@ cudaError_t launch_walk_batch(int dim, const BatchHeader *, const BatchJob *, un
 cudaError_t launch_walk_persistent(const SceneView &, const SolveParams &sp, const Accumulators &acc, int, int,
                                    cudaStream_t s, int lanes, const SavedWalks &, const HandOver &) {
     *acc.next_walk = all_walks(sp);
+    *acc.steps = lanes == 1 ? 1000 : 500;
     return launch(lanes == 1 ? "persistent" : "persistent, 8 lanes", s);
 }
 cudaError_t launch_walk_warp(const SceneView &, const SolveParams &sp, const Accumulators &acc, const SavedWalks &,
                              uint64_t, cudaStream_t s) {
     *acc.next_walk = all_walks(sp);
+    *acc.steps = 1000;
     return launch("one per warp", s);
 }
 cudaError_t launch_walk_chain(const SceneView &, const SolveParams &sp, const Accumulators &acc, SavedWalks src,
                               uint64_t, const ChainBuffers &, int, int, cudaStream_t s) {
     *acc.next_walk = all_walks(sp);
+    *acc.steps = 1000;
     return launch(src.slots ? "chain from saved walks" : "chain", s);
 }
 cudaError_t launch_walk_resume(const SceneView &, const SolveParams &sp, const Accumulators &acc, const ResumeState &rs,
-                               int iters, int, int, cudaStream_t s, int) {
+                               int iters, int, int, cudaStream_t s, int lanes) {
     const uint64_t total = all_walks(sp);
+    *rs.steps_run += lanes == 1 ? 500 : 1000;  // 8 lanes look faster per launch, a whole solve is not
     --sim.to_go;
     *acc.next_walk = sim.to_go > 0 ? total / 2 : total;
     *rs.live = sim.to_go >= 0 ? 5 : 0;

@@ -184,3 +184,39 @@ def test_a_batch_keeps_its_slots_for_the_next_one(sim):
     assert _log(sim) == ["batch 2d", "batch 3d"] * 2
     for s in S:
         s.close()
+
+
+def _tune(sim, S, n, walks, to_go):
+    """wost_scene_autotune (the stand-in's device memory is host memory)."""
+    pts = np.zeros((n, S.dim), np.float32)
+    r = wost.wost_tune_result()
+    sim.sim_to_go(to_go)
+    assert sim.wost_scene_autotune(S.handle, pts.ctypes.data, n, walks, 1e-3, 1e-3, 256, C.byref(r)) == 0
+    assert r.n_tried == 8 and list(r.tried_lanes) == [1] * 4 + [8] * 4
+    assert S.info()["lanes_per_walk"] == r.lanes_per_walk
+    return r
+
+
+def test_tuner_times_what_a_solve_runs(sim):
+    """A sample whose walks do not last the timed launches is timed as whole
+    solves (the stand-in's 8 lanes are twice as fast per launch and half as
+    fast for a solve)."""
+    S = wost.Scene(scenes.config1(n_points=1))
+    r = _tune(sim, S, 64, 400, 1)
+    assert r.lanes_per_walk == 1 and _log(sim)[-8:] == ["chain"] * 4 + ["persistent, 8 lanes"] * 4
+    assert r.steps_per_second == max(r.tried_steps_per_second) > 0
+    sim.sim_reset(1 << 40)
+    r = _tune(sim, S, 64, 400, 10**6)
+    assert r.lanes_per_walk == 8 and _log(sim) == ["resume 256"] * 24
+    S.close()
+
+
+def test_small_solves_of_a_scene_tuned_to_teams_run_one_walk_per_warp(sim):
+    S = wost.Scene(scenes.config1(n_points=1))
+    assert _tune(sim, S, 64, 400, 10**6).lanes_per_walk == 8
+    for walks, kw, want in [(256, {}, "one per warp"), (257, {}, "persistent, 8 lanes"),
+                            (256, dict(lanes_per_walk=8), "persistent, 8 lanes"),
+                            (256, dict(stack_depth=9), "persistent, 8 lanes")]:
+        wost.wost_solve_destroy(_solve(S, 64, walks, **kw))
+        assert _log(sim)[-1] == want, (walks, kw)
+    S.close()
