@@ -281,6 +281,8 @@ struct wost_solve_handle {
     wost_status final_status = WOST_OK;                    // engine requests
     std::mutex mu;
     ~wost_solve_handle() {
+        // a resumable solve drops the walks it has not drawn
+        if (resumable() && !done && cancel_host) *(volatile int *)cancel_host = 1;
         // (a stream of the caller's is used only by a call that failed before
         // its event was recorded: the caller may have destroyed it since)
         if (ev_done && launches) cudaEventSynchronize(ev_done);

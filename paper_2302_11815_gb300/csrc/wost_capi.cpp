@@ -874,11 +874,27 @@ static wost_status advance_locked(wost_solve_handle *h, int iters, cudaStream_t 
     return WOST_OK;
 }
 
-// The next launch of a resumable solve while its caller waits: bounded as
-// wost_solve_advance's or, when every remaining walk is still to be drawn or
-// none is, the chain of launches that runs them all to their ends (caller
-// holds h->mu; the previous launch has completed).
-static wost_status advance_waiting(wost_solve_handle *h) {
+// May a chain over `walks` walks start with `left` more seconds to wait
+// (negative: no limit)?  Nothing but cancelling stops it, and then the walks
+// its lanes hold still run to their ends, which is what destroy and other work
+// have to wait for after a timeout: so only if that takes a quarter of the time
+// left at most, or the whole chain ends within it.  Both with every walk
+// at the step cap: 50 us per step of the last walks (measured 3 to 11) and
+// 1e8 walk steps/s with the lanes full (the lowest rate measured, 212,288
+// triangles in 3D, is 1.05e8), a fifth of it for the whole.
+static bool chain_in_time(const wost_solve_handle *h, uint64_t walks, double left) {
+    if (left < 0) return true;
+    const double steps = h->sp.max_steps,
+                 held = (double)std::min(walks, (uint64_t)resume_slots(h->block, h->resume_blocks, 1));
+    return steps * (50e-6 + held / 1e8) <= 0.25 * left || steps * (50e-6 + (double)walks / 2e7) <= left;
+}
+
+// The next launch of a resumable solve while its caller waits (for `left` more
+// seconds, negative: no limit): bounded as wost_solve_advance's or, when every
+// remaining walk is still to be drawn or none is, the chain of launches that
+// runs them all to their ends (caller holds h->mu; the previous launch has
+// completed).
+static wost_status advance_waiting(wost_solve_handle *h, double left) {
     if (h->lanes != 1 || !h->warp_ok) return advance_locked(h, 2048, h->stream);
     unsigned long long *steps_run = (unsigned long long *)h->rstate.p;
     unsigned int *ctr = (unsigned int *)((char *)h->rstate.p + 8);
@@ -894,6 +910,7 @@ static wost_status advance_waiting(wost_solve_handle *h) {
         src = SavedWalks{(float4 *)h->slots.p, ctr + 2, ctr, ctr + 1, steps_run, 0};
         walks = live;
     }
+    if (!chain_in_time(h, walks, left)) return advance_locked(h, 2048, h->stream);
     ChainBuffers cb{};
     const cudaError_t ce = chain_buffers(h, walks, h->resume_blocks, &cb);
     if (ce == cudaErrorMemoryAllocation) {  // no memory to hand walks over in
@@ -933,6 +950,7 @@ wost_status wost_wait(wost_solve_handle *h, double timeout_s) {
     CK(cudaSetDevice(h->device), "cudaSetDevice");
     auto t0 = std::chrono::steady_clock::now();
     for (;;) {
+        double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         {
             std::lock_guard<std::mutex> lk(h->mu);
             wost_status st = check_done(h);
@@ -941,9 +959,10 @@ wost_status wost_wait(wost_solve_handle *h, double timeout_s) {
             // a resumable solve advances while its caller waits: the next
             // launch as soon as the previous one has completed
             if (h->resumable() && (h->launches == 0 || cudaEventQuery(h->ev_done) == cudaSuccess))
-                if ((st = advance_waiting(h)) != WOST_OK) return st;
+                if ((st = advance_waiting(h, timeout_s < 0 ? -1.0 : std::max(0.0, timeout_s - el))) != WOST_OK)
+                    return st;
         }
-        double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
+        el = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         if (timeout_s >= 0 && el >= timeout_s) return fail(WOST_ERR_TIMEOUT, "solve not finished");
         // (a sleep takes ~70 us at least: short solves are polled)
         if (el < 0.001) std::this_thread::yield();

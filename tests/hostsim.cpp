@@ -27,6 +27,7 @@ struct Sim {
     bool hold = false;  // launches stay in flight (their events are not ready)
     bool launched = false;
     int to_go = 3;      // launches after which a resumable solve has no walk left to draw; one more ends it
+    const int *cancel = nullptr;  // the last launch's cancel flag
     std::string log;
 } sim;
 
@@ -131,7 +132,10 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
     return use(s);
 }
 cudaError_t cudaEventQuery(cudaEvent_t e) { return sim.hold && e->pending ? cudaErrorNotReady : cudaSuccess; }
-cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t e) {
+    if (sim.hold && e->pending) sim.log += sim.cancel && *sim.cancel ? "waiting, cancelled\n" : "waiting\n";
+    return cudaSuccess;
+}
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) {
     *ms = 1.f;
     return cudaSuccess;
@@ -197,11 +201,13 @@ cudaError_t launch_walk_chain(const SceneView &, const SolveParams &sp, const Ac
                               uint64_t, const ChainBuffers &, int, int, cudaStream_t s) {
     *acc.next_walk = all_walks(sp);
     *acc.steps = 1000;
+    sim.cancel = acc.cancel;
     return launch(src.slots ? "chain from saved walks" : "chain", s);
 }
 cudaError_t launch_walk_resume(const SceneView &, const SolveParams &sp, const Accumulators &acc, const ResumeState &rs,
                                int iters, int, int, cudaStream_t s, int lanes) {
     const uint64_t total = all_walks(sp);
+    sim.cancel = acc.cancel;
     *rs.steps_run += lanes == 1 ? 500 : 1000;  // 8 lanes look faster per launch, a whole solve is not
     --sim.to_go;
     *acc.next_walk = sim.to_go > 0 ? total / 2 : total;

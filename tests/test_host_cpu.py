@@ -220,3 +220,63 @@ def test_small_solves_of_a_scene_tuned_to_teams_run_one_walk_per_warp(sim):
         wost.wost_solve_destroy(_solve(S, 64, walks, **kw))
         assert _log(sim)[-1] == want, (walks, kw)
     S.close()
+
+
+def _resumable(S, cap, walks=4):
+    return wost.wost_solve(S.handle, np.zeros((64, S.dim), np.float32), walks, 1e-3, 1e-3, cap, 1, 0, "resumable")
+
+
+@pytest.mark.parametrize("cap,walks,limit,want", [
+    # no limit: the chain of launches that runs every walk to its end
+    (256, 4, -1.0, ["chain"]),
+    (1 << 20, 4, -1.0, ["chain"]),
+    # the whole chain ends within the limit whatever the walks do (0.02, 66 s)
+    (256, 4, 0.5, ["chain"]),
+    (1 << 20, 4, 100.0, ["chain"]),
+    # it does not (862 s), but the walks that the stand-in's 2,048 lanes hold
+    # end within a quarter of the limit (4.6 s)
+    (1 << 16, 4096, 30.0, ["chain"]),
+    # ... or does not: bounded launches until all are drawn, then the last
+    # five's chain, which ends in 3.3 s
+    (1 << 16, 4096, 10.0, ["resume 2048"] * 3 + ["chain from saved walks"]),
+    (1 << 16, 4096, 3.0, ["resume 2048"] * 4),
+    (1 << 20, 4, 5.0, ["resume 2048"] * 4),
+])
+def test_a_limited_wait_starts_no_chain_that_outlasts_it(sim, cap, walks, limit, want):
+    S = wost.Scene(scenes.config1(n_points=1))
+    h = _resumable(S, cap, walks)
+    wost.wost_wait(h, limit)
+    assert _log(sim) == want
+    wost.wost_solve_destroy(h)
+    S.close()
+
+
+@pytest.mark.parametrize("cap,limit,launched", [(1 << 16, 0.02, "resume 2048"), (256, 0.1, "chain")])
+def test_destroying_after_a_timeout_drops_the_walks_not_drawn(sim, cap, limit, launched):
+    S = wost.Scene(scenes.config1(n_points=1))
+    h = _resumable(S, cap)
+    sim.sim_hold(1)  # launches stay in flight
+    with pytest.raises(wost.WostError) as e:
+        wost.wost_wait(h, limit)
+    assert e.value.status == wost.ERR_TIMEOUT
+    assert _log(sim) == [launched]
+    wost.wost_solve_destroy(h)
+    assert _log(sim) == [launched, "waiting, cancelled"]
+    sim.sim_hold(0)
+    h = _resumable(S, 256)  # the next solve has the set's flag cleared
+    wost.wost_wait(h)
+    wost.wost_solve_destroy(h)
+    S.close()
+
+
+def test_an_advanced_solve_ends_in_the_chain_over_its_saved_walks(sim):
+    S = wost.Scene(scenes.config1(n_points=1))
+    for limit in (-1.0, 5.0):
+        sim.sim_reset(1 << 40)
+        h = _resumable(S, 256)
+        for _ in range(3):  # (the stand-in's third launch draws the last walk)
+            wost.wost_solve_advance(h, 7)
+        wost.wost_wait(h, limit)
+        assert _log(sim) == ["resume 7"] * 3 + ["chain from saved walks"]
+        wost.wost_solve_destroy(h)
+    S.close()
