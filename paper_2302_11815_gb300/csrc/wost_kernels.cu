@@ -194,6 +194,11 @@ cudaError_t launch_walk_persistent(const SceneView &sc, const SolveParams &sp, c
     return walk_persistent_launch<false, 1>(sc, sp, acc, src, h, block, blocks, s);
 }
 
+cudaError_t load_chain_kernels(int dim, bool screened) {
+    cudaError_t e = screened ? load_chain_kernels_scr(dim) : load_persistent_forms<false>(dim);
+    return e == cudaSuccess ? load_walk_warp(dim, screened) : e;
+}
+
 // Lane kernels that pass the remaining walks on to one another, then the
 // warp kernel.  A warp of one-lane walks takes 35 us per step (Koch) whether
 // 32 or 8 of its lanes still hold a walk, so once half of the walks of a
@@ -203,6 +208,7 @@ cudaError_t launch_walk_chain(const SceneView &sc, const SolveParams &sp, const 
     const uint64_t resident = (uint64_t)blocks * (uint64_t)block;
     int sms = 0;
     cudaError_t e = sm_count(&sms);
+    if (e == cudaSuccess && walks > kTailWalks) e = load_chain_kernels(sc.dim, sp.sigma > 0.f);
     if (e != cudaSuccess) return e;
     for (int stage = 0; stage < kMaxStages && walks > kTailWalks; ++stage) {
         const int b = stage & 1;

@@ -57,6 +57,10 @@ cudaError_t launch_walk_warp(const SceneView &sc, const SolveParams &sp, const A
 // (block, blocks: the persistent kernel's resident grid)
 cudaError_t launch_walk_chain(const SceneView &sc, const SolveParams &sp, const Accumulators &acc, SavedWalks src,
                               uint64_t walks, const ChainBuffers &cb, int block, int blocks, cudaStream_t s);
+// Loads every kernel of a chain.  The runtime loads a kernel when it is first
+// used, and waits for the device then: the first chain of a process would not
+// return before its first launch has ended.
+cudaError_t load_chain_kernels(int dim, bool screened);
 // slots that the chain's slot array `which` (0, 1) has to hold
 uint64_t chain_capacity(uint64_t walks, int block, int blocks, int which);
 // resumable solves: grid of the fixed launch, its walk slots, one launch

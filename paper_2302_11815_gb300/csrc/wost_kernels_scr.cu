@@ -45,6 +45,7 @@ cudaError_t launch_walk_persistent_scr(const SceneView &sc, const SolveParams &s
                                        cudaStream_t s) {
     return walk_persistent_launch<true, 1>(sc, sp, acc, src, ho, block, blocks, s);
 }
+cudaError_t load_chain_kernels_scr(int dim) { return load_persistent_forms<true>(dim); }
 cudaError_t launch_walk_resume_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                    const ResumeState &rs, int iters, int block, int blocks, cudaStream_t s) {
     return walk_resume_launch<true, 1>(sc, sp, acc, rs, iters, block, blocks, s);

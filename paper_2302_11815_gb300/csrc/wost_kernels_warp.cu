@@ -12,6 +12,10 @@ cudaError_t launch_walk_warp(const SceneView &sc, const SolveParams &sp, const A
     return walk_warp_launch<false>(sc, sp, acc, src, walks, s);
 }
 
+cudaError_t load_walk_warp(int dim, bool screened) {
+    return screened ? load_walk_warp_scr(dim) : walk_warp_load<false>(dim);
+}
+
 cudaError_t launch_walk_warp_batch(int dim, const BatchHeader *hdr, const BatchJob *jobs, unsigned int *guard, int depth,
                                    const SavedWalks &src, unsigned long long *steps_out, bool screened,
                                    cudaStream_t s) {

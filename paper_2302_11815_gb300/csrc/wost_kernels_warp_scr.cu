@@ -11,6 +11,8 @@ cudaError_t launch_walk_warp_scr(const SceneView &sc, const SolveParams &sp, con
     return walk_warp_launch<true>(sc, sp, acc, src, walks, s);
 }
 
+cudaError_t load_walk_warp_scr(int dim) { return walk_warp_load<true>(dim); }
+
 cudaError_t launch_walk_warp_batch_scr(int dim, const BatchHeader *hdr, const BatchJob *jobs, unsigned int *guard,
                                        int depth, const SavedWalks &src, unsigned long long *steps_out,
                                        cudaStream_t s) {

@@ -495,6 +495,18 @@ static cudaError_t walk_persistent_launch(const SceneView &sc, const SolveParams
     return walk_persistent_form<SCR, T, WALKS_KEEP>(sc, sp, acc, src, ho, block, blocks, s);
 }
 
+// loads the forms that a chain runs (load_chain_kernels)
+template <bool SCR>
+static cudaError_t load_persistent_forms(int dim) {
+    cudaFuncAttributes a;
+    auto load = [&](auto *hand, auto *saved) {
+        cudaError_t e = cudaFuncGetAttributes(&a, (const void *)hand);
+        return e == cudaSuccess ? cudaFuncGetAttributes(&a, (const void *)saved) : e;
+    };
+    return dim == 2 ? load(k_walk_persistent<2, SCR, 1, WALKS_HAND_OVER>, k_walk_persistent<2, SCR, 1, WALKS_SAVED>)
+                    : load(k_walk_persistent<3, SCR, 1, WALKS_HAND_OVER>, k_walk_persistent<3, SCR, 1, WALKS_SAVED>);
+}
+
 template <bool SCR, int T>
 static cudaError_t walk_resume_launch(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                       const ResumeState &rs, int iters, int block, int blocks, cudaStream_t s) {
@@ -516,6 +528,9 @@ cudaError_t launch_walk_count_scr(const SceneView &sc, const SolveParams &sp, co
                                   unsigned long long *stats, int block, cudaStream_t s);
 cudaError_t launch_walk_persistent_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                        const SavedWalks &src, const HandOver &ho, int block, int blocks, cudaStream_t s);
+cudaError_t load_chain_kernels_scr(int dim);
+cudaError_t load_walk_warp(int dim, bool screened);
+cudaError_t load_walk_warp_scr(int dim);
 cudaError_t launch_walk_warp_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                  const SavedWalks &src, uint64_t walks, cudaStream_t s);
 cudaError_t launch_walk_resume_scr(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,

@@ -146,6 +146,12 @@ static cudaError_t walk_warp_launch_d(const SceneView &sc, const SolveParams &sp
 }
 
 template <bool SCR>
+static cudaError_t walk_warp_load(int dim) {
+    cudaFuncAttributes a;
+    return cudaFuncGetAttributes(&a, dim == 2 ? (const void *)k_walk_warp<2, SCR> : (const void *)k_walk_warp<3, SCR>);
+}
+
+template <bool SCR>
 static cudaError_t walk_warp_launch(const SceneView &sc, const SolveParams &sp, const Accumulators &acc,
                                     const SavedWalks &src, uint64_t walks, cudaStream_t s) {
     return sc.dim == 2 ? walk_warp_launch_d<2, SCR>(sc, sp, acc, src, walks, s)
