@@ -620,6 +620,14 @@ wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_so
             stream = shared->own_stream;
         }
         std::vector<std::unique_ptr<wost_solve_handle>> hs(n);
+        // a failure after the 3D launch: its stream may not be joined into the
+        // caller's yet, which is all that the solves wait for
+        struct SideJoin {
+            BatchShared *b;
+            ~SideJoin() {
+                if (b && b->side) cudaStreamSynchronize(b->side);
+            }
+        } unjoined{shared.get()};
         int block = descs[0].block_size ? descs[0].block_size
                                         : (scenes[0]->tuned_block ? scenes[0]->tuned_block : 128);
         for (int32_t i = 0; i < n; ++i) {
@@ -714,6 +722,7 @@ wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_so
             CK(cudaStreamWaitEvent(stream, shared->ev_join, 0), "cudaStreamWaitEvent");
         }
         CK(cudaEventRecord(shared->ev_done, stream), "cudaEventRecord");
+        unjoined.b = nullptr;
         for (int32_t i = 0; i < n; ++i) {
             hs[i]->batch = shared;
             hs[i]->ev_start = shared->ev_start;

@@ -8,11 +8,13 @@
 #include <cstring>
 #include <map>
 #include <string>
+#include <vector>
 
 #include "capi_internal.h"
 
 struct CUstream_st {
     bool alive = true;
+    bool busy = false;  // launched on, not waited for since
 };
 struct CUevent_st {
     bool pending = false;
@@ -26,6 +28,8 @@ struct Sim {
     int bad = 0;        // uses of a destroyed stream
     bool hold = false;  // launches stay in flight (their events are not ready)
     bool launched = false;
+    int fail_record = 0;  // the cudaEventRecord that fails, counted from now on (0: none)
+    std::vector<cudaStream_t> streams;
     int to_go = 3;      // launches after which a resumable solve has no walk left to draw; one more ends it
     const int *cancel = nullptr;  // the last launch's cancel flag
     std::string log;
@@ -38,6 +42,7 @@ cudaError_t use(cudaStream_t s) {
 cudaError_t launch(const std::string &what, cudaStream_t s) {
     sim.log += what + "\n";
     sim.launched = true;
+    if (s) s->busy = true;
     return use(s);
 }
 cudaError_t get(void **p, size_t n) {
@@ -57,6 +62,7 @@ void sim_reset(size_t limit) {
     sim.limit = limit;
     sim.bad = 0;
     sim.hold = sim.launched = false;
+    for (cudaStream_t s : sim.streams) s->busy = false;
     sim.to_go = 3;
     sim.log.clear();
 }
@@ -64,6 +70,12 @@ void sim_limit(size_t n) { sim.limit = n; }
 void sim_to_go(int n) { sim.to_go = n; }
 void sim_hold(int on) { sim.hold = on != 0; }
 size_t sim_used(void) { return sim.used; }
+void sim_fail_record(int n) { sim.fail_record = n; }
+int sim_busy(void) {
+    int n = 0;
+    for (cudaStream_t s : sim.streams) n += s->busy;
+    return n;
+}
 int sim_bad(void) { return sim.bad; }
 const char *sim_log(void) { return sim.log.c_str(); }
 
@@ -105,6 +117,7 @@ cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t st) {
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
     *s = new CUstream_st;
+    sim.streams.push_back(*s);
     return cudaSuccess;
 }
 cudaError_t cudaStreamDestroy(cudaStream_t s) {  // (kept, so that later uses are seen)
@@ -112,7 +125,10 @@ cudaError_t cudaStreamDestroy(cudaStream_t s) {  // (kept, so that later uses ar
     s->alive = false;
     return cudaSuccess;
 }
-cudaError_t cudaStreamSynchronize(cudaStream_t s) { return use(s); }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+    if (s) s->busy = false;
+    return use(s);
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t, unsigned) { return use(s); }
 cudaError_t cudaDeviceSynchronize(void) {
     sim.log += "device synchronised\n";
@@ -128,6 +144,7 @@ cudaError_t cudaEventDestroy(cudaEvent_t e) {
     return cudaSuccess;
 }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
+    if (sim.fail_record > 0 && --sim.fail_record == 0) return cudaErrorUnknown;
     e->pending = sim.launched;
     return use(s);
 }

@@ -280,3 +280,20 @@ def test_an_advanced_solve_ends_in_the_chain_over_its_saved_walks(sim):
         assert _log(sim) == ["resume 7"] * 3 + ["chain from saved walks"]
         wost.wost_solve_destroy(h)
     S.close()
+
+
+@pytest.mark.parametrize("failing", [1, 2, 3, 4, 5])
+def test_a_batch_that_fails_leaves_nothing_in_flight(sim, failing):
+    """Its solves' memory goes back at once: both launches, on the call's
+    stream and on the 3D one's, have to be over.  (Records of the call: copies,
+    start, fork, join, end.)"""
+    S = [wost.Scene(scenes.config1(n_points=1)), wost.Scene(scenes.cube_scene(2, neumann_faces=(0,)))]
+    req = [dict(points=np.zeros((64, s.dim), np.float32), walks_per_point=400, epsilon=1e-3, r_min=1e-3, max_steps=256,
+                seed=1) for s in S]
+    sim.sim_fail_record(failing)
+    with pytest.raises(wost.WostError):
+        wost.wost_solve_batch([s.handle for s in S], req)
+    assert _log(sim) == (["batch 2d", "batch 3d"] if failing > 3 else [])
+    assert sim.sim_busy() == 0
+    for s in S:
+        s.close()
