@@ -185,9 +185,15 @@ typedef enum {
 } wost_memory;
 
 typedef enum {
+    /* Plain and persistent solves of at most 16,384 walks run one walk per
+     * warp in one launch (block_size has no effect there), unless the solve
+     * gives stack_depth or visit_limit or asks for 8 lanes per walk.          */
     WOST_KERNEL_PLAIN = 0,      /* one thread per walk, one launch             */
     WOST_KERNEL_PERSISTENT = 1, /* persistent lanes that regenerate finished
-                                   walks from a work counter                   */
+                                   walks from a work counter; the last walks
+                                   go through up to eight more launches that
+                                   pack them together, the last of which runs
+                                   one walk per warp                           */
     WOST_KERNEL_COUNTING = 2,   /* the plain kernel plus per-query work
                                    counters (see wost_solve_work_counts)       */
     WOST_KERNEL_RESUMABLE = 3   /* persistent lanes over a fixed grid, run as a
@@ -225,12 +231,18 @@ typedef struct {
                                   no traversal exceeds).  A smaller value saves
                                   shared memory but a traversal that needs more
                                   drops subtrees and sets guard bit 1, making
-                                  wost_wait / wost_poll return INTERNAL       */
+                                  wost_wait / wost_poll return INTERNAL.  With
+                                  any value given (the scene's own too), and
+                                  with a visit_limit, every traversal is one
+                                  lane's: no walk runs per warp, which can take
+                                  several times as long                       */
     int32_t visit_limit;       /* node visits allowed per traversal, 0 = twice
                                   the tree's nodes plus 8 (more than a correct
                                   traversal makes).  A traversal that reaches
                                   the limit stops and sets guard bit 2        */
-    int32_t lanes_per_walk;    /* 1: one lane per walk over the binary trees;
+    int32_t lanes_per_walk;    /* 1: one lane per walk over the binary trees
+                                  (the last walks, or few of them: one warp
+                                  each, the same walks);
                                   8: a team of 8 lanes per walk over the 8-wide
                                   trees (persistent and resumable Poisson
                                   solves); 0: the scene's choice (set by
@@ -248,7 +260,8 @@ typedef struct {
     uint64_t steps_run;        /* resumable solves: walk steps executed by the
                                   completed launches, finished walks or not;
                                   other kernels: total_steps                   */
-    uint64_t launches;         /* kernel launches of this solve so far          */
+    uint64_t launches;         /* launches of this solve so far (the launches that
+                                  hand walks over to one another count as one) */
 } wost_progress;
 
 /* Starts a solve asynchronously on the stream and returns its handle.
@@ -281,13 +294,16 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *desc, wost_solv
 wost_status wost_solve_advance(wost_solve_handle *solve, int32_t iterations, void *stream);
 
 /* Batching: starts n solves (any scenes of one device, any point counts, walk
- * counts and parameters) in ONE persistent launch per dimension present (2D
- * jobs and 3D jobs run in separate launches, back to back on the stream).
- * Lanes take walks from a shared counter across all jobs, so uneven walk
- * lengths do not idle the GPU.  out[i] (n handles) behaves like a handle from
- * wost_solve; all of them complete together.  descs[i].kernel and block_size
- * are taken from descs[0] (the counting kernel is not allowed here).
- * Errors as for wost_solve; on error no handle is returned. */
+ * counts and parameters) in one persistent launch per dimension present, whose
+ * last walks go through up to eight more, the last with one walk per warp (2D
+ * and 3D jobs run concurrently: the 3D ones on a stream of the library, forked
+ * from and joined into the caller's).  Lanes take walks from a shared counter
+ * across all jobs, so uneven walk lengths do not idle the GPU.  The scenes' own
+ * traversal limits apply, whatever descs[i] gives.  out[i] (n handles) behaves
+ * like a handle from wost_solve; all of them complete together.
+ * descs[i].kernel and block_size are taken from descs[0] (the counting kernel
+ * is not allowed here).  Errors as for wost_solve; on error no handle is
+ * returned. */
 wost_status wost_solve_batch(int32_t n, wost_scene *const *scenes, const wost_solve_desc *descs, void *stream,
                              wost_solve_handle **out);
 

@@ -1,10 +1,12 @@
 // Q.1-Q.4 with one query per warp: for arrays of so few queries that one lane
 // per query leaves most of the GPU idle and waits for the slowest lane's chain
-// of node visits, and for silhouettes in 3D, whose chains are the longest.
-// Bound by the latency of a warp's rounds (few queries) or by instruction issue
-// (many: 2.2 ns per silhouette query around the torus, one lane 5.8).  The
-// answers are those of the one-lane query kernels (wost_kernels.cu), record
-// for record; four queries over 1,000 Koch points 277 -> 128 us.
+// of node visits, and for silhouettes in 3D unless the candidates are few
+// (warp_silhouettes), as their chains are the longest.  Bound by the latency of
+// a warp's rounds (few queries) or by instruction issue (many: 250,000 raster
+// points of a plane by the torus take 0.7 to 3 ns each, by plane; on the plane
+// of the table in wost_kernels.cu 2.2, one lane each 5.8).  The answers are
+// those of the one-lane query kernels (wost_kernels.cu), record for record;
+// four queries over 1,000 Koch points 277 -> 128 us.
 #include <cuda_runtime.h>
 
 #include "wost_walk_warp.cuh"
