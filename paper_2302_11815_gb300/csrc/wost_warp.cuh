@@ -676,7 +676,7 @@ struct WarpQ {
                 else occ_maybe = true;
             }
         };
-        bool ok = !axis && reach < INFINITY;
+        bool ok = !axis && (WALK || reach < INFINITY);
         if (ok)
             ok = search(
                 T, kBrute,
