@@ -35,14 +35,13 @@ __device__ __forceinline__ void init_job_walk(const BatchJob &J, unsigned long l
 // src, ho: walks taken up from (SAVED), and handed over to, another launch (a
 // saved walk keeps its job index).  As in k_walk_persistent, the loop is bound
 // by its instruction supply, so SAVED is a parameter of the template and the
-// stores of a hand-over are behind the loop, and the counter is read by a warp
-// that has itself found nothing to draw, and else every eighth step of lane 0's
-// walk.  Device time of one scene of 3,800 points x 480 walks (Koch level 3: x
-// 100; torus of 18,750 candidates: 17,003 x 32), ms, without hand-over / all of
-// it in the loop, every step / as it is: disk of 356 segments 27.9 / 30.2 / 28.2,
-// flower 9.75 / 10.5 / 10.1, annulus 37.2 / 32.2 / 30.3, crack 26.8 / 18.1 /
-// 17.4, Koch 356 / 341 / 334, torus 146 / 83 / 80.  Read only after a failed
-// draw, 12 mixed scenes with long walks take 358 ms instead of 255.
+// stores of a hand-over are behind the loop.  Device time of one scene of 3,800
+// points x 480 walks (Koch level 3: x 100; torus of 18,750 candidates: 17,003 x
+// 32), ms, without hand-over / all of it in the loop / as it is: disk of 356
+// segments 27.9 / 30.0 / 28.5, flower 9.75 / 10.4 / 10.1, annulus 37.2 / 32.0 /
+// 30.8, crack 26.8 / 18.1 / 17.4, Koch 356 / 339 / 331, torus 146 / 82 / 80.
+// The counter is read on every step: with every fourth to eighth the disk takes
+// 28.0, but serving rounds hand over late (six requests 39.8 -> 41 to 42 ms).
 template <int D, bool SCR, bool SAVED>
 __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hdr,
                                                     const BatchJob *__restrict__ jobs, unsigned long long *counter,
@@ -101,8 +100,7 @@ __global__ void WOST_WALK_BOUNDS k_walk_batch(const BatchHeader *__restrict__ hd
             if (__any_sync(FULL, !drained)) continue;
             break;
         }
-        // (a warp whose walks are all long finds nothing to draw late)
-        if (ho.slots && __any_sync(FULL, drained || (lane == 0 && (w.steps & 7) == 0))) {
+        if (ho.slots) {
             if constexpr (SAVED) first = hand_over_at(ho, src.next, total, lane, held);
             else first = hand_over_at(ho, counter, total, lane, held);
             if (first != 0xffffffffu) break;
