@@ -284,10 +284,10 @@ wost_status wost_solve(wost_scene *scene, const wost_solve_desc *desc, wost_solv
  * on a resumable solve issues the launches itself until every walk has
  * finished: of 2048 iterations each while a solve already advanced has walks
  * left to draw, else launches that run to the walks' ends.  With a time limit
- * the latter run only if they end within it, or if the walks that the lanes
- * hold end within a quarter of it once the solve is cancelled or destroyed,
- * every walk taken to reach max_steps; else launches of 2048 iterations, one of
- * which is in flight at most when the wait times out.  wost_solve_destroy drops
+ * the latter run only if max_steps is at most 2048, or if they end within it, or
+ * if the walks that the lanes hold end within a quarter of it once the solve is
+ * cancelled or destroyed, every walk taken to reach max_steps; else launches of
+ * 2048 iterations, one of which is in flight at most when the wait times out.  wost_solve_destroy drops
  * the walks not drawn yet.  The walks and estimates are those of the other
  * kernels for the same seed.  Errors: INVALID_ARG (not a resumable solve,
  * iterations < 1), CUDA. */

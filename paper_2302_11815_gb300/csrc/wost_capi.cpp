@@ -890,9 +890,12 @@ static wost_status advance_locked(wost_solve_handle *h, int iters, cudaStream_t 
 // left at most, or the whole chain ends within it.  Both with every walk
 // at the step cap: 50 us per step of the last walks (measured 3 to 11) and
 // 1e8 walk steps/s with the lanes full (the lowest rate measured, 212,288
-// triangles in 3D, is 1.05e8), a fifth of it for the whole.
+// triangles in 3D, is 1.05e8), a fifth of it for the whole.  Walks of at most
+// kBounded steps end within a bounded launch as well, so there is nothing to
+// wait for beyond that.
+constexpr int kBounded = 2048;  // iterations of a waiting solve's bounded launch
 static bool chain_in_time(const wost_solve_handle *h, uint64_t walks, double left) {
-    if (left < 0) return true;
+    if (left < 0 || h->sp.max_steps <= kBounded) return true;
     const double steps = h->sp.max_steps,
                  held = (double)std::min(walks, (uint64_t)resume_slots(h->block, h->resume_blocks, 1));
     return steps * (50e-6 + held / 1e8) <= 0.25 * left || steps * (50e-6 + (double)walks / 2e7) <= left;
@@ -904,7 +907,7 @@ static bool chain_in_time(const wost_solve_handle *h, uint64_t walks, double lef
 // runs them all to their ends (caller holds h->mu; the previous launch has
 // completed).
 static wost_status advance_waiting(wost_solve_handle *h, double left) {
-    if (h->lanes != 1 || !h->warp_ok) return advance_locked(h, 2048, h->stream);
+    if (h->lanes != 1 || !h->warp_ok) return advance_locked(h, kBounded, h->stream);
     unsigned long long *steps_run = (unsigned long long *)h->rstate.p;
     unsigned int *ctr = (unsigned int *)((char *)h->rstate.p + 8);
     SavedWalks src{nullptr, nullptr, nullptr, nullptr, steps_run, 0};
@@ -915,16 +918,16 @@ static wost_status advance_waiting(wost_solve_handle *h, double left) {
         wost_status st = resumable_finished(h, &fin, &drained, &live);
         if (st != WOST_OK || fin) return st;
         if (!drained || live > (uint64_t)resume_slots(h->block, h->resume_blocks, 1))
-            return advance_locked(h, 2048, h->stream);
+            return advance_locked(h, kBounded, h->stream);
         src = SavedWalks{(float4 *)h->slots.p, ctr + 2, ctr, ctr + 1, steps_run, 0};
         walks = live;
     }
-    if (!chain_in_time(h, walks, left)) return advance_locked(h, 2048, h->stream);
+    if (!chain_in_time(h, walks, left)) return advance_locked(h, kBounded, h->stream);
     ChainBuffers cb{};
     const cudaError_t ce = chain_buffers(h, walks, h->resume_blocks, &cb);
     if (ce == cudaErrorMemoryAllocation) {  // no memory to hand walks over in
         cudaGetLastError();
-        return advance_locked(h, 2048, h->stream);
+        return advance_locked(h, kBounded, h->stream);
     }
     CK(ce, "cudaMalloc slots");
     h->idle = false;

@@ -241,6 +241,9 @@ def _resumable(S, cap, walks=4):
     (1 << 16, 4096, 10.0, ["resume 2048"] * 3 + ["chain from saved walks"]),
     (1 << 16, 4096, 3.0, ["resume 2048"] * 4),
     (1 << 20, 4, 5.0, ["resume 2048"] * 4),
+    # a bounded launch would run such walks to their ends as well
+    (2048, 4096, 0.1, ["chain"]),
+    (2049, 4096, 0.1, ["resume 2048"] * 4),
 ])
 def test_a_limited_wait_starts_no_chain_that_outlasts_it(sim, cap, walks, limit, want):
     S = wost.Scene(scenes.config1(n_points=1))
