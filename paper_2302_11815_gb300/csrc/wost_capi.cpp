@@ -9,6 +9,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <list>
 #include <memory>
 #include <mutex>
 #include <new>
@@ -35,21 +36,21 @@ wost_status cuda_fail(cudaError_t e, const char *what) {
 
 namespace {
 struct IdleSet {
-    SolvePool *pool;
+    SolvePool *pool = nullptr;
     std::unique_ptr<SolveRes> res;
 };
 struct IdleSets {
     std::mutex mu;
-    std::vector<IdleSet> sets;  // oldest first
-    // moves the sets that `which` names to `out` (to be freed without the lock)
+    std::list<IdleSet> sets;  // oldest first
+    // moves the sets that `which` names to `out` (to be freed without the
+    // lock); allocates nothing, as destructors come here
     template <class F>
-    void move_out(F which, std::vector<IdleSet> &out) {
-        size_t kept = 0;
-        for (IdleSet &q : sets) {
-            if (which(q)) out.push_back(std::move(q));
-            else if (IdleSet &to = sets[kept++]; &to != &q) to = std::move(q);
+    void move_out(F which, std::list<IdleSet> &out) {
+        for (auto q = sets.begin(); q != sets.end();) {
+            const auto next = std::next(q);
+            if (which(*q)) out.splice(out.end(), sets, q);
+            q = next;
         }
-        sets.erase(sets.begin() + (std::ptrdiff_t)kept, sets.end());
     }
 };
 // (never destroyed: at exit the CUDA runtime may be gone before it)
@@ -63,10 +64,10 @@ cudaError_t SolvePool::take(std::unique_ptr<SolveRes> &out) {
     {
         IdleSets &all = idle_sets();
         std::lock_guard<std::mutex> lk(all.mu);
-        for (size_t i = all.sets.size(); i-- > 0;) {
-            if (all.sets[i].pool != this) continue;
-            out = std::move(all.sets[i].res);
-            all.sets.erase(all.sets.begin() + (std::ptrdiff_t)i);
+        for (auto q = all.sets.end(); q != all.sets.begin();) {  // the latest first
+            if ((--q)->pool != this) continue;
+            out = std::move(q->res);
+            all.sets.erase(q);
             return cudaSuccess;
         }
     }
@@ -80,7 +81,12 @@ cudaError_t SolvePool::take(std::unique_ptr<SolveRes> &out) {
 
 void SolvePool::give(std::unique_ptr<SolveRes> r) {
     if (r->bytes() > kIdleBytes) return;
-    std::vector<IdleSet> gone;
+    std::list<IdleSet> one, gone;
+    try {
+        one.emplace_back();
+    } catch (const std::bad_alloc &) {
+        return;
+    }
     IdleSets &all = idle_sets();
     std::lock_guard<std::mutex> lk(all.mu);
     size_t mine = 0, bytes = r->bytes();
@@ -96,11 +102,13 @@ void SolvePool::give(std::unique_ptr<SolveRes> r) {
             return true;
         },
         gone);
-    all.sets.push_back(IdleSet{this, std::move(r)});
+    one.front().pool = this;
+    one.front().res = std::move(r);
+    all.sets.splice(all.sets.end(), one);
 }
 
 void SolvePool::close() {
-    std::vector<IdleSet> gone;
+    std::list<IdleSet> gone;
     IdleSets &all = idle_sets();
     std::lock_guard<std::mutex> lk(all.mu);
     closed = true;
@@ -108,7 +116,7 @@ void SolvePool::close() {
 }
 
 size_t drop_idle(int device) {
-    std::vector<IdleSet> gone;
+    std::list<IdleSet> gone;
     {
         IdleSets &all = idle_sets();
         std::lock_guard<std::mutex> lk(all.mu);

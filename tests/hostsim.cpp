@@ -7,6 +7,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <map>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -19,6 +20,16 @@ struct CUstream_st {
 struct CUevent_st {
     bool pending = false;
 };
+
+// host allocations of the library, refused on demand
+static bool refuse_new = false;
+void *operator new(size_t n) {
+    void *p = refuse_new ? nullptr : std::malloc(n ? n : 1);
+    if (!p) throw std::bad_alloc();
+    return p;
+}
+void operator delete(void *p) noexcept { std::free(p); }
+void operator delete(void *p, size_t) noexcept { std::free(p); }
 
 namespace {
 
@@ -68,6 +79,7 @@ void sim_reset(size_t limit) {
 }
 void sim_limit(size_t n) { sim.limit = n; }
 void sim_to_go(int n) { sim.to_go = n; }
+void sim_refuse_new(int on) { refuse_new = on != 0; }
 void sim_hold(int on) { sim.hold = on != 0; }
 size_t sim_used(void) { return sim.used; }
 void sim_fail_record(int n) { sim.fail_record = n; }

@@ -300,3 +300,28 @@ def test_a_batch_that_fails_leaves_nothing_in_flight(sim, failing):
     assert sim.sim_busy() == 0
     for s in S:
         s.close()
+
+
+def test_destroying_without_host_memory_gives_the_resources_up(sim):
+    """Nothing that destroy does may throw: a set that cannot be kept is freed
+    (in a child process, which would be aborted)."""
+    used = sim.sim_used()
+    S = wost.Scene(scenes.config1(n_points=1))
+    T = wost.Scene(scenes.config1(n_points=1))
+    _finished(S, 64)
+    h = _solve(T)
+    wost.wost_wait(h)
+    pid = os.fork()
+    if pid == 0:
+        code = 1
+        try:
+            sim.sim_refuse_new(1)
+            ok = sim.wost_solve_destroy(h) == 0 and sim.wost_scene_destroy(S.handle) == 0
+            ok = ok and sim.wost_scene_destroy(T.handle) == 0 and sim.sim_used() == used
+            code = 0 if ok else 2
+        finally:
+            os._exit(code)
+    assert os.waitpid(pid, 0)[1] == 0
+    wost.wost_solve_destroy(h)
+    S.close()
+    T.close()
