@@ -86,6 +86,25 @@ def test_static_solves_with_several_hand_overs(wost, name, n, walks):
     S.close()
 
 
+def test_static_solves_in_a_graph(wost):
+    """Captured after a first call of another size, replayed on other points."""
+    S = wost.Scene(SCENES["flower"]())
+    a, b = (torch.from_numpy(_points("flower", 3000, s)).cuda() for s in (1, 2))
+    pts, mean = a.clone(), torch.empty(3000, device="cuda")
+    wost.wost_solve_static(S.handle, pts[:10].contiguous(), 4, 1e-3, 1e-3, 900, 6, 0, mean)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        wost.wost_solve_static(S.handle, pts, 64, 1e-3, 1e-3, 900, 6, 0, mean, stream=torch.cuda.current_stream())
+    for x in (a, b, a):
+        pts.copy_(x)
+        graph.replay()
+        torch.cuda.synchronize()
+        ref = _one_lane(wost, S, x, 64, 900, 6)
+        np.testing.assert_array_equal(mean.cpu().numpy(), ref["mean"].astype(np.float32))
+    S.close()
+
+
 @pytest.mark.parametrize("kernel", ["persistent", "resumable"])
 def test_cancelling_while_a_chain_runs(wost, kernel):
     S = wost.Scene(scenes.config2(grid=8, level=4))
